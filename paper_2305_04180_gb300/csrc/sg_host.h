@@ -14,7 +14,7 @@ struct sg_sim {
   sg::DevCfg dc;
   int n_maps = 0;
   int device = 0;
-  int step_epw = 0;  // envs per warp of k_step (0 = not chosen yet)
+  int sms = 1;       // multiprocessors of the device
   long long atlas_words = 0;
   long long clr_bytes = 0;
   std::vector<sg::MapDesc> maps_host;
@@ -34,6 +34,9 @@ struct sg_sim {
   int persistent_blocks = 0;
   int* order_dev = nullptr;      // work list (cost-sorted env indices) or null
   int* map_order_dev = nullptr;  // env indices grouped by map (stable), for per-CTA map locality
+  int* rank_dev = nullptr;       // position of each env in map_order_dev (two-kernel step)
+  sg::MotionRec* step_rec = nullptr;  // records between the two kernels of a step (null: one kernel)
+  sg::Discs* step_discs = nullptr;  // disc centres of those records (dynamic obstacles)
   unsigned* queue_dev = nullptr; // work-list cursor of the persistent kernel
   unsigned* pipe_sync_dev = nullptr;  // time-sliced pipelined rollout: segment flags, item counter, abort word
   size_t pipe_sync_words = 0;

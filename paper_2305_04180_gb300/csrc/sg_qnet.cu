@@ -1190,8 +1190,10 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       for (int e = 0; e < nv; ++e) {
         const StepScanRec& r = rec[row0 + e];
         float b0, b1;
-        scan_env(c, p, p.maps[r.map], r.nb, r.stepb, r.ax, r.ay, r.aphi, r.asigma,
-                 ((uint64_t)r.anhi << 32) | r.anlo, lane, b0, b1);
+        if (c.scan_fast)
+          scan_rec<false, true>(c, p, r, false, lane, b0, b1);
+        else
+          scan_rec<false, false>(c, p, r, false, lane, b0, b1);
         qt_obs_to_tile(hx, row0 + e, b0, b1, lane < 5 ? r.exa[lane] : 0.0f, B, lane);
         if (use_replay) {
           const long long sl = (long long)((rbase + (unsigned long long)s0) % (unsigned long long)rp.slots);
@@ -1332,10 +1334,9 @@ __global__ void __launch_bounds__(kQtThreads, 1)
         const StepScanRec& r = rec[e];
         const int ie = r.env;
         const uint32_t de = r.done;
-        const MapDesc m = p.maps[r.map];
         float b0, b1;
-        const float mn = scan_env(c, p, m, r.nb, r.stepb, r.ax, r.ay, r.aphi, r.asigma,
-                                  ((uint64_t)r.anhi << 32) | r.anlo, lane, b0, b1);
+        const float mn = c.scan_fast ? scan_rec<false, true>(c, p, r, false, lane, b0, b1)
+                                     : scan_rec<false, false>(c, p, r, false, lane, b0, b1);
         const float rw = (de & 1u) ? -10.0f : (de & 2u) ? 75.0f : reward_finish(c, r.rpart, mn);
         const uint32_t ae = act_sh[e];
         if (use_replay) {
@@ -1351,8 +1352,10 @@ __global__ void __launch_bounds__(kQtThreads, 1)
         if (lane == 0 && rew_seq) rew_seq[(long long)t * n + ie] = rw;
         const float* ex = r.exa;
         if (de) {
-          scan_env(c, p, m, r.nb, r.stepb, r.bx, r.by, r.bphi, r.bsigma, ((uint64_t)r.bnhi << 32) | r.bnlo, lane,
-                   b0, b1);
+          if (c.scan_fast)
+            scan_rec<false, true>(c, p, r, true, lane, b0, b1);
+          else
+            scan_rec<false, false>(c, p, r, true, lane, b0, b1);
           ex = r.exb;
         }
         // the observation t + 1: the next tile row, the outputs, the next ring entry's s

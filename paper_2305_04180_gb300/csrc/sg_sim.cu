@@ -162,77 +162,73 @@ __global__ void __launch_bounds__(128) k_reset(const __grid_constant__ DevCfg c,
   if (kDyn && lane < c.n_dyn) store_obst(p, lane, env, b);
 }
 
-// One vectorized step of every env (sg_sim_step).  A warp takes kE
-// envs (consecutive in the env order grouped by map): its lanes 0.. run the
-// scalar part of the step for one env each (lane_step: state load, delay,
-// Eq. 5, Eq. 6, collision, arrival, truncation, AutoReset draws and the
-// scan-free terms of the observation and of Eq. 11, into shared records),
-// then the whole warp scans each of its envs (lane j marches beam j): the
-// post-motion state always (the observation, or the terminal observation and
-// the reward of a done env), the reset state of a done env.  No warp waits on
-// another.  Every value is the one-env-per-warp step's, in the same float32
-// expressions.  kE envs per warp (6, 7 or 8; the host takes the count whose
-// grid fills its last wave of resident CTAs best: at 65,536 envs 7, 70.8 us
-// per launch, against 72.7 us with 8 and 77 us with 6; 4 per warp 75 us, 16
-// per warp 75 us; 4 or 16 warps per CTA instead of 8 slower).
+// One vectorized step of every env (sg_sim_step), small batches: one kernel.
+// A warp takes kE envs (consecutive in the env order grouped by map): its
+// lanes 0 .. kE - 1 run lane_motion for one env each into shared records,
+// then the whole warp finishes each of its envs (finish_step: lane j marches
+// beam j).  No warp waits on another.  Bound by the latency of one env's
+// chain (state, map, skip values), so kE = 1 while the warps fit the GPU: 16
+// envs took 24.3 us a step when a warp always took 6 to 8, 6.4 us now; 4,096
+// envs 26 and 14 us.
 constexpr int kStepWarps = 8;
 
-// Disc centres of an env for its two scans (dynamic obstacles only).
-struct DiscRec {
-  Discs a, b;
-};
-
-template <bool kDyn, int kE>
-__global__ void __launch_bounds__(32 * kStepWarps, 4) k_step(const __grid_constant__ DevCfg c, SimPtrs p,
+template <bool kDyn, bool kFast, int kE>
+__global__ void __launch_bounds__(32 * kStepWarps, kFast ? 3 : 4) k_step(const __grid_constant__ DevCfg c, SimPtrs p,
                                                              const int* __restrict__ order,
                                                              const uint8_t* __restrict__ act,
                                                              float* __restrict__ obs, float* __restrict__ rew,
                                                              uint8_t* __restrict__ done, float* __restrict__ term) {
-  __shared__ StepScanRec rec[kStepWarps][kE];
-  __shared__ DiscRec drec[kDyn ? kStepWarps : 1][kDyn ? kE : 1];
+  __shared__ MotionRec rec[kStepWarps][kE];
+  __shared__ Discs drec[kDyn ? kStepWarps : 1][kDyn ? kE : 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int base = (blockIdx.x * kStepWarps + warp) * kE;
+  const int base = (blockIdx.x * (blockDim.x >> 5) + warp) * kE;
   if (base >= c.n_envs) return;  // warp-uniform
   const int nv = min(kE, c.n_envs - base);
-  const bool live = lane < nv;
-  const int i = live ? order[base + lane] : 0;
-  Env s;
-  if (live) s = load_env(p, i);
-  // lanes past the warp's envs take part in the warp-wide collision tests only
-  DiscRec* dr = kDyn ? &drec[warp][live ? lane : 0] : nullptr;
-  const uint32_t d = lane_step<kDyn>(c, p, i, live, s, live ? (uint32_t)act[i] : 0u, rec[warp][live ? lane : 0],
-                                     lane, kDyn ? &dr->a : nullptr, kDyn ? &dr->b : nullptr);
-  if (live) {
+  if (lane < nv) {
+    const int i = order[base + lane];
+    Env s = load_env(p, i);
+    lane_motion<kDyn>(c, p, i, s, (uint32_t)act[i], &rec[warp][lane], kDyn ? &drec[warp][lane] : nullptr);
     store_env(p, i, s);
-    done[i] = (uint8_t)d;
   }
   __syncwarp();
-  for (int e = 0; e < nv; ++e) {
-    const StepScanRec& r = rec[warp][e];
-    const int ie = r.env;
-    const MapDesc m = p.maps[r.map];
-    const uint32_t de = r.done;
-    float b0, b1;
-    const DiscRec* de_ = kDyn ? &drec[warp][e] : nullptr;
-    const float mn = scan_env<kDyn, true>(c, p, m, r.nb, r.stepb, r.ax, r.ay, r.aphi, r.asigma,
-                                    ((uint64_t)r.anhi << 32) | r.anlo, lane, b0, b1, kDyn ? &de_->a : nullptr);
-    float rw;
-    if (de & 1u)
-      rw = -10.0f;
-    else if (de & 2u)
-      rw = 75.0f;
-    else
-      rw = reward_finish(c, r.rpart, mn);
-    if (!de) {
-      write_row(obs + (long long)ie * c.obs_dim, b0, b1, r.exa, c.B, lane);
-    } else {
-      if (term) write_row(term + (long long)ie * c.obs_dim, b0, b1, r.exa, c.B, lane);
-      scan_env<kDyn, true>(c, p, m, r.nb, r.stepb, r.bx, r.by, r.bphi, r.bsigma, ((uint64_t)r.bnhi << 32) | r.bnlo, lane,
-                     b0, b1, kDyn ? &de_->b : nullptr);
-      write_row(obs + (long long)ie * c.obs_dim, b0, b1, r.exb, c.B, lane);
-    }
-    if (lane == 0) rew[ie] = rw;
-  }
+#pragma unroll 1
+  for (int e = 0; e < nv; ++e)
+    finish_step<kDyn, kFast, false>(c, p, &rec[warp][e], kDyn ? &drec[warp][e] : nullptr, lane, obs, rew, done, term);
+}
+
+// Large batches: lane_motion with 32 envs per warp (index order: coalesced
+// state), its records in the map-grouped order in global memory (rank[i]: an
+// env's place), and finish_step in a second kernel, whose scans need half of
+// the registers (40 against 78) and so keep 48 warps on an SM.  In one kernel
+// the scalar part ran on 7 of 32 lanes, 130 of 545 warp instructions an
+// env-step.  65,536 envs: 68.1 -> 43.5 us a step, 16,384 envs: 30.4 -> 19.3 us.
+// The second kernel waits on the latency of the march's loads (L2): 4 warps a
+// CTA and one record a warp keep the warp slots full (8 warps or 2 records:
+// 47-49 us); 36 registers spill (57 us).
+template <bool kDyn>
+__global__ void __launch_bounds__(64) k_step_motion(const __grid_constant__ DevCfg c, SimPtrs p,
+                                                    const int* __restrict__ rank, const uint8_t* __restrict__ act,
+                                                    MotionRec* __restrict__ rec, Discs* __restrict__ drec) {
+  pdl_launch_dependents();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= c.n_envs) return;
+  const int at = rank[i];
+  Env s = load_env(p, i);
+  lane_motion<kDyn>(c, p, i, s, (uint32_t)act[i], rec + at, kDyn ? drec + at : nullptr);
+  store_env(p, i, s);
+}
+
+constexpr int kFinishWarps = 4;
+template <bool kDyn>
+__global__ void __launch_bounds__(32 * kFinishWarps, kDyn ? 8 : 12)
+    k_step_finish(const __grid_constant__ DevCfg c, SimPtrs p, const MotionRec* __restrict__ rec,
+                  const Discs* __restrict__ drec, float* __restrict__ obs, float* __restrict__ rew,
+                  uint8_t* __restrict__ done, float* __restrict__ term) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int e = blockIdx.x * kFinishWarps + warp;
+  pdl_wait();
+  if (e < c.n_envs)
+    finish_step<kDyn, true, true>(c, p, rec + e, kDyn ? drec + e : nullptr, lane, obs, rew, done, term);
 }
 
 // K steps of one env with uniformly random actions drawn on the device; the
@@ -365,7 +361,7 @@ struct __align__(16) ObsRec {
   float px, py, pphi;      // pre-reset state (truncated steps)
   float psigma;
   uint32_t pnlo, pnhi;
-  uint32_t pad;
+  uint32_t k0;             // scan_start of the state observed | of the pre-reset state << 8 (0: outside the map)
 };
 static_assert(sizeof(ObsRec) == 80, "observation record is five 16-byte words");
 
@@ -374,8 +370,13 @@ __device__ __forceinline__ uint64_t noise_key(const EnvConst& k, const Env& s) {
 }
 
 // Lane j: record j of the chunk from its step record.
+__device__ __forceinline__ uint32_t rec_start(const DevCfg& c, const EnvConst& k, const Env& s) {
+  if (!c.skip_ok || !in_map(k.m.w, k.m.h, s.x, s.y)) return 0u;
+  return (uint32_t)scan_start(__ldg(k.clr + __float2int_rd(s.y) * k.m.clr_ld + __float2int_rd(s.x)));
+}
 __device__ __forceinline__ void derive_rec(const DevCfg& c, const EnvConst& k, const StepRec& r, ObsRec& o) {
   const Env s = r.post;
+  const uint32_t k0 = rec_start(c, k, s);
   const uint32_t done = r.done;
   const GoalFrame g = goal_frame(k.L, s);
   const uint64_t nk = noise_key(k, s);
@@ -395,28 +396,11 @@ __device__ __forceinline__ void derive_rec(const DevCfg& c, const EnvConst& k, c
     const uint64_t pk = noise_key(k, q);
     o.rpart = reward_partial(c, k.L, q, gp.alpha, gp.ddx, gp.ddy);
     w[3] = make_uint4(fbits(e[4]), fbits(q.x), fbits(q.y), fbits(q.phi));
-    w[4] = make_uint4(fbits(q.sigma), (uint32_t)pk, (uint32_t)(pk >> 32), 0u);
+    w[4] = make_uint4(fbits(q.sigma), (uint32_t)pk, (uint32_t)(pk >> 32), k0 | (rec_start(c, k, q) << 8));
   } else {
     o.ex[4] = e[4];
+    o.k0 = k0;
   }
-}
-
-// The scan of one pose by a whole warp: this lane's beams (with noise drawn
-// from key nk when sigma > 0) into o.b0 / o.b1; returns the minimum
-// noise-free range over all beams.
-template <bool kDyn = false>
-__device__ __forceinline__ float scan_pose(const DevCfg& c, const EnvConst& k, float x, float y, float phi,
-                                           float sigma, uint64_t nk, int lane, ObsRegs& o, const Discs* d = nullptr) {
-  float n0 = 0.0f, n1 = 0.0f;
-  if (sigma > 0.0f) {
-    n0 = box_muller(sm_at(nk, (uint64_t)lane));
-    if (k.nb > 32) n1 = box_muller(sm_at(nk, (uint64_t)(lane + 32)));
-  }
-  float mn = c.range_max;
-  o.b0 = lane < k.nb ? beam_at<kDyn>(c, k, x, y, phi, sigma, k.off0, n0, mn, d) : 1.0f;
-  o.b1 = lane + 32 < k.nb ? beam_at<kDyn>(c, k, x, y, phi, sigma, k.off1, n1, mn, d) : 1.0f;
-  // ranges are >= 0, so their bit patterns order like the values
-  return __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(mn)));
 }
 
 // The motion (delay, Eq. 5, Eq. 6) of steps j0 .. n-1 from state s as if no
@@ -604,7 +588,7 @@ __device__ __forceinline__ void pose_chunk(const DevCfg& c, const SimPtrs& p, co
 // the shared counter: scan, observation, reward, outputs.  With kDyn the
 // scans see the recorded disc centres of each step (dpost; dpre for the
 // pre-reset scan of a truncated step).
-template <bool kDyn = false>
+template <bool kDyn, bool kFast>
 __device__ __forceinline__ void consume_chunk(const DevCfg& c, const EnvConst& k, const ObsRec* buf, unsigned* next,
                                               int i0, int i1, int K, int env, long long n, int lane, ObsRegs& o,
                                               bool& has_last, float* __restrict__ obs_seq,
@@ -625,11 +609,13 @@ __device__ __forceinline__ void consume_chunk(const DevCfg& c, const EnvConst& k
       rew = 75.0f;
     } else if (done) {
       const uint64_t pk = ((uint64_t)R.pnhi << 32) | R.pnlo;
-      rew = reward_finish(c, R.rpart, scan_pose<kDyn>(c, k, R.px, R.py, R.pphi, R.psigma, pk, lane, o,
-                                                      kDyn ? dpre + (i - i0) : nullptr));
+      rew = reward_finish(c, R.rpart,
+                          scan_pose<kDyn, kFast>(c, k.sm, k.nb, k.off0, k.off1, R.px, R.py, R.pphi, R.psigma, pk,
+                                                 (int)(R.k0 >> 8), lane, o.b0, o.b1, kDyn ? dpre + (i - i0) : nullptr));
     }
     const uint64_t nk = ((uint64_t)R.nhi << 32) | R.nlo;
-    const float mn = scan_pose<kDyn>(c, k, R.x, R.y, R.phi, R.sigma, nk, lane, o, kDyn ? dpost + (i - i0) : nullptr);
+    const float mn = scan_pose<kDyn, kFast>(c, k.sm, k.nb, k.off0, k.off1, R.x, R.y, R.phi, R.sigma, nk,
+                                            (int)(R.k0 & 0xFFu), lane, o.b0, o.b1, kDyn ? dpost + (i - i0) : nullptr);
     if (!done) rew = reward_finish(c, R.rpart, mn);
     o.ex = lane < 5 ? R.ex[lane] : 0.0f;
     if (i == K - 1) has_last = true;
@@ -704,7 +690,7 @@ __device__ __forceinline__ Obst load_obst_cg(const SimPtrs& p, int o, int i) {
   return b;
 }
 
-template <bool kDyn>
+template <bool kDyn, bool kFast>
 __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_constant__ DevCfg c, SimPtrs p, int K,
                                                                 int P, const int* __restrict__ order, int seg,
                                                                 unsigned* __restrict__ sync, unsigned wait_iters,
@@ -797,7 +783,7 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
           }
           if (ch >= 1) {
             const int b = (ch - 1) & 1, i0 = s0 + (ch - 1) * kPipeChunk;
-            consume_chunk<kDyn>(c, k, ob + b * kPipeChunk, &next_step[group][b], i0, min(s1, i0 + kPipeChunk), K,
+            consume_chunk<kDyn, kFast>(c, k, ob + b * kPipeChunk, &next_step[group][b], i0, min(s1, i0 + kPipeChunk), K,
                                 env, n, lane, o, has_last, obs_seq, act_seq, rew_seq, done_seq,
                                 dpost + b * kPipeChunk, dpre + b * kPipeChunk);
           }
@@ -812,7 +798,7 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
         for (int ch = 1; ch <= chunks; ++ch) {
           const int b = (ch - 1) & 1, i0 = s0 + (ch - 1) * kPipeChunk;
           named_barrier(bfull + b, nthr);  // chunk ch - 1 written
-          consume_chunk<kDyn>(c, k, ob + b * kPipeChunk, &next_step[group][b], i0, min(s1, i0 + kPipeChunk), K, env,
+          consume_chunk<kDyn, kFast>(c, k, ob + b * kPipeChunk, &next_step[group][b], i0, min(s1, i0 + kPipeChunk), K, env,
                               n, lane, o, has_last, obs_seq, act_seq, rew_seq, done_seq, dpost + b * kPipeChunk,
                               dpre + b * kPipeChunk);
           named_arrive(bfree + b, nthr);
@@ -830,6 +816,10 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
   }
 }
 
+static decltype(&k_rollout_random_pipe<false, true>) pipe_kernel(const DevCfg& c) {
+  if (c.n_dyn > 0) return c.scan_fast ? k_rollout_random_pipe<true, true> : k_rollout_random_pipe<true, false>;
+  return c.scan_fast ? k_rollout_random_pipe<false, true> : k_rollout_random_pipe<false, false>;
+}
 static size_t pipe_smem_bytes(int E, bool dyn) { return (size_t)E * pipe_group_bytes(dyn); }
 static int pipe_envs_per_block(const sg_launch& L) {
   const int E = L.warps_per_block / (1 + L.obs_warps);
@@ -901,6 +891,22 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 constexpr int kWarpsPerBlock = 4;
 
+// A launch whose kernel may start while the kernel before it on the stream
+// still runs (programmatic dependent launch: it waits at pdl_wait).
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), int grid, int block, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 int grid_for(int n_envs) { return (n_envs + kWarpsPerBlock - 1) / kWarpsPerBlock; }
 
 // Host-side cost of an env for the work list: beams x the march work one
@@ -958,6 +964,11 @@ static int make_devcfg(const sg_sim_config* cfg, DevCfg* dc) {
   dc->kmax = (int)kmaxf;
   dc->delay_lo = cfg->delay_lo;
   dc->delay_span = cfg->delay_hi - cfg->delay_lo + 1;
+  // the division by range_max as a product (see div_range)
+  if (cfg->range_max >= 0x1p-20f && cfg->range_max <= 0x1p20f && cfg->march_step >= 0x1p-30f) {
+    dc->rmax_zh = 1.0f / cfg->range_max;
+    dc->rmax_zl = (float)(1.0 / (double)cfg->range_max - (double)dc->rmax_zh);
+  }
   dc->skip_ok = cfg->march_step <= 1.0f ? 1 : 0;
   // a point of a cell with clearance c is at least c - 0.5 cells from every
   // occupied cell centre; keep a margin of one cell above the radius so that
@@ -1155,6 +1166,10 @@ SimPtrs sg_sim_ptrs(sg_sim* s) {
   return p;
 }
 
+// Env counts whose step runs as two kernels.
+constexpr int kStepSplitEnvs = 8192;
+constexpr int kStepSplitMax = 1 << 20;
+
 static void free_sim(sg_sim* s) {
   if (!s) return;
   cudaFree(s->atlas);
@@ -1169,6 +1184,9 @@ static void free_sim(sg_sim* s) {
   cudaFree(s->order_dev);
   cudaFree(s->queue_dev);
   cudaFree(s->map_order_dev);
+  cudaFree(s->rank_dev);
+  cudaFree(s->step_rec);
+  cudaFree(s->step_discs);
   cudaFree(s->dyn);
   cudaFree(s->pipe_sync_dev);
   cudaFree(s->q_sync_dev);
@@ -1223,13 +1241,15 @@ extern "C" int sg_sim_create(const sg_sim_config* cfg, int32_t n_maps, const uin
   }
   dc.n_sec = n_sec;
   dc.sec_scale = (float)((double)n_sec / (2.0 * M_PI));
-  long long sec_bytes = 0;
+  long long sec_bytes = 0, max_planes = 0;
   for (int m = 0; m < n_maps; ++m) {
     const long long plane = (long long)md[m].clr_ld * (map_h[m] + 2 * kClrBorder);
     md[m].sec_plane = n_sec > 1 ? plane : 0;
     md[m].sec_off = n_sec > 1 ? sec_bytes + (long long)kClrBorder * md[m].clr_ld + kClrBorder : 0;
     if (n_sec > 1) sec_bytes += plane * n_sec;
+    max_planes = std::max(max_planes, plane * n_sec);
   }
+  dc.scan_fast = dc.delta == 1.0f && dc.rmax_zh != 0.0f && max_planes < (1ll << 31);
   sg_sim* s = new (std::nothrow) sg_sim();
   if (!s) return SG_E_OOM;
   s->cfg = *cfg;
@@ -1255,6 +1275,12 @@ extern "C" int sg_sim_create(const sg_sim_config* cfg, int32_t n_maps, const uin
   alloc((void**)&s->ustate, sizeof(uint32_t) * 4 * (size_t)n);
   alloc((void**)&s->status_dev, sizeof(uint32_t));
   alloc((void**)&s->map_order_dev, sizeof(int) * n);
+  if (cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess) s->sms = 1;
+  if (dc.scan_fast && n >= kStepSplitEnvs && n <= kStepSplitMax) {
+    alloc((void**)&s->rank_dev, sizeof(int) * n);
+    alloc((void**)&s->step_rec, sizeof(MotionRec) * (size_t)n);
+    if (cfg->n_dyn > 0) alloc((void**)&s->step_discs, sizeof(Discs) * (size_t)n);
+  }
   if (cfg->n_dyn > 0) alloc((void**)&s->dyn, sizeof(float) * 4 * cfg->n_dyn * (size_t)n);
   alloc((void**)&s->q_sync_dev, sizeof(unsigned) * ((size_t)(n + 127) / 128 + 2));
   // maps are preprocessed in groups whose grids fit a staging budget
@@ -1334,6 +1360,11 @@ extern "C" int sg_sim_create(const sg_sim_config* cfg, int32_t n_maps, const uin
     for (int i = 0; i < n; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return env_map[a] < env_map[b]; });
     e = cudaMemcpy(s->map_order_dev, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && s->rank_dev) {
+      std::vector<int> rank((size_t)n);
+      for (int i = 0; i < n; ++i) rank[order[i]] = i;
+      e = cudaMemcpy(s->rank_dev, rank.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
+    }
   }
   if (e == cudaSuccess && env_beams)
     e = cudaMemcpy(s->env_beams_dev, env_beams, sizeof(int) * n, cudaMemcpyHostToDevice);
@@ -1392,33 +1423,31 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
   SG_RANGE("sg_sim_step");
   if (!sim || !act_dev || !obs_dev || !rew_dev || !done_dev) return SG_E_INVAL;
   if (((uintptr_t)obs_dev & 3) || ((uintptr_t)rew_dev & 3) || ((uintptr_t)term_obs_dev & 3)) return SG_E_ALIGN;
-  const bool dyn = sim->dc.n_dyn > 0;
-  auto kern_for = [dyn](int e) {
-    if (e == 6) return dyn ? k_step<true, 6> : k_step<false, 6>;
-    if (e == 7) return dyn ? k_step<true, 7> : k_step<false, 7>;
-    return dyn ? k_step<true, 8> : k_step<false, 8>;
-  };
-  const long long n = sim->dc.n_envs;
-  if (sim->step_epw == 0) {
-    // envs per warp: the count whose grid fills its last wave of resident
-    // CTAs best (chosen once per simulator)
-    int sms = 0;
-    SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, sim->device));
-    double best = -1.0;
-    for (int e = 8; e >= 6; --e) {
-      int bps = 0;
-      SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern_for(e), 32 * kStepWarps, 0));
-      const long long ctas = (n + kStepWarps * e - 1) / (kStepWarps * e), res = (long long)sms * std::max(bps, 1);
-      const double fill = (double)ctas / (double)(((ctas + res - 1) / res) * res);
-      if (fill > best + 1e-9) {
-        best = fill;
-        sim->step_epw = e;
-      }
-    }
+  const DevCfg& dc = sim->dc;
+  const bool dyn = dc.n_dyn > 0, fast = dc.scan_fast != 0;
+  const int n = dc.n_envs;
+  const SimPtrs sp = sg_sim_ptrs(sim);
+  if (sim->step_rec) {
+    (dyn ? k_step_motion<true> : k_step_motion<false>)<<<(n + 63) / 64, 64, 0, stream>>>(
+        dc, sp, sim->rank_dev, act_dev, sim->step_rec, sim->step_discs);
+    SG_CUDA(cudaGetLastError());
+    SG_CUDA(launch_pdl(dyn ? k_step_finish<true> : k_step_finish<false>, (n + kFinishWarps - 1) / kFinishWarps,
+                       32 * kFinishWarps, stream, dc, sp, (const MotionRec*)sim->step_rec, (const Discs*)sim->step_discs, obs_dev, rew_dev,
+                       done_dev, term_obs_dev));
+    return SG_OK;
   }
-  const int per = kStepWarps * sim->step_epw;
-  kern_for(sim->step_epw)<<<(unsigned)((n + per - 1) / per), 32 * kStepWarps, 0, stream>>>(
-      sim->dc, sg_sim_ptrs(sim), sim->map_order_dev, act_dev, obs_dev, rew_dev, done_dev, term_obs_dev);
+  // one env per warp (and per CTA) while that leaves SMs idle, more as the
+  // warps fill the resident slots
+  const int e = !fast ? 8 : n <= 32 * sim->sms ? 1 : n <= 64 * sim->sms ? 2 : n <= 128 * sim->sms ? 4 : 8;
+  const int wpb = std::min(kStepWarps, std::max(1, (n / e + sim->sms - 1) / sim->sms));
+  auto kern = !fast ? (dyn ? k_step<true, false, 8> : k_step<false, false, 8>)
+              : e == 1 ? (dyn ? k_step<true, true, 1> : k_step<false, true, 1>)
+              : e == 2 ? (dyn ? k_step<true, true, 2> : k_step<false, true, 2>)
+              : e == 4 ? (dyn ? k_step<true, true, 4> : k_step<false, true, 4>)
+                       : (dyn ? k_step<true, true, 8> : k_step<false, true, 8>);
+  const int per = wpb * e;
+  kern<<<(n + per - 1) / per, 32 * wpb, 0, stream>>>(dc, sp, sim->map_order_dev, act_dev, obs_dev, rew_dev, done_dev,
+                                                      term_obs_dev);
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
@@ -1454,7 +1483,7 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
           grid = std::min<long long>(nitems, (long long)sim->persistent_blocks);
           SG_CUDA(cudaMemsetAsync(sim->pipe_sync_dev, 0, sizeof(unsigned) * (size_t)(nblk + 2), stream));
         }
-        (dyn ? k_rollout_random_pipe<true> : k_rollout_random_pipe<false>)<<<(unsigned)grid, 32 * G * E, smem,
+        pipe_kernel(sim->dc)<<<(unsigned)grid, 32 * G * E, smem,
                                                                           stream>>>(
             sim->dc, sp, K, L.obs_warps, L.order ? sim->map_order_dev : nullptr, seg,
             seg > 0 ? sim->pipe_sync_dev : nullptr, L.wait_iters > 0 ? (unsigned)L.wait_iters : kPipeWaitIters,
@@ -1531,7 +1560,7 @@ extern "C" int sg_sim_set_launch(sg_sim_t sim, const sg_launch* cfg) {
     const int E = pipe_envs_per_block(L);
     const bool dyn = sim->dc.n_dyn > 0;
     const size_t smem = pipe_smem_bytes(E, dyn);
-    auto kern = dyn ? k_rollout_random_pipe<true> : k_rollout_random_pipe<false>;
+    auto kern = pipe_kernel(sim->dc);
     SG_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (L.segment > 0) {
       // time slicing: a resident grid and the per-CTA segment flags
