@@ -31,6 +31,7 @@ struct sg_sim {
   uint32_t* status_dev = nullptr;
   // launch configuration of the random rollout (sg_sim_set_launch)
   sg_launch launch = {SG_ROLLOUT_GRID, 4, 1, 0, 0, 0, 0, 0};  // no slicing, default wait bound
+  bool launch_set = false;  // else the library chooses by the size of the call
   int persistent_blocks = 0;
   int* order_dev = nullptr;      // work list (cost-sorted env indices) or null
   int* map_order_dev = nullptr;  // env indices grouped by map (stable), for per-CTA map locality
@@ -52,6 +53,23 @@ struct SgRange {
   SgRange& operator=(const SgRange&) = delete;
 };
 #define SG_RANGE(name) SgRange sg_range_(name)
+
+// A launch whose kernel may start while the kernel before it on the stream
+// still runs (programmatic dependent launch: it waits at pdl_wait).
+template <typename... P, typename... A>
+cudaError_t sg_launch_pdl(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 sg::SimPtrs sg_sim_ptrs(sg_sim* s);
 long long sg_state_bytes(const sg_sim* s);

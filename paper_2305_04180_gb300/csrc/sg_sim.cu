@@ -409,9 +409,16 @@ __device__ __forceinline__ void derive_rec(const DevCfg& c, const EnvConst& k, c
 // in step order (every lane the same); the delayed action, the target
 // velocities, sin/cos of each step's heading and the Eq. 6 increments are
 // lane-parallel.  Every value is the float32 expression of kinematics(),
-// evaluated in the same order.  Lane j writes step j's post state (with its
+// evaluated in the same order.  The two ordered loops take kRun steps at a
+// time, their shuffles first: one step at a time each waited for its own
+// shuffles (5,080 cycles for a 32-step run).  More than three steps lose to
+// the instruction cache, which this code shares with the scans: 1,024 envs x
+// 2,000 took 1,514 us one step at a time, 1,403, 1,390, 1,417, 1,555 and 1,800
+// (with unrolled row tests) by 2, 3, 4, 8 and 16.  Lanes past the run keep
+// values that nobody reads.  Lane j writes step j's post state (with its
 // action) to buf[j].post and returns its position and episode step in mx,
 // my, mep; bad is set in the lanes whose action index is out of range.
+constexpr int kRun = 3;
 __device__ __forceinline__ void motion_run(const DevCfg& c, const Env& s, int j0, int n, uint32_t abatch,
                                            StepRec* buf, int lane, bool& bad, float& mx, float& my,
                                            uint32_t& mep) {
@@ -435,20 +442,25 @@ __device__ __forceinline__ void motion_run(const DevCfg& c, const Env& s, int j0
   // Eq. 5 and the heading part of Eq. 6, in step order
   float vl = s.vl, va = s.va, phi = s.phi;
   float jvl = 0.0f, jva = 0.0f, jphi = s.phi;
-  for (int j = j0; j < n; ++j) {
-    const float plj = __shfl_sync(kFull, pl, j), paj = __shfl_sync(kFull, pa, j);
-    vl = s.K * vl + plj;
-    va = s.K * va + paj;
-    float ph = phi + s.dt * va;
-    if (ph >= kPi)
-      ph = ph - 2.0f * kPi;
-    else if (ph < -kPi)
-      ph = ph + 2.0f * kPi;
-    phi = ph;
-    if (lane == j) {
-      jvl = vl;
-      jva = va;
-      jphi = phi;
+  for (int jb = j0; jb < n; jb += kRun) {
+    float plj[kRun], paj[kRun];
+#pragma unroll
+    for (int u = 0; u < kRun; ++u) {
+      plj[u] = __shfl_sync(kFull, pl, (jb + u) & 31);
+      paj[u] = __shfl_sync(kFull, pa, (jb + u) & 31);
+    }
+#pragma unroll
+    for (int u = 0; u < kRun; ++u) {
+      vl = s.K * vl + plj[u];
+      va = s.K * va + paj[u];
+      const float ph = phi + s.dt * va;
+      const float up = ph + 2.0f * kPi, dn = ph - 2.0f * kPi;
+      phi = ph >= kPi ? dn : (ph < -kPi ? up : ph);
+      if (lane == jb + u) {
+        jvl = vl;
+        jva = va;
+        jphi = phi;
+      }
     }
   }
   float sn = s.sphi, cs = s.cphi;
@@ -459,12 +471,21 @@ __device__ __forceinline__ void motion_run(const DevCfg& c, const Env& s, int j0
   const float cprev = lane == j0 ? s.cphi : cu, sprev = lane == j0 ? s.sphi : su;
   const float tx = s.dt * (jvl * cprev), ty = s.dt * (jvl * sprev);
   float x = s.x, y = s.y, jx = s.x, jy = s.y;
-  for (int j = j0; j < n; ++j) {
-    x = x - __shfl_sync(kFull, tx, j);
-    y = y - __shfl_sync(kFull, ty, j);
-    if (lane == j) {
-      jx = x;
-      jy = y;
+  for (int jb = j0; jb < n; jb += kRun) {
+    float txj[kRun], tyj[kRun];
+#pragma unroll
+    for (int u = 0; u < kRun; ++u) {
+      txj[u] = __shfl_sync(kFull, tx, (jb + u) & 31);
+      tyj[u] = __shfl_sync(kFull, ty, (jb + u) & 31);
+    }
+#pragma unroll
+    for (int u = 0; u < kRun; ++u) {
+      x = x - txj[u];
+      y = y - tyj[u];
+      if (lane == jb + u) {
+        jx = x;
+        jy = y;
+      }
     }
   }
   const uint32_t steps = (uint32_t)(lane - j0 + 1);
@@ -890,22 +911,6 @@ int cuda_fail(cudaError_t e, const char* what) {
   } while (0)
 
 constexpr int kWarpsPerBlock = 4;
-
-// A launch whose kernel may start while the kernel before it on the stream
-// still runs (programmatic dependent launch: it waits at pdl_wait).
-template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kern)(P...), int grid, int block, cudaStream_t stream, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
-}
 
 int grid_for(int n_envs) { return (n_envs + kWarpsPerBlock - 1) / kWarpsPerBlock; }
 
@@ -1431,8 +1436,8 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
     (dyn ? k_step_motion<true> : k_step_motion<false>)<<<(n + 63) / 64, 64, 0, stream>>>(
         dc, sp, sim->rank_dev, act_dev, sim->step_rec, sim->step_discs);
     SG_CUDA(cudaGetLastError());
-    SG_CUDA(launch_pdl(dyn ? k_step_finish<true> : k_step_finish<false>, (n + kFinishWarps - 1) / kFinishWarps,
-                       32 * kFinishWarps, stream, dc, sp, (const MotionRec*)sim->step_rec, (const Discs*)sim->step_discs, obs_dev, rew_dev,
+    SG_CUDA(sg_launch_pdl(dyn ? k_step_finish<true> : k_step_finish<false>, (n + kFinishWarps - 1) / kFinishWarps,
+                          32 * kFinishWarps, 0, stream, dc, sp, (const MotionRec*)sim->step_rec, (const Discs*)sim->step_discs, obs_dev, rew_dev,
                        done_dev, term_obs_dev));
     return SG_OK;
   }
@@ -1452,6 +1457,25 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
   return SG_OK;
 }
 
+// The launch of a rollout whose simulator has none set: results never depend
+// on it, so it follows the size of the call.  With random actions the scans of
+// a step wait for the pose chain only, so several warps per env shorten a
+// rollout while the envs alone leave warp slots empty, and the pose chain's
+// run-ahead pays at every size once K fills a chunk.  us (one warp per env /
+// pipelined): 16 envs x 512 steps 1,516 / 184 (15 scan warps), 304 x 512 1,656 /
+// 233 (7), 1,024 x 512 1,951 / 471, 4,096 x 224 1,184 / 726, 16,384 x 32 599 /
+// 497 (3, two envs per CTA).  Few steps of many envs stay with one warp per
+// env (4,096 x 8: 59 / 75; 65,536 x 16: 1,078 / 1,179).
+static sg_launch auto_launch(int n, int K, int sms) {
+  sg_launch L = {SG_ROLLOUT_GRID, 4, 1, 0, 0, 0, 0, 0};
+  if (K < std::min(kPipeChunk, n / 256)) return L;
+  L.kernel = SG_ROLLOUT_PIPE;
+  L.obs_warps = n <= sms ? 15 : n <= 32 * sms ? 7 : 3;
+  L.warps_per_block = n <= sms ? 16 : 8;
+  L.order = 1;
+  return L;
+}
+
 // Q-network rollouts live with the network (sg_qnet.cu).
 int sg_rollout_eps_q(sg_sim* sim, int K, sg_qnet* q, const float* eps, sg_replay* rp, float* obs, float* obs_seq,
                      uint8_t* act_seq, float* rew_seq, uint8_t* done_seq, cudaStream_t stream);
@@ -1464,8 +1488,8 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
   if (((uintptr_t)obs_dev & 3) || ((uintptr_t)obs_seq_dev & 3) || ((uintptr_t)rew_seq_dev & 3)) return SG_E_ALIGN;
   if (policy == SG_POLICY_RANDOM) {
     if (replay) return SG_E_INVAL;  // transitions are recorded by the Q-policy rollout
-    const sg_launch& L = sim->launch;
     const int n = sim->dc.n_envs;
+    const sg_launch L = sim->launch_set ? sim->launch : auto_launch(n, K, sim->sms);
     const SimPtrs sp = sg_sim_ptrs(sim);
     switch (L.kernel) {
       case SG_ROLLOUT_PIPE: {
@@ -1561,7 +1585,10 @@ extern "C" int sg_sim_set_launch(sg_sim_t sim, const sg_launch* cfg) {
     const bool dyn = sim->dc.n_dyn > 0;
     const size_t smem = pipe_smem_bytes(E, dyn);
     auto kern = pipe_kernel(sim->dc);
-    SG_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit is a property of the kernel, shared by every handle: the
+    // largest any launch needs
+    SG_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)pipe_smem_bytes(kPipeMaxGroups, dyn)));
     if (L.segment > 0) {
       // time slicing: a resident grid and the per-CTA segment flags
       SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern,
@@ -1603,6 +1630,7 @@ extern "C" int sg_sim_set_launch(sg_sim_t sim, const sg_launch* cfg) {
   }
   if (L.kernel == SG_ROLLOUT_QUEUE && !sim->queue_dev) SG_CUDA(cudaMalloc(&sim->queue_dev, sizeof(unsigned)));
   sim->launch = L;
+  sim->launch_set = true;
   sim->persistent_blocks =
       (L.kernel == SG_ROLLOUT_QUEUE || (L.kernel == SG_ROLLOUT_PIPE && L.segment > 0)) ? bps * sms : 0;
   return SG_OK;
