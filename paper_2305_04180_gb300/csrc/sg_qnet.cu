@@ -123,6 +123,7 @@ struct ReplayDev {
   uint8_t* term;         // [cap] collided or arrived
   unsigned long long* steps;  // vectorized steps recorded so far
   int slots, n_envs, obs_dim;
+  unsigned long long inv_full, inv_slots;  // floor((2^64 - 1) / (sampled entries of a full ring, slots))
   int reserve;           // newest slots the learner never samples (an actor may be writing them)
 };
 
@@ -145,12 +146,12 @@ struct sg_qnet {
   uint8_t* img = nullptr;    // online BF16 image
   uint8_t* img_t = nullptr;  // target BF16 image
   unsigned long long* step = nullptr;  // optimiser steps taken (device)
-  unsigned* td_fail = nullptr;         // SG_TD_FAIL_* bits of the current TD step (device), cleared per step
+  unsigned* td_fail = nullptr;         // [2] kTdFail* bits of the current TD step, CTAs of its update that are done
   // learner scratch, sized for max_batch
   int max_batch = 0;
-  float* partial = nullptr;  // [max_batch / kTile][P + 1] (last entry: loss)
-  float* y = nullptr;        // [max_batch] TD targets
-  int* idx = nullptr;        // [max_batch] sampled ring entries
+  void* frag = nullptr;      // TdFrag of the 16-sample tiles (mma.sync learner)
+  int td_clusters = 1;       // clusters of k_td_tile that fit the device
+  float* partial = nullptr;  // [tiles of 128][P + 1] (last entry: loss; tcgen05 learner)
   int rollout_mt = 0;        // m-tiles per CTA of the fused rollout (0 = choose by waves)
   int lim_rollout = 0;       // CTA caps of the tcgen05 rollout / learner grids (0 = every SM)
   int lim_learner = 0;
@@ -1396,6 +1397,15 @@ __global__ void k_replay_advance(unsigned long long* steps, int K) { *steps += (
 // Adam moments and the image untouched; the step count does not advance.
 constexpr unsigned kTdFailCopy = 1u;
 constexpr unsigned kTdFailAction = 2u;
+// x mod d with inv = floor((2^64 - 1) / d): the quotient from the high product
+// is at most two too small (x / d - x inv / 2^64 < 2).
+__device__ __forceinline__ unsigned long long mod_inv(unsigned long long x, unsigned long long d,
+                                                      unsigned long long inv) {
+  unsigned long long r = x - __umul64hi(x, inv) * d;
+  if (r >= d) r -= d;
+  if (r >= d) r -= d;
+  return r;
+}
 // Ring entry of sample i of optimiser step `tstep`: uniform over the
 // V = min(steps, slots - reserve) most recently completed slots, so that a
 // rollout running concurrently (which writes the next slots) is never read.
@@ -1408,10 +1418,14 @@ __device__ __forceinline__ long long sample_entry(unsigned long long seed, unsig
   const unsigned long long V = st < usable ? st : usable;
   if (V == 0) return -1;
   const uint64_t h = sm_at(sm_at(sm_at(sm_at(seed, kStreamSample), tstep), (uint64_t)i), 0ull);
-  const unsigned long long j = h % (V * (unsigned long long)rp.n_envs);
-  const unsigned long long back = j / (unsigned long long)rp.n_envs;
-  const unsigned long long slot = (st - 1ull - back) % (unsigned long long)rp.slots;
-  const long long e = (long long)(slot * (unsigned long long)rp.n_envs + j % (unsigned long long)rp.n_envs);
+  // the ring holds at most 2^31 entries, so j and its quotient fit 32 bits;
+  // back < V <= slots, so one correction replaces the modulo of the difference
+  const uint32_t n = (uint32_t)rp.n_envs;
+  const unsigned long long D = V * (unsigned long long)n;
+  const uint32_t j = (uint32_t)(V == usable ? mod_inv(h, D, rp.inv_full) : h % D);
+  const uint32_t back = j / n, last = (uint32_t)mod_inv(st - 1ull, (unsigned long long)rp.slots, rp.inv_slots);
+  const uint32_t slot = last >= back ? last - back : last + (uint32_t)rp.slots - back;
+  const long long e = (long long)slot * n + (j - back * n);
   return SG_IN_BOUNDS(e >= 0 && e < (long long)rp.slots * rp.n_envs) ? e : -1;
 }
 
@@ -1422,64 +1436,6 @@ __device__ __forceinline__ void gather_tile(bf16* X, int ld1, const float* __res
   for (int k = lane; k < ld1; k += 32) {
     const float v = (e >= 0 && k < obs_dim) ? src[(long long)e * obs_dim + k] : 0.0f;
     X[warp * ld1 + k] = __float2bfloat16_rn(v);
-  }
-}
-
-// Double-DQN targets of 16 samples per CTA: a* = argmax_a Q_online(s', a),
-// y = r + gamma (1 - term) Q_target(s', a*).  Also records the sampled entries.
-__global__ void __launch_bounds__(kThreads, 1)
-    k_td_target(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, ImgLayout L, ReplayDev rp,
-                unsigned long long seed, const unsigned long long* __restrict__ step, int batch, float gamma,
-                float* __restrict__ y, int* __restrict__ idx, unsigned* __restrict__ fail) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint8_t* sw = smem;
-  bf16* X = reinterpret_cast<bf16*>(smem + L.bytes);
-  bf16* H1 = X + kTile * L.ld1;
-  bf16* H2 = H1 + kTile * kLdh;
-  float* O = reinterpret_cast<float*>(H2 + kTile * kLdh);
-  __shared__ int rows[kTile];
-  __shared__ int astar[kTile];
-  __shared__ uint64_t bar_img;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kTile + warp;
-  if (lane == 0) {
-    rows[warp] = i < batch ? (int)sample_entry(seed, *step, i, rp) : -1;
-    if (i < batch) idx[i] = rows[warp];
-  }
-  if (threadIdx.x == 0) mbar_init(&bar_img, 1);
-  __syncthreads();
-  // online image (phase 0) while the tile is gathered; a copy that does not
-  // complete makes the targets NaN
-  bool ok = stage_image_bulk(sw, img, L.bytes, &bar_img, 0u, kTcTries);
-  uint32_t phase = 0u;  // the copy in flight
-  gather_tile(X, L.ld1, rp.s2, rows, rp.obs_dim, warp, lane);
-  __syncthreads();
-  if (ok) mlp_tile(qw_at(sw, L), X, H1, H2, O, warp, lane);
-  if (lane == 0) astar[warp] = (int)greedy_action(O + warp * kOutPad, nullptr, L.plain);
-  fence_async_smem();  // this thread's reads of the online image before the bulk copy overwrites it
-  __syncthreads();
-  // the target image over it (phase 1)
-  if (ok) {
-    phase = 1u;
-    ok = stage_image_bulk(sw, img_t, L.bytes, &bar_img, 1u, kTcTries);
-  }
-  if (ok) mlp_tile(qw_at(sw, L), X, H1, H2, O, warp, lane);
-  if (!ok) {
-    if (threadIdx.x == 0) {
-      atomicOr(fail, kTdFailCopy);
-      // the copy that timed out may still be writing shared memory: give it
-      // one more bounded wait before the CTA exits
-      mbar_wait(&bar_img, phase, kTcTries);
-    }
-    if (lane == 0 && i < batch) y[i] = __int_as_float(0x7fc00000);
-  }
-  if (lane == 0 && i < batch && ok) {
-    float qv[5];
-    greedy_action(O + warp * kOutPad, qv, L.plain);
-    const int e = rows[warp];
-    const float r = e >= 0 ? rp.r[e] : 0.0f;
-    const float nt = (e >= 0 && rp.term[e]) ? 0.0f : 1.0f;
-    y[i] = r + gamma * nt * qv[astar[warp]];
   }
 }
 
@@ -1663,84 +1619,606 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// Sum the per-CTA partials in CTA order, Adam (Kingma & Ba) on the FP32
-// master, and the BF16 image entry of each parameter.  The step counter is
-// read here and advanced by k_step_advance afterwards.
-__global__ void k_adam(float* __restrict__ th, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ partial, int nblk, ParamLayout P, ImgLayout L, uint8_t* __restrict__ img,
-                       const unsigned long long* __restrict__ step, float lr, float b1, float b2, float eps,
-                       float* __restrict__ loss, float* __restrict__ grad_out, int batch,
-                       const unsigned* __restrict__ fail) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (*fail) {
-    // no usable gradient this step: NaN out, parameters and moments unchanged
-    const float qnan = __int_as_float(0x7fc00000);
-    if (i == 0 && loss) *loss = qnan;
-    if (grad_out && i < P.total) {
-      const int j = L.plain ? paper_index(i, P, L.n_in) : i;
-      if (j >= 0) grad_out[j] = qnan;
+// ------------------------------------------------------- parameter update
+// Everything that follows the gradient of a TD step, per parameter: Adam
+// (Kingma & Ba) on the FP32 master, the BF16 entry in the image and in the
+// tensor cores' copies, and on a target step the target network's copies.
+// The last CTA of the launch advances the step count and clears the step's
+// failure word, so that nothing else has to run before the next step.  As
+// five launches (reduce + Adam, tensor-core copy, step count, target check, a
+// memset) the same work cost a batch-256 step 25 of its 57 us.
+struct TdUpdate {
+  float* th;
+  float* m;
+  float* v;
+  float* tgt;
+  uint8_t* img;
+  uint8_t* img_t;
+  uint8_t* tc;
+  uint8_t* tc_t;
+  unsigned long long* step;  // null: gradient only (sg_td_grad_noalloc)
+  unsigned* fail;
+  unsigned* tick;            // CTAs that are done (0 between launches)
+  float lr;
+  int every;                 // target period (optimiser steps), <= 0: never
+  float* loss;
+  float* grad;
+  int batch;
+  ParamLayout P;
+  ImgLayout L;
+};
+// What a launch does: read once per thread.  A failed step changes nothing,
+// and its unchanged step count decides about the target.
+struct UpdRun {
+  bool adam, sync;
+  bool sync_failed;  // sync of a failed step
+  float d1, d2;      // 1 - beta1^t, 1 - beta2^t
+};
+constexpr float kBeta1 = 0.9f, kBeta2 = 0.999f, kAdamEps = 1e-8f;
+
+__device__ __forceinline__ UpdRun upd_begin(const TdUpdate& u) {
+  UpdRun r = {false, false, false, 1.0f, 1.0f};
+  if (u.lr != 0.0f) {
+    const unsigned long long st = *u.step;
+    const float t = (float)(st + 1ull);
+    r.adam = true;
+    r.d1 = 1.0f - powf(kBeta1, t);
+    r.d2 = 1.0f - powf(kBeta2, t);
+    if (u.every > 0) {
+      const unsigned long long rem = st % (unsigned long long)u.every;
+      r.sync_failed = rem == 0ull;
+      r.sync = rem + 1ull == (unsigned long long)u.every;
     }
-    return;
   }
-  if (i == 0 && loss) {
-    float acc = 0.0f;
-    for (int b = 0; b < nblk; ++b) acc += partial[(long long)b * partial_stride(P.total) + P.total];
-    *loss = acc / (float)batch;
-  }
-  if (i >= P.total) return;
-  float gsum = 0.0f;
-  for (int b = 0; b < nblk; ++b) gsum += partial[(long long)b * partial_stride(P.total) + i];
-  if (grad_out) {
-    const int j = L.plain ? paper_index(i, P, L.n_in) : i;
-    if (j >= 0) grad_out[j] = gsum;
-  }
-  if (lr == 0.0f) return;
-  const float t = (float)(*step + 1ull);
-  const float mi = b1 * m[i] + (1.0f - b1) * gsum;
-  const float vi = b2 * v[i] + (1.0f - b2) * gsum * gsum;
-  m[i] = mi;
-  v[i] = vi;
-  const float mh = mi / (1.0f - powf(b1, t));
-  const float vh = vi / (1.0f - powf(b2, t));
-  const float nth = th[i] - lr * mh / (sqrtf(vh) + eps);
-  th[i] = nth;
-  // image entry
-  const bf16 hv = __float2bfloat16_rn(nth);
-  if (i < P.b1) {
-    const int r = i / L.n_in, k = i % L.n_in;
-    reinterpret_cast<bf16*>(img + L.w1)[r * L.ld1 + k] = hv;
-  } else if (i < P.w2) {
-    reinterpret_cast<float*>(img + L.b1)[i - P.b1] = nth;
-  } else if (i < P.b2) {
-    const int j = i - P.w2;
-    reinterpret_cast<bf16*>(img + L.w2)[(j / kHid) * kLdh + j % kHid] = hv;
-  } else if (i < P.w3) {
-    reinterpret_cast<float*>(img + L.b2)[i - P.b2] = nth;
-  } else if (i < P.b3) {
-    const int j = i - P.w3;
-    reinterpret_cast<bf16*>(img + L.w3)[(j / kHid) * kLdh + j % kHid] = hv;
+  return r;
+}
+__device__ __forceinline__ void upd_fail(bool failed, UpdRun& r) {
+  if (!failed) return;
+  r.adam = false;
+  r.sync = r.sync_failed;
+}
+
+// The new value of parameter i from its gradient (th, m, v: its old values).
+__device__ __forceinline__ float upd_adam(const TdUpdate& u, const UpdRun& r, int i, float g, float th, float m,
+                                          float v) {
+  const float mi = kBeta1 * m + (1.0f - kBeta1) * g;
+  const float vi = kBeta2 * v + (1.0f - kBeta2) * g * g;
+  u.m[i] = mi;
+  u.v[i] = vi;
+  const float mh = mi / r.d1;
+  const float vh = vi / r.d2;
+  const float nth = th - u.lr * mh / (sqrtf(vh) + kAdamEps);
+  u.th[i] = nth;
+  return nth;
+}
+__device__ __forceinline__ void upd_grad(const TdUpdate& u, int i, float g) {
+  if (!u.grad) return;
+  const int j = u.L.plain ? paper_index(i, u.P, u.L.n_in) : i;
+  if (j >= 0) u.grad[j] = g;
+}
+
+// Elements (r, k .. k + kN - 1) of a weight matrix (1, 2 or 3), one 2- or
+// 4-byte word, in the image and in every tensor-core copy (k even when kN = 2).
+template <int kW, int kN>
+__device__ __forceinline__ void upd_image(uint8_t* img, uint8_t* tc, const ImgLayout& L, int r, int k, float a,
+                                          float b) {
+  const TcImg T = tc_img(L.k1);
+  const uint32_t v = pack_bf16x2(a, b);
+  auto put = [&](uint8_t* at) {
+    if (kN == 2)
+      *reinterpret_cast<uint32_t*>(at) = v;
+    else
+      *reinterpret_cast<uint16_t*>(at) = (uint16_t)v;
+  };
+  if (kW == 1) {
+    put(img + L.w1 + (r * L.ld1 + k) * 2);
+    put(tc + T.w1 + kmajor_offset(r, k, kHid));
+    put(tc + T.w1h + (uint32_t)((r >> 7) * 128 * L.k1 * 2) + kmajor_offset(r & 127, k, 128));
+  } else if (kW == 2) {
+    put(img + L.w2 + (r * kLdh + k) * 2);
+    put(tc + (r < 128 ? T.w2a : T.w2b) + kmajor_offset(r & 127, k, 128));
+    put(tc + T.w2q + (uint32_t)((r >> 6) * 64 * kHid * 2) + kmajor_offset(r & 63, k, 64));
+    put(tc + T.w2f + kmajor_offset(r, k, kHid));
   } else {
-    reinterpret_cast<float*>(img + L.b3)[i - P.b3] = nth;
+    put(img + L.w3 + (r * kLdh + k) * 2);
+    put(tc + T.w3 + kmajor_offset(r, k, 16));
+  }
+}
+template <int kW, int kN>
+__device__ __forceinline__ void upd_images(const TdUpdate& u, const UpdRun& r, int row, int k, float a, float b) {
+  if (r.adam) upd_image<kW, kN>(u.img, u.tc, u.L, row, k, a, b);
+  if (r.sync) upd_image<kW, kN>(u.img_t, u.tc_t, u.L, row, k, a, b);
+}
+// The image entry of bias i.
+__device__ __forceinline__ void upd_bias(const TdUpdate& u, const UpdRun& r, int i, float a) {
+  const ParamLayout& P = u.P;
+  const int at = i < P.w2 ? u.L.b1 + (i - P.b1) * 4 : i < P.w3 ? u.L.b2 + (i - P.b2) * 4 : u.L.b3 + (i - P.b3) * 4;
+  if (r.adam) *reinterpret_cast<float*>(u.img + at) = a;
+  if (r.sync) *reinterpret_cast<float*>(u.img_t + at) = a;
+}
+// Parameter i on its own (gradient g; th, m, v: its old values): everything
+// above for one element.
+__device__ __forceinline__ void upd_one(const TdUpdate& u, const UpdRun& r, int i, float g, float th, float m,
+                                        float v) {
+  upd_grad(u, i, g);
+  if (!r.adam && !r.sync) return;
+  float a = th;
+  if (r.adam) a = upd_adam(u, r, i, g, th, m, v);
+  if (r.sync) u.tgt[i] = a;
+  const ParamLayout& P = u.P;
+  if (i < P.b1) {
+    upd_images<1, 1>(u, r, i / u.L.n_in, i % u.L.n_in, a, a);
+  } else if (i >= P.w2 && i < P.b2) {
+    upd_images<2, 1>(u, r, (i - P.w2) / kHid, (i - P.w2) % kHid, a, a);
+  } else if (i >= P.w3 && i < P.b3) {
+    upd_images<3, 1>(u, r, (i - P.w3) / kHid, (i - P.w3) % kHid, a, a);
+  } else {
+    upd_bias(u, r, i, a);
+  }
+}
+// Every CTA, at its end: the last one advances the step count (of a step that
+// changed the parameters) and clears the failure word.
+__device__ __forceinline__ void upd_end(const TdUpdate& u, bool failed) {
+  if (!u.step) return;
+  __syncthreads();  // this CTA's reads of *step and *fail are done
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(u.tick, 1u) == gridDim.x - 1u) {
+      if (u.lr != 0.0f && !failed) *u.step += 1ull;
+      *u.fail = 0u;
+      *u.tick = 0u;
+    }
   }
 }
 
-__global__ void k_step_advance(unsigned long long* step, const unsigned* __restrict__ fail) {
-  if (!*fail) *step += 1ull;
+// Gradient rows (one per CTA of the gradient kernel) summed in row order and
+// applied, thread per parameter: the tcgen05 learner and the allocation-free
+// gradient.
+__global__ void __launch_bounds__(256) k_adam(TdUpdate u, const float* __restrict__ partial, int nblk) {
+  pdl_launch_dependents();
+  UpdRun run = upd_begin(u);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  float th = 0.0f, m = 0.0f, v = 0.0f;
+  if (u.lr != 0.0f && i < u.P.total) th = u.th[i], m = u.m[i], v = u.v[i];
+  pdl_wait();
+  const bool failed = *u.fail != 0u;
+  if (i <= u.P.total) {
+    const long long ld = partial_stride(u.P.total);
+    float g = 0.0f;
+#pragma unroll 8
+    for (int b = 0; b < nblk; ++b) g += partial[(long long)b * ld + i];
+    if (failed) g = __int_as_float(0x7fc00000);
+    upd_fail(failed, run);
+    if (i < u.P.total)
+      upd_one(u, run, i, g, th, m, v);
+    else if (u.loss)
+      *u.loss = g / (float)u.batch;
+  }
+  upd_end(u, failed);
 }
 
-// Target network <- online network when the optimiser step count is a
-// multiple of `every` (checked on the device, so the call can be replayed
-// from a CUDA graph).
-__global__ void k_target_sync(const unsigned long long* __restrict__ step, int every, const float* __restrict__ th,
-                              float* __restrict__ tgt, const uint8_t* __restrict__ img, uint8_t* __restrict__ img_t,
-                              int P, int img_words, const uint8_t* __restrict__ tc, uint8_t* __restrict__ tc_t,
-                              int tc_words) {
-  if (every <= 0 || (*step % (unsigned long long)every) != 0ull) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < P) tgt[i] = th[i];
-  if (i < img_words) reinterpret_cast<uint32_t*>(img_t)[i] = reinterpret_cast<const uint32_t*>(img)[i];
-  if (i < tc_words) reinterpret_cast<uint32_t*>(tc_t)[i] = reinterpret_cast<const uint32_t*>(tc)[i];
+// --------------------------------------------------- mma.sync learner
+// Small batches, in 16-sample tiles.  A cluster of three CTAs takes a tile:
+// rank 0 the forward on s, ranks 1 and 2 those of the online and the target
+// network on s' (each CTA holds its network's image for all its tiles); the
+// next-state Q-values go to rank 0 through distributed shared memory, which
+// forms the targets and runs the backward pass.  The weight gradients are
+// sums over the batch of outer products, so rank 0 stores its operands
+// (dZ2, H1, dZ1, X: 8 KB each at most) as the fragments that k_td_update's
+// MMAs take, and no CTA writes a 330 KB gradient of its own.  Bound by the
+// latency of the chain gather - three layers - backward: at batch 256 the
+// two forwards in a row of one kernel, then a forward and the backward of a
+// second, took 30 of the step's 57 us.
+constexpr int kTpRanks = 3;
+constexpr int kVecDb2 = kHid, kVecW3 = 2 * kHid, kVecB3 = kVecW3 + kOut * kHid, kVecHub = kVecB3 + kOut;
+constexpr int kVecLd = (kVecHub + 1 + 31) / 32 * 32;  // db1 | db2 | dW3 | db3 | Huber sum
+constexpr int kFragTile = 16 * 32;                    // 16-byte words of a 16 x 256 operand
+struct TdFrag {
+  uint4* z2;   // [tiles][16 unit blocks][32 lanes]: A fragments of dZ2^T
+  uint4* h1;   // [tiles][16 unit pairs][32]: B fragments of H1
+  uint4* z1;   // [tiles][16][32]: A fragments of dZ1^T
+  uint4* x;    // [tiles][k1 / 16][32]: B fragments of X
+  float* vec;  // [tiles][kVecLd]
+};
+inline size_t td_frag_bytes(int tiles, int k1) {
+  return (size_t)tiles * ((3 * kFragTile + k1 / 16 * 32) * 16 + kVecLd * 4);
 }
+inline TdFrag td_frag(void* base, int tiles, int k1) {
+  TdFrag f;
+  f.z2 = static_cast<uint4*>(base);
+  f.h1 = f.z2 + (size_t)tiles * kFragTile;
+  f.z1 = f.h1 + (size_t)tiles * kFragTile;
+  f.x = f.z1 + (size_t)tiles * kFragTile;
+  f.vec = reinterpret_cast<float*>(f.x + (size_t)tiles * (k1 / 16 * 32));
+  return f;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+// A float into the same variable of another CTA of the cluster.
+__device__ __forceinline__ void st_cluster(float* p, uint32_t rank, float v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
+}
+
+// B fragments of k-step k0 of 16 samples X[16][ldx] (two n-tiles of 8).
+__device__ __forceinline__ void load_x16(uint32_t (&x)[4], const bf16* X, int ldx, int k0, int lane) {
+  ldsm_x4(x, X + ((lane & 7) + (lane >> 4) * 8) * ldx + k0 + ((lane >> 3) & 1) * 8);
+}
+// Hidden layer of 16 samples, 16 warps of 16 units: the weights are the A
+// operand, so that each is read from shared memory once per tile.
+__device__ __forceinline__ void tp_layer(const bf16* X, int ldx, int nks, const bf16* W, int ldw, const float* b,
+                                         bf16* H, int warp, int lane) {
+  const int g = lane >> 2, q = lane & 3, u0 = 16 * warp;
+  float c[2][4] = {};
+#pragma unroll 4
+  for (int ks = 0; ks < nks; ++ks) {
+    uint32_t a[4], x[4];
+    load_a_row(a, W, ldw, u0, 16 * ks, lane);
+    load_x16(x, X, ldx, 16 * ks, lane);
+    mma_bf16(c[0], a, x[0], x[1]);
+    mma_bf16(c[1], a, x[2], x[3]);
+  }
+  const float bl = b[u0 + g], bh = b[u0 + g + 8];
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      H[(8 * t + 2 * q + (j & 1)) * kLdh + u0 + g + (j >> 1) * 8] =
+          __float2bfloat16_rn(fmaxf(c[t][j] + (j >> 1 ? bh : bl), 0.f));
+}
+
+// dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
+__device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w, d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
+}
+
+__global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
+    k_td_tile(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, ImgLayout L, ReplayDev rp,
+              unsigned long long seed, const unsigned long long* __restrict__ step, int batch, float gamma, TdFrag f,
+              unsigned* __restrict__ fail) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint8_t* sw = smem;
+  bf16* X = reinterpret_cast<bf16*>(smem + L.bytes);
+  bf16* H1 = X + kTile * L.ld1;
+  bf16* H2 = H1 + kTile * kLdh;  // becomes dZ1
+  bf16* Z2 = H2 + kTile * kLdh;
+  float* O = reinterpret_cast<float*>(Z2 + kTile * kLdh);
+  float* DO = O + kTile * kOutPad;  // dL/d(head outputs) [16][8]
+  __shared__ uint64_t bar_w1, bar_w2;
+  __shared__ float next_q[2][2][kTile * kOutPad];  // rank 0: head outputs of s' by tile parity and network
+  __shared__ int rows[kTile];
+  __shared__ float hub[kTile];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q = lane & 3, g = lane >> 2;
+  const uint32_t rank = cluster_rank();
+  const int ntiles = (batch + kTile - 1) / kTile, stride = (int)gridDim.x / kTpRanks;
+  cluster_arrive();  // every CTA of the cluster has started before the first remote store
+  if (tid == 0) {
+    mbar_init(&bar_w1, 1);
+    mbar_init(&bar_w2, 1);
+  }
+  pdl_wait();
+  pdl_launch_dependents();
+  __syncthreads();
+  if (tid == 0) {
+    // layer 1 starts when W1 and the vectors behind W2 are here
+    const uint8_t* src = rank == 2 ? img_t : img;
+    mbar_expect_tx(&bar_w1, (uint32_t)(L.w2 + L.bytes - L.w3));
+    bulk_g2s(sw, src, (uint32_t)L.w2, &bar_w1);
+    bulk_g2s(sw + L.w3, src + L.w3, (uint32_t)(L.bytes - L.w3), &bar_w1);
+    mbar_expect_tx(&bar_w2, (uint32_t)(L.w3 - L.w2));
+    for (int off = L.w2; off < L.w3; off += kStageChunk)
+      bulk_g2s(sw + off, src + off, (uint32_t)min(kStageChunk, L.w3 - off), &bar_w2);
+  }
+  const QW w = qw_at(sw, L);
+  const unsigned long long tstep = *step;
+  bool ok = true, first = true;
+  for (int tile = (int)blockIdx.x / kTpRanks, it = 0; tile < ntiles; tile += stride, ++it) {
+    {
+      const int i = tile * kTile + warp;
+      const int e = i < batch ? (int)sample_entry(seed, tstep, i, rp) : -1;
+      const float* src = (rank == 0 ? rp.s : rp.s2) + (long long)e * rp.obs_dim;
+      for (int k = lane; k < L.ld1; k += 32)
+        X[warp * L.ld1 + k] = __float2bfloat16_rn(e >= 0 && k < rp.obs_dim ? src[k] : 0.0f);
+      if (lane == 0) rows[warp] = e;
+    }
+    ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w1, 0u, kTcTries)));
+    // this sample's reward, flag and action on their way during the forward
+    int e = -1, act = 0;
+    float rwd = 0.0f, nt = 1.0f;
+    if (rank == 0 && tid < kTile) {
+      e = rows[tid];
+      if (e >= 0) {
+        act = rp.a[e];
+        rwd = rp.r[e];
+        nt = rp.term[e] ? 0.0f : 1.0f;
+      }
+    }
+    if (ok) tp_layer(X, L.ld1, L.k1 / 16, w.W1, L.ld1, w.b1, H1, warp, lane);
+    ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w2, 0u, kTcTries)));
+    first = false;
+    if (ok) tp_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, warp, lane);
+    __syncthreads();
+    if (ok && warp == 0) head_layer(H2, w, O, 0, lane);
+    __syncthreads();
+    if (it == 0) cluster_wait();  // the start's arrival
+    if (rank != 0 && tid < kTile * kOutPad)
+      st_cluster(&next_q[it & 1][rank - 1][tid], 0u, ok ? O[tid] : __int_as_float(0x7fc00000));
+    cluster_arrive();
+    cluster_wait();
+    if (rank != 0) continue;
+    if (!ok) continue;
+    // y = r + gamma (1 - term) Q_target(s', argmax_a Q_online(s', a));
+    // dL/dQ(s, a) = clip(Q(s, a) - y, -1, 1) / B, back through the head's combine
+    if (tid < kTile) {
+      float qv[5], qn[5];
+      const int astar = (int)greedy_action(&next_q[it & 1][0][tid * kOutPad], nullptr, L.plain);
+      greedy_action(&next_q[it & 1][1][tid * kOutPad], qn, L.plain);
+      greedy_action(O + tid * kOutPad, qv, L.plain);
+      float* dO = DO + tid * kOutPad;
+      float gq = 0.0f, hl = 0.0f;
+#pragma unroll
+      for (int k = 0; k < kOutPad; ++k) dO[k] = 0.0f;
+      if (e >= 0) {
+        float qs = qn[0], qa = qv[0];
+#pragma unroll
+        for (int k = 1; k < 5; ++k) {
+          if (k == astar) qs = qn[k];
+          if (k == act) qa = qv[k];
+        }
+        const float y = rwd + gamma * nt * qs;
+        float d;
+        if (act >= 5) {
+          // outside the action table: no loss term, and no update this step
+          atomicOr(fail, kTdFailAction);
+          act = 0;
+          d = __int_as_float(0x7fc00000);
+        } else {
+          d = qa - y;
+        }
+        const float ad = fabsf(d);
+        hl = ad <= 1.0f ? 0.5f * d * d : ad - 0.5f;
+        // a NaN target stays NaN through the clip
+        gq = (isnan(d) ? d : fminf(fmaxf(d, -1.0f), 1.0f)) / (float)batch;
+        if (L.plain) {
+          for (int k = 0; k < 5; ++k) dO[k] = k == act ? gq : 0.0f;
+        } else {
+          dO[0] = gq;
+          for (int k = 0; k < 5; ++k) dO[1 + k] = (k == act ? gq : 0.0f) - gq / 5.0f;
+        }
+      }
+      hub[tid] = hl;
+    }
+    __syncthreads();
+    float* vec = f.vec + (long long)tile * kVecLd;
+    // the head's gradient on the CUDA cores (FP32), half of the threads each:
+    // dW3[o][j] = sum_s dO[s][o] H2[s][j] and db3, the Huber sum; dH2 = dO W3
+    // masked by the ReLU into dZ2, db2
+    if (tid < kHid) {
+      float acc[kOut];
+#pragma unroll
+      for (int o = 0; o < kOut; ++o) acc[o] = 0.0f;
+#pragma unroll 4
+      for (int s = 0; s < kTile; ++s) {
+        const float h = __bfloat162float(H2[s * kLdh + tid]);
+        float d[kOutPad];
+        load_do(DO + s * kOutPad, d);
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) acc[o] += d[o] * h;
+      }
+#pragma unroll
+      for (int o = 0; o < kOut; ++o) vec[kVecW3 + o * kHid + tid] = acc[o];
+      if (tid < kOut) {
+        float b3 = 0.0f;
+        for (int s = 0; s < kTile; ++s) b3 += DO[s * kOutPad + tid];
+        vec[kVecB3 + tid] = b3;
+      }
+      if (tid == kHid - 1) {
+        float h = 0.0f;
+        for (int s = 0; s < kTile; ++s) h += hub[s];
+        vec[kVecHub] = h;
+      }
+    } else {
+      const int j = tid - kHid;
+      float w3[kOut];
+#pragma unroll
+      for (int o = 0; o < kOut; ++o) w3[o] = __bfloat162float(w.W3[o * kLdh + j]);
+      float db2 = 0.0f;
+#pragma unroll 4
+      for (int s = 0; s < kTile; ++s) {
+        float dh = 0.0f, d[kOutPad];
+        load_do(DO + s * kOutPad, d);
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) dh += d[o] * w3[o];
+        const float v = __bfloat162float(H2[s * kLdh + j]) > 0.0f ? dh : 0.0f;
+        Z2[s * kLdh + j] = __float2bfloat16_rn(v);
+        db2 += v;
+      }
+      vec[kVecDb2 + j] = db2;
+    }
+    __syncthreads();
+    uint32_t r4[4];
+    load_a_col(r4, Z2, kLdh, 16 * warp, 0, lane);
+    f.z2[((long long)tile * 16 + warp) * 32 + lane] = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+    ldsm_x4_t(r4, H1 + ((lane & 7) + ((lane >> 3) & 1) * 8) * kLdh + 16 * warp + (lane >> 4) * 8);
+    f.h1[((long long)tile * 16 + warp) * 32 + lane] = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+    // dH1 = dZ2 W2, masked by the ReLU into dZ1 (over H2), db1 from the FP32 values
+    {
+      const int u0 = 16 * warp;
+      float c[2][4] = {};
+#pragma unroll 4
+      for (int k0 = 0; k0 < kHid; k0 += 16) {
+        uint32_t a[4], x[4];
+        load_a_col(a, w.W2, kLdh, u0, k0, lane);
+        load_x16(x, Z2, kLdh, k0, lane);
+        mma_bf16(c[0], a, x[0], x[1]);
+        mma_bf16(c[1], a, x[2], x[3]);
+      }
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int at = (8 * t + 2 * q + (j & 1)) * kLdh + u0 + g + (j >> 1) * 8;
+          if (!(__bfloat162float(H1[at]) > 0.f)) c[t][j] = 0.f;
+          H2[at] = __float2bfloat16_rn(c[t][j]);
+        }
+      // the 16 samples of a unit: s and s + 8, then a tree over s mod 8
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float v = (c[0][2 * h] + c[1][2 * h]) + (c[0][2 * h + 1] + c[1][2 * h + 1]);
+        v += __shfl_xor_sync(kFull, v, 1);
+        v += __shfl_xor_sync(kFull, v, 2);
+        if (q == 0) vec[u0 + g + 8 * h] = v;
+      }
+    }
+    __syncthreads();
+    load_a_col(r4, H2, kLdh, 16 * warp, 0, lane);
+    f.z1[((long long)tile * 16 + warp) * 32 + lane] = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+    const int nx = L.k1 / 16;
+    if (warp < nx) {
+      ldsm_x4_t(r4, X + ((lane & 7) + ((lane >> 3) & 1) * 8) * L.ld1 + 16 * warp + (lane >> 4) * 8);
+      f.x[((long long)tile * nx + warp) * 32 + lane] = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+    }
+    __syncthreads();  // X and the activations are rewritten by the next tile
+  }
+  if (!ok && tid == 0) {
+    // no update this step; a copy that timed out may still be writing: one
+    // more bounded wait for each before the CTA exits
+    atomicOr(fail, kTdFailCopy);
+    mbar_wait(&bar_w1, 0u, kTcTries);
+    mbar_wait(&bar_w2, 0u, kTcTries);
+  }
+}
+
+// The weight gradients from k_td_tile's fragments, and the update, one item per
+// CTA: a 16 x 16 block of W2 or W1 (per tile two MMAs, a 16-sample outer
+// product from zero), or 64 entries of the vectors.  Every warp takes a run of
+// consecutive tiles.  Up to 16 tiles each tile's product has a slot of its own
+// in shared memory (four warps, one round of loads each); above, each warp adds
+// its tiles up (eight warps).  A thread then adds the slots of two neighbouring
+// parameters in order, in FP32, and updates both.  No gradient goes through
+// memory: bound by the latency of the loads (old values before the wait) and of
+// one Adam update; with one warp a block that had eight updates in a row
+// it took 16 K cycles at batch 256, now 4 K (a whole step 23.0 -> 16.6 us).
+constexpr int kTuItem = 256;  // floats of an item
+constexpr int kTuSlots = 16;
+template <int kWarps, bool kSlots>
+__global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f, int ntiles) {
+  __shared__ float sum[kSlots ? kTuSlots : kWarps][kTuItem];
+  pdl_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
+  const int nx = u.L.k1 / 16, n2 = 256, n1 = 16 * nx;
+  const int item = blockIdx.x;
+  const bool w2 = item < n2, mat = item < n2 + n1;
+  const int mb = w2 ? item >> 4 : (item - n2) / nx, nb = w2 ? item & 15 : (item - n2) % nx;
+  // this thread's parameters: columns k, k + 1 of row r, or vector entry ve
+  const int r = mb * 16 + t / 8, k = nb * 16 + 2 * (t % 8), ve = (item - n2 - n1) * 64 + t;
+  int at = 0;
+  bool live[2];
+  if (mat) {
+    at = w2 ? u.P.w2 + r * kHid + k : u.P.w1 + r * u.L.n_in + k;
+    live[0] = t < 128 && (w2 || k < u.L.n_in);
+    live[1] = t < 128 && (w2 || k + 1 < u.L.n_in);
+  } else {
+    at = ve < kVecDb2 ? u.P.b1 + ve : ve < kVecW3 ? u.P.b2 + (ve - kVecDb2)
+                                    : ve < kVecB3 ? u.P.w3 + (ve - kVecW3) : u.P.b3 + (ve - kVecB3);
+    live[0] = t < 64 && ve < kVecHub;
+    live[1] = false;
+  }
+  UpdRun run = upd_begin(u);
+  // the old values (nothing before this launch writes them) before the wait
+  float th[2] = {}, m[2] = {}, v[2] = {};
+  if (u.lr != 0.0f) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (live[h]) th[h] = u.th[at + h], m[h] = u.m[at + h], v[h] = u.v[at + h];
+  }
+  pdl_wait();
+  const unsigned fail = __ldcg(u.fail);
+  const int per = (ntiles + kWarps - 1) / kWarps, t0 = warp * per, t1 = min(ntiles, t0 + per);
+  if (mat) {
+    const uint4* fa = (w2 ? f.z2 : f.z1) + mb * 32 + lane;
+    const uint4* fb = (w2 ? f.h1 : f.x) + nb * 32 + lane;
+    const int lb = w2 ? kFragTile : nx * 32;
+    const int g = lane >> 2, q = lane & 3;
+    float acc[2][4] = {};
+    auto put = [&](float* s) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          *reinterpret_cast<float2*>(s + (g + 8 * j) * 16 + 8 * h + 2 * q) = make_float2(acc[h][2 * j], acc[h][2 * j + 1]);
+    };
+#pragma unroll 4
+    for (int i = t0; i < t1; ++i) {
+      const uint4 a = __ldcg(fa + (long long)i * kFragTile), b = __ldcg(fb + (long long)i * lb);
+      const uint32_t ar[4] = {a.x, a.y, a.z, a.w};
+      float d[2][4] = {};
+      mma_bf16(d[0], ar, b.x, b.y);
+      mma_bf16(d[1], ar, b.z, b.w);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[h][j] = kSlots ? d[h][j] : acc[h][j] + d[h][j];
+      if (kSlots) put(sum[i]);
+    }
+    if (!kSlots) put(sum[warp]);
+  } else {
+    const int e = (item - n2 - n1) * 64 + 2 * lane;
+    float2 acc = make_float2(0.0f, 0.0f);
+    if (e <= kVecHub) {
+#pragma unroll 4
+      for (int i = t0; i < t1; ++i) {
+        const float2 x = __ldcg(reinterpret_cast<const float2*>(f.vec + (long long)i * kVecLd + e));
+        acc.x = kSlots ? x.x : acc.x + x.x;
+        acc.y = kSlots ? x.y : acc.y + x.y;
+        if (kSlots) *reinterpret_cast<float2*>(sum[i] + 2 * lane) = acc;
+      }
+    }
+    if (!kSlots) *reinterpret_cast<float2*>(sum[warp] + 2 * lane) = acc;
+  }
+  __syncthreads();
+  const bool failed = fail != 0u;
+  upd_fail(failed, run);
+  const int slots = kSlots ? ntiles : kWarps;
+  auto total = [&](int i) {
+    float g = sum[0][i];
+#pragma unroll 4
+    for (int s = 1; s < slots; ++s) g += sum[s][i];
+    return failed ? __int_as_float(0x7fc00000) : g;
+  };
+  if (mat) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!live[h]) continue;
+      const float g = total(2 * t + h);
+      upd_grad(u, at + h, g);
+      if (run.adam) th[h] = upd_adam(u, run, at + h, g, th[h], m[h], v[h]);
+      if (run.sync) u.tgt[at + h] = th[h];
+    }
+    if (live[0]) {
+      // the padding column beside an odd last input stays zero
+      if (w2)
+        upd_images<2, 2>(u, run, r, k, th[0], th[1]);
+      else
+        upd_images<1, 2>(u, run, r, k, th[0], th[1]);
+    }
+  } else if (live[0]) {
+    upd_one(u, run, at, total(t), th[0], m[0], v[0]);
+  } else if (ve == kVecHub && t < 64 && u.loss) {
+    *u.loss = total(t) / (float)u.batch;
+  }
+  upd_end(u, failed);
+}
+inline int td_update_items(int k1) { return 256 + 16 * (k1 / 16) + (kVecHub + 1 + 63) / 64; }
 
 
 // ------------------------------------------------ tcgen05 learner (batch >= 128)
@@ -2008,8 +2486,7 @@ __global__ void __launch_bounds__(kLtThreads, 1)
     k_td_tc(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, const uint8_t* __restrict__ timg,
             const uint8_t* __restrict__ timg_t, ImgLayout L, ParamLayout P, ReplayDev rp, unsigned long long seed,
             const unsigned long long* __restrict__ step, int batch, float gamma, float* __restrict__ q2,
-            int* __restrict__ idx, unsigned* __restrict__ sync, float* __restrict__ partial,
-            unsigned* __restrict__ fail) {
+            unsigned* __restrict__ sync, float* __restrict__ partial, unsigned* __restrict__ fail) {
   extern __shared__ __align__(1024) uint8_t tsm[];
   __shared__ uint64_t bar_ld[2], bar_mm[2], bar_layer;
   __shared__ uint32_t tslot;
@@ -2067,7 +2544,6 @@ __global__ void __launch_bounds__(kLtThreads, 1)
         const int i = tile * kLtRows + tid;
         const int e = i < batch ? (int)sample_entry(seed, tstep, i, rp) : -1;
         rows_sh[tid] = e;
-        if (net == 0 && i < batch) idx[i] = e;
       }
       __syncthreads();
       lt_load_x(xs, rp.s2, rows_sh, L.n_in, L.k1, tid);
@@ -2396,21 +2872,12 @@ int set_smem_attr(const void* fn, size_t bytes) {
   return SG_OK;
 }
 
-// The online weights' copy in the tensor cores' layout follows every change
-// of the online image (stream-ordered, so also inside captured graphs).
-int refresh_tc_image(sg_qnet* q, cudaStream_t st) {
-  k_tc_image<<<44, 256, 0, st>>>(q->img, q->IL, q->img_tc);
-  SG_CUDA(cudaGetLastError());
-  return SG_OK;
-}
-
 int rebuild_image(sg_qnet* q, const float* th, uint8_t* img, cudaStream_t st) {
   const int n = image_elems(q->IL);
   k_build_image<<<(n + 255) / 256, 256, 0, st>>>(th, img, q->IL, q->PL);
   SG_CUDA(cudaGetLastError());
-  if (img == q->img) return refresh_tc_image(q, st);
-  // the target image's tensor-core copy (read by the tcgen05 learner)
-  k_tc_image<<<44, 256, 0, st>>>(q->img_t, q->IL, q->img_tc_t);
+  // the copy in the tensor cores' layout (a TD step updates both in place)
+  k_tc_image<<<44, 256, 0, st>>>(img, q->IL, img == q->img ? q->img_tc : q->img_tc_t);
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
@@ -2426,8 +2893,7 @@ void free_qnet(sg_qnet* q) {
   cudaFree(q->step);
   cudaFree(q->td_fail);
   cudaFree(q->partial);
-  cudaFree(q->y);
-  cudaFree(q->idx);
+  cudaFree(q->frag);
   cudaFree(q->img_tc);
   cudaFree(q->img_tc_t);
   cudaFree(q->q2);
@@ -2460,7 +2926,9 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   q->max_batch = (max_batch + kTile - 1) / kTile * kTile;
   cudaGetDevice(&q->device);
   const size_t P = (size_t)q->PL.total;
-  const size_t nblk = (size_t)q->max_batch / kTile;
+  const bool large = q->max_batch >= kLtMinBatch;
+  const size_t tiles16 = (size_t)(std::min(q->max_batch, kLtMinBatch) + kTile - 1) / kTile;
+  const size_t tiles128 = large ? (size_t)(q->max_batch + kLtRows - 1) / kLtRows : 0;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void** p, size_t b) {
     if (e == cudaSuccess) e = cudaMalloc(p, b);
@@ -2472,10 +2940,9 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   alloc((void**)&q->img, (size_t)q->IL.bytes);
   alloc((void**)&q->img_t, (size_t)q->IL.bytes);
   alloc((void**)&q->step, 8);
-  alloc((void**)&q->td_fail, 4);
-  alloc((void**)&q->partial, nblk * partial_stride(P) * 4);
-  alloc((void**)&q->y, (size_t)q->max_batch * 4);
-  alloc((void**)&q->idx, (size_t)q->max_batch * 4);
+  alloc((void**)&q->td_fail, 8);
+  alloc(&q->frag, td_frag_bytes((int)tiles16, q->IL.k1));
+  if (large) alloc((void**)&q->partial, tiles128 * partial_stride(P) * 4);
   alloc((void**)&q->img_tc, tc_img(q->IL.k1).bytes);
   alloc((void**)&q->img_tc_t, tc_img(q->IL.k1).bytes);
   alloc((void**)&q->q2, (size_t)2 * q->max_batch * 5 * 4);
@@ -2490,7 +2957,7 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   if (e == cudaSuccess) e = cudaMemset(q->adam_m, 0, P * 4);
   if (e == cudaSuccess) e = cudaMemset(q->adam_v, 0, P * 4);
   if (e == cudaSuccess) e = cudaMemset(q->step, 0, 8);
-  if (e == cudaSuccess) e = cudaMemset(q->td_fail, 0, 4);
+  if (e == cudaSuccess) e = cudaMemset(q->td_fail, 0, 8);
   if (e == cudaSuccess) e = cudaMemset(q->img, 0, (size_t)q->IL.bytes);
   if (e == cudaSuccess) e = cudaMemset(q->img_t, 0, (size_t)q->IL.bytes);
   if (e == cudaSuccess) {
@@ -2517,11 +2984,25 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
       (rc = set_smem_attr((const void*)k_rollout_q<2, false>, fwd_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<1, true>, fwd_smem(widest))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<2, true>, fwd_smem(widest, 32))) ||
-      (rc = set_smem_attr((const void*)k_td_target, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_td_grad, grad_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_td_tile, grad_smem(widest))) ||
       (rc = set_smem_attr((const void*)k_td_tc, kTcSmemLaunch))) {
     free_qnet(q);
     return rc;
+  }
+  // clusters of the small-batch learner that run at once: more tiles than
+  // that loop over a resident grid, which stages its weights once
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(kTpRanks * 64);
+  lc.blockDim = dim3(kThreads);
+  lc.dynamicSmemBytes = grad_smem(q->IL);
+  cudaLaunchAttribute la[1];
+  la[0].id = cudaLaunchAttributeClusterDimension;
+  la[0].val.clusterDim.x = kTpRanks, la[0].val.clusterDim.y = 1, la[0].val.clusterDim.z = 1;
+  lc.attrs = la;
+  lc.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&q->td_clusters, k_td_tile, &lc) != cudaSuccess || q->td_clusters < 1) {
+    cudaGetLastError();
+    q->td_clusters = std::max(1, q->sms / (kTpRanks + 1));
   }
   *out = q;
   return SG_OK;
@@ -2673,6 +3154,8 @@ extern "C" int sg_replay_create(int32_t slots_per_env, int32_t n_envs, int32_t o
   r->d.n_envs = n_envs;
   r->d.obs_dim = obs_dim;
   r->d.reserve = reserve_slots;
+  r->d.inv_full = ~0ull / ((unsigned long long)(slots_per_env - reserve_slots) * (unsigned long long)n_envs);
+  r->d.inv_slots = ~0ull / (unsigned long long)slots_per_env;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void** p, size_t b) {
     if (e == cudaSuccess) e = cudaMalloc(p, b);
@@ -2876,44 +3359,37 @@ extern "C" int sg_td_train_step(sg_qnet_t q, sg_replay_t rp, int32_t batch, floa
   SG_RANGE("sg_td_train_step");
   if (!q || !rp || batch < 1 || batch > q->max_batch || rp->d.obs_dim != q->n_in) return SG_E_INVAL;
   if (!(gamma >= 0.0f && gamma <= 1.0f) || !(lr >= 0.0f)) return SG_E_INVAL;
-  SG_CUDA(cudaMemsetAsync(q->td_fail, 0, 4, stream));
-  int nblk;
+  TdUpdate u;
+  u.th = q->master, u.m = q->adam_m, u.v = q->adam_v, u.tgt = q->target;
+  u.img = q->img, u.img_t = q->img_t, u.tc = q->img_tc, u.tc_t = q->img_tc_t;
+  u.step = q->step, u.fail = q->td_fail, u.tick = q->td_fail + 1;
+  u.lr = lr, u.every = target_every, u.loss = loss_dev, u.grad = grad_dev, u.batch = batch;
+  u.P = q->PL, u.L = q->IL;
+  const int cap = q->lim_learner > 0 ? std::min(q->lim_learner, q->sms) : q->sms;
   if (batch >= kLtMinBatch) {
     // tcgen05 learner: 128-sample tiles, one partial gradient row per tile
     const int ntiles = (batch + kLtRows - 1) / kLtRows;
-    nblk = ntiles;
     SG_CUDA(cudaMemsetAsync(q->td_sync, 0, (size_t)(1 + ntiles) * 4, stream));
-    const int cap = q->lim_learner > 0 ? std::min(q->lim_learner, q->sms) : q->sms;
     k_td_tc<<<std::min(4 * ntiles, cap), kLtThreads, kTcSmemLaunch, stream>>>(
-        q->img, q->img_t, q->img_tc, q->img_tc_t, q->IL, q->PL, rp->d, seed, q->step, batch, gamma, q->q2, q->idx,
-        q->td_sync, q->partial, q->td_fail);
+        q->img, q->img_t, q->img_tc, q->img_tc_t, q->IL, q->PL, rp->d, seed, q->step, batch, gamma, q->q2, q->td_sync,
+        q->partial, q->td_fail);
     SG_CUDA(cudaGetLastError());
-  } else {
-    // mma.sync learner: 16-sample tiles
-    nblk = (batch + kTile - 1) / kTile;
-    k_td_target<<<nblk, kThreads, fwd_smem(q->IL), stream>>>(q->img, q->img_t, q->IL, rp->d, seed, q->step, batch,
-                                                              gamma, q->y, q->idx, q->td_fail);
-    SG_CUDA(cudaGetLastError());
-    k_td_grad<<<nblk, kThreads, grad_smem(q->IL), stream>>>(q->img, q->IL, q->PL, rp->d, q->idx, q->y, batch,
-                                                            q->partial, q->td_fail);
-    SG_CUDA(cudaGetLastError());
+    SG_CUDA(sg_launch_pdl(k_adam, (q->PL.total + 256) / 256, 256, 0, stream, u, (const float*)q->partial, ntiles));
+    return SG_OK;
   }
-  const int P = q->PL.total;
-  k_adam<<<(P + 255) / 256, 256, 0, stream>>>(q->master, q->adam_m, q->adam_v, q->partial, nblk, q->PL, q->IL, q->img,
-                                               q->step, lr, 0.9f, 0.999f, 1e-8f, loss_dev, grad_dev, batch,
-                                               q->td_fail);
-  SG_CUDA(cudaGetLastError());
-  if (int rc = refresh_tc_image(q, stream)) return rc;
-  if (lr > 0.0f) {
-    k_step_advance<<<1, 1, 0, stream>>>(q->step, q->td_fail);
-    SG_CUDA(cudaGetLastError());
-    const int words = q->IL.bytes / 4;
-    const int tc_words = (int)(tc_img(q->IL.k1).bytes / 4);
-    const int n = std::max(P, std::max(words, tc_words));
-    k_target_sync<<<(n + 255) / 256, 256, 0, stream>>>(q->step, target_every, q->master, q->target, q->img, q->img_t,
-                                                        P, words, q->img_tc, q->img_tc_t, tc_words);
-    SG_CUDA(cudaGetLastError());
-  }
+  // mma.sync learner: 16-sample tiles, a cluster each, evenly over the rounds
+  const int ntiles = (batch + kTile - 1) / kTile;
+  const int fit = std::max(1, std::min(q->td_clusters, cap / kTpRanks));
+  const int rounds = (ntiles + fit - 1) / fit, clusters = (ntiles + rounds - 1) / rounds;
+  const TdFrag f = td_frag(q->frag, ntiles, q->IL.k1);
+  SG_CUDA(sg_launch_pdl(k_td_tile, clusters * kTpRanks, kThreads, grad_smem(q->IL), stream, (const uint8_t*)q->img,
+                        (const uint8_t*)q->img_t, q->IL, rp->d, (unsigned long long)seed,
+                        (const unsigned long long*)q->step, (int)batch, gamma, f, q->td_fail));
+  const int items = td_update_items(q->IL.k1);
+  if (ntiles <= kTuSlots)
+    SG_CUDA(sg_launch_pdl(k_td_update<4, true>, items, 128, 0, stream, u, f, ntiles));
+  else
+    SG_CUDA(sg_launch_pdl(k_td_update<8, false>, items, 256, 0, stream, u, f, ntiles));
   return SG_OK;
 }
 
@@ -3054,9 +3530,12 @@ extern "C" int sg_td_grad_noalloc(const float* params_dev, const float* target_p
   SG_CUDA(cudaGetLastError());
   k_td_grad<<<nblk, kThreads, grad_smem(IL), stream>>>(img, IL, PL, b, idx, y, batch, partial, fail);
   SG_CUDA(cudaGetLastError());
-  k_adam<<<(PL.total + 255) / 256, 256, 0, stream>>>(nullptr, nullptr, nullptr, partial, nblk, PL, IL, nullptr,
-                                                      nullptr, 0.0f, 0.9f, 0.999f, 1e-8f, loss_dev, grad_dev, batch,
-                                                      fail);
+  TdUpdate u;
+  std::memset(&u, 0, sizeof(u));  // no parameters: loss and gradient only
+  u.fail = fail;
+  u.loss = loss_dev, u.grad = grad_dev, u.batch = batch;
+  u.P = PL, u.L = IL;
+  k_adam<<<(PL.total + 256) / 256, 256, 0, stream>>>(u, partial, nblk);
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
