@@ -121,7 +121,7 @@ struct ReplayDev {
   uint8_t* a;            // [cap]
   float* r;              // [cap]
   uint8_t* term;         // [cap] collided or arrived
-  unsigned long long* steps;  // vectorized steps recorded so far
+  unsigned long long* steps;  // vectorized steps recorded so far; behind it the CTA count of replay_advance
   int slots, n_envs, obs_dim;
   unsigned long long inv_full, inv_slots;  // floor((2^64 - 1) / (sampled entries of a full ring, slots))
   int reserve;           // newest slots the learner never samples (an actor may be writing them)
@@ -227,13 +227,15 @@ __device__ __forceinline__ void stage_image(uint8_t* dst, const uint8_t* __restr
 // for its phase `parity` (bounded).  CTA-wide; false when the copy did not
 // complete within the bound.
 constexpr int kStageChunk = 32 * 1024;
+__device__ __forceinline__ void stage_image_issue(uint8_t* dst, const uint8_t* __restrict__ src, int bytes,
+                                                  uint64_t* bar) {
+  mbar_expect_tx(bar, (uint32_t)bytes);
+  for (int off = 0; off < bytes; off += kStageChunk)
+    bulk_g2s(dst + off, src + off, (uint32_t)min(kStageChunk, bytes - off), bar);
+}
 __device__ __forceinline__ bool stage_image_bulk(uint8_t* dst, const uint8_t* __restrict__ src, int bytes,
                                                  uint64_t* bar, uint32_t parity, uint32_t tries) {
-  if (threadIdx.x == 0) {
-    mbar_expect_tx(bar, (uint32_t)bytes);
-    for (int off = 0; off < bytes; off += kStageChunk)
-      bulk_g2s(dst + off, src + off, (uint32_t)min(kStageChunk, bytes - off), bar);
-  }
+  if (threadIdx.x == 0) stage_image_issue(dst, src, bytes, bar);
   return __syncthreads_and(mbar_wait(bar, parity, tries));
 }
 
@@ -260,78 +262,61 @@ __device__ __forceinline__ QW qw_at(const uint8_t* base, const ImgLayout& L) {
   return w;
 }
 
-// One hidden layer for R = 16 * MT rows and R warps: Hout[R][256] =
-// bf16(ReLU(Xin * W^T + b)).  The 32 output n-tiles of 8 columns are spread
-// over the warps (32 / R per warp), each warp covering all MT m-tiles so
-// that one B fragment serves MT MMAs.
-template <int MT>
-__device__ __forceinline__ void hidden_layer(const bf16* Xin, int ldx, int kdim, const bf16* W, int ldw,
-                                             const float* b, bf16* Hout, int warp, int lane) {
-  constexpr int kWarps = 16 * MT;
-  constexpr int kNt = 32 / kWarps;
-  const int g = lane >> 2, q = lane & 3;
-#pragma unroll
-  for (int t = 0; t < kNt; ++t) {
-    const int n0 = 8 * (warp + kWarps * t);
-    float acc[MT][4];
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt) acc[mt][0] = acc[mt][1] = acc[mt][2] = acc[mt][3] = 0.f;
-    for (int k0 = 0; k0 < kdim; k0 += 16) {
-      uint32_t b0, b1;
-      load_b_col(b0, b1, W, ldw, k0, n0, lane);
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt) {
-        uint32_t a[4];
-        load_a_row(a, Xin, ldx, 16 * mt, k0, lane);
-        mma_bf16(acc[mt], a, b0, b1);
-      }
-    }
-    const int n = n0 + 2 * q;
-    const float bn = b[n], bn1 = b[n + 1];
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-      const int r0 = 16 * mt + g;
-      *reinterpret_cast<uint32_t*>(Hout + r0 * kLdh + n) =
-          pack_bf16x2(fmaxf(acc[mt][0] + bn, 0.f), fmaxf(acc[mt][1] + bn1, 0.f));
-      *reinterpret_cast<uint32_t*>(Hout + (r0 + 8) * kLdh + n) =
-          pack_bf16x2(fmaxf(acc[mt][2] + bn, 0.f), fmaxf(acc[mt][3] + bn1, 0.f));
-    }
+// B fragments of k-step k0 of 16 samples X[16][ldx] (two n-tiles of 8).
+__device__ __forceinline__ void load_x16(uint32_t (&x)[4], const bf16* X, int ldx, int k0, int lane) {
+  ldsm_x4(x, X + ((lane & 7) + (lane >> 4) * 8) * ldx + k0 + ((lane >> 3) & 1) * 8);
+}
+// One hidden layer of 16 rows by 16 warps of 16 units: H[16][256] = bf16(ReLU(X
+// W^T + b)).  Bound by shared-memory reads: with the weights as the A operand
+// each is read once and the 16 rows once per warp (256 KB a layer of 256
+// inputs); with the rows as A and 8 units per warp and pass it was 384 KB.
+__device__ __forceinline__ void hidden_layer(const bf16* X, int ldx, int nks, const bf16* W, int ldw, const float* b,
+                                         bf16* H, int warp, int lane) {
+  const int g = lane >> 2, q = lane & 3, u0 = 16 * warp;
+  float c[2][4] = {};
+#pragma unroll 4
+  for (int ks = 0; ks < nks; ++ks) {
+    uint32_t a[4], x[4];
+    load_a_row(a, W, ldw, u0, 16 * ks, lane);
+    load_x16(x, X, ldx, 16 * ks, lane);
+    mma_bf16(c[0], a, x[0], x[1]);
+    mma_bf16(c[1], a, x[2], x[3]);
   }
+  const float bl = b[u0 + g], bh = b[u0 + g + 8];
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      H[(8 * t + 2 * q + (j & 1)) * kLdh + u0 + g + (j >> 1) * 8] =
+          __float2bfloat16_rn(fmaxf(c[t][j] + (j >> 1 ? bh : bl), 0.f));
 }
 
-// Head for the 16 rows of m-tile mt (one warp): O[16][8] = H2 * W3^T + b3
-// (FP32), two accumulator chains (even / odd k-steps) summed in a fixed order.
-__device__ __forceinline__ void head_layer(const bf16* H2, const QW& w, float* O, int mt, int lane) {
+// dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
+__device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w, d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
+}
+
+// Head of 16 rows (one warp): O[16][8] = H2 * W3^T + b3 (FP32), two
+// accumulator chains (even / odd k-steps) summed in a fixed order.
+__device__ __forceinline__ void head_layer(const bf16* H2, const QW& w, float* O, int lane) {
   const int g = lane >> 2, q = lane & 3;
   float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
   for (int k0 = 0; k0 < kHid; k0 += 32) {
-    uint32_t a[4], b0, b1;
-    load_a_row(a, H2, kLdh, 16 * mt, k0, lane);
-    load_b_col(b0, b1, w.W3, kLdh, k0, 0, lane);
-    mma_bf16(acc0, a, b0, b1);
-    load_a_row(a, H2, kLdh, 16 * mt, k0 + 16, lane);
-    load_b_col(b0, b1, w.W3, kLdh, k0 + 16, 0, lane);
-    mma_bf16(acc1, a, b0, b1);
+    uint32_t a[4], b[4];
+    // W3 rows 0..7, columns k0 .. k0 + 31: the B fragments of both k-steps
+    ldsm_x4(b, w.W3 + (lane & 7) * kLdh + k0 + (lane >> 3) * 8);
+    load_a_row(a, H2, kLdh, 0, k0, lane);
+    mma_bf16(acc0, a, b[0], b[1]);
+    load_a_row(a, H2, kLdh, 0, k0 + 16, lane);
+    mma_bf16(acc1, a, b[2], b[3]);
   }
   const int n = 2 * q;
-  const int r0 = 16 * mt + g;
-  O[r0 * kOutPad + n] = (acc0[0] + acc1[0]) + w.b3[n];
-  O[r0 * kOutPad + n + 1] = (acc0[1] + acc1[1]) + w.b3[n + 1];
-  O[(r0 + 8) * kOutPad + n] = (acc0[2] + acc1[2]) + w.b3[n];
-  O[(r0 + 8) * kOutPad + n + 1] = (acc0[3] + acc1[3]) + w.b3[n + 1];
-}
-
-// Full forward of a tile of 16 * MT rows by 16 * MT warps (contains block
-// barriers; every thread of the block must call it).
-template <int MT = 1>
-__device__ __forceinline__ void mlp_tile(const QW& w, const bf16* X, bf16* H1, bf16* H2, float* O, int warp,
-                                         int lane) {
-  hidden_layer<MT>(X, w.ld1, w.k1, w.W1, w.ld1, w.b1, H1, warp, lane);
-  __syncthreads();
-  hidden_layer<MT>(H1, kLdh, kHid, w.W2, kLdh, w.b2, H2, warp, lane);
-  __syncthreads();
-  if (warp < MT) head_layer(H2, w, O, warp, lane);
-  __syncthreads();
+  O[g * kOutPad + n] = (acc0[0] + acc1[0]) + w.b3[n];
+  O[g * kOutPad + n + 1] = (acc0[1] + acc1[1]) + w.b3[n + 1];
+  O[(g + 8) * kOutPad + n] = (acc0[2] + acc1[2]) + w.b3[n];
+  O[(g + 8) * kOutPad + n + 1] = (acc0[3] + acc1[3]) + w.b3[n + 1];
 }
 
 __device__ __forceinline__ void group_barrier(int id, int nthreads) {
@@ -339,15 +324,16 @@ __device__ __forceinline__ void group_barrier(int id, int nthreads) {
 }
 
 // The forward of one 16-row tile by a group of 16 warps that synchronise
-// among themselves on named barrier `bar` (the other warps of the CTA run
-// on); wg = the warp's index in its group.
-__device__ __forceinline__ void mlp_tile_group(const QW& w, const bf16* X, bf16* H1, bf16* H2, float* O, int wg,
-                                               int lane, int bar) {
-  hidden_layer<1>(X, w.ld1, w.k1, w.W1, w.ld1, w.b1, H1, wg, lane);
+// among themselves on named barrier `bar` (0: the whole CTA is the group;
+// otherwise the other warps of the CTA run on); wg = the warp's index in its
+// group.
+__device__ __forceinline__ void mlp_tile(const QW& w, const bf16* X, bf16* H1, bf16* H2, float* O, int wg, int lane,
+                                         int bar = 0) {
+  hidden_layer(X, w.ld1, w.k1 / 16, w.W1, w.ld1, w.b1, H1, wg, lane);
   group_barrier(bar, 512);
-  hidden_layer<1>(H1, kLdh, kHid, w.W2, kLdh, w.b2, H2, wg, lane);
+  hidden_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, wg, lane);
   group_barrier(bar, 512);
-  if (wg == 0) head_layer(H2, w, O, 0, lane);
+  if (wg == 0) head_layer(H2, w, O, lane);
   group_barrier(bar, 512);
 }
 
@@ -797,6 +783,19 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
   if (warp == 0) tmem_free(tacc, 512);
 }
 
+// One thread of every CTA of a rollout, after the CTA's last use of the ring's
+// step counter: the last CTA advances it by the K steps recorded and leaves
+// the CTA count (behind it) zero for the next launch.
+__device__ __forceinline__ void replay_advance(const ReplayDev& rp, int use_replay, int K) {
+  if (!use_replay) return;
+  unsigned* done = reinterpret_cast<unsigned*>(rp.steps + 1);
+  __threadfence();
+  if (atomicAdd(done, 1u) == gridDim.x - 1u) {
+    *done = 0u;
+    *rp.steps += (unsigned long long)K;
+  }
+}
+
 // VEM eps-greedy rollout with the network fused in: per step, the 16 envs of
 // a group write their observations to a BF16 tile, the tile goes through the
 // network on the tensor cores, every env takes argmax Q or (with probability
@@ -804,7 +803,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
 // replay ring.  One warp per env; 16 envs per group, MT groups per CTA
 // sharing the weight image.  The groups synchronise only among themselves
 // (named barriers), so one group's env step overlaps the other's network.
-template <int MT, bool kDyn>
+template <int MT, bool kDyn, bool kFast>
 __global__ void __launch_bounds__(512 * MT, 1)
     k_rollout_q(const __grid_constant__ DevCfg c, SimPtrs p, const uint8_t* __restrict__ img, ImgLayout L, int K,
                 const float* __restrict__ eps, ReplayDev rp, int use_replay, const int* __restrict__ order, int epc,
@@ -818,7 +817,12 @@ __global__ void __launch_bounds__(512 * MT, 1)
   bf16* H1 = X + kRows * L.ld1;
   bf16* H2 = H1 + kRows * kLdh;
   float* O = reinterpret_cast<float*>(H2 + kRows * kLdh);
-  stage_image(sw, img, L.bytes);
+  __shared__ uint64_t bar_img;
+  if (threadIdx.x == 0) {
+    // the weights on their way while the envs take their first observation
+    mbar_init(&bar_img, 1);
+    stage_image_issue(sw, img, L.bytes, &bar_img);
+  }
   for (int i = threadIdx.x; i < kRows * L.ld1; i += blockDim.x) X[i] = __float2bfloat16_rn(0.0f);
   const QW w = qw_at(sw, L);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -852,17 +856,27 @@ __global__ void __launch_bounds__(512 * MT, 1)
     }
     const Noise z = noise_for(k, s.sigma, s.ep_id, s.ep_step, lane);
     Aux aux;
-    observe<kDyn>(c, k, s, z, lane, o, aux, &dsc);  // the current observation, from the state
+    observe<kDyn, kFast>(c, k, s, z, lane, o, aux, &dsc);  // the current observation, from the state
     eps_i = eps[env];
     akey = sm_at(sm_at(c.seed, kStreamAction), (uint64_t)env);
   }
   const unsigned long long rbase = use_replay ? *rp.steps : 0ull;
   uint32_t ra_batch = 0, ex_batch = 0;
-  __syncthreads();
+  __syncthreads();  // the barrier is initialised
+  if (!__syncthreads_and(mbar_wait(&bar_img, 0u, kTcTries))) {
+    // no weights: the launch's outputs are incomplete; one more bounded wait
+    // for the copy before the CTA exits
+    if (threadIdx.x == 0) {
+      atomicOr(p.status, SG_DEV_TIMEOUT);
+      mbar_wait(&bar_img, 0u, kTcTries);
+      replay_advance(rp, use_replay, K);
+    }
+    return;
+  }
   for (int i = 0; i < K; ++i) {
     if (live) obs_to_tile(Xg + wg * L.ld1, o, c.B, lane);
     group_barrier(bar, 512);
-    mlp_tile_group(w, Xg, H1g, H2g, Og, wg, lane, bar);
+    mlp_tile(w, Xg, H1g, H2g, Og, wg, lane, bar);
     if (!live) continue;
     if ((i & 31) == 0) {
       // lane l draws the random action and the exploration uniform of step t + l
@@ -883,7 +897,7 @@ __global__ void __launch_bounds__(512 * MT, 1)
       s2row = rp.s2 + e * rp.obs_dim;
       write_obs(srow, o, c.B, lane);
     }
-    const StepOut r = env_step<kDyn>(c, p, k, s, a, lane, o, s2row, &b, &dsc);
+    const StepOut r = env_step<kDyn, kFast>(c, p, k, s, a, lane, o, s2row, &b, &dsc);
     if (use_replay) {
       if (!r.done) write_obs(s2row, o, c.B, lane);
       if (lane == 0) {
@@ -904,6 +918,8 @@ __global__ void __launch_bounds__(512 * MT, 1)
     if (lane == 0) store_env(p, env, s);
     if (kDyn && lane < c.n_dyn) store_obst(p, lane, env, b);
   }
+  __syncthreads();  // this CTA's reads of the step counter are done
+  if (threadIdx.x == 0) replay_advance(rp, use_replay, K);
 }
 
 // ---------------------------------------- tcgen05 fused eps-greedy rollout
@@ -1385,9 +1401,8 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 0) tmem_free(tacc, 256);
+  if (tid == 0) replay_advance(rp, use_replay, K);
 }
-
-__global__ void k_replay_advance(unsigned long long* steps, int K) { *steps += (unsigned long long)K; }
 
 // ------------------------------------------------------------ learner
 // Why a TD step produced no update (bits of a device word cleared at the
@@ -1847,39 +1862,6 @@ __device__ __forceinline__ void st_cluster(float* p, uint32_t rank, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
 }
 
-// B fragments of k-step k0 of 16 samples X[16][ldx] (two n-tiles of 8).
-__device__ __forceinline__ void load_x16(uint32_t (&x)[4], const bf16* X, int ldx, int k0, int lane) {
-  ldsm_x4(x, X + ((lane & 7) + (lane >> 4) * 8) * ldx + k0 + ((lane >> 3) & 1) * 8);
-}
-// Hidden layer of 16 samples, 16 warps of 16 units: the weights are the A
-// operand, so that each is read from shared memory once per tile.
-__device__ __forceinline__ void tp_layer(const bf16* X, int ldx, int nks, const bf16* W, int ldw, const float* b,
-                                         bf16* H, int warp, int lane) {
-  const int g = lane >> 2, q = lane & 3, u0 = 16 * warp;
-  float c[2][4] = {};
-#pragma unroll 4
-  for (int ks = 0; ks < nks; ++ks) {
-    uint32_t a[4], x[4];
-    load_a_row(a, W, ldw, u0, 16 * ks, lane);
-    load_x16(x, X, ldx, 16 * ks, lane);
-    mma_bf16(c[0], a, x[0], x[1]);
-    mma_bf16(c[1], a, x[2], x[3]);
-  }
-  const float bl = b[u0 + g], bh = b[u0 + g + 8];
-#pragma unroll
-  for (int t = 0; t < 2; ++t)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      H[(8 * t + 2 * q + (j & 1)) * kLdh + u0 + g + (j >> 1) * 8] =
-          __float2bfloat16_rn(fmaxf(c[t][j] + (j >> 1 ? bh : bl), 0.f));
-}
-
-// dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
-__device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
-  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
-  d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w, d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
-}
-
 __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     k_td_tile(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, ImgLayout L, ReplayDev rp,
               unsigned long long seed, const unsigned long long* __restrict__ step, int batch, float gamma, TdFrag f,
@@ -1942,12 +1924,12 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
         nt = rp.term[e] ? 0.0f : 1.0f;
       }
     }
-    if (ok) tp_layer(X, L.ld1, L.k1 / 16, w.W1, L.ld1, w.b1, H1, warp, lane);
+    if (ok) hidden_layer(X, L.ld1, L.k1 / 16, w.W1, L.ld1, w.b1, H1, warp, lane);
     ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w2, 0u, kTcTries)));
     first = false;
-    if (ok) tp_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, warp, lane);
+    if (ok) hidden_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, warp, lane);
     __syncthreads();
-    if (ok && warp == 0) head_layer(H2, w, O, 0, lane);
+    if (ok && warp == 0) head_layer(H2, w, O, lane);
     __syncthreads();
     if (it == 0) cluster_wait();  // the start's arrival
     if (rank != 0 && tid < kTile * kOutPad)
@@ -2980,10 +2962,14 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   const ImgLayout widest = img_layout(69);
   if ((rc = set_smem_attr((const void*)k_qnet_forward_tc, kTcSmemLaunch)) ||
       (rc = set_smem_attr((const void*)k_rollout_q_tc, qt_smem().bytes)) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<1, false>, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<2, false>, fwd_smem(widest, 32))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<1, true>, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<2, true>, fwd_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, false, false>, fwd_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, false, true>, fwd_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, false, false>, fwd_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, false, true>, fwd_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, true, false>, fwd_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, true, true>, fwd_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, true, false>, fwd_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, true, true>, fwd_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_td_tile, grad_smem(widest))) ||
       (rc = set_smem_attr((const void*)k_td_tc, kTcSmemLaunch))) {
     free_qnet(q);
@@ -3165,8 +3151,8 @@ extern "C" int sg_replay_create(int32_t slots_per_env, int32_t n_envs, int32_t o
   alloc((void**)&r->d.a, (size_t)cap);
   alloc((void**)&r->d.r, (size_t)cap * 4);
   alloc((void**)&r->d.term, (size_t)cap);
-  alloc((void**)&r->d.steps, 8);
-  if (e == cudaSuccess) e = cudaMemset(r->d.steps, 0, 8);
+  alloc((void**)&r->d.steps, 16);
+  if (e == cudaSuccess) e = cudaMemset(r->d.steps, 0, 16);
   if (e != cudaSuccess) {
     cudaFree(r->d.s);
     cudaFree(r->d.s2);
@@ -3330,26 +3316,23 @@ int sg_rollout_eps_q(sg_sim* sim, int K, sg_qnet* q, const float* eps, sg_replay
         sim->dc, sg_sim_ptrs(sim), q->img, q->img_tc, q->IL, K, eps, rd, rp ? 1 : 0, sim->map_order_dev, seg,
         seg > 0 ? sim->q_sync_dev : nullptr, obs, obs_seq, act_seq, rew_seq, done_seq);
   } else {
-    // envs per CTA: the full tile, or fewer (down to half of it) when the
-    // tiles would leave SMs idle (one CTA per SM: the staged image takes the
-    // shared memory); 4,096 envs: 152 CTAs of 27 instead of 128 of 32
+    // envs per CTA: the full tile, or fewer when the tiles would leave SMs
+    // idle (one CTA per SM: the staged image takes the shared memory), down
+    // to one: a CTA's steps wait on its slowest env and on its warps' issue
+    // slots; 4,096 envs: 152 CTAs of 27 instead of 128 of 32
     const int rows = 16 * mt;
-    const int epc = (n + rows - 1) / rows < sms ? std::max(rows / 2, (n + sms - 1) / sms) : rows;
+    const int epc = (n + rows - 1) / rows < sms ? (n + sms - 1) / sms : rows;
     const int grid = (n + epc - 1) / epc;
-    if (mt == 2)
-      (dyn ? k_rollout_q<2, true> : k_rollout_q<2, false>)<<<grid, 1024, fwd_smem(q->IL, 32), stream>>>(
-          sim->dc, sg_sim_ptrs(sim), q->img, q->IL, K, eps, rd, rp ? 1 : 0, sim->map_order_dev, epc, obs, obs_seq,
-          act_seq, rew_seq, done_seq);
-    else
-      (dyn ? k_rollout_q<1, true> : k_rollout_q<1, false>)<<<grid, 512, fwd_smem(q->IL), stream>>>(
-          sim->dc, sg_sim_ptrs(sim), q->img, q->IL, K, eps, rd, rp ? 1 : 0, sim->map_order_dev, epc, obs, obs_seq,
-          act_seq, rew_seq, done_seq);
+    const bool fast = sim->dc.scan_fast != 0;
+    auto kern = mt == 2 ? (dyn ? (fast ? k_rollout_q<2, true, true> : k_rollout_q<2, true, false>)
+                               : (fast ? k_rollout_q<2, false, true> : k_rollout_q<2, false, false>))
+                        : (dyn ? (fast ? k_rollout_q<1, true, true> : k_rollout_q<1, true, false>)
+                               : (fast ? k_rollout_q<1, false, true> : k_rollout_q<1, false, false>));
+    kern<<<grid, 512 * mt, fwd_smem(q->IL, rows), stream>>>(sim->dc, sg_sim_ptrs(sim), q->img, q->IL, K, eps, rd,
+                                                            rp ? 1 : 0, sim->map_order_dev, epc, obs, obs_seq, act_seq,
+                                                            rew_seq, done_seq);
   }
   SG_CUDA(cudaGetLastError());
-  if (rp) {
-    k_replay_advance<<<1, 1, 0, stream>>>(rp->d.steps, K);
-    SG_CUDA(cudaGetLastError());
-  }
   return SG_OK;
 }
 
