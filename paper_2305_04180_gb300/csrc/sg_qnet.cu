@@ -291,12 +291,6 @@ __device__ __forceinline__ void hidden_layer(const bf16* X, int ldx, int nks, co
           __float2bfloat16_rn(fmaxf(c[t][j] + (j >> 1 ? bh : bl), 0.f));
 }
 
-// dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
-__device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
-  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
-  d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w, d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
-}
-
 // Head of 16 rows (one warp): O[16][8] = H2 * W3^T + b3 (FP32), two
 // accumulator chains (even / odd k-steps) summed in a fixed order.
 __device__ __forceinline__ void head_layer(const bf16* H2, const QW& w, float* O, int lane) {
@@ -381,27 +375,32 @@ __device__ __forceinline__ void obs_to_tile(bf16* row, const ObsRegs& o, int B, 
 
 // ------------------------------------------------ tcgen05 batched forward
 // Q[M][5] of obs[M][n_in] on the fifth-generation tensor cores, 128 rows per
-// tile.  A persistent CTA (one per SM) holds all weights in shared memory
-// (W1, W2, W3: one set of bulk asynchronous copies (TMA) from a copy of the
-// online network in the tensor cores' layout, k_tc_image) and the whole
-// 512-column tensor memory.  Per tile: the threads convert the 128 input
-// rows to BF16 (X, shared memory); one thread issues the MMAs of a layer
-// (tcgen05.mma, FP32 accumulators in tensor memory) and commits them to an
-// mbarrier; the eight warps read the accumulators back (tcgen05.ld; warps w
-// and w + 4 take the rows of lane quarter w % 4 and half of the columns
-// each), add the bias, apply ReLU, round to BF16 and store the pairs back
-// into the first half of the columns they read (tcgen05.st): the hidden
-// activations never leave tensor memory and are the A operand of the next
-// layer's MMAs.  Tensor-memory columns:
-//   [0, 256)   layer 1 accumulators; H1 in [0, 64) (units 0..127) and [128, 192) (128..255)
-//   [256, 512) layer 2 accumulators; H2 in [256, 320) and [384, 448); head accumulators at 320
-// The tensor cores run the next tile's layer 1 beside this tile's layer-2
-// epilogue, and this tile's head beside the next tile's layer-1 epilogue;
-// only layer 2 (N = 256) is waited for by all warps.
-// Shared memory: X 128 x k1 | W1 256 x k1 | W2 256 x 256 | W3 16 x 256,
-// in the canonical K-major layout of sg_tc.cuh.  Same BF16 recipe as the
-// mma.sync kernels (BF16 inputs, weights and hidden activations, FP32 sums);
-// only the summation order differs.
+// tile.  A persistent CTA (one per SM) holds W1 and W2 in shared memory (one
+// set of bulk asynchronous copies (TMA) from a copy of the online network in
+// the tensor cores' layout, k_tc_image) and the whole 512-column tensor
+// memory.  Per tile: the threads convert the 128 input rows to BF16 (X, shared
+// memory); one thread issues the MMAs of a hidden layer (tcgen05.mma, FP32
+// accumulators in tensor memory) and commits them to an mbarrier; 16 warps
+// read the accumulators back (warps w, w + 4, .. take the rows of lane quarter
+// w % 4 and 64 columns each) and add the bias, apply ReLU and round to BF16.
+// H1 goes back into the first half of the columns it was read from
+// (tcgen05.st) and is the A operand of layer 2's MMAs.  H2 is read in the
+// fragment shape of mma.sync and never leaves the registers: the head (6
+// outputs) is eight m16n8k16 a warp on its 64 columns, the four column groups'
+// sums meet in shared memory and three more warps write the Q-values.
+// Tensor-memory columns:
+//   [0, 256)   layer 1 accumulators; H1 in the first half of each 64
+//   [256, 512) layer 2 accumulators
+// Bound by the tensor cores' layer 2 (2,048 cycles a tile) with the two
+// epilogues behind it; the next tile's layer 1 runs beside the layer-2
+// epilogue.  As a tcgen05 layer of its own the head (16 MMAs at their
+// 88-cycle floor for any N up to 128, and H2's store) sat in that chain, and
+// row-wise input loads took 24 lines a warp instruction: 2^20 rows of 37
+// inputs 185 -> 154 us.
+// Shared memory: X 128 x k1 | W1 256 x k1 | W2 256 x 256 (the canonical K-major
+// layout of sg_tc.cuh) | head sums.  Same BF16 recipe as the mma.sync kernels
+// (BF16 inputs, weights and hidden activations, FP32 sums); only the
+// summation order differs.
 constexpr int kTcRows = 128;
 constexpr uint32_t kTcTries = 1u << 24;  // bound of every mbarrier wait (polls)
 // The launch takes the whole shared memory of an SM (one CTA per SM either
@@ -409,7 +408,7 @@ constexpr uint32_t kTcTries = 1u << 24;  // bound of every mbarrier wait (polls)
 constexpr uint32_t kTcSmemLaunch = 227u * 1024u - 4096u;
 
 struct TcSmem {
-  uint32_t x, w1, w2, w3, bytes;
+  uint32_t x, w1, w2, part, bytes;
 };
 __host__ __device__ inline uint32_t tc_up(uint32_t v) { return (v + 1023u) & ~1023u; }
 __host__ __device__ inline TcSmem tc_smem(int k1) {
@@ -417,12 +416,12 @@ __host__ __device__ inline TcSmem tc_smem(int k1) {
   t.x = 0;
   t.w1 = tc_up(t.x + (uint32_t)(kTcRows * k1 * 2));
   t.w2 = tc_up(t.w1 + (uint32_t)(kHid * k1 * 2));
-  t.w3 = tc_up(t.w2 + (uint32_t)(kHid * kHid * 2));
-  t.bytes = tc_up(t.w3 + (uint32_t)(16 * kHid * 2));
+  t.part = tc_up(t.w2 + (uint32_t)(kHid * kHid * 2));  // head sums [2][4][128][8] float
+  t.bytes = tc_up(t.part + (uint32_t)(2 * 4 * kTcRows * kOutPad * 4));
   return t;
 }
-// k1 <= 80 (n_in <= 69): 197 KB, inside the launch's shared memory
-static_assert(kTcRows * 80 * 2 + 1024 + kHid * 80 * 2 + kHid * kHid * 2 + 16 * kHid * 2 + 1024 <= kTcSmemLaunch,
+// k1 <= 80 (n_in <= 69): 220 KB, inside the launch's shared memory
+static_assert(kTcRows * 80 * 2 + 1024 + kHid * 80 * 2 + kHid * kHid * 2 + 32 * 1024 + 1024 <= kTcSmemLaunch,
               "tcgen05 forward: operands exceed the shared memory");
 // The weight copy in global memory: blocks identical to their shared-memory
 // images, so that each is one bulk copy.
@@ -505,7 +504,8 @@ __device__ __forceinline__ void tc_epilogue_hidden(uint32_t tacc, const float* b
 // w / 4).
 constexpr int kTfEpiWarps = 16;
 constexpr int kTfEpiThreads = kTfEpiWarps * 32;
-constexpr int kTfThreads = kTfEpiThreads + 32;  // + the MMA-issue warp
+constexpr int kTfWriters = 96;                               // Q-value writers
+constexpr int kTfThreads = kTfEpiThreads + 32 + kTfWriters;  // + the MMA-issue warp
 constexpr int kTfCols = kHid / (kTfEpiWarps / 4);
 static_assert(kTfCols % 32 == 0, "each epilogue warp's columns hold whole 16-column chunks and head accumulators");
 
@@ -541,13 +541,9 @@ __device__ __forceinline__ void tc_epilogue_tmem(uint32_t tacc, const float* bia
   tmem_st_wait();
 }
 // Tensor-memory column (relative to the layer's accumulators) of K step ks
-// of the packed activations, and of head accumulator q (four of 16 columns
-// in the halves the epilogue leaves free).
+// of the packed activations.
 __host__ __device__ constexpr uint32_t tf_a_col(int ks) {
   return (uint32_t)((ks / (kTfCols / 16)) * kTfCols + (ks % (kTfCols / 16)) * 8);
-}
-__host__ __device__ constexpr uint32_t tf_head_col(int q) {
-  return (uint32_t)(kTfCols / 2 + (q / (kTfCols / 32)) * kTfCols + (q % (kTfCols / 32)) * 16);
 }
 
 // One layer from a tensor-memory A operand (the packed activations of
@@ -562,66 +558,94 @@ __device__ __forceinline__ void tc_layer_ta(uint32_t d, uint32_t a, uint32_t b_s
     tc_mma_bf16_ta(d, a + tf_a_col(ks), smem_desc(b_smem + (uint32_t)ks * 2 * lb, lb, 128), idesc, ks > 0 ? 1u : 0u);
 }
 
-// Input rows of a tile into the X operand (BF16, zero padded) in two steps:
-// tc_fetch_x loads this thread's values (the kTfEpiThreads / 128 threads of
-// a row take interleaved 8-column groups, at most kTcMaxGroups each),
-// tc_store_x converts and stores them.
-constexpr int kTcXStride = kTfEpiThreads / kTcRows;
-constexpr int kTcMaxGroups = (80 / 8 + kTcXStride - 1) / kTcXStride;
-struct TcXRegs {
-  float v[kTcMaxGroups][8];
-};
-__device__ __forceinline__ void tc_fetch_x(TcXRegs& x, const float* __restrict__ obs, const ImgLayout& L, int M,
-                                           int tile, int tid) {
-  const int row = tid & (kTcRows - 1), grow = tile * kTcRows + row, ng = L.k1 / 8;
-  const float* src = obs + (long long)grow * L.n_in;
+// Layer-2 epilogue and head of a warp's 64 columns [tacc + 64 (warp / 4), + 64):
+// its 32 rows in two halves of 16, bias and ReLU into A fragments, times the
+// columns' W3 fragments w3 (b0, b1 of each 16-column step); the sums of row r to
+// out[8 r ..].
+__device__ __forceinline__ void tf_epilogue_head(uint32_t tacc, const float* bias, const uint32_t (&w3)[8], float* out,
+                                                 int warp, int lane) {
+  static_assert(kTfCols == 64, "one fragment load per half");
+  const int g = lane >> 2, q = lane & 3;
+  const uint32_t t = tacc + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * kTfCols);
+  const float2* b2 = reinterpret_cast<const float2*>(bias + (warp >> 2) * kTfCols) + q;
+  uint32_t r[2][32];
+  tmem_ld_frag64_nowait(t, r[0]);
+  tmem_ld_frag64_nowait(t + (16u << 16), r[1]);
+  tmem_ld_wait();
 #pragma unroll
-  for (int it = 0; it < kTcMaxGroups; ++it) {
-    const int kg = (tid >> 7) + kTcXStride * it;
+  for (int h = 0; h < 2; ++h) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int k = kg * 8 + j;
-      x.v[it][j] = (kg < ng && grow < M && k < L.n_in) ? __ldg(src + k) : 0.0f;
+    for (int i = 0; i < 4; ++i) {
+      uint32_t a[4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float2 bb = b2[4 * (2 * i + j)];
+        const uint32_t* v = r[h] + 4 * (2 * i + j);
+        a[2 * j] = pack_bf16x2_relu(__uint_as_float(v[0]) + bb.x, __uint_as_float(v[1]) + bb.y);
+        a[2 * j + 1] = pack_bf16x2_relu(__uint_as_float(v[2]) + bb.x, __uint_as_float(v[3]) + bb.y);
+      }
+      mma_bf16(acc, a, w3[2 * i], w3[2 * i + 1]);
     }
+    float* o = out + ((warp & 3) * 32 + 16 * h + g) * kOutPad + 2 * q;
+    *reinterpret_cast<float2*>(o) = make_float2(acc[0], acc[1]);
+    *reinterpret_cast<float2*>(o + 8 * kOutPad) = make_float2(acc[2], acc[3]);
   }
 }
-__device__ __forceinline__ void tc_store_x(uint8_t* xs, const TcXRegs& x, const ImgLayout& L, int tid) {
-  const int row = tid & (kTcRows - 1), ng = L.k1 / 8;
+
+// Input rows of a tile into the X operand (BF16; its padding columns are zero
+// from the start) in two steps: tc_fetch_x loads the tile's floats, which are
+// contiguous, in order over the threads (a line a warp instruction),
+// tc_store_x converts and stores them.  div: ceil(2^20 / n_in), exact for the
+// index / n_in of at most 128 x 69 floats.
+constexpr int kTcXFloats = (kTcRows * 69 + kTfEpiThreads - 1) / kTfEpiThreads;
+__device__ __forceinline__ void tc_fetch_x(float (&x)[kTcXFloats], const float* __restrict__ obs, int n_in, int M,
+                                           int tile, int tid) {
+  const long long first = (long long)tile * kTcRows;
+  const int total = (int)min((long long)kTcRows, M - first) * n_in;
+  const float* src = obs + first * n_in;
 #pragma unroll
-  for (int it = 0; it < kTcMaxGroups; ++it) {
-    const int kg = (tid >> 7) + kTcXStride * it;
-    if (kg < ng)
-      *reinterpret_cast<uint4*>(xs + kmajor_offset(row, kg * 8, kTcRows)) =
-          make_uint4(pack_bf16x2(x.v[it][0], x.v[it][1]), pack_bf16x2(x.v[it][2], x.v[it][3]),
-                     pack_bf16x2(x.v[it][4], x.v[it][5]), pack_bf16x2(x.v[it][6], x.v[it][7]));
+  for (int i = 0; i < kTcXFloats; ++i) {
+    const int e = tid + i * kTfEpiThreads;
+    x[i] = e < total ? __ldg(src + e) : 0.0f;
+  }
+}
+__device__ __forceinline__ void tc_store_x(uint8_t* xs, const float (&x)[kTcXFloats], int n_in, uint32_t div, int tid) {
+#pragma unroll
+  for (int i = 0; i < kTcXFloats; ++i) {
+    const int e = tid + i * kTfEpiThreads;
+    if (e < kTcRows * n_in) {
+      const int row = (int)(((uint32_t)e * div) >> 20), k = e - row * n_in;
+      *reinterpret_cast<bf16*>(xs + kmajor_offset(row, k, kTcRows)) = __float2bfloat16_rn(x[i]);
+    }
   }
   fence_async_smem();
 }
 
-// Warps 0..15 run the epilogues, convert the inputs and write Q; warp 16
-// (one lane) copies the weights and issues every MMA, so that the issue, which
-// waits while the tensor cores' queue is full, never holds up an epilogue.
-// The two sides meet on mbarriers, one phase per tile each: bar_x (X
-// stored), bar_h1 (H1 stored and the previous tile's head read), bar_h2 (H2
-// stored), and the MMA commits bar_l1, bar_l2, bar_hd (layer 1, layer 2,
-// head complete).  Order on the tensor cores per tile t: layer 2 (t) once H1
-// (t) is stored and the head of t - 1 is read; layer 1 (t + 1) once layer 2
-// (t) is complete and X (t + 1) is stored; the head (t) once H2 (t) is stored.
+// Warps 0..15 run the epilogues and convert the inputs, warp 16 (one lane)
+// copies the weights and issues every MMA, so that the issue, which waits
+// while the tensor cores' queue is full, never holds up an epilogue, and warps
+// 17..19 write Q.  They meet on mbarriers, one phase per tile each: bar_x (X
+// stored), bar_h1 (H1 stored and the previous tile's layer 2 read), and the
+// MMA commits bar_l1, bar_l2 (layer complete); the head sums of tile t pass
+// through named barriers 1 + t % 2 (written) and 3 + t % 2 (read).  Order on
+// the tensor cores: layer 2 (t) once H1 (t) is stored; layer 1 (t + 1) once
+// layer 2 (t) is complete and X (t + 1) is stored.
 __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t* __restrict__ img,
                                                                 const uint8_t* __restrict__ timg, ImgLayout L,
                                                                 const float* __restrict__ obs, int M,
                                                                 float* __restrict__ qout) {
   extern __shared__ __align__(1024) uint8_t tsm[];
-  __shared__ uint64_t bar_w, bar_l1, bar_l2, bar_hd, bar_x, bar_h1, bar_h2, bar_drain;
+  __shared__ uint64_t bar_w, bar_l1, bar_l2, bar_x, bar_h1, bar_drain;
   __shared__ uint32_t tslot;
   __shared__ int s_fail;
   __shared__ __align__(16) float sb1[kHid];
   __shared__ __align__(16) float sb2[kHid];
-  __shared__ float sb3[kOutPad];
   const TcSmem T = tc_smem(L.k1);
   const TcImg G = tc_img(L.k1);
   uint8_t* xs = tsm + T.x;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  float* part = reinterpret_cast<float*>(tsm + T.part);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ntiles = (M + kTcRows - 1) / kTcRows;
   // this CTA's tiles: blockIdx.x + i gridDim.x, i < my_tiles
   const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
@@ -629,17 +653,17 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
     sb1[i] = __ldg(reinterpret_cast<const float*>(img + L.b1) + i);
     sb2[i] = __ldg(reinterpret_cast<const float*>(img + L.b2) + i);
   }
-  if (tid < kOutPad) sb3[tid] = __ldg(reinterpret_cast<const float*>(img + L.b3) + tid);
+  for (int i = tid; i < kTcRows * L.k1 / 8; i += kTfThreads)
+    reinterpret_cast<uint4*>(xs)[i] = make_uint4(0u, 0u, 0u, 0u);
+  fence_async_smem();
   if (warp == 0) tmem_alloc(&tslot, 512);
   if (tid == 0) {
     mbar_init(&bar_w, 1);
     mbar_init(&bar_l1, 1);
     mbar_init(&bar_l2, 1);
-    mbar_init(&bar_hd, 1);
     mbar_init(&bar_drain, 1);
     mbar_init(&bar_x, kTfEpiThreads);
     mbar_init(&bar_h1, kTfEpiThreads);
-    mbar_init(&bar_h2, kTfEpiThreads);
     s_fail = 0;
   }
   tc_fence_before();
@@ -647,11 +671,11 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
   tc_fence_after();
   const uint32_t tacc = tslot, tacc2 = tacc + 256u;
   volatile int* fail = &s_fail;
-  if (warp == kTfEpiThreads / 32) {
-    if ((tid & 31) == 0 && my_tiles > 0) {
+  constexpr int kHandover = kTfEpiThreads + kTfWriters;
+  if (warp == kTfEpiWarps) {
+    if (lane == 0 && my_tiles > 0) {
       // ---- MMA issue
-      const uint32_t sx = smem_u32(xs), sw1 = smem_u32(tsm + T.w1), sw2 = smem_u32(tsm + T.w2),
-                     sw3 = smem_u32(tsm + T.w3);
+      const uint32_t sx = smem_u32(xs), sw1 = smem_u32(tsm + T.w1), sw2 = smem_u32(tsm + T.w2);
       auto issue_l1 = [&]() {
         const uint32_t idesc = idesc_bf16_f32(kTcRows, kHid);
         const uint32_t la = kTcRows * 16, lb = kHid * 16;
@@ -660,11 +684,10 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
                       smem_desc(sw1 + (uint32_t)ks * 2 * lb, lb, 128), idesc, ks > 0 ? 1u : 0u);
         tc_commit(&bar_l1);
       };
-      // the resident weights: W1, W2 (one 256-row operand), W3
-      mbar_expect_tx(&bar_w, G.w2a + kHid * kHid * 2u + 16u * kHid * 2u);
+      // the resident weights: W1, W2 (one 256-row operand)
+      mbar_expect_tx(&bar_w, G.w2a + kHid * kHid * 2u);
       bulk_g2s(tsm + T.w1, timg + G.w1, G.w2a, &bar_w);
       bulk_g2s(tsm + T.w2, timg + G.w2f, kHid * kHid * 2u, &bar_w);
-      bulk_g2s(tsm + T.w3, timg + G.w3, 16u * kHid * 2u, &bar_w);
       bool ok = mbar_wait_or_fail(&bar_w, 0, kTcTries, fail) && mbar_wait_or_fail(&bar_x, 0, kTcTries, fail);
       if (ok) {
         tc_fence_after();
@@ -685,20 +708,6 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
           tc_fence_after();
           issue_l1();
         }
-        // head (t): N = 16 (6 used) into four accumulators in layer-2
-        // columns the epilogue has read and left free, K step ks into
-        // accumulator ks % 4
-        ok = mbar_wait_or_fail(&bar_h2, par, kTcTries, fail);
-        if (!ok) break;
-        tc_fence_after();
-        {
-          const uint32_t idesc = idesc_bf16_f32(kTcRows, 16);
-#pragma unroll 1
-          for (int ks = 0; ks < kHid / 16; ++ks)
-            tc_mma_bf16_ta(tacc2 + tf_head_col(ks & 3), tacc2 + tf_a_col(ks),
-                           smem_desc(sw3 + (uint32_t)ks * 2 * 256, 256, 128), idesc, ks >= 4 ? 1u : 0u);
-        }
-        tc_commit(&bar_hd);
       }
       // every MMA of this thread, and the weight copies, complete before the
       // tensor memory is freed (bounded waits)
@@ -706,76 +715,81 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
       mbar_wait(&bar_drain, 0, kTcTries);
       mbar_wait(&bar_w, 0, kTcTries);
     }
+  } else if (warp > kTfEpiWarps) {
+    // ---- read-out: rows of tile i from the four column groups' head sums
+    // (NaN where a wait ran out)
+    float b3[kOut];
+#pragma unroll
+    for (int j = 0; j < kOut; ++j) b3[j] = __ldg(reinterpret_cast<const float*>(img + L.b3) + j);
+    for (int i = 0; i < my_tiles; ++i) {
+      group_barrier(1 + (i & 1), kHandover);
+      const bool good = *fail == 0;
+      const long long first = ((long long)blockIdx.x + (long long)i * gridDim.x) * kTcRows;
+      for (int r = tid - kTfEpiThreads - 32; r < kTcRows; r += kTfWriters) {
+        const float* p = part + (i & 1) * 4 * kTcRows * kOutPad + r * kOutPad;
+        float o[kOutPad];
+#pragma unroll
+        for (int j = 0; j < kOutPad; j += 2) {
+          float2 v[4];
+#pragma unroll
+          for (int gq = 0; gq < 4; ++gq) v[gq] = *reinterpret_cast<const float2*>(p + gq * kTcRows * kOutPad + j);
+          o[j] = (v[0].x + v[1].x) + (v[2].x + v[3].x);
+          o[j + 1] = (v[0].y + v[1].y) + (v[2].y + v[3].y);
+        }
+        if (first + r < M) {
+          float qv[5];
+#pragma unroll
+          for (int j = 0; j < kOut; ++j) o[j] += b3[j];
+          greedy_action(o, qv, L.plain);
+#pragma unroll
+          for (int a = 0; a < 5; ++a) qout[(first + r) * 5 + a] = good ? qv[a] : __int_as_float(0x7fc00000);
+        }
+      }
+      __threadfence_block();
+      asm volatile("bar.arrive %0, %1;\n" ::"r"(3 + (i & 1)), "n"(kHandover) : "memory");
+    }
   } else {
-    // ---- epilogues, inputs, read-out (warps 0..7)
+    // ---- epilogues, inputs (warps 0..15)
     bool ok = true;
-    const int row = tid & (kTcRows - 1);
     auto wait = [&](uint64_t* bar, uint32_t par) {
       ok = __all_sync(0xffffffffu, ok && mbar_wait_or_fail(bar, par, kTcTries, fail));
       if (ok) tc_fence_after();
     };
-    // Q rows of local tile i from the four head accumulators (NaN where a
-    // wait ran out)
-    auto write_rows = [&](int i) {
-      uint32_t h[4][8];
-      if (ok && warp < 4) {
+    const uint32_t div = ((1u << 20) + (uint32_t)L.n_in - 1u) / (uint32_t)L.n_in;
+    // this lane's W3 fragments: outputs g, columns 64 (warp / 4) + 16 i + 2 q ..
+    uint32_t w3[8];
+    {
+      const bf16* w = reinterpret_cast<const bf16*>(img + L.w3) + (lane >> 2) * kLdh + (warp >> 2) * kTfCols + 2 * (lane & 3);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) tmem_ld8_nowait(tacc2 + tf_head_col(q) + ((uint32_t)(warp * 32) << 16), h[q]);
-        tmem_ld_wait();
-      }
-      const int grow = ((int)blockIdx.x + i * (int)gridDim.x) * kTcRows + row;
-      if (warp < 4 && grow < M) {
-        float qv[5];
-        if (ok) {
-          float o[kOut];
-#pragma unroll
-          for (int j = 0; j < kOut; ++j)
-            o[j] = ((__uint_as_float(h[0][j]) + __uint_as_float(h[1][j])) +
-                    (__uint_as_float(h[2][j]) + __uint_as_float(h[3][j]))) +
-                   sb3[j];
-          greedy_action(o, qv, L.plain);
-        } else {
-#pragma unroll
-          for (int a = 0; a < 5; ++a) qv[a] = __int_as_float(0x7fc00000);
-        }
-#pragma unroll
-        for (int a = 0; a < 5; ++a) qout[(long long)grow * 5 + a] = qv[a];
-      }
-    };
-    TcXRegs xr;
+      for (int i = 0; i < 8; ++i) w3[i] = __ldg(reinterpret_cast<const uint32_t*>(w + 8 * i));
+    }
+    float xr[kTcXFloats];
     if (my_tiles > 0) {
-      tc_fetch_x(xr, obs, L, M, blockIdx.x, tid);
-      tc_store_x(xs, xr, L, tid);
+      tc_fetch_x(xr, obs, L.n_in, M, blockIdx.x, tid);
+      tc_store_x(xs, xr, L.n_in, div, tid);
       mbar_arrive(&bar_x);
     }
     for (int it = 0; it < my_tiles; ++it) {
       const uint32_t par = (uint32_t)it & 1u;
       wait(&bar_l1, par);
       if (ok) tc_epilogue_tmem(tacc, sb1, warp);  // H1 over the layer-1 accumulators
-      if (it > 0) {
-        wait(&bar_hd, par ^ 1u);
-        write_rows(it - 1);
-        // the read-out (warps 0..3) is on the critical path: the other
-        // warps' input loads start after it
-        asm volatile("bar.sync 1, %0;\n" ::"n"(kTfEpiThreads) : "memory");
-      }
       tc_fence_before();
       mbar_arrive(&bar_h1);
       // X is free (layer 1 of t is complete): the next tile's inputs while layer 2 runs
       if (ok && it + 1 < my_tiles) {
-        tc_fetch_x(xr, obs, L, M, (int)blockIdx.x + (it + 1) * (int)gridDim.x, tid);
-        tc_store_x(xs, xr, L, tid);
+        tc_fetch_x(xr, obs, L.n_in, M, (int)blockIdx.x + (it + 1) * (int)gridDim.x, tid);
+        tc_store_x(xs, xr, L.n_in, div, tid);
         mbar_arrive(&bar_x);
       }
+      if (it >= 2) group_barrier(3 + (it & 1), kHandover);  // the sums of t - 2 are read
       wait(&bar_l2, par);
-      if (ok) tc_epilogue_tmem(tacc2, sb2, warp);  // H2 over the layer-2 accumulators
-      tc_fence_before();
-      mbar_arrive(&bar_h2);
+      if (ok)
+        tf_epilogue_head(tacc2, sb2, w3, part + ((it & 1) * 4 + (warp >> 2)) * kTcRows * kOutPad, warp, lane);
+      __threadfence_block();
+      asm volatile("bar.arrive %0, %1;\n" ::"r"(1 + (it & 1)), "n"(kHandover) : "memory");
     }
-    if (my_tiles > 0) {
-      wait(&bar_hd, (uint32_t)(my_tiles - 1) & 1u);
-      write_rows(my_tiles - 1);
-    }
+    // the read-out's last arrivals
+    for (int it = max(my_tiles, 2); it < my_tiles + 2; ++it) group_barrier(3 + (it & 1), kHandover);
     tc_fence_before();
   }
   __syncthreads();
@@ -1860,6 +1874,12 @@ __device__ __forceinline__ void st_cluster(float* p, uint32_t rank, float v) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
+}
+
+// dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
+__device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w, d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
 }
 
 __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
