@@ -150,15 +150,12 @@ struct sg_qnet {
   // learner scratch, sized for max_batch
   int max_batch = 0;
   void* frag = nullptr;      // TdFrag of the 16-sample tiles (mma.sync learner)
-  int td_clusters = 1;       // clusters of k_td_tile that fit the device
-  float* partial = nullptr;  // [tiles of 128][P + 1] (last entry: loss; tcgen05 learner)
+  int td_clusters = 1;       // clusters of k_td_tile / k_td_tc that fit the device
   int rollout_mt = 0;        // m-tiles per CTA of the fused rollout (0 = choose by waves)
   int lim_rollout = 0;       // CTA caps of the tcgen05 rollout / learner grids (0 = every SM)
   int lim_learner = 0;
   uint8_t* img_tc = nullptr; // the online weights in the tensor cores' shared-memory layout (batched forward)
   uint8_t* img_tc_t = nullptr; // the target weights in the same layout (tcgen05 learner)
-  float* q2 = nullptr;       // [2][max_batch][5] Q-values of the sampled next states (tcgen05 learner)
-  unsigned* td_sync = nullptr;  // [1 + max_batch / 128] job counter and per-tile counters (tcgen05 learner)
   int sms = 0;               // multiprocessors of the device (persistent grids)
 };
 
@@ -474,28 +471,6 @@ __global__ void k_tc_image(const uint8_t* __restrict__ img, ImgLayout L, uint8_t
       dst = T.w3 + kmajor_offset(n, kg * 8, 16);
     }
     *reinterpret_cast<uint4*>(out + dst) = v;
-  }
-}
-
-// Hidden-layer epilogue: this thread's row r = 32 (warp % 4) + lane, columns
-// [128 (warp / 4), + 128) of the accumulator plus bias, ReLU, rounded to BF16
-// into the H operand.
-__device__ __forceinline__ void tc_epilogue_hidden(uint32_t tacc, const float* bias, uint8_t* hs,
-                                                   int warp, int lane) {
-  const int quarter = warp & 3, r = quarter * 32 + lane, c0 = (warp >> 2) * 128;
-  for (int c = c0; c < c0 + 128; c += 32) {
-    float v[32];
-    tmem_ld32(tacc + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      uint32_t w[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int k = c + 8 * g + 2 * j;
-        w[j] = pack_bf16x2(fmaxf(v[8 * g + 2 * j] + bias[k], 0.f), fmaxf(v[8 * g + 2 * j + 1] + bias[k + 1], 0.f));
-      }
-      *reinterpret_cast<uint4*>(hs + kmajor_offset(r, c + 8 * g, kTcRows)) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
   }
 }
 
@@ -1665,7 +1640,7 @@ struct TdUpdate {
   uint8_t* img_t;
   uint8_t* tc;
   uint8_t* tc_t;
-  unsigned long long* step;  // null: gradient only (sg_td_grad_noalloc)
+  unsigned long long* step;
   unsigned* fail;
   unsigned* tick;            // CTAs that are done (0 between launches)
   float lr;
@@ -1788,7 +1763,6 @@ __device__ __forceinline__ void upd_one(const TdUpdate& u, const UpdRun& r, int 
 // Every CTA, at its end: the last one advances the step count (of a step that
 // changed the parameters) and clears the failure word.
 __device__ __forceinline__ void upd_end(const TdUpdate& u, bool failed) {
-  if (!u.step) return;
   __syncthreads();  // this CTA's reads of *step and *fail are done
   if (threadIdx.x == 0) {
     __threadfence();
@@ -1800,30 +1774,20 @@ __device__ __forceinline__ void upd_end(const TdUpdate& u, bool failed) {
   }
 }
 
-// Gradient rows (one per CTA of the gradient kernel) summed in row order and
-// applied, thread per parameter: the tcgen05 learner and the allocation-free
-// gradient.
-__global__ void __launch_bounds__(256) k_adam(TdUpdate u, const float* __restrict__ partial, int nblk) {
-  pdl_launch_dependents();
-  UpdRun run = upd_begin(u);
+// Gradient rows (one per CTA of the gradient kernel) summed in row order,
+// thread per parameter: the allocation-free gradient.
+__global__ void __launch_bounds__(256) k_grad_sum(TdUpdate u, const float* __restrict__ partial, int nblk) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float th = 0.0f, m = 0.0f, v = 0.0f;
-  if (u.lr != 0.0f && i < u.P.total) th = u.th[i], m = u.m[i], v = u.v[i];
-  pdl_wait();
-  const bool failed = *u.fail != 0u;
-  if (i <= u.P.total) {
-    const long long ld = partial_stride(u.P.total);
-    float g = 0.0f;
+  if (i > u.P.total) return;
+  const long long ld = partial_stride(u.P.total);
+  float g = 0.0f;
 #pragma unroll 8
-    for (int b = 0; b < nblk; ++b) g += partial[(long long)b * ld + i];
-    if (failed) g = __int_as_float(0x7fc00000);
-    upd_fail(failed, run);
-    if (i < u.P.total)
-      upd_one(u, run, i, g, th, m, v);
-    else if (u.loss)
-      *u.loss = g / (float)u.batch;
-  }
-  upd_end(u, failed);
+  for (int b = 0; b < nblk; ++b) g += partial[(long long)b * ld + i];
+  if (*u.fail) g = __int_as_float(0x7fc00000);
+  if (i < u.P.total)
+    upd_grad(u, i, g);
+  else if (u.loss)
+    *u.loss = g / (float)u.batch;
 }
 
 // --------------------------------------------------- mma.sync learner
@@ -1839,6 +1803,8 @@ __global__ void __launch_bounds__(256) k_adam(TdUpdate u, const float* __restric
 // two forwards in a row of one kernel, then a forward and the backward of a
 // second, took 30 of the step's 57 us.
 constexpr int kTpRanks = 3;
+constexpr int kLtRows = 128;             // samples of a tile of the tcgen05 learner
+constexpr int kLtSub = kLtRows / kTile;  // its 16-sample fragment tiles
 constexpr int kVecDb2 = kHid, kVecW3 = 2 * kHid, kVecB3 = kVecW3 + kOut * kHid, kVecHub = kVecB3 + kOut;
 constexpr int kVecLd = (kVecHub + 1 + 31) / 32 * 32;  // db1 | db2 | dW3 | db3 | Huber sum
 constexpr int kFragTile = 16 * 32;                    // 16-byte words of a 16 x 256 operand
@@ -1847,18 +1813,22 @@ struct TdFrag {
   uint4* h1;   // [tiles][16 unit pairs][32]: B fragments of H1
   uint4* z1;   // [tiles][16][32]: A fragments of dZ1^T
   uint4* x;    // [tiles][k1 / 16][32]: B fragments of X
-  float* vec;  // [tiles][kVecLd]
+  uint4* h2;   // [tiles][16][32]: A fragments of H2^T (128-sample learner)
+  float* dout; // [tiles][16][8]: dL/d(head outputs), the Huber term in column 7 (128-sample learner)
+  float* vec;  // [tiles][kVecLd]; [tiles / 8][kVecLd] of the 128-sample learner
 };
 inline size_t td_frag_bytes(int tiles, int k1) {
-  return (size_t)tiles * ((3 * kFragTile + k1 / 16 * 32) * 16 + kVecLd * 4);
+  return (size_t)tiles * ((4 * kFragTile + k1 / 16 * 32) * 16 + (kTile * kOutPad + kVecLd) * 4);
 }
 inline TdFrag td_frag(void* base, int tiles, int k1) {
   TdFrag f;
   f.z2 = static_cast<uint4*>(base);
   f.h1 = f.z2 + (size_t)tiles * kFragTile;
   f.z1 = f.h1 + (size_t)tiles * kFragTile;
-  f.x = f.z1 + (size_t)tiles * kFragTile;
-  f.vec = reinterpret_cast<float*>(f.x + (size_t)tiles * (k1 / 16 * 32));
+  f.h2 = f.z1 + (size_t)tiles * kFragTile;
+  f.x = f.h2 + (size_t)tiles * kFragTile;
+  f.dout = reinterpret_cast<float*>(f.x + (size_t)tiles * (k1 / 16 * 32));
+  f.vec = f.dout + (size_t)tiles * kTile * kOutPad;
   return f;
 }
 
@@ -2112,7 +2082,56 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
 // it took 16 K cycles at batch 256, now 4 K (a whole step 23.0 -> 16.6 us).
 constexpr int kTuItem = 256;  // floats of an item
 constexpr int kTuSlots = 16;
-template <int kWarps, bool kSlots>
+constexpr int kBigB3 = kHid, kBigHub = kBigB3 + kOut;  // vectors of a 128-sample tile: db1 | db3 | Huber sum
+// x in three BF16 terms (24 bits: exact for a normal x not near the smallest).
+__device__ __forceinline__ void split_bf16(float x, float (&t)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    t[i] = __bfloat162float(__float2bfloat16_rn(x));
+    x -= t[i];
+  }
+}
+// The head's part of a 128-sample learner step for 16 units, over fragment
+// tiles t0 .. t1 - 1: dW3[o][n] = sum_s dO[s][o] H2[s][n] and M[n][o] = sum over the
+// samples with H2[s][n] > 0 of dO[s][o], from which db2[n] = sum_o W3[o][n] M[n][o].
+// dO in three BF16 terms against the exact BF16 H2 and 0 / 1: FP32 sums of
+// exact products, as on the CUDA cores (there 100 instructions a tile and warp).
+__device__ __forceinline__ void upd_head(const TdFrag& f, int blk, int t0, int t1, float* out, int lane) {
+  const int g = lane >> 2, q = lane & 3;
+  float acc[2][4] = {};
+#pragma unroll 2
+  for (int i = t0; i < t1; ++i) {
+    const uint4 a = __ldcg(f.h2 + (long long)i * kFragTile + blk * 32 + lane);
+    const float* d = f.dout + ((long long)i * kTile + 2 * q) * kOutPad + g;
+    float t[4][3];
+    split_bf16(__ldcg(d), t[0]);
+    split_bf16(__ldcg(d + kOutPad), t[1]);
+    split_bf16(__ldcg(d + 8 * kOutPad), t[2]);
+    split_bf16(__ldcg(d + 9 * kOutPad), t[3]);
+    const uint32_t ar[4] = {a.x, a.y, a.z, a.w};
+    uint32_t ar1[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      ar1[j] = ((ar[j] & 0x7FFFu) ? 0x3F80u : 0u) | ((ar[j] & 0x7FFF0000u) ? 0x3F800000u : 0u);
+    float s[2][4] = {};
+#pragma unroll
+    for (int n = 2; n >= 0; --n) {
+      const uint32_t b0 = pack_bf16x2(t[0][n], t[1][n]), b1 = pack_bf16x2(t[2][n], t[3][n]);
+      mma_bf16(s[0], ar, b0, b1);
+      mma_bf16(s[1], ar1, b0, b1);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[h][j] += s[h][j];
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      *reinterpret_cast<float2*>(out + 128 * h + (g + 8 * j) * kOutPad + 2 * q) = make_float2(acc[h][2 * j], acc[h][2 * j + 1]);
+}
+template <int kWarps, bool kSlots, bool kBig>
 __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f, int ntiles) {
   __shared__ float sum[kSlots ? kTuSlots : kWarps][kTuItem];
   pdl_launch_dependents();
@@ -2122,13 +2141,32 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
   const bool w2 = item < n2, mat = item < n2 + n1;
   const int mb = w2 ? item >> 4 : (item - n2) / nx, nb = w2 ? item & 15 : (item - n2) % nx;
   // this thread's parameters: columns k, k + 1 of row r, or vector entry ve
+  constexpr int kHub = kBig ? kBigHub : kVecHub;
+  constexpr int kVecItems = (kHub + 1 + 63) / 64;
   const int r = mb * 16 + t / 8, k = nb * 16 + 2 * (t % 8), ve = (item - n2 - n1) * 64 + t;
+  const bool head = kBig && item >= n2 + n1 + kVecItems;
+  const int hb = item - n2 - n1 - kVecItems;
+  float w3[kOut];  // b2 of the head items: W3's column, before this launch changes it
   int at = 0;
   bool live[2];
   if (mat) {
     at = w2 ? u.P.w2 + r * kHid + k : u.P.w1 + r * u.L.n_in + k;
     live[0] = t < 128 && (w2 || k < u.L.n_in);
     live[1] = t < 128 && (w2 || k + 1 < u.L.n_in);
+  } else if (head) {
+    const int n = hb * 16 + t % 16, o = t / 16;  // dW3[o][n], then db2[n]
+    at = o < kOut ? u.P.w3 + o * kHid + n : u.P.b2 + n;
+    live[0] = o <= kOut;
+    live[1] = false;
+    if (o == kOut) {
+#pragma unroll
+      for (int i = 0; i < kOut; ++i)
+        w3[i] = __bfloat162float(reinterpret_cast<const bf16*>(u.img + u.L.w3)[i * kLdh + n]);
+    }
+  } else if (kBig) {
+    at = ve < kBigB3 ? u.P.b1 + ve : u.P.b3 + (ve - kBigB3);
+    live[0] = t < 64 && ve < kBigHub;
+    live[1] = false;
   } else {
     at = ve < kVecDb2 ? u.P.b1 + ve : ve < kVecW3 ? u.P.b2 + (ve - kVecDb2)
                                     : ve < kVecB3 ? u.P.w3 + (ve - kVecW3) : u.P.b3 + (ve - kVecB3);
@@ -2145,7 +2183,9 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
   }
   pdl_wait();
   const unsigned fail = __ldcg(u.fail);
-  const int per = (ntiles + kWarps - 1) / kWarps, t0 = warp * per, t1 = min(ntiles, t0 + per);
+  // fragment tiles, or the vectors of 128-sample tiles
+  const int nt = kBig && !mat && !head ? (ntiles + kLtSub - 1) / kLtSub : ntiles;
+  const int per = (nt + kWarps - 1) / kWarps, t0 = warp * per, t1 = min(nt, t0 + per);
   if (mat) {
     const uint4* fa = (w2 ? f.z2 : f.z1) + mb * 32 + lane;
     const uint4* fb = (w2 ? f.h1 : f.x) + nb * 32 + lane;
@@ -2173,10 +2213,12 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
       if (kSlots) put(sum[i]);
     }
     if (!kSlots) put(sum[warp]);
+  } else if (head) {
+    upd_head(f, hb, t0, t1, sum[warp], lane);
   } else {
     const int e = (item - n2 - n1) * 64 + 2 * lane;
     float2 acc = make_float2(0.0f, 0.0f);
-    if (e <= kVecHub) {
+    if (e <= kHub) {
 #pragma unroll 4
       for (int i = t0; i < t1; ++i) {
         const float2 x = __ldcg(reinterpret_cast<const float2*>(f.vec + (long long)i * kVecLd + e));
@@ -2213,140 +2255,78 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
       else
         upd_images<1, 2>(u, run, r, k, th[0], th[1]);
     }
+  } else if (head) {
+    if (live[0]) {
+      float gr = 0.0f;
+      if (t < kOut * 16) {
+        gr = total((t % 16) * kOutPad + t / 16);
+      } else {
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) gr += w3[o] * total(128 + (t % 16) * kOutPad + o);
+      }
+      upd_one(u, run, at, gr, th[0], m[0], v[0]);
+    }
   } else if (live[0]) {
     upd_one(u, run, at, total(t), th[0], m[0], v[0]);
-  } else if (ve == kVecHub && t < 64 && u.loss) {
+  } else if (ve == kHub && t < 64 && u.loss) {
     *u.loss = total(t) / (float)u.batch;
   }
   upd_end(u, failed);
 }
-inline int td_update_items(int k1) { return 256 + 16 * (k1 / 16) + (kVecHub + 1 + 63) / 64; }
+inline int td_update_items(int k1, bool big) {
+  return 256 + 16 * (k1 / 16) + (big ? (kBigHub + 1 + 63) / 64 + 16 : (kVecHub + 1 + 63) / 64);
+}
 
 
-// ------------------------------------------------ tcgen05 learner (batch >= 128)
-// The TD step for large batches on the fifth-generation tensor cores, in
-// 128-sample tiles (one per CTA, 8 warps, the whole shared memory, 512
-// tensor-memory columns):
-//   k_td_target_tc: per (network, tile) job the forward of Q_online(s') or
-//     Q_target(s') (the fused rollout's layer order, weights streamed through
-//     two 32 KB buffers); the Q-values go to global memory.
-//   k_td_grad_tc: per tile y = r + gamma (1 - term) Q_target(s', argmax
-//     Q_online(s')), the forward on s keeping H1 and H2, dQ -> dO (dueling
-//     combine), dW3 / db3 / dH2 / dZ2 / db2 on the CUDA cores, then on the
-//     tensor cores dW2 = dZ2^T H1, dH1 = dZ2 W2^T (-> dZ1, db1) and
-//     dW1 = dZ1^T X; the tile's gradient goes to its own partial row, so the
-//     reduction (k_adam, in tile order) is fixed.
-// The weight-gradient and backpropagation products read their operands
-// transposed: a K-major tile [rows][cols] (core matrices of 8 rows x 16
-// bytes, LBO = rows x 16 between 8-column groups, SBO = 128 between 8-row
-// groups) is, for the transposed product, an MN-major operand whose core
-// matrices are the same 128 bytes (8 consecutive MN elements per 16-byte
-// row, 8 K rows): SBO = rows x 16 between 8-element MN groups, LBO = 128
-// between 8-row K groups, and the instruction descriptor's transpose bit of
-// that operand set.  The same BF16 recipe as the mma.sync learner (BF16
-// weights, activations and backpropagated dZ, FP32 sums; dW3, db and the
-// head on the CUDA cores in FP32).
-constexpr int kLtRows = 128;
-constexpr int kLtThreads = 256;
-// Below this batch the 16-sample mma.sync learner is faster (its CTAs spread
-// over more SMs); measured on one GB300: 58 vs 98 us per step at batch 256,
-// 120 vs 98 us at 4,096 with the two-kernel tcgen05 learner.
+// ------------------------------------------------ tcgen05 learner (large batches)
+// The tiles of k_td_tile with 128 samples, on the fifth-generation tensor
+// cores: a cluster of three CTAs takes a tile (rank 0 the forward on s and the
+// backward pass, ranks 1 and 2 the online and target network's Q(s')), every
+// CTA with its network's W1, W2 and W3 resident in shared memory (bulk copies,
+// once per launch).  Thread 0 issues the MMAs; 16 warps run the epilogues on
+// their lane quarter and 64 columns.  Accumulators are read in the fragment
+// shape of mma.sync (tcgen05.ld.16x256b), so that an epilogue packs its BF16
+// pairs back into tensor memory as the next layer's A operand
+// (tcgen05.st.16x128b) and, with one movmatrix per 8 x 8 block, writes the
+// operands that k_td_update sums the weight gradients from:
+//   [0, 256)   layer 1, H1 (first half of each 64), head in [32, 48), then dH1
+//   [256, 512) layer 2, H2, then dZ2 over it
+// dH1 = dZ2 W2 reads W2's shared-memory operand transposed: a K-major tile of R
+// rows is, MN-major, the same 128-byte core matrices with SBO = 16 R between
+// 8-element MN groups and LBO = 128 between 8-row K groups.
+// Bound by the latency of its chain (gather, three layers, dO, dH1, about 18 K
+// cycles).  In place of the learner whose jobs streamed W2 through two 32 KB
+// buffers, ran a forward for each of two roles a tile and wrote a 330 KB
+// gradient row per tile: batch 4,096 76 -> 45.6 us.
+// Below this batch the 16-sample learner's CTAs spread over more SMs and its
+// chain is shorter.
 constexpr int kLtMinBatch = 2048;
-constexpr uint32_t kLtBuf = 32u * 1024u;
 
 struct LtSmem {
-  uint32_t x, h1, h2, b0, b1, dout, bias, bytes;
+  uint32_t x, w1, w2, w3, dout, bias, w3f, red, next, bytes;
 };
 __host__ __device__ inline LtSmem lt_smem(int k1) {
   LtSmem t;
   t.x = 0;
-  t.h1 = tc_up((uint32_t)(kLtRows * k1 * 2));
-  t.h2 = t.h1 + (uint32_t)(kLtRows * kHid * 2);
-  t.b0 = t.h2 + (uint32_t)(kLtRows * kHid * 2);
-  t.b1 = t.b0 + kLtBuf;
-  t.dout = t.b1 + kLtBuf;                          // dO [128][8] float
-  t.bias = t.dout + (uint32_t)(kLtRows * kOutPad * 4);  // b1, b2 [256] float, b3 [8], reduction scratch [4][256]
-  t.bytes = t.bias + (uint32_t)((2 * kHid + kOutPad + 4 * kHid) * 4);
+  t.w1 = (uint32_t)(kLtRows * k1 * 2);
+  t.w2 = t.w1 + (uint32_t)(kHid * k1 * 2);
+  t.w3 = t.w2 + (uint32_t)(kHid * kHid * 2);
+  t.dout = t.w3 + 16u * kHid * 2u;                       // dO [128][8] float
+  t.bias = t.dout + (uint32_t)(kLtRows * kOutPad * 4);   // b1, b2 [256] float
+  t.w3f = t.bias + 2u * kHid * 4u;                       // W3 [6][256] float
+  t.red = t.w3f + (uint32_t)(kOut * kHid * 4);           // column sums [4][256] float
+  t.next = t.red + 4u * kHid * 4u;                       // Q(s') [tile parity][network][128][5] float
+  t.bytes = t.next + 2u * 2u * kLtRows * 5u * 4u;
   return t;
 }
+static_assert(128 * 80 * 2 + 256 * 80 * 2 + 256 * 256 * 2 + 16 * 256 * 2 + 128 * 32 + 2048 + 6144 + 4096 + 10240 <=
+                  227 * 1024 - 1024,
+              "tcgen05 learner: shared memory");
 
 // Instruction descriptor with the operands' major-ness: trans_a / trans_b = 1
 // reads A / B MN-major (bits 15 / 16).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32_t(int M, int N, int trans_a, int trans_b) {
   return idesc_bf16_f32(M, N) | ((uint32_t)trans_a << 15) | ((uint32_t)trans_b << 16);
-}
-
-// nks MMAs of K = 16: A at a0 + ks * ka, B at b0 + ks * kb (shared-memory
-// byte addresses), each with its own leading / stride byte offsets.
-__device__ __forceinline__ void lt_mma(uint32_t tacc, uint32_t a0, uint32_t lba, uint32_t sba, uint32_t ka,
-                                       uint32_t b0, uint32_t lbb, uint32_t sbb, uint32_t kb, uint32_t idesc, int nks,
-                                       bool accumulate) {
-  for (int ks = 0; ks < nks; ++ks)
-    tc_mma_bf16(tacc, smem_desc(a0 + (uint32_t)ks * ka, lba, sba), smem_desc(b0 + (uint32_t)ks * kb, lbb, sbb), idesc,
-                (accumulate || ks > 0) ? 1u : 0u);
-}
-
-// The two weight buffers of a CTA, run by thread 0: a copy into buffer b
-// waits (bounded) until the MMAs that read it are done.
-struct LtStream {
-  uint64_t* ld;
-  uint64_t* mm;
-  uint8_t* buf[2];
-  uint32_t pl[2], pm[2];
-  bool ld_out[2], mm_out[2];
-  bool ok;
-  __device__ __forceinline__ void load(int b, const void* src, uint32_t bytes) {
-    if (!ok) return;
-    if (mm_out[b]) {
-      ok = mbar_wait(&mm[b], pm[b], kTcTries);
-      pm[b] ^= 1u;
-      mm_out[b] = false;
-      if (!ok) return;
-    }
-    mbar_expect_tx(&ld[b], bytes);
-    bulk_g2s(buf[b], src, bytes, &ld[b]);
-    ld_out[b] = true;
-  }
-  __device__ __forceinline__ bool ready(int b) {
-    if (!ok) return false;
-    if (ld_out[b]) {
-      ok = mbar_wait(&ld[b], pl[b], kTcTries);
-      pl[b] ^= 1u;
-      ld_out[b] = false;
-    }
-    if (ok) tc_fence_after();
-    return ok;
-  }
-  __device__ __forceinline__ void done(int b) {
-    tc_commit(&mm[b]);
-    mm_out[b] = true;
-  }
-  __device__ __forceinline__ void drain() {
-    for (int b = 0; b < 2; ++b) {
-      if (mm_out[b]) mbar_wait(&mm[b], pm[b], kTcTries);
-      if (ld_out[b]) mbar_wait(&ld[b], pl[b], kTcTries);
-    }
-  }
-};
-
-// Rows of a tile: sample i's ring entry (or -1 past the batch) into X (BF16,
-// K-major, zero padded); the two threads of a row take alternate 8-column
-// groups.
-__device__ __forceinline__ void lt_load_x(uint8_t* xs, const float* __restrict__ src, const int* rows_sh, int n_in,
-                                          int k1, int tid) {
-  const int row = tid & (kLtRows - 1);
-  const int e = rows_sh[row];
-  for (int kg = tid >> 7; kg < k1 / 8; kg += 2) {
-    float v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int k = kg * 8 + j;
-      v[j] = (e >= 0 && k < n_in) ? __ldg(src + (long long)e * n_in + k) : 0.0f;
-    }
-    *reinterpret_cast<uint4*>(xs + kmajor_offset(row, kg * 8, kLtRows)) =
-        make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
-  }
-  fence_async_smem();
 }
 
 // A CTA-wide barrier that also orders the tensor-core work around it.
@@ -2355,503 +2335,383 @@ __device__ __forceinline__ void lt_sync() {
   __syncthreads();
   tc_fence_after();
 }
-
-// Thread 0: the two W1 halves of timg into the two buffers (issued before the
-// tile's inputs are gathered, so that the copies overlap the gathers).
-__device__ __forceinline__ void lt_prefetch_w1(LtStream& S, const uint8_t* __restrict__ timg, const ImgLayout& L) {
-  const TcImg G = tc_img(L.k1);
-  const uint32_t w1h = 128u * (uint32_t)L.k1 * 2u;
-  S.load(0, timg + G.w1h, w1h);
-  S.load(1, timg + G.w1h + w1h, w1h);
+__device__ __forceinline__ uint32_t movmatrix(uint32_t a) {
+  uint32_t d;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(d) : "r"(a));
+  return d;
 }
-
-// The forward of one tile (X in xs) through the network whose tensor-core
-// image is timg (W1 already on its way, lt_prefetch_w1), the hidden
-// activations left in h1s / h2s (BF16, K-major), the head's 16 columns in
-// tensor-memory columns [0, 16).  Thread 0 issues the MMAs and copies; every
-// thread runs the epilogues.  Returns false when a wait ran out (then
-// nothing after it was issued).
-__device__ __forceinline__ bool lt_forward(LtStream& S, uint64_t* bar_layer, uint32_t& player, uint32_t tacc,
-                                           const uint8_t* __restrict__ timg, const ImgLayout& L, uint8_t* xs,
-                                           uint8_t* h1s, uint8_t* h2s, const float* b1, const float* b2, int tid,
-                                           bool& layer_out) {
-  const TcImg G = tc_img(L.k1);
-  const int warp = tid >> 5, lane = tid & 31;
-  const uint32_t w2q = 64u * kHid * 2u;
-  const uint32_t sx = smem_u32(xs), sh1 = smem_u32(h1s), sh2 = smem_u32(h2s);
-  const uint32_t kA = kLtRows * 16u;  // K-group stride of a 128-row K-major tile
-  if (tid == 0) {
-    // layer 1 in two 128-unit halves (W1 halves in the two buffers)
-    for (int h = 0; h < 2; ++h)
-      if (S.ready(h)) {
-        lt_mma(tacc + 128u * h, sx, kA, 128, 2 * kA, smem_u32(S.buf[h]), 128u * 16u, 128, 2u * 128u * 16u,
-               idesc_bf16_f32(kLtRows, 128), L.k1 / 16, false);
-        S.done(h);
-      }
-    if (S.ok) tc_commit(bar_layer);
-    // W2 in 32 KB pieces: the two K halves of its first 128 rows follow as
-    // soon as the buffers are free
-    S.load(0, timg + G.w2a, w2q);
-    S.load(1, timg + G.w2a + w2q, w2q);
+// 16 samples x 64 units in C-fragment pairs (p[2 j]: sample g, p[2 j + 1]: g + 8,
+// units 8 j + 2 q, + 1) as k_td_update's operands of four 16-unit blocks: A
+// fragments of the transpose, or B fragments.
+template <bool kA>
+__device__ __forceinline__ void lt_put_frags(uint4* out, const uint32_t (&p)[16], int lane) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const uint32_t l0 = movmatrix(p[4 * b]), l1 = movmatrix(p[4 * b + 1]);
+    const uint32_t h0 = movmatrix(p[4 * b + 2]), h1 = movmatrix(p[4 * b + 3]);
+    out[b * 32 + lane] = kA ? make_uint4(l0, h0, l1, h1) : make_uint4(l0, l1, h0, h1);
   }
-  layer_out = true;
-  bool ok = __syncthreads_and(mbar_wait(bar_layer, player, kTcTries));
-  player ^= 1u;
-  layer_out = !ok;
-  if (!ok) return false;
-  tc_fence_after();
-  tc_epilogue_hidden(tacc, b1, h1s, warp, lane);
-  fence_async_smem();
-  lt_sync();
-  if (tid == 0) {
-    // layer 2 in two 128-unit halves (N = 128: an MMA of M = 128 costs
-    // about as much at N = 64 as at 128), each from two 32 KB K-half pieces
-    // of its rows (piece c: K steps 8 c .. 8 c + 7, in buffer c); the second
-    // half's pieces are copied in as the first half's are consumed
-    for (int h = 0; h < 2; ++h)
-      for (int c = 0; c < 2; ++c) {
-        if (h == 1) S.load(c, timg + G.w2b + (uint32_t)c * w2q, w2q);
-        if (S.ready(c)) {
-          lt_mma(tacc + 128u * h, sh1 + (uint32_t)(16 * c) * kA, kA, 128, 2 * kA, smem_u32(S.buf[c]), 128u * 16u,
-                 128, 2u * 128u * 16u, idesc_bf16_f32(kLtRows, 128), kHid / 32, c > 0);
-          S.done(c);
-        }
+}
+// Hidden-layer epilogue of a warp's 32 rows x 64 columns at t: bias, ReLU, BF16
+// pairs back into the first half of the columns; with kOut != 0 also as
+// fragments (1: B, 2: A) to out (the next 16 samples 16 blocks on), and mask[h]
+// bit 4 j + e = whether element e of octet j is positive.
+template <int kPut>
+__device__ __forceinline__ void lt_epilogue(uint32_t t, const float* bias, uint4* out, uint32_t (&mask)[2], int lane) {
+  const float2* b2 = reinterpret_cast<const float2*>(bias) + (lane & 3);
+  uint32_t r[2][32];
+  tmem_ld_frag64_nowait(t, r[0]);
+  tmem_ld_frag64_nowait(t + (16u << 16), r[1]);
+  tmem_ld_wait();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t p[16], mk = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float2 b = b2[4 * j];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const uint32_t w = pack_bf16x2(fmaxf(__uint_as_float(r[h][4 * j + 2 * e]) + b.x, 0.f),
+                                       fmaxf(__uint_as_float(r[h][4 * j + 2 * e + 1]) + b.y, 0.f));
+        p[2 * j + e] = w;
+        if (kPut) mk |= ((w & 0x7FFFu) ? 1u : 0u) << (4 * j + 2 * e) | ((w & 0x7FFF0000u) ? 2u : 0u) << (4 * j + 2 * e);
       }
-    if (S.ok) tc_commit(bar_layer);
-    S.load(0, timg + G.w3, 16u * kHid * 2u);  // the head's weights next
-  }
-  layer_out = true;
-  ok = __syncthreads_and(mbar_wait(bar_layer, player, kTcTries));
-  player ^= 1u;
-  layer_out = !ok;
-  if (!ok) return false;
-  tc_fence_after();
-  tc_epilogue_hidden(tacc, b2, h2s, warp, lane);
-  fence_async_smem();
-  lt_sync();
-  if (tid == 0) {
-    if (S.ready(0)) {
-      lt_mma(tacc, sh2, kA, 128, 2 * kA, smem_u32(S.buf[0]), 16u * 16u, 128, 2u * 16u * 16u,
-             idesc_bf16_f32(kLtRows, 16), kHid / 16, false);
-      S.done(0);
-      tc_commit(bar_layer);
+    }
+    tmem_st_frag32(t + ((uint32_t)(16 * h) << 16), p);
+    if (kPut) {
+      lt_put_frags<kPut == 2>(out + h * kFragTile, p, lane);
+      mask[h] = mk;
     }
   }
-  layer_out = true;
-  ok = __syncthreads_and(mbar_wait(bar_layer, player, kTcTries));
-  player ^= 1u;
-  layer_out = !ok;
-  if (ok) tc_fence_after();
-  return ok;
+  tmem_st_wait();
 }
 
-// Sum of this lane's 32 values over the warp's 32 lanes, column by column:
-// afterwards lane l holds the sum of column l (fixed butterfly order).
-__device__ __forceinline__ float lt_colsum32(float (&v)[32], int lane) {
-#pragma unroll
-  for (int w = 16; w >= 1; w >>= 1) {
-    const bool upper = (lane & w) != 0;
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const float send = upper ? v[i] : v[i + w];
-      const float keep = upper ? v[i + w] : v[i];
-      v[i] = keep + __shfl_xor_sync(kFull, send, w);
-    }
-  }
-  return v[0];
-}
-
-// Bias vectors of a network's image into shared memory.
-__device__ __forceinline__ void lt_biases(const uint8_t* __restrict__ im, const ImgLayout& L, float* b1, float* b2,
-                                          float* b3, int tid) {
-  for (int i = tid; i < kHid; i += kLtThreads) {
-    b1[i] = __ldg(reinterpret_cast<const float*>(im + L.b1) + i);
-    b2[i] = __ldg(reinterpret_cast<const float*>(im + L.b2) + i);
-  }
-  if (tid < kOutPad) b3[tid] = __ldg(reinterpret_cast<const float*>(im + L.b3) + tid);
-  __syncthreads();
-}
-
-// The tensor-core work of one TD step in one kernel.  CTAs take jobs in start
-// order from a device counter: jobs [0, 2 ntiles) are the next-state
-// forwards (Q_online(s') of tile t, then Q_target(s') of tile t; Q-values to
-// q2[net][i][5], then the tile's counter in sync is raised), jobs
-// [2 ntiles, 4 ntiles) the tiles' loss and gradient in two halves per tile
-// (role 0: dW3, db3, db2, the loss, dW2; role 1: dH1, db1, dW1), each from its
-// own forward on s, into partial[tile].  A gradient job runs its forward
-// first and only then waits (bounded) for its tile's two next-state jobs:
-// those were taken earlier by CTAs that are running and never wait, so the
-// wait ends for any grid size.
-// sync: [0] the job counter, [1 + t] next-state jobs done for tile t; zero at
-// launch.
-__global__ void __launch_bounds__(kLtThreads, 1)
+__global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     k_td_tc(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, const uint8_t* __restrict__ timg,
-            const uint8_t* __restrict__ timg_t, ImgLayout L, ParamLayout P, ReplayDev rp, unsigned long long seed,
-            const unsigned long long* __restrict__ step, int batch, float gamma, float* __restrict__ q2,
-            unsigned* __restrict__ sync, float* __restrict__ partial, unsigned* __restrict__ fail) {
+            const uint8_t* __restrict__ timg_t, ImgLayout L, ReplayDev rp, unsigned long long seed,
+            const unsigned long long* __restrict__ step, int batch, float gamma, TdFrag f,
+            unsigned* __restrict__ fail) {
   extern __shared__ __align__(1024) uint8_t tsm[];
-  __shared__ uint64_t bar_ld[2], bar_mm[2], bar_layer;
+  __shared__ uint64_t bar_w1, bar_w2, bar_mma;
   __shared__ uint32_t tslot;
   __shared__ int rows_sh[kLtRows];
-  __shared__ float y_sh[kLtRows];
-  __shared__ float hub_sh[kLtRows / 32];
-  __shared__ int job_sh, flag_sh;
+  __shared__ float dsum_sh[4][kOutPad];
   const LtSmem T = lt_smem(L.k1);
   const TcImg G = tc_img(L.k1);
   uint8_t* xs = tsm + T.x;
-  uint8_t* h1s = tsm + T.h1;
-  uint8_t* h2s = tsm + T.h2;
   float* dout = reinterpret_cast<float*>(tsm + T.dout);
   float* b1 = reinterpret_cast<float*>(tsm + T.bias);
   float* b2 = b1 + kHid;
-  float* b3 = b2 + kHid;
-  float* red = b3 + kOutPad;  // [4][256] column sums of the four lane quarters
+  float* w3f = reinterpret_cast<float*>(tsm + T.w3f);
+  float* red = reinterpret_cast<float*>(tsm + T.red);
+  float* next_q = reinterpret_cast<float*>(tsm + T.next);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ntiles = (batch + kLtRows - 1) / kLtRows;
-  const uint32_t w2q = 64u * kHid * 2u;
-  const uint32_t kA = kLtRows * 16u;
-  const bf16* W3g = reinterpret_cast<const bf16*>(img + L.w3);
+  const int g = lane >> 2, q = lane & 3, quarter = warp & 3, grp = warp >> 2;
+  const uint32_t rank = cluster_rank();
+  const int ntiles = (batch + kLtRows - 1) / kLtRows, stride = (int)gridDim.x / kTpRanks;
+  cluster_arrive();  // every CTA of the cluster has started before the first remote store
   if (warp == 0) tmem_alloc(&tslot, 512);
   if (tid == 0) {
-    mbar_init(&bar_ld[0], 1);
-    mbar_init(&bar_ld[1], 1);
-    mbar_init(&bar_mm[0], 1);
-    mbar_init(&bar_mm[1], 1);
-    mbar_init(&bar_layer, 1);
+    mbar_init(&bar_w1, 1);
+    mbar_init(&bar_w2, 1);
+    mbar_init(&bar_mma, 1);
   }
+  pdl_wait();
+  pdl_launch_dependents();
   lt_sync();
-  const uint32_t tacc = tslot;
-  LtStream S;
-  S.ld = bar_ld;
-  S.mm = bar_mm;
-  S.buf[0] = tsm + T.b0;
-  S.buf[1] = tsm + T.b1;
-  S.pl[0] = S.pl[1] = S.pm[0] = S.pm[1] = 0u;
-  S.ld_out[0] = S.ld_out[1] = S.mm_out[0] = S.mm_out[1] = false;
-  S.ok = true;
-  uint32_t player = 0;
-  bool layer_out = false, ok = true;
+  const uint32_t tacc = tslot, tacc2 = tacc + 256u;
+  const uint32_t tw = ((uint32_t)(quarter * 32) << 16) + (uint32_t)(64 * grp);  // this warp's lanes and columns
+  const uint32_t sx = smem_u32(xs), sw1 = smem_u32(tsm + T.w1), sw2 = smem_u32(tsm + T.w2),
+                 sw3 = smem_u32(tsm + T.w3);
+  const uint8_t* im = rank == 2 ? img_t : img;
+  if (tid == 0) {
+    const uint8_t* src = rank == 2 ? timg_t : timg;
+    mbar_expect_tx(&bar_w1, G.w2a);
+    bulk_g2s(tsm + T.w1, src + G.w1, G.w2a, &bar_w1);
+    mbar_expect_tx(&bar_w2, kHid * kHid * 2u + 16u * kHid * 2u);
+    bulk_g2s(tsm + T.w2, src + G.w2f, kHid * kHid * 2u, &bar_w2);
+    bulk_g2s(tsm + T.w3, src + G.w3, 16u * kHid * 2u, &bar_w2);
+  }
+  for (int i = tid; i < 2 * kHid; i += kThreads)
+    b1[i] = __ldg(reinterpret_cast<const float*>(im + (i < kHid ? L.b1 : L.b2)) + (i & (kHid - 1)));
+  if (rank == 0)
+    for (int i = tid; i < kOut * kHid; i += kThreads)
+      w3f[i] = __bfloat162float(reinterpret_cast<const bf16*>(im + L.w3)[(i >> 8) * kLdh + (i & (kHid - 1))]);
+  for (int i = tid; i < kLtRows * L.k1 / 8; i += kThreads)
+    reinterpret_cast<uint4*>(xs)[i] = make_uint4(0u, 0u, 0u, 0u);
+  float b3[kOut];
+#pragma unroll
+  for (int j = 0; j < kOut; ++j) b3[j] = __ldg(reinterpret_cast<const float*>(im + L.b3) + j);
   const unsigned long long tstep = *step;
-  for (;;) {
-    if (tid == 0) job_sh = (int)atomicAdd(sync, 1u);
-    __syncthreads();
-    const int job = job_sh;
-    __syncthreads();  // every thread has the job before the next one is taken
-    if (job >= 4 * ntiles || !ok) break;
-    if (job < 2 * ntiles) {
-      const int net = job >= ntiles ? 1 : 0, tile = job - net * ntiles;
-      lt_biases(net ? img_t : img, L, b1, b2, b3, tid);
-      if (tid == 0) lt_prefetch_w1(S, net ? timg_t : timg, L);
-      if (tid < kLtRows) {
-        const int i = tile * kLtRows + tid;
-        const int e = i < batch ? (int)sample_entry(seed, tstep, i, rp) : -1;
-        rows_sh[tid] = e;
-      }
-      __syncthreads();
-      lt_load_x(xs, rp.s2, rows_sh, L.n_in, L.k1, tid);
-      lt_sync();
-      ok = lt_forward(S, &bar_layer, player, tacc, net ? timg_t : timg, L, xs, h1s, h2s, b1, b2, tid, layer_out);
-      if (warp < 4) {
-        const int i = tile * kLtRows + warp * 32 + lane;
-        float v[32];
-        if (ok) tmem_ld32(tacc + ((uint32_t)(warp * 32) << 16), v);
-        if (i < batch) {
-          float qv[5];
-          if (ok) {
-            float o[kOut];
-#pragma unroll
-            for (int j = 0; j < kOut; ++j) o[j] = v[j] + b3[j];
-            greedy_action(o, qv, L.plain);
-          } else {
-#pragma unroll
-            for (int a = 0; a < 5; ++a) qv[a] = __int_as_float(0x7fc00000);
-          }
-#pragma unroll
-          for (int a = 0; a < 5; ++a) q2[((long long)net * batch + i) * 5 + a] = qv[a];
-        }
-      }
-      // publish (also after a failure, whose Q-values are NaN): the values
-      // before the tile's counter (release)
-      __threadfence();
-      __syncthreads();
-      if (tid == 0) atomicAdd(sync + 1 + tile, 1u);
-      lt_sync();
-      continue;
-    }
-    // gradient jobs: role 0 of a tile computes dW3, db3, db2, the loss and
-    // dW2; role 1 (on another CTA, from the same forward) dH1, db1 and dW1
-    const int role = job >= 3 * ntiles ? 1 : 0;
-    const int tile = job - (2 + role) * ntiles;
-    float* pg = partial + (long long)tile * partial_stride(P.total);
-    if (tid == 0) lt_prefetch_w1(S, timg, L);
-    lt_biases(img, L, b1, b2, b3, tid);
-    // the tile's samples (the same counter-RNG draws as the next-state jobs)
+  const int nx = L.k1 / 16;
+  bool ok = true, first = true, mma_out = false;
+  uint32_t phase = 0u;
+  // wait for the MMAs committed last, by every thread
+  auto mma_wait = [&]() {
+    mma_out = true;
+    ok = __syncthreads_and(ok && mbar_wait(&bar_mma, phase, kTcTries));
+    phase ^= 1u;
+    if (ok) mma_out = false;
+    tc_fence_after();
+  };
+  for (int tile = (int)blockIdx.x / kTpRanks, it = 0; tile < ntiles; tile += stride, ++it) {
     if (tid < kLtRows) {
       const int i = tile * kLtRows + tid;
       rows_sh[tid] = i < batch ? (int)sample_entry(seed, tstep, i, rp) : -1;
     }
     __syncthreads();
-    lt_load_x(xs, rp.s, rows_sh, L.n_in, L.k1, tid);
-    lt_sync();
-    ok = lt_forward(S, &bar_layer, player, tacc, timg, L, xs, h1s, h2s, b1, b2, tid, layer_out);
-    if (!ok) break;
-    // the tile's two next-state jobs (taken earlier by running CTAs, which
-    // never wait) publish their Q-values; bounded wait
-    if (tid == 0) {
-      unsigned it = 0;
-      while (qt_ld_acquire(sync + 1 + tile) < 2u && ++it < kQtWaitIters) __nanosleep(256);
-      flag_sh = it < kQtWaitIters ? 1 : 0;
-    }
-    __syncthreads();
-    if (!flag_sh) {
-      ok = false;
-      break;
-    }
-    // double-DQN targets y = r + gamma (1 - term) Q_target(s', argmax_a Q_online(s', a))
-    if (tid < kLtRows) {
-      const int i = tile * kLtRows + tid, e = rows_sh[tid];
-      float y = 0.0f;
-      if (e >= 0) {
-        const float* qo = q2 + (long long)i * 5;
-        const float* qt = q2 + ((long long)batch + i) * 5;
-        int astar = 0;
-        float best = __ldcg(qo);
-        for (int a = 1; a < 5; ++a) {
-          const float v = __ldcg(qo + a);
-          if (v > best) {
-            best = v;
-            astar = a;
-          }
+    {
+      // a row per warp and pass: its floats are contiguous
+      const float* src = rank == 0 ? rp.s : rp.s2;
+      float v[8][3];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int e = rows_sh[warp * 8 + u];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int k = lane + 32 * c;
+          v[u][c] = e >= 0 && k < L.n_in ? __ldg(src + (long long)e * L.n_in + k) : 0.0f;
         }
-        const float nt = rp.term[e] ? 0.0f : 1.0f;
-        y = rp.r[e] + gamma * nt * __ldcg(qt + astar);
-        if (isnan(best)) y = best;  // a failed next-state job
       }
-      y_sh[tid] = y;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          if (lane + 32 * c < L.n_in)
+            *reinterpret_cast<bf16*>(xs + kmajor_offset(warp * 8 + u, lane + 32 * c, kLtRows)) =
+                __float2bfloat16_rn(v[u][c]);
     }
-    __syncthreads();
+    fence_async_smem();
+    lt_sync();
+    int e = -1, act = 0;
+    float rwd = 0.0f, nt = 1.0f;
+    if (rank == 0 && tid < kLtRows) {
+      // this sample's reward, flag and action on their way during the forward
+      e = rows_sh[tid];
+      if (e >= 0) {
+        act = rp.a[e];
+        rwd = rp.r[e];
+        nt = rp.term[e] ? 0.0f : 1.0f;
+      }
+    }
+    if (tid == 0 && ok && (!first || mbar_wait(&bar_w1, 0u, kTcTries))) {
+      tc_fence_after();
+      for (int ks = 0; ks < nx; ++ks)
+        tc_mma_bf16(tacc, smem_desc(sx + (uint32_t)ks * 2u * kLtRows * 16u, kLtRows * 16u, 128),
+                    smem_desc(sw1 + (uint32_t)ks * 2u * kHid * 16u, kHid * 16u, 128), idesc_bf16_f32(kLtRows, kHid),
+                    ks > 0 ? 1u : 0u);
+      tc_commit(&bar_mma);
+    }
+    if (rank == 0) {
+      // X's B fragments: a core matrix is an 8 x 8 block of 16-byte rows
+      for (int w = warp; w < kLtSub * nx; w += kThreads / 32) {
+        const int st = w / nx, kb = w % nx, mat = lane >> 3;  // matrices: samples 0-7, 8-15 of inputs 0-7, then 8-15
+        uint32_t r4[4];
+        ldsm_x4_t(r4, xs + kmajor_offset(st * 16 + (mat & 1) * 8 + (lane & 7), kb * 16 + (mat >> 1) * 8, kLtRows));
+        f.x[((long long)(tile * kLtSub + st) * nx + kb) * 32 + lane] = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+      }
+    }
+    mma_wait();
+    // this warp's fragment tiles: samples 32 quarter .., units 64 grp ..
+    const long long fo = (long long)(tile * kLtSub + 2 * quarter) * kFragTile + 4 * grp * 32;
+    uint32_t mask1[2] = {0u, 0u}, mask2[2] = {0u, 0u};
+    if (ok) {
+      if (rank == 0)
+        lt_epilogue<1>(tacc + tw, b1 + 64 * grp, f.h1 + fo, mask1, lane);
+      else
+        lt_epilogue<0>(tacc + tw, b1 + 64 * grp, nullptr, mask1, lane);
+    }
+    lt_sync();
+    if (tid == 0 && ok && (!first || mbar_wait(&bar_w2, 0u, kTcTries))) {
+      tc_fence_after();
+      tc_layer_ta(tacc2, tacc, sw2, kHid);
+      tc_commit(&bar_mma);
+    }
+    first = false;
+    mma_wait();
+    if (ok) {
+      if (rank == 0)
+        lt_epilogue<2>(tacc2 + tw, b2 + 64 * grp, f.h2 + fo, mask2, lane);
+      else
+        lt_epilogue<0>(tacc2 + tw, b2 + 64 * grp, nullptr, mask2, lane);
+    }
+    lt_sync();
+    if (tid == 0 && ok) {
+      tc_layer_ta(tacc + 32u, tacc2, sw3, 16);
+      tc_commit(&bar_mma);
+    }
+    mma_wait();
+    float qv[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    if (warp < 4) {
+      uint32_t v[8];
+      float o[kOut];
+      if (ok) {
+        tmem_ld8_nowait(tacc + 32u + ((uint32_t)(warp * 32) << 16), v);
+        tmem_ld_wait();
+      }
+#pragma unroll
+      for (int j = 0; j < kOut; ++j) o[j] = (ok ? __uint_as_float(v[j]) : __int_as_float(0x7fc00000)) + b3[j];
+      greedy_action(o, qv, L.plain);
+    }
+    if (it == 0) cluster_wait();  // the start's arrival
+    if (rank != 0 && warp < 4) {
+#pragma unroll
+      for (int a = 0; a < 5; ++a)
+        st_cluster(next_q + (((it & 1) * 2 + (int)rank - 1) * kLtRows + tid) * 5 + a, 0u, qv[a]);
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (rank != 0 || !ok) {
+      lt_sync();  // the head is read before the next tile's layer 1
+      continue;
+    }
+    // double-DQN targets y = r + gamma (1 - term) Q_target(s', argmax_a Q_online(s', a));
     // dL/dQ(s, a) = clip(Q(s, a) - y) / B, back through the head's combine
     if (warp < 4) {
-      const int r = warp * 32 + lane, e = rows_sh[r];
-      float v[32];
-      tmem_ld32(tacc + ((uint32_t)(warp * 32) << 16), v);
-      float hl = 0.0f;
-      float* dO = dout + r * kOutPad;
-      for (int k = 0; k < kOutPad; ++k) dO[k] = 0.0f;
+      const float* qo = next_q + ((it & 1) * 2 * kLtRows + tid) * 5;
+      const float* qt = qo + kLtRows * 5;
+      float d8[kOutPad] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       if (e >= 0) {
-        float o[kOut], qv[5];
+        float best = qo[0], qs = qt[0], qa = qv[0];
 #pragma unroll
-        for (int j = 0; j < kOut; ++j) o[j] = v[j] + b3[j];
-        greedy_action(o, qv, L.plain);
-        int a = rp.a[e];
+        for (int a = 1; a < 5; ++a) {
+          if (qo[a] > best) best = qo[a], qs = qt[a];
+          if (act == a) qa = qv[a];
+        }
+        const float y = isnan(best) ? best : rwd + gamma * nt * qs;  // NaN: a failed next-state forward
         float d;
-        if (a >= 5) {
+        if (act >= 5) {
           atomicOr(fail, kTdFailAction);
-          a = 0;
+          act = 0;
           d = __int_as_float(0x7fc00000);
         } else {
-          d = qv[a] - y_sh[r];
+          d = qa - y;
         }
         const float ad = fabsf(d);
-        hl = ad <= 1.0f ? 0.5f * d * d : ad - 0.5f;
         const float gq = (isnan(d) ? d : fminf(fmaxf(d, -1.0f), 1.0f)) / (float)batch;
         if (L.plain) {
-          for (int k = 0; k < 5; ++k) dO[k] = k == a ? gq : 0.0f;
+#pragma unroll
+          for (int k = 0; k < 5; ++k) d8[k] = k == act ? gq : 0.0f;
         } else {
-          dO[0] = gq;
-          for (int k = 0; k < 5; ++k) dO[1 + k] = (k == a ? gq : 0.0f) - gq / 5.0f;
+          d8[0] = gq;
+#pragma unroll
+          for (int k = 0; k < 5; ++k) d8[1 + k] = (k == act ? gq : 0.0f) - gq / 5.0f;
         }
+        d8[7] = ad <= 1.0f ? 0.5f * d * d : ad - 0.5f;  // the Huber term beside dO
       }
-      // the tile's Huber sum: lanes in order, then warps in order
-      for (int off = 16; off > 0; off >>= 1) hl += __shfl_xor_sync(kFull, hl, off);
-      if (lane == 0) hub_sh[warp] = hl;
+      float4* dO = reinterpret_cast<float4*>(dout + tid * kOutPad);
+      float4* dg = reinterpret_cast<float4*>(f.dout + ((long long)tile * kLtRows + tid) * kOutPad);
+      dO[0] = dg[0] = make_float4(d8[0], d8[1], d8[2], d8[3]);
+      dO[1] = dg[1] = make_float4(d8[4], d8[5], d8[6], d8[7]);
     }
-    lt_sync();
-    // CUDA cores, thread per hidden unit n: dW3[o][n] = sum_s dO[s][o] H2[s][n],
-    // dZ2[s][n] = (H2 > 0) sum_o dO[s][o] W3[o][n] written over H2 (BF16),
-    // db2[n] = sum_s dZ2[s][n] (FP32)
+    __syncthreads();
+    // dZ2 = (H2 > 0) dO W3 (FP32, then BF16) over H2, and its fragments
     {
-      const int n = tid;
-      float w3c[kOut];
+      float d[4][kOut];
 #pragma unroll
-      for (int o = 0; o < kOut; ++o) w3c[o] = __bfloat162float(W3g[o * kLdh + n]);
-      float acc3[kOut];
+      for (int i = 0; i < 4; ++i) {
+        const float* p = dout + (quarter * 32 + 8 * i + g) * kOutPad;
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        const float2 b = *reinterpret_cast<const float2*>(p + 4);
+        d[i][0] = a.x, d[i][1] = a.y, d[i][2] = a.z, d[i][3] = a.w, d[i][4] = b.x, d[i][5] = b.y;
+      }
+      uint32_t p[2][16];
 #pragma unroll
-      for (int o = 0; o < kOut; ++o) acc3[o] = 0.0f;
-      float db2 = 0.0f;
-      // four rows at a time: their loads are independent of the stores
-      for (int r0 = 0; r0 < kLtRows; r0 += 4) {
-        bf16* hp[4];
-        float h[4];
+      for (int j = 0; j < 8; ++j) {
+        float z[4][2] = {};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          hp[u] = reinterpret_cast<bf16*>(h2s + kmajor_offset(r0 + u, n, kLtRows));
-          h[u] = __bfloat162float(*hp[u]);
-        }
-        bf16 z[4];
+        for (int o = 0; o < kOut; ++o) {
+          const float2 w = *reinterpret_cast<const float2*>(w3f + o * kHid + 64 * grp + 8 * j + 2 * q);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float* dO = dout + (r0 + u) * kOutPad;
-          float dh = 0.0f;
-#pragma unroll
-          for (int o = 0; o < kOut; ++o) {
-            acc3[o] += dO[o] * h[u];
-            dh += dO[o] * w3c[o];
+          for (int i = 0; i < 4; ++i) {
+            z[i][0] += d[i][o] * w.x;
+            z[i][1] += d[i][o] * w.y;
           }
-          const float dz = h[u] > 0.0f ? dh : 0.0f;
-          db2 += dz;
-          z[u] = __float2bfloat16_rn(dz);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) *hp[u] = z[u];
-      }
-      if (role == 0) {
-#pragma unroll
-        for (int o = 0; o < kOut; ++o) pg[P.w3 + o * kHid + n] = acc3[o];
-        pg[P.b2 + n] = db2;
-        if (n < kOut) {
-          float acc = 0.0f;
-          for (int r = 0; r < kLtRows; ++r) acc += dout[r * kOutPad + n];
-          pg[P.b3 + n] = acc;
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t mk = mask2[i >> 1] >> (4 * j + 2 * (i & 1));
+          p[i >> 1][2 * j + (i & 1)] = pack_bf16x2((mk & 1u) ? z[i][0] : 0.0f, (mk & 2u) ? z[i][1] : 0.0f);
         }
-        if (n == 0) pg[P.total] = ((hub_sh[0] + hub_sh[1]) + hub_sh[2]) + hub_sh[3];
       }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        tmem_st_frag32(tacc2 + tw + ((uint32_t)(16 * h) << 16), p[h]);
+        lt_put_frags<true>(f.z2 + fo + h * kFragTile, p[h], lane);
+      }
+      tmem_st_wait();
     }
-    fence_async_smem();
     lt_sync();
-    if (role == 0) {
-      // tensor cores: dW2 = dZ2^T H1 (M = out unit in two halves, N = in unit,
-      // K = sample; both operands transposed) into columns [0, 512); the W2
-      // quarters of dH1 stream in meanwhile
-      if (tid == 0) {
-        for (int h = 0; h < 2; ++h)
-          lt_mma(tacc + 256u * h, smem_u32(h2s) + 16u * (uint32_t)h * kA, 128, kA, 2u * 128u, smem_u32(h1s), 128, kA,
-                 2u * 128u, idesc_bf16_f32_t(kLtRows, kHid, 1, 1), kLtRows / 16, false);
-        tc_commit(&bar_layer);
-      }
-      layer_out = true;
-      ok = __syncthreads_and(mbar_wait(&bar_layer, player, kTcTries));
-      player ^= 1u;
-      layer_out = !ok;
-      if (!ok) break;
-      tc_fence_after();
-      {
-        // warp w: rows of lane quarter w % 4 (out unit 32 (w % 4) + lane of half
-        // w / 4), 32 columns at a time through a 32 x 32 float tile of buffer 1
-        // (rotated by the row: conflict-free both ways), then stored row by row
-        // with the warp's 32 lanes on 32 consecutive columns (coalesced)
-        const int quarter = warp & 3, h = warp >> 2, n0 = 128 * h + quarter * 32;
-        float* st = reinterpret_cast<float*>(S.buf[1]) + warp * 32 * 32;
-        for (int c = 0; c < kHid; c += 32) {
-          float v[32];
-          tmem_ld32(tacc + ((uint32_t)(quarter * 32) << 16) + 256u * h + (uint32_t)c, v);
-#pragma unroll
-          for (int k = 0; k < 32; ++k) st[lane * 32 + ((k + lane) & 31)] = v[k];
-          __syncwarp();
-#pragma unroll 8
-          for (int r = 0; r < 32; ++r) pg[P.w2 + (long long)(n0 + r) * kHid + c + lane] = st[r * 32 + ((lane + r) & 31)];
-          __syncwarp();
-        }
-      }
-      fence_async_smem();  // the staging reads before buffer 1 takes a bulk copy
-      lt_sync();
-      continue;
-    }  // role 0
-    // dH1 = dZ2 W2^T (A = dZ2 K-major over the out unit, B = W2 quarters
-    // transposed) into columns [0, 256)
+    // dH1 = dZ2 W2 (W2's rows, the units of layer 2, are K: MN-major)
     if (tid == 0) {
-      for (int q = 0; q < 4; ++q) {
-        const int b = q & 1;
-        if (q < 2) S.load(b, timg + G.w2q + (uint32_t)q * w2q, w2q);
-        if (q == 2) {
-          S.load(0, timg + G.w2q + 2u * w2q, w2q);
-          S.load(1, timg + G.w2q + 3u * w2q, w2q);
-        }
-        if (S.ready(b)) {
-          lt_mma(tacc, smem_u32(h2s) + (uint32_t)(8 * q) * kA, kA, 128, 2u * kA, smem_u32(S.buf[b]), 128, 64u * 16u,
-                 2u * 128u, idesc_bf16_f32_t(kLtRows, kHid, 0, 1), 64 / 16, q > 0);
-          S.done(b);
-        }
-      }
-      if (S.ok) tc_commit(&bar_layer);
+      for (int ks = 0; ks < kHid / 16; ++ks)
+        tc_mma_bf16_ta(tacc, tacc2 + tf_a_col(ks), smem_desc(sw2 + (uint32_t)ks * 2u * 128u, 128, kHid * 16u),
+                       idesc_bf16_f32_t(kLtRows, kHid, 0, 1), ks > 0 ? 1u : 0u);
+      tc_commit(&bar_mma);
     }
-    layer_out = true;
-    ok = __syncthreads_and(mbar_wait(&bar_layer, player, kTcTries));
-    player ^= 1u;
-    layer_out = !ok;
-    if (!ok) break;
-    tc_fence_after();
-    {
-      // dZ1 = (H1 > 0) dH1 written over H1 (BF16); db1 from the FP32 values
-      const int quarter = warp & 3, r = quarter * 32 + lane, c0 = (warp >> 2) * 128;
-      for (int c = c0; c < c0 + 128; c += 32) {
-        float v[32];
-        tmem_ld32(tacc + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+    float* vec = f.vec + (long long)tile * kVecLd;
+    if (warp < 4) {
+      // db3 and the Huber sum meanwhile: lanes, then warps in order
+      const float* dO = dout + tid * kOutPad;
+      float s[kOutPad];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          uint4* hp = reinterpret_cast<uint4*>(h1s + kmajor_offset(r, c + 8 * g, kLtRows));
-          const uint4 hv = *hp;
-          const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
-          uint32_t w[4];
+      for (int k = 0; k < kOutPad; ++k) {
+        s[k] = dO[k];
+        for (int off = 16; off > 0; off >>= 1) s[k] += __shfl_xor_sync(kFull, s[k], off);
+        if (lane == 0) dsum_sh[warp][k] = s[k];
+      }
+    }
+    mma_wait();
+    if (ok) {
+      // dZ1 = (H1 > 0) dH1: its fragments (BF16), db1 from the FP32 values
+      uint32_t r[2][32];
+      tmem_ld_frag64_nowait(tacc + tw, r[0]);
+      tmem_ld_frag64_nowait(tacc + tw + (16u << 16), r[1]);
+      tmem_ld_wait();
+      float cs[16] = {};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const bool m0 = (hw[j] & 0xFFFFu) != 0u && !(hw[j] & 0x8000u);
-            const bool m1 = (hw[j] >> 16) != 0u && !(hw[j] & 0x80000000u);
-            v[8 * g + 2 * j] = m0 ? v[8 * g + 2 * j] : 0.0f;
-            v[8 * g + 2 * j + 1] = m1 ? v[8 * g + 2 * j + 1] : 0.0f;
-            w[j] = pack_bf16x2(v[8 * g + 2 * j], v[8 * g + 2 * j + 1]);
+      for (int h = 0; h < 2; ++h) {
+        uint32_t p[16];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const uint32_t mk = mask1[h] >> (4 * j + 2 * i);
+            const float a = (mk & 1u) ? __uint_as_float(r[h][4 * j + 2 * i]) : 0.0f;
+            const float b = (mk & 2u) ? __uint_as_float(r[h][4 * j + 2 * i + 1]) : 0.0f;
+            cs[2 * j] += a;
+            cs[2 * j + 1] += b;
+            p[2 * j + i] = pack_bf16x2(a, b);
           }
-          *hp = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-        const float s = lt_colsum32(v, lane);
-        red[quarter * kHid + c + lane] = s;
+        lt_put_frags<true>(f.z1 + fo + h * kFragTile, p, lane);
       }
-    }
-    fence_async_smem();
-    lt_sync();
-    if (tid < kHid) pg[P.b1 + tid] = ((red[tid] + red[kHid + tid]) + red[2 * kHid + tid]) + red[3 * kHid + tid];
-    // dW1 = dZ1^T X (M = hidden unit in two halves, N = input feature,
-    // K = sample; both operands transposed) into columns [0, 2 k1)
-    if (tid == 0) {
-      for (int h = 0; h < 2; ++h)
-        lt_mma(tacc + (uint32_t)(h * L.k1), smem_u32(h1s) + 16u * (uint32_t)h * kA, 128, kA, 2u * 128u, smem_u32(xs),
-               128, kA, 2u * 128u, idesc_bf16_f32_t(kLtRows, L.k1, 1, 1), kLtRows / 16, false);
-      tc_commit(&bar_layer);
-    }
-    layer_out = true;
-    ok = __syncthreads_and(mbar_wait(&bar_layer, player, kTcTries));
-    player ^= 1u;
-    layer_out = !ok;
-    if (!ok) break;
-    tc_fence_after();
-    {
-      // dW1 rows (hidden unit j, n_in inputs) staged over the dead H1 / H2
-      // tiles with an odd row stride (conflict-free), then copied out: the
-      // block is contiguous in the partial row (coalesced)
-      const int quarter = warp & 3, h = warp >> 2, j = 128 * h + quarter * 32 + lane;
-      const int sn = L.n_in | 1;
-      float* st = reinterpret_cast<float*>(h1s);  // 256 x sn floats <= 70 KB of the 128 KB
-      for (int c = 0; c < L.k1; c += 32) {
-        float v[32];
-        tmem_ld32(tacc + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(h * L.k1 + c), v);
 #pragma unroll
-        for (int k = 0; k < 32; ++k)
-          if (c + k < L.n_in) st[j * sn + c + k] = v[k];
+      for (int j = 0; j < 16; ++j) {
+        for (int off = 4; off < 32; off <<= 1) cs[j] += __shfl_xor_sync(kFull, cs[j], off);
+        if (g == 0) red[quarter * kHid + 64 * grp + 8 * (j >> 1) + 2 * q + (j & 1)] = cs[j];
       }
-      lt_sync();
-      for (int t = tid; t < kHid * L.n_in; t += kLtThreads) pg[P.w1 + t] = st[(t / L.n_in) * sn + t % L.n_in];
     }
-    lt_sync();  // the tile's buffers and tensor memory are reused by the next tile
+    lt_sync();  // also: tensor memory and X are free for the next tile
+    if (ok) {
+      if (tid < kHid) {
+        vec[tid] = ((red[tid] + red[kHid + tid]) + red[2 * kHid + tid]) + red[3 * kHid + tid];
+      } else if (tid < kHid + kOutPad && tid != kHid + kOut) {
+        const int k = tid - kHid;
+        vec[k < kOut ? kBigB3 + k : kBigHub] =
+            ((dsum_sh[0][k] + dsum_sh[1][k]) + dsum_sh[2][k]) + dsum_sh[3][k];
+      }
+    }
   }
-  if (!ok && tid == 0) atomicOr(fail, kTdFailCopy);
-  if (tid == 0) {
-    S.drain();
-    if (layer_out) mbar_wait(&bar_layer, player, kTcTries);
+  if (!ok && tid == 0) {
+    // no update this step; what is in flight gets one more bounded wait
+    atomicOr(fail, kTdFailCopy);
+    mbar_wait(&bar_w1, 0u, kTcTries);
+    mbar_wait(&bar_w2, 0u, kTcTries);
+    if (mma_out) mbar_wait(&bar_mma, phase ^ 1u, kTcTries);
   }
   lt_sync();
   if (warp == 0) tmem_free(tacc, 512);
 }
-
 
 // ------------------------------------------------------------- host side
 
@@ -2894,12 +2754,9 @@ void free_qnet(sg_qnet* q) {
   cudaFree(q->img_t);
   cudaFree(q->step);
   cudaFree(q->td_fail);
-  cudaFree(q->partial);
   cudaFree(q->frag);
   cudaFree(q->img_tc);
   cudaFree(q->img_tc_t);
-  cudaFree(q->q2);
-  cudaFree(q->td_sync);
   delete q;
 }
 }  // namespace
@@ -2928,9 +2785,8 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   q->max_batch = (max_batch + kTile - 1) / kTile * kTile;
   cudaGetDevice(&q->device);
   const size_t P = (size_t)q->PL.total;
-  const bool large = q->max_batch >= kLtMinBatch;
-  const size_t tiles16 = (size_t)(std::min(q->max_batch, kLtMinBatch) + kTile - 1) / kTile;
-  const size_t tiles128 = large ? (size_t)(q->max_batch + kLtRows - 1) / kLtRows : 0;
+  // fragment tiles of the largest batch: whole 128-sample tiles from kLtMinBatch
+  const int tiles = q->max_batch >= kLtMinBatch ? (q->max_batch + kLtRows - 1) / kLtRows * kLtSub : q->max_batch / kTile;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void** p, size_t b) {
     if (e == cudaSuccess) e = cudaMalloc(p, b);
@@ -2943,12 +2799,9 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   alloc((void**)&q->img_t, (size_t)q->IL.bytes);
   alloc((void**)&q->step, 8);
   alloc((void**)&q->td_fail, 8);
-  alloc(&q->frag, td_frag_bytes((int)tiles16, q->IL.k1));
-  if (large) alloc((void**)&q->partial, tiles128 * partial_stride(P) * 4);
+  alloc(&q->frag, td_frag_bytes(tiles, q->IL.k1));
   alloc((void**)&q->img_tc, tc_img(q->IL.k1).bytes);
   alloc((void**)&q->img_tc_t, tc_img(q->IL.k1).bytes);
-  alloc((void**)&q->q2, (size_t)2 * q->max_batch * 5 * 4);
-  alloc((void**)&q->td_sync, (size_t)(1 + (q->max_batch + kLtRows - 1) / kLtRows) * 4);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&q->sms, cudaDevAttrMultiProcessorCount, q->device);
   if (e != cudaSuccess) {
     free_qnet(q);
@@ -2991,11 +2844,11 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
       (rc = set_smem_attr((const void*)k_rollout_q<2, true, false>, fwd_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<2, true, true>, fwd_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_td_tile, grad_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_td_tc, kTcSmemLaunch))) {
+      (rc = set_smem_attr((const void*)k_td_tc, lt_smem(80).bytes))) {
     free_qnet(q);
     return rc;
   }
-  // clusters of the small-batch learner that run at once: more tiles than
+  // clusters of the learners that run at once (one CTA per SM): more tiles than
   // that loop over a resident grid, which stages its weights once
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(kTpRanks * 64);
@@ -3368,31 +3221,28 @@ extern "C" int sg_td_train_step(sg_qnet_t q, sg_replay_t rp, int32_t batch, floa
   u.step = q->step, u.fail = q->td_fail, u.tick = q->td_fail + 1;
   u.lr = lr, u.every = target_every, u.loss = loss_dev, u.grad = grad_dev, u.batch = batch;
   u.P = q->PL, u.L = q->IL;
+  // a cluster per tile, evenly over the rounds
   const int cap = q->lim_learner > 0 ? std::min(q->lim_learner, q->sms) : q->sms;
-  if (batch >= kLtMinBatch) {
-    // tcgen05 learner: 128-sample tiles, one partial gradient row per tile
-    const int ntiles = (batch + kLtRows - 1) / kLtRows;
-    SG_CUDA(cudaMemsetAsync(q->td_sync, 0, (size_t)(1 + ntiles) * 4, stream));
-    k_td_tc<<<std::min(4 * ntiles, cap), kLtThreads, kTcSmemLaunch, stream>>>(
-        q->img, q->img_t, q->img_tc, q->img_tc_t, q->IL, q->PL, rp->d, seed, q->step, batch, gamma, q->q2, q->td_sync,
-        q->partial, q->td_fail);
-    SG_CUDA(cudaGetLastError());
-    SG_CUDA(sg_launch_pdl(k_adam, (q->PL.total + 256) / 256, 256, 0, stream, u, (const float*)q->partial, ntiles));
+  const int fit = std::max(1, std::min(q->td_clusters, cap / kTpRanks));
+  const bool big = batch >= kLtMinBatch;
+  const int rows = big ? kLtRows : kTile, ntiles = (batch + rows - 1) / rows;
+  const int rounds = (ntiles + fit - 1) / fit, grid = (ntiles + rounds - 1) / rounds * kTpRanks;
+  const int frags = big ? ntiles * kLtSub : ntiles, items = td_update_items(q->IL.k1, big);
+  const TdFrag f = td_frag(q->frag, frags, q->IL.k1);
+  const uint8_t *im = q->img, *im_t = q->img_t, *tc = q->img_tc, *tc_t = q->img_tc_t;
+  const unsigned long long* step = q->step;
+  if (big) {
+    SG_CUDA(sg_launch_pdl(k_td_tc, grid, kThreads, lt_smem(q->IL.k1).bytes, stream, im, im_t, tc, tc_t, q->IL, rp->d,
+                          seed, step, batch, gamma, f, q->td_fail));
+    SG_CUDA(sg_launch_pdl(k_td_update<8, false, true>, items, 256, 0, stream, u, f, frags));
     return SG_OK;
   }
-  // mma.sync learner: 16-sample tiles, a cluster each, evenly over the rounds
-  const int ntiles = (batch + kTile - 1) / kTile;
-  const int fit = std::max(1, std::min(q->td_clusters, cap / kTpRanks));
-  const int rounds = (ntiles + fit - 1) / fit, clusters = (ntiles + rounds - 1) / rounds;
-  const TdFrag f = td_frag(q->frag, ntiles, q->IL.k1);
-  SG_CUDA(sg_launch_pdl(k_td_tile, clusters * kTpRanks, kThreads, grad_smem(q->IL), stream, (const uint8_t*)q->img,
-                        (const uint8_t*)q->img_t, q->IL, rp->d, (unsigned long long)seed,
-                        (const unsigned long long*)q->step, (int)batch, gamma, f, q->td_fail));
-  const int items = td_update_items(q->IL.k1);
+  SG_CUDA(sg_launch_pdl(k_td_tile, grid, kThreads, grad_smem(q->IL), stream, im, im_t, q->IL, rp->d, seed, step, batch,
+                        gamma, f, q->td_fail));
   if (ntiles <= kTuSlots)
-    SG_CUDA(sg_launch_pdl(k_td_update<4, true>, items, 128, 0, stream, u, f, ntiles));
+    SG_CUDA(sg_launch_pdl(k_td_update<4, true, false>, items, 128, 0, stream, u, f, ntiles));
   else
-    SG_CUDA(sg_launch_pdl(k_td_update<8, false>, items, 256, 0, stream, u, f, ntiles));
+    SG_CUDA(sg_launch_pdl(k_td_update<8, false, false>, items, 256, 0, stream, u, f, ntiles));
   return SG_OK;
 }
 
@@ -3538,7 +3388,7 @@ extern "C" int sg_td_grad_noalloc(const float* params_dev, const float* target_p
   u.fail = fail;
   u.loss = loss_dev, u.grad = grad_dev, u.batch = batch;
   u.P = PL, u.L = IL;
-  k_adam<<<(PL.total + 256) / 256, 256, 0, stream>>>(u, partial, nblk);
+  k_grad_sum<<<(PL.total + 256) / 256, 256, 0, stream>>>(u, partial, nblk);
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
