@@ -98,7 +98,7 @@ __global__ void k_clr_cols(const uint8_t* __restrict__ g, const PrepMap* __restr
     if (cy - dd >= 0) best = min(best, max((int)col[(long long)(cy - dd) * d.w], dd));
     if (cy + dd < d.h) best = min(best, max((int)col[(long long)(cy + dd) * d.w], dd));
   }
-  clr[d.clr_off + (long long)cy * d.clr_ld + cx] = (uint8_t)(best == 0 ? 0 : max(1, best - 1));
+  clr[d.clr_off + skip_off(cx, cy, d.clr_ld)] = (uint8_t)(best == 0 ? 0 : max(1, best - 1));
 }
 
 // Sector skip planes (see MapDesc in sg_device.cuh).  Block (x, y): 256
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) k_sector_skip(const uint32_t* __restrict_
   const MapDesc d = maps[m];
   const long long local = i - cell_prefix[m];
   const int cx = (int)(local % d.w), cy = (int)(local / d.w);
-  const int own = clr[d.clr_off + (long long)cy * d.clr_ld + cx];
+  const int own = clr[d.clr_off + skip_off(cx, cy, d.clr_ld)];
   if (own == 0) return;  // occupied: the plane keeps its 0
   const uint32_t* rows = atlas + d.word_off;
   int J = kSecRadius;
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256) k_sector_skip(const uint32_t* __restrict_
       break;
     }
   }
-  sec[d.sec_off + (long long)sector * d.sec_plane + (long long)cy * d.clr_ld + cx] = (uint8_t)max(J, own);
+  sec[d.sec_off + (long long)sector * d.sec_plane + skip_off(cx, cy, d.clr_ld)] = (uint8_t)max(J, own);
 }
 
 // Episode 0 of every env; one warp per env.
@@ -372,7 +372,7 @@ __device__ __forceinline__ uint64_t noise_key(const EnvConst& k, const Env& s) {
 // Lane j: record j of the chunk from its step record.
 __device__ __forceinline__ uint32_t rec_start(const DevCfg& c, const EnvConst& k, const Env& s) {
   if (!c.skip_ok || !in_map(k.m.w, k.m.h, s.x, s.y)) return 0u;
-  return (uint32_t)scan_start(__ldg(k.clr + __float2int_rd(s.y) * k.m.clr_ld + __float2int_rd(s.x)));
+  return (uint32_t)scan_start(__ldg(k.clr + skip_off(__float2int_rd(s.x), __float2int_rd(s.y), k.m.clr_ld)));
 }
 __device__ __forceinline__ void derive_rec(const DevCfg& c, const EnvConst& k, const StepRec& r, ObsRec& o) {
   const Env s = r.post;
@@ -544,7 +544,7 @@ __device__ __forceinline__ void pose_chunk(const DevCfg& c, const SimPtrs& p, co
       if (mx < 0.0f || my < 0.0f || mx >= (float)k.m.w || my >= (float)k.m.h) {
         done = 1u;
       } else {
-        const int own = __ldg(k.clr + __float2int_rd(my) * k.m.clr_ld + __float2int_rd(mx));
+        const int own = __ldg(k.clr + skip_off(__float2int_rd(mx), __float2int_rd(my), k.m.clr_ld));
         slow = own < c.clr_collide;
       }
       const float ddx = k.L.gx - mx, ddy = k.L.gy - my;
@@ -1224,9 +1224,9 @@ extern "C" int sg_sim_create(const sg_sim_config* cfg, int32_t n_maps, const uin
     md[m].h = map_h[m];
     md[m].row_words = ((map_w[m] + 127) / 128) * 4;  // rows padded to 16 bytes
     md[m].clr_ld = map_w[m] + 2 * kClrBorder;
-    md[m].clr_off = clr_bytes + (long long)kClrBorder * md[m].clr_ld + kClrBorder;
+    md[m].clr_off = clr_bytes + skip_corner(md[m].clr_ld);
     words += (long long)md[m].row_words * map_h[m];
-    clr_bytes += (long long)md[m].clr_ld * (map_h[m] + 2 * kClrBorder);
+    clr_bytes += skip_plane_bytes(md[m].clr_ld, map_h[m]);
     max_cells = std::max(max_cells, (size_t)map_w[m] * (size_t)map_h[m]);
   }
   for (int i = 0; i < n; ++i) {
@@ -1248,9 +1248,9 @@ extern "C" int sg_sim_create(const sg_sim_config* cfg, int32_t n_maps, const uin
   dc.sec_scale = (float)((double)n_sec / (2.0 * M_PI));
   long long sec_bytes = 0, max_planes = 0;
   for (int m = 0; m < n_maps; ++m) {
-    const long long plane = (long long)md[m].clr_ld * (map_h[m] + 2 * kClrBorder);
+    const long long plane = skip_plane_bytes(md[m].clr_ld, map_h[m]);
     md[m].sec_plane = n_sec > 1 ? plane : 0;
-    md[m].sec_off = n_sec > 1 ? sec_bytes + (long long)kClrBorder * md[m].clr_ld + kClrBorder : 0;
+    md[m].sec_off = n_sec > 1 ? sec_bytes + skip_corner(md[m].clr_ld) : 0;
     if (n_sec > 1) sec_bytes += plane * n_sec;
     max_planes = std::max(max_planes, plane * n_sec);
   }
@@ -1507,8 +1507,7 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
           grid = std::min<long long>(nitems, (long long)sim->persistent_blocks);
           SG_CUDA(cudaMemsetAsync(sim->pipe_sync_dev, 0, sizeof(unsigned) * (size_t)(nblk + 2), stream));
         }
-        pipe_kernel(sim->dc)<<<(unsigned)grid, 32 * G * E, smem,
-                                                                          stream>>>(
+        pipe_kernel(sim->dc)<<<(unsigned)grid, 32 * G * E, smem, stream>>>(
             sim->dc, sp, K, L.obs_warps, L.order ? sim->map_order_dev : nullptr, seg,
             seg > 0 ? sim->pipe_sync_dev : nullptr, L.wait_iters > 0 ? (unsigned)L.wait_iters : kPipeWaitIters,
             obs_dev, obs_seq_dev, act_seq_dev, rew_seq_dev, done_seq_dev);
@@ -1709,6 +1708,16 @@ extern "C" int sg_sim_get_atlas(sg_sim_t sim, uint32_t* atlas_host, size_t* word
   return SG_OK;
 }
 
+// The h x w interior of a skip plane (its cell (0, 0) at dev) in row order.
+static int download_plane(const MapDesc& d, const uint8_t* dev, uint8_t* host) {
+  const long long corner = skip_corner(d.clr_ld);
+  std::vector<uint8_t> plane((size_t)skip_plane_bytes(d.clr_ld, d.h));
+  SG_CUDA(cudaMemcpy(plane.data(), dev - corner, plane.size(), cudaMemcpyDeviceToHost));
+  for (int y = 0; y < d.h; ++y)
+    for (int x = 0; x < d.w; ++x) host[(size_t)y * d.w + x] = plane[(size_t)(corner + skip_off(x, y, d.clr_ld))];
+  return SG_OK;
+}
+
 extern "C" int sg_sim_get_clearance(sg_sim_t sim, uint8_t* host, size_t* bytes, int64_t* offs_host) {
   SG_RANGE("sg_sim_get_clearance");
   if (!sim || !bytes) return SG_E_INVAL;
@@ -1720,8 +1729,7 @@ extern "C" int sg_sim_get_clearance(sg_sim_t sim, uint8_t* host, size_t* bytes, 
     size_t off = 0;
     for (int m = 0; m < sim->n_maps; ++m) {
       const MapDesc& d = sim->maps_host[m];
-      SG_CUDA(cudaMemcpy2D(host + off, (size_t)d.w, sim->clr + d.clr_off, (size_t)d.clr_ld, (size_t)d.w,
-                           (size_t)d.h, cudaMemcpyDeviceToHost));
+      if (int rc = download_plane(d, sim->clr + d.clr_off, host + off)) return rc;
       off += (size_t)d.w * d.h;
     }
   }
@@ -1749,8 +1757,7 @@ extern "C" int sg_sim_get_sector_skip(sg_sim_t sim, uint8_t* host, size_t* bytes
     for (int m = 0; m < sim->n_maps; ++m) {
       const MapDesc& d = sim->maps_host[m];
       for (int p = 0; p < S; ++p) {
-        SG_CUDA(cudaMemcpy2D(host + off, (size_t)d.w, sim->sec + d.sec_off + (long long)p * d.sec_plane,
-                             (size_t)d.clr_ld, (size_t)d.w, (size_t)d.h, cudaMemcpyDeviceToHost));
+        if (int rc = download_plane(d, sim->sec + d.sec_off + (long long)p * d.sec_plane, host + off)) return rc;
         off += (size_t)d.w * d.h;
       }
     }
