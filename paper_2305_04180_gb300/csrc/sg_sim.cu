@@ -660,6 +660,14 @@ __host__ __device__ constexpr size_t pipe_group_bytes(bool dyn) {
   return kPipeChunk * (sizeof(StepRec) + 2 * sizeof(ObsRec)) +
          (dyn ? 4 * kPipeChunk * sizeof(Discs) + kMaxDyn * sizeof(Obst) : 0);
 }
+// With this many observation warps a rollout lasts as long as its pose chains,
+// so the first of them only helps the pose warp: it derives the observation
+// records and draws the actions of the chunk after next, and the pose warp
+// takes no scans (one more buffer of step records, two of actions).  16 envs x
+// 1,000 steps: 228 -> 204 us, 152 envs x 512 166 -> 133.
+constexpr int kPipeHelper = 15;
+constexpr size_t kPipeHelperBytes = kPipeChunk * sizeof(StepRec) + 2 * kPipeChunk * sizeof(uint32_t);
+constexpr int kPipeHelperBar = 1 + 4 * 3;  // named barriers 13, 14: step records of buffer b written
 static_assert(pipe_group_bytes(false) % 16 == 0 && pipe_group_bytes(true) % 16 == 0, "16-byte aligned groups");
 
 // Time slicing (seg > 0): the rollout is cut into segments of seg steps and
@@ -711,7 +719,7 @@ __device__ __forceinline__ Obst load_obst_cg(const SimPtrs& p, int o, int i) {
   return b;
 }
 
-template <bool kDyn, bool kFast>
+template <bool kDyn, bool kFast, bool kHelped>
 __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_constant__ DevCfg c, SimPtrs p, int K,
                                                                 int P, const int* __restrict__ order, int seg,
                                                                 unsigned* __restrict__ sync, unsigned wait_iters,
@@ -740,6 +748,8 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
   Discs* dpost = reinterpret_cast<Discs*>(ob + 2 * kPipeChunk);
   Discs* dpre = dpost + 2 * kPipeChunk;
   Obst* dst = reinterpret_cast<Obst*>(dpre + 2 * kPipeChunk);
+  StepRec* st2 = kHelped ? reinterpret_cast<StepRec*>(base + pipe_group_bytes(kDyn)) : st;
+  uint32_t* acts = reinterpret_cast<uint32_t*>(st2 + kPipeChunk);  // [2][kPipeChunk] (kHelped)
   const int bfull = 1 + 4 * group, bfree = 3 + 4 * group, nthr = 32 * G;
   const long long n = c.n_envs;
   for (int iter = 0;; ++iter) {
@@ -789,20 +799,27 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
             // the state carried between chunks is the last step record's post
             // state, so nothing of the pose chain stays live while this warp
             // takes observation records
-            Env s = ch > 0 ? unpack_env(reinterpret_cast<const uint4*>(&st[kPipeChunk - 1].post))
+            StepRec* sb = b ? st2 : st;
+            Env s = ch > 0 ? unpack_env(reinterpret_cast<const uint4*>(&(b ? st : st2)[kPipeChunk - 1].post))
                            : (sync ? load_env_cg(p, env) : load_env(p, env));
             if (kDyn && ch == 0 && lane < c.n_dyn) dst[lane] = sync ? load_obst_cg(p, lane, env) : load_obst(p, lane, env);
             const int i0 = ch * kPipeChunk, nst = min(Kl, i0 + kPipeChunk) - i0;
             // lane l draws the action of step i0 + l (t counts every step)
-            const uint64_t akey = sm_at(sm_at(c.seed, kStreamAction), (uint64_t)env);
-            const uint32_t abatch = random_action_for(c, akey, s.t + (uint32_t)lane);
-            pose_chunk<kDyn>(c, p, k, s, nst, abatch, st, lane, dst, dpost + b * kPipeChunk,
+            uint32_t abatch;
+            if (kHelped && ch >= 2)
+              abatch = acts[b * kPipeChunk + lane];
+            else
+              abatch = random_action_for(c, sm_at(sm_at(c.seed, kStreamAction), (uint64_t)env), s.t + (uint32_t)lane);
+            pose_chunk<kDyn>(c, p, k, s, nst, abatch, sb, lane, dst, dpost + b * kPipeChunk,
                              dpre + b * kPipeChunk);
             __syncwarp();
-            if (lane < nst) derive_rec(c, k, st[lane], ob[b * kPipeChunk + lane]);
+            if (kHelped)
+              named_arrive(kPipeHelperBar + b, 64);
+            else if (lane < nst)
+              derive_rec(c, k, sb[lane], ob[b * kPipeChunk + lane]);
             named_arrive(bfull + b, nthr);
           }
-          if (ch >= 1) {
+          if (ch >= 1 && !kHelped) {
             const int b = (ch - 1) & 1, i0 = s0 + (ch - 1) * kPipeChunk;
             consume_chunk<kDyn, kFast>(c, k, ob + b * kPipeChunk, &next_step[group][b], i0, min(s1, i0 + kPipeChunk), K,
                                 env, n, lane, o, has_last, obs_seq, act_seq, rew_seq, done_seq,
@@ -812,9 +829,21 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
         // the last two chunks' consumption completes the free barriers' phases
         for (int ch = max(chunks, 2); ch < chunks + 2; ++ch) named_barrier(bfree + (ch & 1), nthr);
         if (lane == 0 && chunks > 0)
-          store_env(p, env, unpack_env(reinterpret_cast<const uint4*>(&st[Kl - 1 - (chunks - 1) * kPipeChunk].post)));
+          store_env(p, env, unpack_env(reinterpret_cast<const uint4*>(
+                                &((chunks & 1) ? st : st2)[Kl - 1 - (chunks - 1) * kPipeChunk].post)));
         if (kDyn && lane < c.n_dyn) store_obst(p, lane, env, dst[lane]);
         if (sync) __threadfence();
+      } else if (kHelped && role == 1) {
+        const uint64_t akey = sm_at(sm_at(c.seed, kStreamAction), (uint64_t)env);
+        const uint32_t t0 = (sync ? __ldcg(p.u + 2 * n + env) : p.u[2 * n + env]) + (uint32_t)lane;
+        for (int ch = 0; ch < chunks; ++ch) {
+          const int b = ch & 1, nst = min(Kl, (ch + 1) * kPipeChunk) - ch * kPipeChunk;
+          named_barrier(kPipeHelperBar + b, 64);  // the pose chain of chunk ch
+          if (lane < nst) derive_rec(c, k, (b ? st2 : st)[lane], ob[b * kPipeChunk + lane]);
+          named_arrive(bfull + b, nthr);
+          acts[b * kPipeChunk + lane] = random_action_for(c, akey, t0 + (uint32_t)((ch + 2) * kPipeChunk));
+          named_arrive(bfree + b, nthr);
+        }
       } else {
         for (int ch = 1; ch <= chunks; ++ch) {
           const int b = (ch - 1) & 1, i0 = s0 + (ch - 1) * kPipeChunk;
@@ -837,11 +866,18 @@ __global__ void __launch_bounds__(512, 2) k_rollout_random_pipe(const __grid_con
   }
 }
 
-static decltype(&k_rollout_random_pipe<false, true>) pipe_kernel(const DevCfg& c) {
-  if (c.n_dyn > 0) return c.scan_fast ? k_rollout_random_pipe<true, true> : k_rollout_random_pipe<true, false>;
-  return c.scan_fast ? k_rollout_random_pipe<false, true> : k_rollout_random_pipe<false, false>;
+template <bool kHelped>
+static decltype(&k_rollout_random_pipe<false, true, false>) pipe_pick(const DevCfg& c) {
+  if (c.n_dyn > 0)
+    return c.scan_fast ? k_rollout_random_pipe<true, true, kHelped> : k_rollout_random_pipe<true, false, kHelped>;
+  return c.scan_fast ? k_rollout_random_pipe<false, true, kHelped> : k_rollout_random_pipe<false, false, kHelped>;
 }
-static size_t pipe_smem_bytes(int E, bool dyn) { return (size_t)E * pipe_group_bytes(dyn); }
+static decltype(&k_rollout_random_pipe<false, true, false>) pipe_kernel(const DevCfg& c, const sg_launch& L) {
+  return L.obs_warps >= kPipeHelper ? pipe_pick<true>(c) : pipe_pick<false>(c);
+}
+static size_t pipe_smem_bytes(int E, bool dyn, bool helped) {
+  return (size_t)E * pipe_group_bytes(dyn) + (helped ? kPipeHelperBytes : 0);
+}
 static int pipe_envs_per_block(const sg_launch& L) {
   const int E = L.warps_per_block / (1 + L.obs_warps);
   return E < 1 ? 1 : (E > kPipeMaxGroups ? kPipeMaxGroups : E);
@@ -1462,7 +1498,7 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
 // a step wait for the pose chain only, so several warps per env shorten a
 // rollout while the envs alone leave warp slots empty, and the pose chain's
 // run-ahead pays at every size once K fills a chunk.  us (one warp per env /
-// pipelined): 16 envs x 512 steps 1,516 / 184 (15 scan warps), 304 x 512 1,656 /
+// pipelined): 16 envs x 1,000 steps 2,515 / 204 (15 scan warps), 304 x 512 1,656 /
 // 233 (7), 1,024 x 512 1,951 / 471, 4,096 x 224 1,184 / 726, 16,384 x 32 599 /
 // 497 (3, two envs per CTA).  Few steps of many envs stay with one warp per
 // env (4,096 x 8: 59 / 75; 65,536 x 16: 1,078 / 1,179).
@@ -1496,7 +1532,7 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
         const int G = 1 + L.obs_warps;
         const int E = pipe_envs_per_block(L);
         const bool dyn = sim->dc.n_dyn > 0;
-        const size_t smem = pipe_smem_bytes(E, dyn);
+        const size_t smem = pipe_smem_bytes(E, dyn, L.obs_warps >= kPipeHelper);
         const int nblk = (n + E - 1) / E;
         int seg = L.segment < K ? L.segment : 0;  // one segment needs no slicing
         long long grid = nblk;
@@ -1507,7 +1543,7 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
           grid = std::min<long long>(nitems, (long long)sim->persistent_blocks);
           SG_CUDA(cudaMemsetAsync(sim->pipe_sync_dev, 0, sizeof(unsigned) * (size_t)(nblk + 2), stream));
         }
-        pipe_kernel(sim->dc)<<<(unsigned)grid, 32 * G * E, smem, stream>>>(
+        pipe_kernel(sim->dc, L)<<<(unsigned)grid, 32 * G * E, smem, stream>>>(
             sim->dc, sp, K, L.obs_warps, L.order ? sim->map_order_dev : nullptr, seg,
             seg > 0 ? sim->pipe_sync_dev : nullptr, L.wait_iters > 0 ? (unsigned)L.wait_iters : kPipeWaitIters,
             obs_dev, obs_seq_dev, act_seq_dev, rew_seq_dev, done_seq_dev);
@@ -1582,12 +1618,12 @@ extern "C" int sg_sim_set_launch(sg_sim_t sim, const sg_launch* cfg) {
   if (L.kernel == SG_ROLLOUT_PIPE) {
     const int E = pipe_envs_per_block(L);
     const bool dyn = sim->dc.n_dyn > 0;
-    const size_t smem = pipe_smem_bytes(E, dyn);
-    auto kern = pipe_kernel(sim->dc);
+    const size_t smem = pipe_smem_bytes(E, dyn, L.obs_warps >= kPipeHelper);
+    auto kern = pipe_kernel(sim->dc, L);
     // the limit is a property of the kernel, shared by every handle: the
     // largest any launch needs
     SG_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pipe_smem_bytes(kPipeMaxGroups, dyn)));
+                                 (int)pipe_smem_bytes(kPipeMaxGroups, dyn, true)));
     if (L.segment > 0) {
       // time slicing: a resident grid and the per-CTA segment flags
       SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern,
