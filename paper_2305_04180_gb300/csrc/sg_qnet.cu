@@ -575,8 +575,8 @@ __device__ __forceinline__ void tf_epilogue_head(uint32_t tacc, const float* bia
 // index / n_in of at most 128 x 69 floats.
 constexpr int kTcXFloats = (kTcRows * 69 + kTfEpiThreads - 1) / kTfEpiThreads;
 __device__ __forceinline__ void tc_fetch_x(float (&x)[kTcXFloats], const float* __restrict__ obs, int n_in, int M,
-                                           int tile, int tid) {
-  const long long first = (long long)tile * kTcRows;
+                                           long long tile, int tid) {
+  const long long first = tile * kTcRows;
   const int total = (int)min((long long)kTcRows, M - first) * n_in;
   const float* src = obs + first * n_in;
 #pragma unroll
@@ -600,7 +600,10 @@ __device__ __forceinline__ void tc_store_x(uint8_t* xs, const float (&x)[kTcXFlo
 // Warps 0..15 run the epilogues and convert the inputs, warp 16 (one lane)
 // copies the weights and issues every MMA, so that the issue, which waits
 // while the tensor cores' queue is full, never holds up an epilogue, and warps
-// 17..19 write Q.  They meet on mbarriers, one phase per tile each: bar_x (X
+// 17..19 write Q.  The input loads (2,000 cycles) follow the layer-1 epilogue,
+// beside layer 2: issued before it they hold its tensor-memory waits (188 us a
+// call of 2^20 rows), and on warps 17..19 alone they are too slow (217 us).
+// They meet on mbarriers, one phase per tile each: bar_x (X
 // stored), bar_h1 (H1 stored and the previous tile's layer 2 read), and the
 // MMA commits bar_l1, bar_l2 (layer complete); the head sums of tile t pass
 // through named barriers 1 + t % 2 (written) and 3 + t % 2 (read).  Order on
@@ -693,14 +696,16 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
   } else if (warp > kTfEpiWarps) {
     // ---- read-out: rows of tile i from the four column groups' head sums
     // (NaN where a wait ran out)
+    const int w = tid - kTfEpiThreads - 32;
+    auto tile_of = [&](int i) { return (long long)blockIdx.x + (long long)i * gridDim.x; };
     float b3[kOut];
 #pragma unroll
     for (int j = 0; j < kOut; ++j) b3[j] = __ldg(reinterpret_cast<const float*>(img + L.b3) + j);
     for (int i = 0; i < my_tiles; ++i) {
       group_barrier(1 + (i & 1), kHandover);
       const bool good = *fail == 0;
-      const long long first = ((long long)blockIdx.x + (long long)i * gridDim.x) * kTcRows;
-      for (int r = tid - kTfEpiThreads - 32; r < kTcRows; r += kTfWriters) {
+      const long long first = tile_of(i) * kTcRows;
+      for (int r = w; r < kTcRows; r += kTfWriters) {
         const float* p = part + (i & 1) * 4 * kTcRows * kOutPad + r * kOutPad;
         float o[kOutPad];
 #pragma unroll
@@ -725,12 +730,12 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
     }
   } else {
     // ---- epilogues, inputs (warps 0..15)
+    const uint32_t div = ((1u << 20) + (uint32_t)L.n_in - 1u) / (uint32_t)L.n_in;
     bool ok = true;
     auto wait = [&](uint64_t* bar, uint32_t par) {
       ok = __all_sync(0xffffffffu, ok && mbar_wait_or_fail(bar, par, kTcTries, fail));
       if (ok) tc_fence_after();
     };
-    const uint32_t div = ((1u << 20) + (uint32_t)L.n_in - 1u) / (uint32_t)L.n_in;
     // this lane's W3 fragments: outputs g, columns 64 (warp / 4) + 16 i + 2 q ..
     uint32_t w3[8];
     {
@@ -752,7 +757,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
       mbar_arrive(&bar_h1);
       // X is free (layer 1 of t is complete): the next tile's inputs while layer 2 runs
       if (ok && it + 1 < my_tiles) {
-        tc_fetch_x(xr, obs, L.n_in, M, (int)blockIdx.x + (it + 1) * (int)gridDim.x, tid);
+        tc_fetch_x(xr, obs, L.n_in, M, (long long)blockIdx.x + (long long)(it + 1) * gridDim.x, tid);
         tc_store_x(xs, xr, L.n_in, div, tid);
         mbar_arrive(&bar_x);
       }
@@ -850,6 +855,7 @@ __global__ void __launch_bounds__(512 * MT, 1)
     akey = sm_at(sm_at(c.seed, kStreamAction), (uint64_t)env);
   }
   const unsigned long long rbase = use_replay ? *rp.steps : 0ull;
+  uint32_t slot_t = use_replay ? (uint32_t)(rbase % (unsigned long long)rp.slots) : 0u;  // ring slot of step i
   uint32_t ra_batch = 0, ex_batch = 0;
   __syncthreads();  // the barrier is initialised
   if (!__syncthreads_and(mbar_wait(&bar_img, 0u, kTcTries))) {
@@ -881,7 +887,8 @@ __global__ void __launch_bounds__(512 * MT, 1)
     float* srow = nullptr;
     float* s2row = nullptr;
     if (use_replay) {
-      e = (long long)((rbase + (unsigned long long)i) % (unsigned long long)rp.slots) * rp.n_envs + env;
+      e = (long long)slot_t * rp.n_envs + env;
+      slot_t = slot_t + 1u == (uint32_t)rp.slots ? 0u : slot_t + 1u;
       srow = rp.s + e * rp.obs_dim;
       s2row = rp.s2 + e * rp.obs_dim;
       write_obs(srow, o, c.B, lane);
@@ -1208,6 +1215,8 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       }
     }
     fence_async_smem();
+    // ring slot of step t
+    int slot = use_replay ? (int)((rbase + (unsigned long long)s0) % (unsigned long long)rp.slots) : 0;
     for (int t = s0; t < s1; ++t) {
       // ---- the network on the tile of observations t ----
       tc_fence_before();
@@ -1327,10 +1336,8 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       // 16 to 64 beams) are handed out row by row through a shared counter,
       // so that no warp waits at the next step's barrier for a slow one
       __syncthreads();
-      const long long slot_t =
-          use_replay ? (long long)((rbase + (unsigned long long)t) % (unsigned long long)rp.slots) : 0;
-      const long long slot_n =
-          use_replay ? (long long)((rbase + (unsigned long long)t + 1ull) % (unsigned long long)rp.slots) : 0;
+      const long long slot_t = slot, slot_n = slot + 1 == rp.slots ? 0 : slot + 1;
+      slot = (int)slot_n;
       const int rows = (int)min((long long)kQtEnvs, n - (long long)blk * kQtEnvs);
       for (;;) {
         int e = 0;
@@ -1410,14 +1417,13 @@ __device__ __forceinline__ unsigned long long mod_inv(unsigned long long x, unsi
   if (r >= d) r -= d;
   return r;
 }
-// Ring entry of sample i of optimiser step `tstep`: uniform over the
+// Ring entry of sample i of optimiser step `tstep` with st = *rp.steps: uniform over the
 // V = min(steps, slots - reserve) most recently completed slots, so that a
 // rollout running concurrently (which writes the next slots) is never read.
 // With j = h mod (V n_envs): slot = (steps - 1 - j / n_envs) mod slots,
 // env = j mod n_envs.
-__device__ __forceinline__ long long sample_entry(unsigned long long seed, unsigned long long tstep, int i,
-                                                  const ReplayDev& rp) {
-  const unsigned long long st = *rp.steps;
+__device__ __forceinline__ long long sample_entry(unsigned long long seed, unsigned long long tstep,
+                                                  unsigned long long st, int i, const ReplayDev& rp) {
   const unsigned long long usable = (unsigned long long)(rp.slots - rp.reserve);
   const unsigned long long V = st < usable ? st : usable;
   if (V == 0) return -1;
@@ -1873,14 +1879,14 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   const uint32_t rank = cluster_rank();
   const int ntiles = (batch + kTile - 1) / kTile, stride = (int)gridDim.x / kTpRanks;
   cluster_arrive();  // every CTA of the cluster has started before the first remote store
-  if (tid == 0) {
+  if (tid == kThreads - 1) {
     mbar_init(&bar_w1, 1);
     mbar_init(&bar_w2, 1);
   }
   pdl_wait();
   pdl_launch_dependents();
-  __syncthreads();
-  if (tid == 0) {
+  const unsigned long long tstep = __ldcg(step), st = __ldcg(rp.steps);
+  if (tid == kThreads - 1) {
     // layer 1 starts when W1 and the vectors behind W2 are here
     const uint8_t* src = rank == 2 ? img_t : img;
     mbar_expect_tx(&bar_w1, (uint32_t)(L.w2 + L.bytes - L.w3));
@@ -1890,13 +1896,13 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     for (int off = L.w2; off < L.w3; off += kStageChunk)
       bulk_g2s(sw + off, src + off, (uint32_t)min(kStageChunk, L.w3 - off), &bar_w2);
   }
+  __syncthreads();
   const QW w = qw_at(sw, L);
-  const unsigned long long tstep = *step;
   bool ok = true, first = true;
   for (int tile = (int)blockIdx.x / kTpRanks, it = 0; tile < ntiles; tile += stride, ++it) {
     {
       const int i = tile * kTile + warp;
-      const int e = i < batch ? (int)sample_entry(seed, tstep, i, rp) : -1;
+      const int e = i < batch ? (int)sample_entry(seed, tstep, st, i, rp) : -1;
       const float* src = (rank == 0 ? rp.s : rp.s2) + (long long)e * rp.obs_dim;
       for (int k = lane; k < L.ld1; k += 32)
         X[warp * L.ld1 + k] = __float2bfloat16_rn(e >= 0 && k < rp.obs_dim ? src[k] : 0.0f);
@@ -2082,56 +2088,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
 // it took 16 K cycles at batch 256, now 4 K (a whole step 23.0 -> 16.6 us).
 constexpr int kTuItem = 256;  // floats of an item
 constexpr int kTuSlots = 16;
-constexpr int kBigB3 = kHid, kBigHub = kBigB3 + kOut;  // vectors of a 128-sample tile: db1 | db3 | Huber sum
-// x in three BF16 terms (24 bits: exact for a normal x not near the smallest).
-__device__ __forceinline__ void split_bf16(float x, float (&t)[3]) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    t[i] = __bfloat162float(__float2bfloat16_rn(x));
-    x -= t[i];
-  }
-}
-// The head's part of a 128-sample learner step for 16 units, over fragment
-// tiles t0 .. t1 - 1: dW3[o][n] = sum_s dO[s][o] H2[s][n] and M[n][o] = sum over the
-// samples with H2[s][n] > 0 of dO[s][o], from which db2[n] = sum_o W3[o][n] M[n][o].
-// dO in three BF16 terms against the exact BF16 H2 and 0 / 1: FP32 sums of
-// exact products, as on the CUDA cores (there 100 instructions a tile and warp).
-__device__ __forceinline__ void upd_head(const TdFrag& f, int blk, int t0, int t1, float* out, int lane) {
-  const int g = lane >> 2, q = lane & 3;
-  float acc[2][4] = {};
-#pragma unroll 2
-  for (int i = t0; i < t1; ++i) {
-    const uint4 a = __ldcg(f.h2 + (long long)i * kFragTile + blk * 32 + lane);
-    const float* d = f.dout + ((long long)i * kTile + 2 * q) * kOutPad + g;
-    float t[4][3];
-    split_bf16(__ldcg(d), t[0]);
-    split_bf16(__ldcg(d + kOutPad), t[1]);
-    split_bf16(__ldcg(d + 8 * kOutPad), t[2]);
-    split_bf16(__ldcg(d + 9 * kOutPad), t[3]);
-    const uint32_t ar[4] = {a.x, a.y, a.z, a.w};
-    uint32_t ar1[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      ar1[j] = ((ar[j] & 0x7FFFu) ? 0x3F80u : 0u) | ((ar[j] & 0x7FFF0000u) ? 0x3F800000u : 0u);
-    float s[2][4] = {};
-#pragma unroll
-    for (int n = 2; n >= 0; --n) {
-      const uint32_t b0 = pack_bf16x2(t[0][n], t[1][n]), b1 = pack_bf16x2(t[2][n], t[3][n]);
-      mma_bf16(s[0], ar, b0, b1);
-      mma_bf16(s[1], ar1, b0, b1);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[h][j] += s[h][j];
-  }
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-      *reinterpret_cast<float2*>(out + 128 * h + (g + 8 * j) * kOutPad + 2 * q) = make_float2(acc[h][2 * j], acc[h][2 * j + 1]);
-}
-template <int kWarps, bool kSlots, bool kBig>
+template <int kWarps, bool kSlots>
 __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f, int ntiles) {
   __shared__ float sum[kSlots ? kTuSlots : kWarps][kTuItem];
   pdl_launch_dependents();
@@ -2141,32 +2098,13 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
   const bool w2 = item < n2, mat = item < n2 + n1;
   const int mb = w2 ? item >> 4 : (item - n2) / nx, nb = w2 ? item & 15 : (item - n2) % nx;
   // this thread's parameters: columns k, k + 1 of row r, or vector entry ve
-  constexpr int kHub = kBig ? kBigHub : kVecHub;
-  constexpr int kVecItems = (kHub + 1 + 63) / 64;
   const int r = mb * 16 + t / 8, k = nb * 16 + 2 * (t % 8), ve = (item - n2 - n1) * 64 + t;
-  const bool head = kBig && item >= n2 + n1 + kVecItems;
-  const int hb = item - n2 - n1 - kVecItems;
-  float w3[kOut];  // b2 of the head items: W3's column, before this launch changes it
   int at = 0;
   bool live[2];
   if (mat) {
     at = w2 ? u.P.w2 + r * kHid + k : u.P.w1 + r * u.L.n_in + k;
     live[0] = t < 128 && (w2 || k < u.L.n_in);
     live[1] = t < 128 && (w2 || k + 1 < u.L.n_in);
-  } else if (head) {
-    const int n = hb * 16 + t % 16, o = t / 16;  // dW3[o][n], then db2[n]
-    at = o < kOut ? u.P.w3 + o * kHid + n : u.P.b2 + n;
-    live[0] = o <= kOut;
-    live[1] = false;
-    if (o == kOut) {
-#pragma unroll
-      for (int i = 0; i < kOut; ++i)
-        w3[i] = __bfloat162float(reinterpret_cast<const bf16*>(u.img + u.L.w3)[i * kLdh + n]);
-    }
-  } else if (kBig) {
-    at = ve < kBigB3 ? u.P.b1 + ve : u.P.b3 + (ve - kBigB3);
-    live[0] = t < 64 && ve < kBigHub;
-    live[1] = false;
   } else {
     at = ve < kVecDb2 ? u.P.b1 + ve : ve < kVecW3 ? u.P.b2 + (ve - kVecDb2)
                                     : ve < kVecB3 ? u.P.w3 + (ve - kVecW3) : u.P.b3 + (ve - kVecB3);
@@ -2183,9 +2121,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
   }
   pdl_wait();
   const unsigned fail = __ldcg(u.fail);
-  // fragment tiles, or the vectors of 128-sample tiles
-  const int nt = kBig && !mat && !head ? (ntiles + kLtSub - 1) / kLtSub : ntiles;
-  const int per = (nt + kWarps - 1) / kWarps, t0 = warp * per, t1 = min(nt, t0 + per);
+  const int per = (ntiles + kWarps - 1) / kWarps, t0 = warp * per, t1 = min(ntiles, t0 + per);
   if (mat) {
     const uint4* fa = (w2 ? f.z2 : f.z1) + mb * 32 + lane;
     const uint4* fb = (w2 ? f.h1 : f.x) + nb * 32 + lane;
@@ -2213,12 +2149,10 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
       if (kSlots) put(sum[i]);
     }
     if (!kSlots) put(sum[warp]);
-  } else if (head) {
-    upd_head(f, hb, t0, t1, sum[warp], lane);
   } else {
     const int e = (item - n2 - n1) * 64 + 2 * lane;
     float2 acc = make_float2(0.0f, 0.0f);
-    if (e <= kHub) {
+    if (e <= kVecHub) {
 #pragma unroll 4
       for (int i = t0; i < t1; ++i) {
         const float2 x = __ldcg(reinterpret_cast<const float2*>(f.vec + (long long)i * kVecLd + e));
@@ -2255,28 +2189,291 @@ __global__ void __launch_bounds__(32 * kWarps) k_td_update(TdUpdate u, TdFrag f,
       else
         upd_images<1, 2>(u, run, r, k, th[0], th[1]);
     }
-  } else if (head) {
-    if (live[0]) {
-      float gr = 0.0f;
-      if (t < kOut * 16) {
-        gr = total((t % 16) * kOutPad + t / 16);
-      } else {
-#pragma unroll
-        for (int o = 0; o < kOut; ++o) gr += w3[o] * total(128 + (t % 16) * kOutPad + o);
-      }
-      upd_one(u, run, at, gr, th[0], m[0], v[0]);
-    }
   } else if (live[0]) {
     upd_one(u, run, at, total(t), th[0], m[0], v[0]);
-  } else if (ve == kHub && t < 64 && u.loss) {
+  } else if (ve == kVecHub && t < 64 && u.loss) {
     *u.loss = total(t) / (float)u.batch;
   }
   upd_end(u, failed);
 }
-inline int td_update_items(int k1, bool big) {
-  return 256 + 16 * (k1 / 16) + (big ? (kBigHub + 1 + 63) / 64 + 16 : (kVecHub + 1 + 63) / 64);
+inline int td_update_items(int k1) { return 256 + 16 * (k1 / 16) + (kVecHub + 1 + 63) / 64; }
+
+// The same for the 128-sample learner, whose batches have hundreds of fragment
+// tiles: a cluster of kSplit CTAs per item, a run of the tiles each, partial
+// sums added in CTA order through distributed shared memory (each CTA updates
+// an eighth of the item).  Items: 64 x 64 blocks of W2 and W1 (a warp 16 x 32, so
+// that a fragment serves two or four warps; the tiles' operands, contiguous, by
+// bulk copies in two stages of eight tiles), W3 and b2 of 64 units, the
+// remaining vectors.  Bound by L2 reads (each operand four times) and the
+// latency of the chain; 16 x 16 items of one CTA read each operand 16 times,
+// 88 MB at batch 4,096 (45.6 us a step, 34.5 now with the rolled epilogues).
+constexpr int kSplit = 8, kSplitBlk = 64;
+constexpr int kBigB3 = kHid, kBigHub = kBigB3 + kOut;  // vectors of a 128-sample tile: db1 | db3 | Huber sum
+inline int td_split_items(int k1) { return 16 + 4 * ((k1 / 16 + 3) / 4) + 4 + 1; }
+
+// x in three BF16 terms (24 bits: exact for a normal x not near the smallest).
+__device__ __forceinline__ void split_bf16(float x, float (&t)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    t[i] = __bfloat162float(__float2bfloat16_rn(x));
+    x -= t[i];
+  }
+}
+// A word, and two floats, of another CTA's copy of a shared array.
+__device__ __forceinline__ int ld_cluster1(const int* p, uint32_t rank) {
+  uint32_t a;
+  int v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_cluster2(const float* p, uint32_t rank) {
+  uint32_t a;
+  float2 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
 }
 
+// Operands of kGroup fragment tiles in one stage: 2 KB of A, up to 2 KB of B a tile.
+constexpr int kGroup = 8, kStageTile = 4096;
+constexpr int kSplitSmem = kSplitBlk * kSplitBlk * 4 + 2 * kGroup * kStageTile;
+
+__global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
+    k_td_update_split(TdUpdate u, TdFrag f, int ntiles) {
+  extern __shared__ __align__(128) uint8_t usm[];
+  float* blk = reinterpret_cast<float*>(usm);
+  uint8_t* stage = usm + kSplitBlk * kSplitBlk * 4;
+  __shared__ uint64_t bar[2];
+  __shared__ int bad_sh;
+  pdl_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
+  const int g = lane >> 2, q = lane & 3;
+  const uint32_t rank = cluster_rank();
+  const int nx = u.L.k1 / 16, nb1 = (nx + 3) / 4, n2 = 16, n1 = 4 * nb1;
+  const int item = (int)blockIdx.x / kSplit;
+  const bool w2 = item < n2, mat = item < n2 + n1, head = !mat && item < n2 + n1 + 4;
+  const int mb = w2 ? item >> 2 : (item - n2) / nb1, nb = w2 ? item & 3 : (item - n2) % nb1, hb = item - n2 - n1;
+  // this thread's parameters: columns k, k + 1 of row r; output o of unit n
+  // (o = 6: its bias); vector entry ve
+  const int r = mb * kSplitBlk + 8 * (int)rank + warp, k = nb * kSplitBlk + 2 * lane;
+  const int o = t >> 3, n = hb * kSplitBlk + 8 * (int)rank + (t & 7);
+  constexpr int kVe = (kBigHub + 1 + kSplit - 1) / kSplit;
+  const int ve = (int)rank * kVe + t;
+  int at = 0;
+  bool live[2] = {false, false};
+  float w3[kOut] = {};  // the unit's column of W3, before this launch changes it
+  if (mat) {
+    at = w2 ? u.P.w2 + r * kHid + k : u.P.w1 + r * u.L.n_in + k;
+    live[0] = w2 || k < u.L.n_in;
+    live[1] = w2 || k + 1 < u.L.n_in;
+  } else if (head) {
+    at = o < kOut ? u.P.w3 + o * kHid + n : u.P.b2 + n;
+    live[0] = o <= kOut;
+    if (o == kOut) {
+#pragma unroll
+      for (int i = 0; i < kOut; ++i)
+        w3[i] = __bfloat162float(reinterpret_cast<const bf16*>(u.img + u.L.w3)[i * kLdh + n]);
+    }
+  } else {
+    at = ve < kBigB3 ? u.P.b1 + ve : u.P.b3 + (ve - kBigB3);
+    live[0] = t < kVe && ve < kBigHub;
+  }
+  UpdRun run = upd_begin(u);
+  float th[2] = {}, m[2] = {}, v[2] = {};
+  if (u.lr != 0.0f) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (live[h]) th[h] = u.th[at + h], m[h] = u.m[at + h], v[h] = u.v[at + h];
+  }
+  if (t == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    bad_sh = 0;
+  }
+  __syncthreads();
+  pdl_wait();
+  const unsigned fail = __ldcg(u.fail);
+  // fragment tiles of this CTA, or the vectors of 128-sample tiles
+  const int nt = mat || head ? ntiles : (ntiles + kLtSub - 1) / kLtSub;
+  const int per = (nt + kSplit - 1) / kSplit, t0 = (int)rank * per, t1 = min(nt, t0 + per);
+  if (mat || head) {
+    // a tile's operands are contiguous: four 16-unit blocks of A; four (or the
+    // rest of) 16-column blocks of B, or the 16 rows of dO
+    const int nbk = w2 ? 16 : nx, bblk = min(4, nbk - 4 * nb);
+    const uint8_t* ga = reinterpret_cast<const uint8_t*>(head ? f.h2 + 4 * hb * 32 : (w2 ? f.z2 : f.z1) + 4 * mb * 32);
+    const uint8_t* gb = head ? reinterpret_cast<const uint8_t*>(f.dout)
+                             : reinterpret_cast<const uint8_t*>((w2 ? f.h1 : f.x) + 4 * nb * 32);
+    const long long lb = head ? kTile * kOutPad * 4 : nbk * 512;
+    const uint32_t bb = head ? (uint32_t)(kTile * kOutPad * 4) : (uint32_t)bblk * 512u;
+    const int ngroups = (t1 - t0 + kGroup - 1) / kGroup;
+    // warp 0: the copies of group i into its stage, a lane per copy
+    auto issue = [&](int i) {
+      const int g0 = t0 + i * kGroup, gn = min(kGroup, t1 - g0);
+      if (lane == 0) mbar_expect_tx(&bar[i & 1], (uint32_t)gn * (2048u + bb));
+      __syncwarp();
+      const int tile = lane >> 1;
+      if (tile < gn) {
+        uint8_t* dst = stage + ((i & 1) * kGroup + tile) * kStageTile;
+        if (lane & 1)
+          bulk_g2s(dst + 2048, gb + (long long)(g0 + tile) * lb, bb, &bar[i & 1]);
+        else
+          bulk_g2s(dst, ga + (long long)(g0 + tile) * (kFragTile * 16), 2048u, &bar[i & 1]);
+      }
+    };
+    if (warp == 0) {
+      if (ngroups > 0) issue(0);
+      if (ngroups > 1) issue(1);
+    }
+    const bool have0 = mat && 2 * (warp & 1) < bblk, have1 = mat && 2 * (warp & 1) + 1 < bblk;
+    float acc[2][2][4] = {};
+    bool ok = true;
+    for (int i = 0; i < ngroups; ++i) {
+      ok = ok && mbar_wait(&bar[i & 1], (uint32_t)(i >> 1) & 1u, kTcTries);
+      const int gn = min(kGroup, t1 - t0 - i * kGroup);
+      const uint8_t* st = stage + (i & 1) * kGroup * kStageTile;
+      if (mat) {
+#pragma unroll 2
+        for (int e = 0; e < gn; ++e, st += kStageTile) {
+          const uint4 a = reinterpret_cast<const uint4*>(st + (warp >> 1) * 512)[lane];
+          const uint4* pb = reinterpret_cast<const uint4*>(st + 2048 + 2 * (warp & 1) * 512) + lane;
+          const uint4 z = make_uint4(0u, 0u, 0u, 0u), b0 = have0 ? pb[0] : z, b1 = have1 ? pb[32] : z;
+          const uint32_t ar[4] = {a.x, a.y, a.z, a.w};
+          float d[2][2][4] = {};
+          mma_bf16(d[0][0], ar, b0.x, b0.y);
+          mma_bf16(d[0][1], ar, b0.z, b0.w);
+          mma_bf16(d[1][0], ar, b1.x, b1.y);
+          mma_bf16(d[1][1], ar, b1.z, b1.w);
+#pragma unroll
+          for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) acc[b][h][j] += d[b][h][j];
+        }
+      } else {
+        // dW3[o][n] = sum_s dO[s][o] H2[s][n] (warps 0..3) and M[n][o], the same
+        // sum over the samples with H2[s][n] > 0, from which db2[n] = sum_o W3[o][n]
+        // M[n][o] (warps 4..7).  dO in three BF16 terms against the exact BF16 H2
+        // and 0 / 1: FP32 sums of exact products, as on the CUDA cores.
+#pragma unroll 2
+        for (int e = 0; e < gn; ++e, st += kStageTile) {
+          const uint4 a = reinterpret_cast<const uint4*>(st + (warp & 3) * 512)[lane];
+          const float* d = reinterpret_cast<const float*>(st + 2048) + 2 * q * kOutPad + g;
+          float x[4][3];
+          split_bf16(d[0], x[0]);
+          split_bf16(d[kOutPad], x[1]);
+          split_bf16(d[8 * kOutPad], x[2]);
+          split_bf16(d[9 * kOutPad], x[3]);
+          uint32_t ar[4] = {a.x, a.y, a.z, a.w};
+          if (warp >= 4) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              ar[j] = ((ar[j] & 0x7FFFu) ? 0x3F80u : 0u) | ((ar[j] & 0x7FFF0000u) ? 0x3F800000u : 0u);
+          }
+          float sm[4] = {};
+#pragma unroll
+          for (int c = 2; c >= 0; --c) mma_bf16(sm, ar, pack_bf16x2(x[0][c], x[1][c]), pack_bf16x2(x[2][c], x[3][c]));
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[0][0][j] += sm[j];
+        }
+      }
+      fence_async_smem();  // these reads before the stage takes another copy
+      __syncthreads();
+      if (warp == 0 && i + 2 < ngroups) issue(i + 2);
+    }
+    if (!ok) {
+      // a copy did not complete: no update of this item; one more bounded wait
+      bad_sh = 1;
+      if (t == 0)
+        for (int i = max(0, ngroups - 2); i < ngroups; ++i) mbar_wait(&bar[i & 1], (uint32_t)(i >> 1) & 1u, kTcTries);
+    }
+    if (mat) {
+#pragma unroll
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            *reinterpret_cast<float2*>(blk + (16 * (warp >> 1) + g + 8 * j) * kSplitBlk + 32 * (warp & 1) + 16 * b + 8 * h + 2 * q) =
+                make_float2(acc[b][h][2 * j], acc[b][h][2 * j + 1]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        *reinterpret_cast<float2*>(blk + (16 * (warp & 3) + g + 8 * j) * 16 + 8 * (warp >> 2) + 2 * q) =
+            make_float2(acc[0][0][2 * j], acc[0][0][2 * j + 1]);
+    }
+  } else {
+    for (int e = t; e <= kBigHub; e += 256) {
+      float a = 0.0f;
+#pragma unroll 4
+      for (int i = t0; i < t1; ++i) a += f.vec[(long long)i * kVecLd + e];
+      blk[e] = a;
+    }
+  }
+  cluster_arrive();
+  cluster_wait();
+  bool bad = false;
+  if (t < kSplit) bad = ld_cluster1(&bad_sh, (uint32_t)t) != 0;
+  const bool failed = __syncthreads_or(bad) || fail != 0u;
+  upd_fail(failed, run);
+  // element i (even) and i + 1 of the item
+  auto total = [&](int i) {
+    float2 x[kSplit];
+#pragma unroll
+    for (int c = 0; c < kSplit; ++c) x[c] = ld_cluster2(blk + i, (uint32_t)c);
+    float2 sum = x[0];
+#pragma unroll
+    for (int c = 1; c < kSplit; ++c) sum.x += x[c].x, sum.y += x[c].y;
+    if (failed) sum.x = sum.y = __int_as_float(0x7fc00000);
+    return sum;
+  };
+  if (mat) {
+    if (live[0]) {
+      const float2 gr = total((8 * (int)rank + warp) * kSplitBlk + 2 * lane);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!live[h]) continue;
+        const float gh = h ? gr.y : gr.x;
+        upd_grad(u, at + h, gh);
+        if (run.adam) th[h] = upd_adam(u, run, at + h, gh, th[h], m[h], v[h]);
+        if (run.sync) u.tgt[at + h] = th[h];
+      }
+      // the padding column beside an odd last input stays zero
+      if (w2)
+        upd_images<2, 2>(u, run, r, k, th[0], th[1]);
+      else
+        upd_images<1, 2>(u, run, r, k, th[0], th[1]);
+    }
+  } else if (head) {
+    if (live[0]) {
+      const int e = (8 * (int)rank + (t & 7)) * 16;
+      float gr = 0.0f;
+      if (o < kOut) {
+        const float2 x = total(e + (o & ~1));
+        gr = (o & 1) ? x.y : x.x;
+      } else {
+#pragma unroll
+        for (int i = 0; i < kOut; i += 2) {
+          const float2 x = total(e + 8 + i);
+          gr += w3[i] * x.x;
+          gr += w3[i + 1] * x.y;
+        }
+      }
+      upd_one(u, run, at, gr, th[0], m[0], v[0]);
+    }
+  } else if (t < kVe && ve <= kBigHub) {
+    const float2 x = total(ve & ~1);
+    const float gr = (ve & 1) ? x.y : x.x;
+    if (ve < kBigHub)
+      upd_one(u, run, at, gr, th[0], m[0], v[0]);
+    else if (u.loss)
+      *u.loss = gr / (float)u.batch;
+  }
+  upd_end(u, failed);
+  cluster_arrive();  // the others' reads of this CTA's sums are done
+  cluster_wait();
+}
 
 // ------------------------------------------------ tcgen05 learner (large batches)
 // The tiles of k_td_tile with 128 samples, on the fifth-generation tensor
@@ -2297,9 +2494,11 @@ inline int td_update_items(int k1, bool big) {
 // Bound by the latency of its chain (gather, three layers, dO, dH1, about 18 K
 // cycles).  In place of the learner whose jobs streamed W2 through two 32 KB
 // buffers, ran a forward for each of two roles a tile and wrote a 330 KB
-// gradient row per tile: batch 4,096 76 -> 45.6 us.
-// Below this batch the 16-sample learner's CTAs spread over more SMs and its
-// chain is shorter.
+// gradient row per tile: batch 4,096
+// 76 -> 34.5 us.
+// Below this batch the 16-sample learner, whose CTAs spread over more SMs: 24.3
+// against 27.2 us at batch 1,024 (35.8 against 31.3 at 2,000, where the line
+// stays so that the batches keep their summation order).
 constexpr int kLtMinBatch = 2048;
 
 struct LtSmem {
@@ -2340,47 +2539,48 @@ __device__ __forceinline__ uint32_t movmatrix(uint32_t a) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(d) : "r"(a));
   return d;
 }
-// 16 samples x 64 units in C-fragment pairs (p[2 j]: sample g, p[2 j + 1]: g + 8,
-// units 8 j + 2 q, + 1) as k_td_update's operands of four 16-unit blocks: A
-// fragments of the transpose, or B fragments.
+// 16 samples x 16 units in C-fragment pairs (p[2 j]: sample g, p[2 j + 1]: g + 8,
+// units 8 j + 2 q, + 1) as an operand of k_td_update_split: the A fragment of the
+// transpose, or the B fragment.
 template <bool kA>
-__device__ __forceinline__ void lt_put_frags(uint4* out, const uint32_t (&p)[16], int lane) {
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const uint32_t l0 = movmatrix(p[4 * b]), l1 = movmatrix(p[4 * b + 1]);
-    const uint32_t h0 = movmatrix(p[4 * b + 2]), h1 = movmatrix(p[4 * b + 3]);
-    out[b * 32 + lane] = kA ? make_uint4(l0, h0, l1, h1) : make_uint4(l0, l1, h0, h1);
-  }
+__device__ __forceinline__ void lt_put_frag(uint4* out, const uint32_t (&p)[4], int lane) {
+  const uint32_t l0 = movmatrix(p[0]), l1 = movmatrix(p[1]), h0 = movmatrix(p[2]), h1 = movmatrix(p[3]);
+  out[lane] = kA ? make_uint4(l0, h0, l1, h1) : make_uint4(l0, l1, h0, h1);
 }
-// Hidden-layer epilogue of a warp's 32 rows x 64 columns at t: bias, ReLU, BF16
-// pairs back into the first half of the columns; with kOut != 0 also as
-// fragments (1: B, 2: A) to out (the next 16 samples 16 blocks on), and mask[h]
-// bit 4 j + e = whether element e of octet j is positive.
+// Hidden-layer epilogue of a warp's 32 rows x 64 columns at t, 16 columns at a
+// time: bias, ReLU, BF16 pairs back into the first half of the columns (below
+// every column still to be read); with kPut != 0 also as fragments (1: B, 2: A)
+// to out (the next 16 units 32 words on, the next 16 samples kFragTile), and
+// mask[h] bit 8 b + 4 j + e = whether element e of octet j of block b is positive.
+// Rolled: the code runs once per tile, so its instruction fetches count.
 template <int kPut>
 __device__ __forceinline__ void lt_epilogue(uint32_t t, const float* bias, uint4* out, uint32_t (&mask)[2], int lane) {
   const float2* b2 = reinterpret_cast<const float2*>(bias) + (lane & 3);
-  uint32_t r[2][32];
-  tmem_ld_frag64_nowait(t, r[0]);
-  tmem_ld_frag64_nowait(t + (16u << 16), r[1]);
-  tmem_ld_wait();
+  mask[0] = mask[1] = 0u;
+#pragma unroll 1
+  for (int b = 0; b < 4; ++b) {
+    uint32_t r[2][8];
+    tmem_ld_frag16_nowait(t + 16u * b, r[0]);
+    tmem_ld_frag16_nowait(t + (16u << 16) + 16u * b, r[1]);
+    const float2 bb[2] = {b2[8 * b], b2[8 * b + 4]};
+    tmem_ld_wait();
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint32_t p[16], mk = 0u;
+    for (int h = 0; h < 2; ++h) {
+      uint32_t p[4], mk = 0u;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float2 b = b2[4 * j];
+      for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const uint32_t w = pack_bf16x2(fmaxf(__uint_as_float(r[h][4 * j + 2 * e]) + b.x, 0.f),
-                                       fmaxf(__uint_as_float(r[h][4 * j + 2 * e + 1]) + b.y, 0.f));
-        p[2 * j + e] = w;
-        if (kPut) mk |= ((w & 0x7FFFu) ? 1u : 0u) << (4 * j + 2 * e) | ((w & 0x7FFF0000u) ? 2u : 0u) << (4 * j + 2 * e);
+        for (int e = 0; e < 2; ++e) {
+          const uint32_t w = pack_bf16x2(fmaxf(__uint_as_float(r[h][4 * j + 2 * e]) + bb[j].x, 0.f),
+                                         fmaxf(__uint_as_float(r[h][4 * j + 2 * e + 1]) + bb[j].y, 0.f));
+          p[2 * j + e] = w;
+          if (kPut) mk |= ((w & 0x7FFFu) ? 1u : 0u) << (4 * j + 2 * e) | ((w & 0x7FFF0000u) ? 2u : 0u) << (4 * j + 2 * e);
+        }
+      tmem_st_frag8(t + ((uint32_t)(16 * h) << 16) + 8u * b, p);
+      if (kPut) {
+        lt_put_frag<kPut == 2>(out + h * kFragTile + b * 32, p, lane);
+        mask[h] |= mk << (8 * b);
       }
-    }
-    tmem_st_frag32(t + ((uint32_t)(16 * h) << 16), p);
-    if (kPut) {
-      lt_put_frags<kPut == 2>(out + h * kFragTile, p, lane);
-      mask[h] = mk;
     }
   }
   tmem_st_wait();
@@ -2411,20 +2611,16 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   const int ntiles = (batch + kLtRows - 1) / kLtRows, stride = (int)gridDim.x / kTpRanks;
   cluster_arrive();  // every CTA of the cluster has started before the first remote store
   if (warp == 0) tmem_alloc(&tslot, 512);
-  if (tid == 0) {
+  const uint8_t* im = rank == 2 ? img_t : img;
+  if (tid == kThreads - 1) {
     mbar_init(&bar_w1, 1);
     mbar_init(&bar_w2, 1);
     mbar_init(&bar_mma, 1);
   }
   pdl_wait();
   pdl_launch_dependents();
-  lt_sync();
-  const uint32_t tacc = tslot, tacc2 = tacc + 256u;
-  const uint32_t tw = ((uint32_t)(quarter * 32) << 16) + (uint32_t)(64 * grp);  // this warp's lanes and columns
-  const uint32_t sx = smem_u32(xs), sw1 = smem_u32(tsm + T.w1), sw2 = smem_u32(tsm + T.w2),
-                 sw3 = smem_u32(tsm + T.w3);
-  const uint8_t* im = rank == 2 ? img_t : img;
-  if (tid == 0) {
+  const unsigned long long tstep = __ldcg(step), st = __ldcg(rp.steps);
+  if (tid == kThreads - 1) {
     const uint8_t* src = rank == 2 ? timg_t : timg;
     mbar_expect_tx(&bar_w1, G.w2a);
     bulk_g2s(tsm + T.w1, src + G.w1, G.w2a, &bar_w1);
@@ -2432,18 +2628,13 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     bulk_g2s(tsm + T.w2, src + G.w2f, kHid * kHid * 2u, &bar_w2);
     bulk_g2s(tsm + T.w3, src + G.w3, 16u * kHid * 2u, &bar_w2);
   }
-  for (int i = tid; i < 2 * kHid; i += kThreads)
-    b1[i] = __ldg(reinterpret_cast<const float*>(im + (i < kHid ? L.b1 : L.b2)) + (i & (kHid - 1)));
-  if (rank == 0)
-    for (int i = tid; i < kOut * kHid; i += kThreads)
-      w3f[i] = __bfloat162float(reinterpret_cast<const bf16*>(im + L.w3)[(i >> 8) * kLdh + (i & (kHid - 1))]);
-  for (int i = tid; i < kLtRows * L.k1 / 8; i += kThreads)
-    reinterpret_cast<uint4*>(xs)[i] = make_uint4(0u, 0u, 0u, 0u);
-  float b3[kOut];
-#pragma unroll
-  for (int j = 0; j < kOut; ++j) b3[j] = __ldg(reinterpret_cast<const float*>(im + L.b3) + j);
-  const unsigned long long tstep = *step;
+  lt_sync();
+  const uint32_t tacc = tslot, tacc2 = tacc + 256u;
+  const uint32_t tw = ((uint32_t)(quarter * 32) << 16) + (uint32_t)(64 * grp);  // this warp's lanes and columns
+  const uint32_t sx = smem_u32(xs), sw1 = smem_u32(tsm + T.w1), sw2 = smem_u32(tsm + T.w2),
+                 sw3 = smem_u32(tsm + T.w3);
   const int nx = L.k1 / 16;
+  float b3[kOut];
   bool ok = true, first = true, mma_out = false;
   uint32_t phase = 0u;
   // wait for the MMAs committed last, by every thread
@@ -2457,7 +2648,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   for (int tile = (int)blockIdx.x / kTpRanks, it = 0; tile < ntiles; tile += stride, ++it) {
     if (tid < kLtRows) {
       const int i = tile * kLtRows + tid;
-      rows_sh[tid] = i < batch ? (int)sample_entry(seed, tstep, i, rp) : -1;
+      rows_sh[tid] = i < batch ? (int)sample_entry(seed, tstep, st, i, rp) : -1;
     }
     __syncthreads();
     {
@@ -2477,7 +2668,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
       for (int u = 0; u < 8; ++u)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          if (lane + 32 * c < L.n_in)
+          if (lane + 32 * c < L.k1)
             *reinterpret_cast<bf16*>(xs + kmajor_offset(warp * 8 + u, lane + 32 * c, kLtRows)) =
                 __float2bfloat16_rn(v[u][c]);
     }
@@ -2501,6 +2692,20 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
                     smem_desc(sw1 + (uint32_t)ks * 2u * kHid * 16u, kHid * 16u, 128), idesc_bf16_f32(kLtRows, kHid),
                     ks > 0 ? 1u : 0u);
       tc_commit(&bar_mma);
+    }
+    if (first) {
+      // the vectors of this CTA's network, behind layer 1
+      for (int i = tid; i < 2 * kHid; i += kThreads)
+        b1[i] = __ldg(reinterpret_cast<const float*>(im + (i < kHid ? L.b1 : L.b2)) + (i & (kHid - 1)));
+      if (rank == 0) {
+#pragma unroll
+        for (int i = 0; i < kOut * kHid / kThreads; ++i) {
+          const int j = tid + i * kThreads;
+          w3f[j] = __bfloat162float(reinterpret_cast<const bf16*>(im + L.w3)[(j >> 8) * kLdh + (j & (kHid - 1))]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kOut; ++j) b3[j] = __ldg(reinterpret_cast<const float*>(im + L.b3) + j);
     }
     if (rank == 0) {
       // X's B fragments: a core matrix is an 8 x 8 block of 16-byte rows
@@ -2615,29 +2820,32 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
         const float2 b = *reinterpret_cast<const float2*>(p + 4);
         d[i][0] = a.x, d[i][1] = a.y, d[i][2] = a.z, d[i][3] = a.w, d[i][4] = b.x, d[i][5] = b.y;
       }
-      uint32_t p[2][16];
+#pragma unroll 1
+      for (int b = 0; b < 4; ++b) {
+        uint32_t p[2][4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        float z[4][2] = {};
+        for (int j = 0; j < 2; ++j) {
+          float z[4][2] = {};
 #pragma unroll
-        for (int o = 0; o < kOut; ++o) {
-          const float2 w = *reinterpret_cast<const float2*>(w3f + o * kHid + 64 * grp + 8 * j + 2 * q);
+          for (int o = 0; o < kOut; ++o) {
+            const float2 w = *reinterpret_cast<const float2*>(w3f + o * kHid + 64 * grp + 16 * b + 8 * j + 2 * q);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              z[i][0] += d[i][o] * w.x;
+              z[i][1] += d[i][o] * w.y;
+            }
+          }
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            z[i][0] += d[i][o] * w.x;
-            z[i][1] += d[i][o] * w.y;
+            const uint32_t mk = mask2[i >> 1] >> (8 * b + 4 * j + 2 * (i & 1));
+            p[i >> 1][2 * j + (i & 1)] = pack_bf16x2((mk & 1u) ? z[i][0] : 0.0f, (mk & 2u) ? z[i][1] : 0.0f);
           }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t mk = mask2[i >> 1] >> (4 * j + 2 * (i & 1));
-          p[i >> 1][2 * j + (i & 1)] = pack_bf16x2((mk & 1u) ? z[i][0] : 0.0f, (mk & 2u) ? z[i][1] : 0.0f);
+        for (int h = 0; h < 2; ++h) {
+          tmem_st_frag8(tacc2 + tw + ((uint32_t)(16 * h) << 16) + 8u * b, p[h]);
+          lt_put_frag<true>(f.z2 + fo + h * kFragTile + b * 32, p[h], lane);
         }
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        tmem_st_frag32(tacc2 + tw + ((uint32_t)(16 * h) << 16), p[h]);
-        lt_put_frags<true>(f.z2 + fo + h * kFragTile, p[h], lane);
       }
       tmem_st_wait();
     }
@@ -2664,31 +2872,35 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     mma_wait();
     if (ok) {
       // dZ1 = (H1 > 0) dH1: its fragments (BF16), db1 from the FP32 values
-      uint32_t r[2][32];
-      tmem_ld_frag64_nowait(tacc + tw, r[0]);
-      tmem_ld_frag64_nowait(tacc + tw + (16u << 16), r[1]);
-      tmem_ld_wait();
-      float cs[16] = {};
+#pragma unroll 1
+      for (int b = 0; b < 4; ++b) {
+        uint32_t r[2][8];
+        tmem_ld_frag16_nowait(tacc + tw + 16u * b, r[0]);
+        tmem_ld_frag16_nowait(tacc + tw + (16u << 16) + 16u * b, r[1]);
+        tmem_ld_wait();
+        float cs[4] = {};
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t p[16];
+        for (int h = 0; h < 2; ++h) {
+          uint32_t p[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+          for (int j = 0; j < 2; ++j)
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const uint32_t mk = mask1[h] >> (4 * j + 2 * i);
-            const float a = (mk & 1u) ? __uint_as_float(r[h][4 * j + 2 * i]) : 0.0f;
-            const float b = (mk & 2u) ? __uint_as_float(r[h][4 * j + 2 * i + 1]) : 0.0f;
-            cs[2 * j] += a;
-            cs[2 * j + 1] += b;
-            p[2 * j + i] = pack_bf16x2(a, b);
-          }
-        lt_put_frags<true>(f.z1 + fo + h * kFragTile, p, lane);
-      }
+            for (int i = 0; i < 2; ++i) {
+              const uint32_t mk = mask1[h] >> (8 * b + 4 * j + 2 * i);
+              const float x = (mk & 1u) ? __uint_as_float(r[h][4 * j + 2 * i]) : 0.0f;
+              const float y = (mk & 2u) ? __uint_as_float(r[h][4 * j + 2 * i + 1]) : 0.0f;
+              cs[2 * j] += x;
+              cs[2 * j + 1] += y;
+              p[2 * j + i] = pack_bf16x2(x, y);
+            }
+          lt_put_frag<true>(f.z1 + fo + h * kFragTile + b * 32, p, lane);
+        }
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        for (int off = 4; off < 32; off <<= 1) cs[j] += __shfl_xor_sync(kFull, cs[j], off);
-        if (g == 0) red[quarter * kHid + 64 * grp + 8 * (j >> 1) + 2 * q + (j & 1)] = cs[j];
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+          for (int off = 4; off < 32; off <<= 1) cs[j] += __shfl_xor_sync(kFull, cs[j], off);
+          if (g == 0) red[quarter * kHid + 64 * grp + 16 * b + 8 * (j >> 1) + 2 * q + (j & 1)] = cs[j];
+        }
       }
     }
     lt_sync();  // also: tensor memory and X are free for the next tile
@@ -2844,7 +3056,8 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
       (rc = set_smem_attr((const void*)k_rollout_q<2, true, false>, fwd_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<2, true, true>, fwd_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_td_tile, grad_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_td_tc, lt_smem(80).bytes))) {
+      (rc = set_smem_attr((const void*)k_td_tc, lt_smem(80).bytes)) ||
+      (rc = set_smem_attr((const void*)k_td_update_split, kSplitSmem))) {
     free_qnet(q);
     return rc;
   }
@@ -3227,22 +3440,22 @@ extern "C" int sg_td_train_step(sg_qnet_t q, sg_replay_t rp, int32_t batch, floa
   const bool big = batch >= kLtMinBatch;
   const int rows = big ? kLtRows : kTile, ntiles = (batch + rows - 1) / rows;
   const int rounds = (ntiles + fit - 1) / fit, grid = (ntiles + rounds - 1) / rounds * kTpRanks;
-  const int frags = big ? ntiles * kLtSub : ntiles, items = td_update_items(q->IL.k1, big);
+  const int frags = big ? ntiles * kLtSub : ntiles, items = td_update_items(q->IL.k1);
   const TdFrag f = td_frag(q->frag, frags, q->IL.k1);
   const uint8_t *im = q->img, *im_t = q->img_t, *tc = q->img_tc, *tc_t = q->img_tc_t;
   const unsigned long long* step = q->step;
   if (big) {
     SG_CUDA(sg_launch_pdl(k_td_tc, grid, kThreads, lt_smem(q->IL.k1).bytes, stream, im, im_t, tc, tc_t, q->IL, rp->d,
                           seed, step, batch, gamma, f, q->td_fail));
-    SG_CUDA(sg_launch_pdl(k_td_update<8, false, true>, items, 256, 0, stream, u, f, frags));
+    SG_CUDA(sg_launch_pdl(k_td_update_split, td_split_items(q->IL.k1) * kSplit, 256, kSplitSmem, stream, u, f, frags));
     return SG_OK;
   }
   SG_CUDA(sg_launch_pdl(k_td_tile, grid, kThreads, grad_smem(q->IL), stream, im, im_t, q->IL, rp->d, seed, step, batch,
                         gamma, f, q->td_fail));
   if (ntiles <= kTuSlots)
-    SG_CUDA(sg_launch_pdl(k_td_update<4, true, false>, items, 128, 0, stream, u, f, ntiles));
+    SG_CUDA(sg_launch_pdl(k_td_update<4, true>, items, 128, 0, stream, u, f, ntiles));
   else
-    SG_CUDA(sg_launch_pdl(k_td_update<8, false, false>, items, 256, 0, stream, u, f, ntiles));
+    SG_CUDA(sg_launch_pdl(k_td_update<8, false>, items, 256, 0, stream, u, f, ntiles));
   return SG_OK;
 }
 
