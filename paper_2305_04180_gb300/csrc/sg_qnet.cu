@@ -923,15 +923,15 @@ __global__ void __launch_bounds__(512 * MT, 1)
 // network.  Per step the network runs on the tile on the tensor cores
 // (tcgen05 MMAs into 256 tensor-memory columns, epilogues split over the 8
 // warps of each lane quarter), warps 0-3 take the greedy actions from the
-// head, the first 16 warps step the tile's envs the way sg_sim_step does (8
-// envs per warp, one per lane: the scalar part, lane_step), and then every
-// warp takes whole-warp scans row by row from a shared counter, writing the
-// next observation as the tile's BF16 row and the FP32 outputs and ring
-// entries.  Same VEM draws, same simulator values as k_rollout_q; the Q
+// head, the first four warps run what every env of the tile takes, one env per
+// lane (lane_motion, as in sg_sim_step), and then every warp takes the rest row
+// by row from a shared counter (bit-row collision test, scan, AutoReset),
+// writing the next observation as the tile's BF16 row and the FP32 outputs
+// and ring entries.  Same VEM draws, same simulator values as k_rollout_q; the Q
 // values differ from it only in the summation order.
 //
 // Shared memory is kept small (136 KB) so that L1 keeps room for the maps the
-// scans read: the input tile (at most 20 KB) and the step records (16 KB,
+// scans read: the input tile (at most 20 KB) and the step records (10 KB,
 // from byte 32 K) live inside the hidden-activation buffer, which holds H1
 // and H2 during the network only, and all of W1 (two 128-row halves) and W2
 // (four 32 KB pieces: the K halves of its two 128-row halves) stream through
@@ -944,12 +944,11 @@ constexpr int kQtWarps = 32;
 constexpr int kQtThreads = kQtWarps * 32;
 constexpr uint32_t kQtBuf = 32u * 1024u;
 constexpr uint32_t kQtRecOff = 32u * 1024u;
-// The env steps of a tile (the scalar part, lane_step) run on the first
-// kQtEnvs / kQtStepLanes warps, kQtStepLanes envs per warp (one per lane):
-// 16 warps of 8 envs measured fastest (32 x 4: 406.2, 16 x 8: 414.5,
-// 8 x 16: 411.4, 4 x 32: 400.5 M env-steps/s at 65,536 envs).
-constexpr int kQtStepLanes = 8;  // records in the activation buffer (input tile: 256 k1 <= 20 KB)
-static_assert(kQtRecOff + kQtEnvs * 128u <= (uint32_t)(kQtEnvs * kHid * 2), "records fit the activation buffer");
+// The env steps of a tile: what every env takes, one env per lane of the first
+// four warps (lane_motion); the bit-row collision test and AutoReset, which
+// few take, go with the scans, a warp per row.  With 16 warps of 8 lanes doing
+// the whole scalar step, 65,536 envs x 32 steps took 4,112 us (3,664 now).
+static_assert(kQtRecOff + kQtEnvs * sizeof(MotionRec) <= (uint32_t)(kQtEnvs * kHid * 2), "records fit the activation buffer");
 
 struct QtSmem {
   uint32_t hx, b0, b1, w3, bytes;
@@ -1083,6 +1082,7 @@ constexpr unsigned kQtWaitIters = 1u << 22;  // x ~256 ns sleeps: about a second
 // takes its first observation from the replay ring (the entry the previous
 // segment wrote), or scans it when there is no ring.  sync: [nblk] segments
 // done per block, item counter, abort word; zero at launch.
+template <bool kFast>
 __global__ void __launch_bounds__(kQtThreads, 1)
     k_rollout_q_tc(const __grid_constant__ DevCfg c, SimPtrs p, const uint8_t* __restrict__ img,
                    const uint8_t* __restrict__ timg, ImgLayout L, int K, const float* __restrict__ eps, ReplayDev rp,
@@ -1104,7 +1104,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   const TcImg G = tc_img(L.k1);
   uint8_t* hx = tsm + T.hx;  // the input tile, then H1, then H2
   uint8_t* w3s = tsm + T.w3;
-  StepScanRec* rec = reinterpret_cast<StepScanRec*>(tsm + T.hx + kQtRecOff);  // during the env steps only
+  MotionRec* rec = reinterpret_cast<MotionRec*>(tsm + T.hx + kQtRecOff);  // during the env steps only
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long n = c.n_envs;
   const int nblk = (int)((n + kQtEnvs - 1) / kQtEnvs);
@@ -1179,11 +1179,9 @@ __global__ void __launch_bounds__(kQtThreads, 1)
     const int nv = max(0, min(4, (int)n - slot0));
     const bool live = lane < nv;
     const int env = live ? order[slot0 + lane] : 0;
-    // the env-step lanes: row srow of the tile
-    const bool stepper = warp < kQtEnvs / kQtStepLanes;
-    const int srow = warp * kQtStepLanes + lane;
-    const bool slive = stepper && lane < kQtStepLanes && (long long)blk * kQtEnvs + srow < n;
-    const int senv = slive ? order[blk * kQtEnvs + srow] : 0;
+    // the env-step lanes: row tid of the tile
+    const bool slive = tid < kQtEnvs && (long long)blk * kQtEnvs + tid < n;
+    const int senv = slive ? order[blk * kQtEnvs + tid] : 0;
     // the tile: zero (padding columns, rows without an env), then the first
     // observation of the segment
     for (int i = tid; i < kQtEnvs * L.k1 / 8; i += kQtThreads)
@@ -1198,19 +1196,21 @@ __global__ void __launch_bounds__(kQtThreads, 1)
           *reinterpret_cast<bf16*>(hx + kmajor_offset(row0 + e, k, kQtEnvs)) = __float2bfloat16_rn(__ldcg(src + k));
       }
     } else {
-      if (live) lane_observe(c, p, env, load_env_l2(p, env), rec[row0 + lane]);
+      if (live) lane_observe(c, p, env, load_env_l2(p, env), rec + row0 + lane);
       __syncwarp();
       for (int e = 0; e < nv; ++e) {
-        const StepScanRec& r = rec[row0 + e];
-        float b0, b1;
-        if (c.scan_fast)
-          scan_rec<false, true>(c, p, r, false, lane, b0, b1);
-        else
-          scan_rec<false, false>(c, p, r, false, lane, b0, b1);
-        qt_obs_to_tile(hx, row0 + e, b0, b1, lane < 5 ? r.exa[lane] : 0.0f, B, lane);
+        const MotionRec* r = rec + row0 + e;
+        const uint4 w0 = rec_word<false>(r, 0), w1 = rec_word<false>(r, 1);
+        const RecScan q = rec_scan(c, rec_word<false>(r, 3), rec_word<false>(r, 4), lane);
+        ObsRegs o;
+        scan_pose<false, kFast>(c, q.sm, q.nb, q.off0, q.off1, __uint_as_float(w0.x), __uint_as_float(w0.y),
+                                __uint_as_float(w0.z), __uint_as_float(w0.w), ((uint64_t)w1.y << 32) | w1.x, q.k0, lane,
+                                o.b0, o.b1);
+        o.ex = lane < 5 ? r->ex[lane] : 0.0f;
+        qt_obs_to_tile(hx, row0 + e, o.b0, o.b1, o.ex, B, lane);
         if (use_replay) {
           const long long sl = (long long)((rbase + (unsigned long long)s0) % (unsigned long long)rp.slots);
-          write_row(rp.s + (sl * rp.n_envs + r.env) * rp.obs_dim, b0, b1, r.exa, B, lane);
+          write_obs(rp.s + (sl * rp.n_envs + r->env) * rp.obs_dim, o, B, lane);
         }
       }
     }
@@ -1308,29 +1308,21 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
-      // ---- the env steps of the tile: one env per lane of the stepping warps ----
-      if (stepper) {
-        Env s;
-        uint32_t a = 0;
-        if (slive) {
-          // the state stays in shared memory between the steps of a segment
-          // (stored to global memory at its last step)
-          s = t == s0 ? load_env_l2(p, senv) : env_sh[srow];
-          if (t == s0) akey_sh[srow] = sm_at(sm_at(c.seed, kStreamAction), (uint64_t)senv);
-          // VEM (Sec. 3.1.1): with probability eps_i the random action of step t
-          const uint64_t h = sm_at(akey_sh[srow], (uint64_t)s.t);
-          const uint32_t ra = (uint32_t)(sm_at(h, 0ull) >> 32) % (uint32_t)c.n_actions;
-          const bool explore = u24_hi(sm_at(h, 1ull)) < __ldg(eps + senv);
-          a = explore ? ra : (uint32_t)greedy[srow];
-        }
-        const uint32_t d = lane_step(c, p, senv, slive, s, a, rec[slive ? srow : 0], lane);
-        if (slive) {
-          env_sh[srow] = s;
-          if (t + 1 == s1) store_env(p, senv, s);
-          act_sh[srow] = (uint8_t)a;
-          if (act_seq) act_seq[(long long)t * n + senv] = (uint8_t)a;
-          if (done_seq) done_seq[(long long)t * n + senv] = (uint8_t)d;
-        }
+      // ---- the env steps of the tile: one env per lane of the first warps ----
+      if (slive) {
+        // the state stays in shared memory between the steps of a segment
+        // (stored to global memory at its end)
+        Env s = t == s0 ? load_env_l2(p, senv) : env_sh[tid];
+        if (t == s0) akey_sh[tid] = sm_at(sm_at(c.seed, kStreamAction), (uint64_t)senv);
+        // VEM (Sec. 3.1.1): with probability eps_i the random action of step t
+        const uint64_t h = sm_at(akey_sh[tid], (uint64_t)s.t);
+        const uint32_t ra = (uint32_t)(sm_at(h, 0ull) >> 32) % (uint32_t)c.n_actions;
+        const bool explore = u24_hi(sm_at(h, 1ull)) < __ldg(eps + senv);
+        const uint32_t a = explore ? ra : (uint32_t)greedy[tid];
+        lane_motion<false>(c, p, senv, s, a, rec + tid, nullptr);
+        env_sh[tid] = s;
+        act_sh[tid] = (uint8_t)a;
+        if (act_seq) act_seq[(long long)t * n + senv] = (uint8_t)a;
       }
       // every record of the tile is written; the scans (one or two per env,
       // 16 to 64 beams) are handed out row by row through a shared counter,
@@ -1344,39 +1336,59 @@ __global__ void __launch_bounds__(kQtThreads, 1)
         if (lane == 0) e = atomicAdd(&scan_next, 1);
         e = __shfl_sync(kFull, e, 0);
         if (e >= rows) break;
-        const StepScanRec& r = rec[e];
-        const int ie = r.env;
-        const uint32_t de = r.done;
-        float b0, b1;
-        const float mn = c.scan_fast ? scan_rec<false, true>(c, p, r, false, lane, b0, b1)
-                                     : scan_rec<false, false>(c, p, r, false, lane, b0, b1);
-        const float rw = (de & 1u) ? -10.0f : (de & 2u) ? 75.0f : reward_finish(c, r.rpart, mn);
-        const uint32_t ae = act_sh[e];
+        const MotionRec* r = rec + e;
+        const uint4 w1 = rec_word<false>(r, 1), w3 = rec_word<false>(r, 3);
+        const int ie = (int)w3.w;
+        const RecScan q = rec_scan(c, w3, rec_word<false>(r, 4), lane);
+        uint32_t d = w1.w;
+        ObsRegs o;
+        float mn;
+        {
+          const uint4 w0 = rec_word<false>(r, 0);
+          const float x = __uint_as_float(w0.x), y = __uint_as_float(w0.y);
+          if (d & kRecSlow) {
+            const MapDesc m = p.maps[p.env_map[ie]];
+            d = (d & 7u) | (collide_rows_warp(c, m, p.atlas + m.word_off, x, y, lane) ? 1u : 0u);
+          }
+          mn = scan_pose<false, kFast>(c, q.sm, q.nb, q.off0, q.off1, x, y, __uint_as_float(w0.z),
+                                       __uint_as_float(w0.w), ((uint64_t)w1.y << 32) | w1.x, q.k0, lane, o.b0, o.b1);
+        }
+        o.ex = lane < 5 ? r->ex[lane] : 0.0f;
+        const float rw = (d & 1u) ? -10.0f : (d & 2u) ? 75.0f : reward_finish(c, __uint_as_float(w1.z), mn);
         if (use_replay) {
           // transition t: s2 is the observation after the step, before a reset
           const long long en = slot_t * rp.n_envs + ie;
-          write_row(rp.s2 + en * rp.obs_dim, b0, b1, r.exa, B, lane);
+          write_obs(rp.s2 + en * rp.obs_dim, o, B, lane);
           if (lane == 0) {
-            rp.a[en] = (uint8_t)ae;
+            rp.a[en] = act_sh[e];
             rp.r[en] = rw;
-            rp.term[en] = (de & 3u) ? 1 : 0;
+            rp.term[en] = (d & 3u) ? 1 : 0;
           }
         }
-        if (lane == 0 && rew_seq) rew_seq[(long long)t * n + ie] = rw;
-        const float* ex = r.exa;
-        if (de) {
-          if (c.scan_fast)
-            scan_rec<false, true>(c, p, r, true, lane, b0, b1);
-          else
-            scan_rec<false, false>(c, p, r, true, lane, b0, b1);
-          ex = r.exb;
+        if (lane == 0) {
+          if (rew_seq) rew_seq[(long long)t * n + ie] = rw;
+          if (done_seq) done_seq[(long long)t * n + ie] = (uint8_t)d;
+        }
+        if (d) {
+          // AutoReset (Sec. 3.2.5): a new episode, observed at its step 0
+          const MapDesc m = p.maps[p.env_map[ie]];
+          const Layout L2 = layout_of(c, m);
+          Env s;
+          s.t = env_sh[e].t;
+          const uint32_t ep = env_sh[e].ep_id + 1u;
+          __syncwarp();
+          reset_env(c, m, p.clr + m.clr_off, L2, sm_at(sm_at(c.seed, kStreamReset), (uint64_t)ie), s, ep, lane);
+          if (lane == 0) env_sh[e] = s;
+          o.ex = obs_extra(c, L2, s, goal_frame(L2, s), lane);
+          scan_pose<false, kFast>(c, q.sm, q.nb, q.off0, q.off1, s.x, s.y, s.phi, s.sigma,
+                                  sm_at(sm_at(sm_at(c.seed, kStreamNoise), (uint64_t)ie), (uint64_t)s.ep_id << 32),
+                                  lane_scan_start(c, p, m, s.x, s.y), lane, o.b0, o.b1);
         }
         // the observation t + 1: the next tile row, the outputs, the next ring entry's s
-        qt_obs_to_tile(hx, e, b0, b1, lane < 5 ? ex[lane] : 0.0f, B, lane);
-        if (obs_seq) write_row(obs_seq + ((long long)t * n + ie) * c.obs_dim, b0, b1, ex, B, lane);
-        if (t == K - 1 && obs_out) write_row(obs_out + (long long)ie * c.obs_dim, b0, b1, ex, B, lane);
-        if (use_replay && t + 1 < K)
-          write_row(rp.s + (slot_n * rp.n_envs + ie) * rp.obs_dim, b0, b1, ex, B, lane);
+        qt_obs_to_tile(hx, e, o.b0, o.b1, o.ex, B, lane);
+        if (obs_seq) write_obs(obs_seq + ((long long)t * n + ie) * c.obs_dim, o, B, lane);
+        if (t == K - 1 && obs_out) write_obs(obs_out + (long long)ie * c.obs_dim, o, B, lane);
+        if (use_replay && t + 1 < K) write_obs(rp.s + (slot_n * rp.n_envs + ie) * rp.obs_dim, o, B, lane);
       }
       fence_async_smem();
     }
@@ -1384,6 +1396,8 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       if (tid == 0) atomicOr(p.status, SG_DEV_TIMEOUT);
       break;  // CTA-uniform: the launch's outputs from here on are incomplete
     }
+    __syncthreads();  // the last step's resets are in env_sh
+    if (slive) store_env(p, senv, env_sh[tid]);
     if (!sync) break;
     // publish the block's segment: its env state and ring entries are stored
     __threadfence();
@@ -3046,7 +3060,8 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   // cannot lower it below what a wider one launches with.
   const ImgLayout widest = img_layout(69);
   if ((rc = set_smem_attr((const void*)k_qnet_forward_tc, kTcSmemLaunch)) ||
-      (rc = set_smem_attr((const void*)k_rollout_q_tc, qt_smem().bytes)) ||
+      (rc = set_smem_attr((const void*)k_rollout_q_tc<false>, qt_smem().bytes)) ||
+      (rc = set_smem_attr((const void*)k_rollout_q_tc<true>, qt_smem().bytes)) ||
       (rc = set_smem_attr((const void*)k_rollout_q<1, false, false>, fwd_smem(widest))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<1, false, true>, fwd_smem(widest))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<2, false, false>, fwd_smem(widest, 32))) ||
@@ -3398,7 +3413,7 @@ int sg_rollout_eps_q(sg_sim* sim, int K, sg_qnet* q, const float* eps, sg_replay
       grid = std::min(nblk * ((K + seg - 1) / seg), cap);
       SG_CUDA(cudaMemsetAsync(sim->q_sync_dev, 0, sizeof(unsigned) * (size_t)(nblk + 2), stream));
     }
-    k_rollout_q_tc<<<grid, kQtThreads, qt_smem().bytes, stream>>>(
+    (sim->dc.scan_fast ? k_rollout_q_tc<true> : k_rollout_q_tc<false>)<<<grid, kQtThreads, qt_smem().bytes, stream>>>(
         sim->dc, sg_sim_ptrs(sim), q->img, q->img_tc, q->IL, K, eps, rd, rp ? 1 : 0, sim->map_order_dev, seg,
         seg > 0 ? sim->q_sync_dev : nullptr, obs, obs_seq, act_seq, rew_seq, done_seq);
   } else {
