@@ -660,12 +660,13 @@ __host__ __device__ constexpr size_t pipe_group_bytes(bool dyn) {
   return kPipeChunk * (sizeof(StepRec) + 2 * sizeof(ObsRec)) +
          (dyn ? 4 * kPipeChunk * sizeof(Discs) + kMaxDyn * sizeof(Obst) : 0);
 }
-// With this many observation warps a rollout lasts as long as its pose chains,
-// so the first of them only helps the pose warp: it derives the observation
+// With 15 observation warps a rollout lasts as long as its pose chains, and with
+// moving obstacles (whose motion and draws lengthen the chain) from seven on, so
+// the first of them only helps the pose warp: it derives the observation
 // records and draws the actions of the chunk after next, and the pose warp
-// takes no scans (one more buffer of step records, two of actions).  16 envs x
-// 1,000 steps: 228 -> 204 us, 152 envs x 512 166 -> 133.
-constexpr int kPipeHelper = 15;
+// takes no scans (one more buffer of step records, two of actions; one env per
+// CTA).  16 envs x 1,000 steps: 228 -> 204 us, 152 envs x 512 166 -> 133; seven
+// warps, 1,024 envs: with discs 888 -> 801, without 1,321 -> 1,392.
 constexpr size_t kPipeHelperBytes = kPipeChunk * sizeof(StepRec) + 2 * kPipeChunk * sizeof(uint32_t);
 constexpr int kPipeHelperBar = 1 + 4 * 3;  // named barriers 13, 14: step records of buffer b written
 static_assert(pipe_group_bytes(false) % 16 == 0 && pipe_group_bytes(true) % 16 == 0, "16-byte aligned groups");
@@ -872,15 +873,18 @@ static decltype(&k_rollout_random_pipe<false, true, false>) pipe_pick(const DevC
     return c.scan_fast ? k_rollout_random_pipe<true, true, kHelped> : k_rollout_random_pipe<true, false, kHelped>;
   return c.scan_fast ? k_rollout_random_pipe<false, true, kHelped> : k_rollout_random_pipe<false, false, kHelped>;
 }
-static decltype(&k_rollout_random_pipe<false, true, false>) pipe_kernel(const DevCfg& c, const sg_launch& L) {
-  return L.obs_warps >= kPipeHelper ? pipe_pick<true>(c) : pipe_pick<false>(c);
-}
-static size_t pipe_smem_bytes(int E, bool dyn, bool helped) {
-  return (size_t)E * pipe_group_bytes(dyn) + (helped ? kPipeHelperBytes : 0);
-}
 static int pipe_envs_per_block(const sg_launch& L) {
   const int E = L.warps_per_block / (1 + L.obs_warps);
   return E < 1 ? 1 : (E > kPipeMaxGroups ? kPipeMaxGroups : E);
+}
+static bool pipe_helped(const DevCfg& c, const sg_launch& L) {
+  return L.obs_warps >= (c.n_dyn > 0 ? 7 : 15) && pipe_envs_per_block(L) == 1;
+}
+static decltype(&k_rollout_random_pipe<false, true, false>) pipe_kernel(const DevCfg& c, const sg_launch& L) {
+  return pipe_helped(c, L) ? pipe_pick<true>(c) : pipe_pick<false>(c);
+}
+static size_t pipe_smem_bytes(int E, bool dyn, bool helped) {
+  return (size_t)E * pipe_group_bytes(dyn) + (helped ? kPipeHelperBytes : 0);
 }
 
 
@@ -1499,15 +1503,16 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
 // rollout while the envs alone leave warp slots empty, and the pose chain's
 // run-ahead pays at every size once K fills a chunk.  us (one warp per env /
 // pipelined): 16 envs x 1,000 steps 2,515 / 204 (15 scan warps), 304 x 512 1,656 /
-// 233 (7), 1,024 x 512 1,951 / 471, 4,096 x 224 1,184 / 726, 16,384 x 32 599 /
+// 158 (15; 180 with 7), 456 x 512 269 with 15 and 201 with 7, 1,024 x 512 1,951 /
+// 395 (7), 4,096 x 224 1,184 / 622 (7; 627 with 3), 16,384 x 32 599 /
 // 497 (3, two envs per CTA).  Few steps of many envs stay with one warp per
 // env (4,096 x 8: 59 / 75; 65,536 x 16: 1,078 / 1,179).
 static sg_launch auto_launch(int n, int K, int sms) {
   sg_launch L = {SG_ROLLOUT_GRID, 4, 1, 0, 0, 0, 0, 0};
   if (K < std::min(kPipeChunk, n / 256)) return L;
   L.kernel = SG_ROLLOUT_PIPE;
-  L.obs_warps = n <= sms ? 15 : n <= 32 * sms ? 7 : 3;
-  L.warps_per_block = n <= sms ? 16 : 8;
+  L.obs_warps = n <= 2 * sms ? 15 : n <= 32 * sms ? 7 : 3;
+  L.warps_per_block = n <= 2 * sms ? 16 : 8;
   L.order = 1;
   return L;
 }
@@ -1532,7 +1537,7 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
         const int G = 1 + L.obs_warps;
         const int E = pipe_envs_per_block(L);
         const bool dyn = sim->dc.n_dyn > 0;
-        const size_t smem = pipe_smem_bytes(E, dyn, L.obs_warps >= kPipeHelper);
+        const size_t smem = pipe_smem_bytes(E, dyn, pipe_helped(sim->dc, L));
         const int nblk = (n + E - 1) / E;
         int seg = L.segment < K ? L.segment : 0;  // one segment needs no slicing
         long long grid = nblk;
@@ -1618,7 +1623,7 @@ extern "C" int sg_sim_set_launch(sg_sim_t sim, const sg_launch* cfg) {
   if (L.kernel == SG_ROLLOUT_PIPE) {
     const int E = pipe_envs_per_block(L);
     const bool dyn = sim->dc.n_dyn > 0;
-    const size_t smem = pipe_smem_bytes(E, dyn, L.obs_warps >= kPipeHelper);
+    const size_t smem = pipe_smem_bytes(E, dyn, pipe_helped(sim->dc, L));
     auto kern = pipe_kernel(sim->dc, L);
     // the limit is a property of the kernel, shared by every handle: the
     // largest any launch needs
