@@ -1096,7 +1096,8 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   __shared__ int ok_sh;
   __shared__ int greedy[kQtEnvs];
   __shared__ uint8_t act_sh[kQtEnvs];
-  __shared__ int scan_next;
+  __shared__ int scan_next, row_heavy, row_light;
+  __shared__ uint8_t row_list[kQtEnvs];
   __shared__ Env env_sh[kQtEnvs];                 // the tile's env states within a segment
   __shared__ unsigned long long akey_sh[kQtEnvs];  // their action-stream keys
   __shared__ float sb1[kHid], sb2[kHid], sb3[kOutPad];
@@ -1304,7 +1305,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       // the next input tile starts from zero (H2 is dead after the head)
       for (int i = tid; i < kQtEnvs * L.k1 / 8; i += kQtThreads)
         reinterpret_cast<uint4*>(hx)[i] = make_uint4(0u, 0u, 0u, 0u);
-      if (tid == 0) scan_next = 0;
+      if (tid == 0) scan_next = row_heavy = row_light = 0;
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
@@ -1324,18 +1325,34 @@ __global__ void __launch_bounds__(kQtThreads, 1)
         act_sh[tid] = (uint8_t)a;
         if (act_seq) act_seq[(long long)t * n + senv] = (uint8_t)a;
       }
+      const int rows = (int)min((long long)kQtEnvs, n - (long long)blk * kQtEnvs);
+      if (tid < kQtEnvs) {
+        // the rows in the order they are handed out: two-beam lanes and resets
+        // first, so that no long row is the last
+        const bool heavy = slive && ((rec[tid].nbk & 0xFFu) > 32u || (rec[tid].done & 7u));
+        const unsigned hm = __ballot_sync(kFull, heavy), lm = __ballot_sync(kFull, slive && !heavy);
+        const unsigned below = (1u << lane) - 1u;
+        int hb = 0, lb = 0;
+        if (lane == 0) {
+          hb = atomicAdd(&row_heavy, __popc(hm));
+          lb = atomicAdd(&row_light, __popc(lm));
+        }
+        hb = __shfl_sync(kFull, hb, 0) + __popc(hm & below);
+        lb = __shfl_sync(kFull, lb, 0) + __popc(lm & below);
+        if (slive) row_list[heavy ? hb : rows - 1 - lb] = (uint8_t)tid;
+      }
       // every record of the tile is written; the scans (one or two per env,
       // 16 to 64 beams) are handed out row by row through a shared counter,
       // so that no warp waits at the next step's barrier for a slow one
       __syncthreads();
       const long long slot_t = slot, slot_n = slot + 1 == rp.slots ? 0 : slot + 1;
       slot = (int)slot_n;
-      const int rows = (int)min((long long)kQtEnvs, n - (long long)blk * kQtEnvs);
       for (;;) {
         int e = 0;
         if (lane == 0) e = atomicAdd(&scan_next, 1);
         e = __shfl_sync(kFull, e, 0);
         if (e >= rows) break;
+        e = row_list[e];
         const MotionRec* r = rec + e;
         const uint4 w1 = rec_word<false>(r, 1), w3 = rec_word<false>(r, 3);
         const int ie = (int)w3.w;
