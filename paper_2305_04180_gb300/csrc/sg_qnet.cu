@@ -267,21 +267,27 @@ __device__ __forceinline__ void load_x16(uint32_t (&x)[4], const bf16* X, int ld
 // W^T + b)).  Bound by shared-memory reads: with the weights as the A operand
 // each is read once and the 16 rows once per warp (256 KB a layer of 256
 // inputs); with the rows as A and 8 units per warp and pass it was 384 KB.
+// kRows = 8: rows 0..7 only (the others keep what H holds): half of the MMAs.
+template <int kRows = 16>
 __device__ __forceinline__ void hidden_layer(const bf16* X, int ldx, int nks, const bf16* W, int ldw, const float* b,
-                                         bf16* H, int warp, int lane) {
+                                             bf16* H, int warp, int lane) {
+  constexpr int kNt = kRows / 8;
   const int g = lane >> 2, q = lane & 3, u0 = 16 * warp;
-  float c[2][4] = {};
+  float c[kNt][4] = {};
 #pragma unroll 4
   for (int ks = 0; ks < nks; ++ks) {
     uint32_t a[4], x[4];
     load_a_row(a, W, ldw, u0, 16 * ks, lane);
-    load_x16(x, X, ldx, 16 * ks, lane);
+    if (kNt == 2)
+      load_x16(x, X, ldx, 16 * ks, lane);
+    else
+      load_b_col(x[0], x[1], X, ldx, 16 * ks, 0, lane);
     mma_bf16(c[0], a, x[0], x[1]);
-    mma_bf16(c[1], a, x[2], x[3]);
+    if (kNt == 2) mma_bf16(c[kNt - 1], a, x[2], x[3]);
   }
   const float bl = b[u0 + g], bh = b[u0 + g + 8];
 #pragma unroll
-  for (int t = 0; t < 2; ++t)
+  for (int t = 0; t < kNt; ++t)
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       H[(8 * t + 2 * q + (j & 1)) * kLdh + u0 + g + (j >> 1) * 8] =
@@ -317,12 +323,13 @@ __device__ __forceinline__ void group_barrier(int id, int nthreads) {
 // The forward of one 16-row tile by a group of 16 warps that synchronise
 // among themselves on named barrier `bar` (0: the whole CTA is the group;
 // otherwise the other warps of the CTA run on); wg = the warp's index in its
-// group.
+// group.  kRows = 8: the rows from 8 on hold no sample.
+template <int kRows = 16>
 __device__ __forceinline__ void mlp_tile(const QW& w, const bf16* X, bf16* H1, bf16* H2, float* O, int wg, int lane,
                                          int bar = 0) {
-  hidden_layer(X, w.ld1, w.k1 / 16, w.W1, w.ld1, w.b1, H1, wg, lane);
+  hidden_layer<kRows>(X, w.ld1, w.k1 / 16, w.W1, w.ld1, w.b1, H1, wg, lane);
   group_barrier(bar, 512);
-  hidden_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, wg, lane);
+  hidden_layer<kRows>(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, wg, lane);
   group_barrier(bar, 512);
   if (wg == 0) head_layer(H2, w, O, lane);
   group_barrier(bar, 512);
@@ -422,11 +429,10 @@ static_assert(kTcRows * 80 * 2 + 1024 + kHid * 80 * 2 + kHid * kHid * 2 + 32 * 1
               "tcgen05 forward: operands exceed the shared memory");
 // The weight copy in global memory: blocks identical to their shared-memory
 // images, so that each is one bulk copy.
-// For the fused rollout also W1 in two 128-row halves and W2 in four
-// 64-row quarters, and for the batched forward W2 as one 256-row operand
-// (each its own canonical operand).
+// For the fused rollout W1 and W2 in two 128-row halves each, for the batched
+// forward and the learner as one 256-row operand each (all canonical operands).
 struct TcImg {
-  uint32_t w1, w2a, w2b, w3, w1h, w2q, w2f, bytes;
+  uint32_t w1, w2a, w2b, w3, w1h, w2f, bytes;
 };
 __host__ __device__ inline TcImg tc_img(int k1) {
   TcImg t;
@@ -435,8 +441,7 @@ __host__ __device__ inline TcImg tc_img(int k1) {
   t.w2b = t.w2a + 128u * kHid * 2u;
   t.w3 = t.w2b + 128u * kHid * 2u;
   t.w1h = t.w3 + 16u * kHid * 2u;
-  t.w2q = t.w1h + (uint32_t)(kHid * k1 * 2);
-  t.w2f = t.w2q + (uint32_t)(kHid * kHid * 2);
+  t.w2f = t.w1h + (uint32_t)(kHid * k1 * 2);
   t.bytes = t.w2f + (uint32_t)(kHid * kHid * 2);
   return t;
 }
@@ -461,9 +466,7 @@ __global__ void k_tc_image(const uint8_t* __restrict__ img, ImgLayout L, uint8_t
       const int j = c - n1, n = j % kHid, kg = j / kHid;
       v = __ldg(reinterpret_cast<const uint4*>(img + L.w2 + ((size_t)n * kLdh + kg * 8) * 2));
       dst = n < 128 ? T.w2a + kmajor_offset(n, kg * 8, 128) : T.w2b + kmajor_offset(n - 128, kg * 8, 128);
-      // in its 64-row quarter and in the 256-row operand
-      *reinterpret_cast<uint4*>(out + T.w2q + (uint32_t)((n >> 6) * 64 * kHid * 2) +
-                                kmajor_offset(n & 63, kg * 8, 64)) = v;
+      // in the 256-row operand
       *reinterpret_cast<uint4*>(out + T.w2f + kmajor_offset(n, kg * 8, kHid)) = v;
     } else {
       const int j = c - n1 - n2, n = j % 16, kg = j / 16;
@@ -871,7 +874,10 @@ __global__ void __launch_bounds__(512 * MT, 1)
   for (int i = 0; i < K; ++i) {
     if (live) obs_to_tile(Xg + wg * L.ld1, o, c.B, lane);
     group_barrier(bar, 512);
-    mlp_tile(w, Xg, H1g, H2g, Og, wg, lane, bar);
+    if (MT == 1 && epc <= 8)
+      mlp_tile<8>(w, Xg, H1g, H2g, Og, wg, lane, bar);
+    else
+      mlp_tile(w, Xg, H1g, H2g, Og, wg, lane, bar);
     if (!live) continue;
     if ((i & 31) == 0) {
       // lane l draws the random action and the exploration uniform of step t + l
@@ -1758,7 +1764,6 @@ __device__ __forceinline__ void upd_image(uint8_t* img, uint8_t* tc, const ImgLa
   } else if (kW == 2) {
     put(img + L.w2 + (r * kLdh + k) * 2);
     put(tc + (r < 128 ? T.w2a : T.w2b) + kmajor_offset(r & 127, k, 128));
-    put(tc + T.w2q + (uint32_t)((r >> 6) * 64 * kHid * 2) + kmajor_offset(r & 63, k, 64));
     put(tc + T.w2f + kmajor_offset(r, k, kHid));
   } else {
     put(img + L.w3 + (r * kLdh + k) * 2);
