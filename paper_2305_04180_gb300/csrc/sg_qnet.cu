@@ -259,6 +259,10 @@ __device__ __forceinline__ QW qw_at(const uint8_t* base, const ImgLayout& L) {
   return w;
 }
 
+__device__ __forceinline__ void group_barrier(int id, int nthreads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
+}
+
 // B fragments of k-step k0 of 16 samples X[16][ldx] (two n-tiles of 8).
 __device__ __forceinline__ void load_x16(uint32_t (&x)[4], const bf16* X, int ldx, int k0, int lane) {
   ldsm_x4(x, X + ((lane & 7) + (lane >> 4) * 8) * ldx + k0 + ((lane >> 3) & 1) * 8);
@@ -268,9 +272,11 @@ __device__ __forceinline__ void load_x16(uint32_t (&x)[4], const bf16* X, int ld
 // each is read once and the 16 rows once per warp (256 KB a layer of 256
 // inputs); with the rows as A and 8 units per warp and pass it was 384 KB.
 // kRows = 8: rows 0..7 only (the others keep what H holds): half of the MMAs.
+// With bar >= 0 H may be X: the 16 warps meet on that named barrier between
+// their last read and their stores.
 template <int kRows = 16>
 __device__ __forceinline__ void hidden_layer(const bf16* X, int ldx, int nks, const bf16* W, int ldw, const float* b,
-                                             bf16* H, int warp, int lane) {
+                                             bf16* H, int warp, int lane, int bar = -1) {
   constexpr int kNt = kRows / 8;
   const int g = lane >> 2, q = lane & 3, u0 = 16 * warp;
   float c[kNt][4] = {};
@@ -286,6 +292,7 @@ __device__ __forceinline__ void hidden_layer(const bf16* X, int ldx, int nks, co
     if (kNt == 2) mma_bf16(c[kNt - 1], a, x[2], x[3]);
   }
   const float bl = b[u0 + g], bh = b[u0 + g + 8];
+  if (bar >= 0) group_barrier(bar, 512);
 #pragma unroll
   for (int t = 0; t < kNt; ++t)
 #pragma unroll
@@ -316,20 +323,16 @@ __device__ __forceinline__ void head_layer(const bf16* H2, const QW& w, float* O
   O[(g + 8) * kOutPad + n + 1] = (acc0[3] + acc1[3]) + w.b3[n + 1];
 }
 
-__device__ __forceinline__ void group_barrier(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
-}
-
 // The forward of one 16-row tile by a group of 16 warps that synchronise
 // among themselves on named barrier `bar` (0: the whole CTA is the group;
 // otherwise the other warps of the CTA run on); wg = the warp's index in its
-// group.  kRows = 8: the rows from 8 on hold no sample.
+// group.  kRows = 8: the rows from 8 on hold no sample.  H2 may be H1.
 template <int kRows = 16>
 __device__ __forceinline__ void mlp_tile(const QW& w, const bf16* X, bf16* H1, bf16* H2, float* O, int wg, int lane,
                                          int bar = 0) {
   hidden_layer<kRows>(X, w.ld1, w.k1 / 16, w.W1, w.ld1, w.b1, H1, wg, lane);
   group_barrier(bar, 512);
-  hidden_layer<kRows>(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, wg, lane);
+  hidden_layer<kRows>(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, wg, lane, H2 == H1 ? bar : -1);
   group_barrier(bar, 512);
   if (wg == 0) head_layer(H2, w, O, lane);
   group_barrier(bar, 512);
@@ -812,8 +815,9 @@ __global__ void __launch_bounds__(512 * MT, 1)
   bf16* X = reinterpret_cast<bf16*>(smem + L.bytes);
   constexpr int kRows = 16 * MT;
   bf16* H1 = X + kRows * L.ld1;
-  bf16* H2 = H1 + kRows * kLdh;
-  float* O = reinterpret_cast<float*>(H2 + kRows * kLdh);
+  // layer 2 over layer 1: at most 48 (padded) inputs then fit 196 KB of shared
+  // memory with 32 envs, which leaves the scans 60 KB of L1 instead of 28
+  float* O = reinterpret_cast<float*>(H1 + kRows * kLdh);
   __shared__ uint64_t bar_img;
   if (threadIdx.x == 0) {
     // the weights on their way while the envs take their first observation
@@ -826,7 +830,6 @@ __global__ void __launch_bounds__(512 * MT, 1)
   const int grp = warp >> 4, wg = warp & 15, bar = 1 + grp;
   bf16* Xg = X + grp * 16 * L.ld1;
   bf16* H1g = H1 + grp * 16 * kLdh;
-  bf16* H2g = H2 + grp * 16 * kLdh;
   float* Og = O + grp * 16 * kOutPad;
   // CTAs take envs grouped by map, so that one CTA's scans share cache lines;
   // epc <= kRows envs per CTA (fewer than the tile when that spreads the
@@ -875,9 +878,9 @@ __global__ void __launch_bounds__(512 * MT, 1)
     if (live) obs_to_tile(Xg + wg * L.ld1, o, c.B, lane);
     group_barrier(bar, 512);
     if (MT == 1 && epc <= 8)
-      mlp_tile<8>(w, Xg, H1g, H2g, Og, wg, lane, bar);
+      mlp_tile<8>(w, Xg, H1g, H1g, Og, wg, lane, bar);
     else
-      mlp_tile(w, Xg, H1g, H2g, Og, wg, lane, bar);
+      mlp_tile(w, Xg, H1g, H1g, Og, wg, lane, bar);
     if (!live) continue;
     if ((i & 31) == 0) {
       // lane l draws the random action and the exploration uniform of step t + l
@@ -2973,6 +2976,8 @@ namespace {
 size_t fwd_smem(const ImgLayout& L, int rows = kTile) {
   return (size_t)L.bytes + (size_t)rows * L.ld1 * 2 + 2ull * rows * kLdh * 2 + (size_t)rows * kOutPad * 4;
 }
+// The fused rollout's: one activation buffer.
+size_t roll_smem(const ImgLayout& L, int rows) { return fwd_smem(L, rows) - (size_t)rows * kLdh * 2; }
 size_t grad_smem(const ImgLayout& L) {
   return (size_t)L.bytes + (size_t)kTile * L.ld1 * 2 + 3ull * kTile * kLdh * 2 + 2ull * kTile * kOutPad * 4;
 }
@@ -3084,14 +3089,14 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   if ((rc = set_smem_attr((const void*)k_qnet_forward_tc, kTcSmemLaunch)) ||
       (rc = set_smem_attr((const void*)k_rollout_q_tc<false>, qt_smem().bytes)) ||
       (rc = set_smem_attr((const void*)k_rollout_q_tc<true>, qt_smem().bytes)) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<1, false, false>, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<1, false, true>, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<2, false, false>, fwd_smem(widest, 32))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<2, false, true>, fwd_smem(widest, 32))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<1, true, false>, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<1, true, true>, fwd_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<2, true, false>, fwd_smem(widest, 32))) ||
-      (rc = set_smem_attr((const void*)k_rollout_q<2, true, true>, fwd_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, false, false>, roll_smem(widest, 16))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, false, true>, roll_smem(widest, 16))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, false, false>, roll_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, false, true>, roll_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, true, false>, roll_smem(widest, 16))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<1, true, true>, roll_smem(widest, 16))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, true, false>, roll_smem(widest, 32))) ||
+      (rc = set_smem_attr((const void*)k_rollout_q<2, true, true>, roll_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_td_tile, grad_smem(widest))) ||
       (rc = set_smem_attr((const void*)k_td_tc, lt_smem(80).bytes)) ||
       (rc = set_smem_attr((const void*)k_td_update_split, kSplitSmem))) {
@@ -3451,7 +3456,7 @@ int sg_rollout_eps_q(sg_sim* sim, int K, sg_qnet* q, const float* eps, sg_replay
                                : (fast ? k_rollout_q<2, false, true> : k_rollout_q<2, false, false>))
                         : (dyn ? (fast ? k_rollout_q<1, true, true> : k_rollout_q<1, true, false>)
                                : (fast ? k_rollout_q<1, false, true> : k_rollout_q<1, false, false>));
-    kern<<<grid, 512 * mt, fwd_smem(q->IL, rows), stream>>>(sim->dc, sg_sim_ptrs(sim), q->img, q->IL, K, eps, rd,
+    kern<<<grid, 512 * mt, roll_smem(q->IL, rows), stream>>>(sim->dc, sg_sim_ptrs(sim), q->img, q->IL, K, eps, rd,
                                                             rp ? 1 : 0, sim->map_order_dev, epc, obs, obs_seq, act_seq,
                                                             rew_seq, done_seq);
   }
