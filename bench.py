@@ -477,8 +477,8 @@ def run_extras(flush, which, l2_read=None):
         ft()
     ms_t = _time_cuda(ft, 20, flush)
     out["td_train_step"] = {"batch": w.extra["batch"], "ms": ms_t, "samples_per_s": w.extra["batch"] / (ms_t / 1e3),
-                            "gpu_launches_per_call": 5, "loss": float(loss.item()),
-                            "kernel": "k_td_target + k_td_grad (16-sample mma.sync tiles) + k_adam"}
+                            "gpu_launches_per_call": 2, "loss": float(loss.item()),
+                            "kernel": "k_td_tile (16-sample mma.sync tiles) + k_td_update"}
     # the learned loop's batch, 4,096: the tcgen05 learner (k_td_tc).  FLOPs
     # per sample of the step's definition: three forwards (online and target
     # on s', online on s) and the backward (dW1, dW2, dW3, dH1, dH2)
@@ -492,7 +492,7 @@ def run_extras(flush, which, l2_read=None):
     bwd = 2.0 * (256 * n_in + 256 * 256 + 256 * 256 + 6 * 256 + 6 * 256)
     flop = 4096 * (3 * fwd + bwd)
     out["td_train_step_4096"] = {"batch": 4096, "ms": ms_t4, "samples_per_s": 4096 / (ms_t4 / 1e3),
-                                 "kernel": "k_td_tc (tcgen05, 128-sample tiles) + k_adam",
+                                 "kernel": "k_td_tc (tcgen05, 128-sample tiles) + k_td_update_split",
                                  "roofline": {"bound": "tensor", "achieved": flop / (ms_t4 / 1e3) / 1e12,
                                               "peak": peak_tf, "unit": "TFLOP/s",
                                               "frac": flop / (ms_t4 / 1e3) / 1e12 / peak_tf,

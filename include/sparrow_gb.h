@@ -247,7 +247,9 @@ int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t qnet, cons
  *                     after each episode end) and then joins obs_warps
  *                     (1..15) warps that compute the scans, observations and
  *                     rewards of the previous chunk, taking steps from a
- *                     shared counter; min(3, max(1, warps_per_block /
+ *                     shared counter (with one env per CTA and 15 of them,
+ *                     or 7 with moving obstacles, the first helps the pose
+ *                     warp instead, which then takes no scans); min(3, max(1, warps_per_block /
  *                     (1 + obs_warps))) envs per CTA, warps_per_block 1..16;
  *                     order 0 = index order, 1 = envs grouped by map (CTAs
  *                     share maps, so fewer maps compete for each SM's L1).
@@ -417,13 +419,15 @@ int sg_qnet_set_rollout_rows(sg_qnet_t q, int32_t rows);
 
 /*
  * At most rollout_ctas CTAs (one per SM) for the tcgen05 fused rollout run
- * with this network, and at most learner_ctas for its tcgen05 TD step (0 =
- * every SM, the default; negative: SG_E_INVAL).  The ASL framework runs the
+ * with this network, and at most learner_ctas (rounded to whole clusters of
+ * three, one at least) for the tile kernel of its TD step (0 = every SM, the
+ * default; negative: SG_E_INVAL).  The ASL framework runs the
  * actor and the learner in parallel (Sec. 3.1, Alg. 1 and 2): a rollout and
  * a learning step launched on concurrent streams (or graph branches) with
  * caps that add up to the SM count each keep SMs of their own instead of
- * taking turns.  Results do not depend on the caps (the rollout's items and
- * the learner's jobs are taken from device counters by whichever CTAs run).
+ * taking turns.  Results do not depend on the caps (the rollout's items are
+ * taken from a device counter by whichever CTAs run, the learner's clusters
+ * loop over its tiles).
  */
 int sg_qnet_set_grid_limit(sg_qnet_t q, int32_t rollout_ctas, int32_t learner_ctas);
 

@@ -939,33 +939,32 @@ __global__ void __launch_bounds__(512 * MT, 1)
 // and ring entries.  Same VEM draws, same simulator values as k_rollout_q; the Q
 // values differ from it only in the summation order.
 //
-// Shared memory is kept small (136 KB) so that L1 keeps room for the maps the
-// scans read: the input tile (at most 20 KB) and the step records (10 KB,
-// from byte 32 K) live inside the hidden-activation buffer, which holds H1
-// and H2 during the network only, and all of W1 (two 128-row halves) and W2
-// (four 32 KB pieces: the K halves of its two 128-row halves) stream through
-// two 32 KB buffers by bulk copies
-// every step, each copy issued as soon as its buffer's previous MMAs are
+// Shared memory is kept small (102 KB) so that L1 keeps room for the maps the
+// scans read: the hidden activations stay in tensor memory (an epilogue packs
+// its BF16 pairs into the first half of the columns it read, the next layer's A
+// operand; layer 1 in columns [0, 256), layer 2 in [256, 512), the head in
+// [16, 32); in shared memory, 136 KB, 65,536 envs x 32 steps took 3,566 us against
+// 3,518), and all of W1 (two 128-row halves) and W2 (four 32 KB pieces: the K
+// halves of its two 128-row halves) stream through two 32 KB buffers by bulk
+// copies every step, each copy issued as soon as its buffer's previous MMAs are
 // done (both W1 halves during the env steps, the first two W2 pieces during
 // the layer-1 epilogue); W3 stays.
 constexpr int kQtEnvs = 128;
 constexpr int kQtWarps = 32;
 constexpr int kQtThreads = kQtWarps * 32;
 constexpr uint32_t kQtBuf = 32u * 1024u;
-constexpr uint32_t kQtRecOff = 32u * 1024u;
+constexpr uint32_t kQtRecOff = (uint32_t)(kQtEnvs * 80 * 2);  // step records behind the input tile (k1 <= 80)
 // The env steps of a tile: what every env takes, one env per lane of the first
 // four warps (lane_motion); the bit-row collision test and AutoReset, which
 // few take, go with the scans, a warp per row.  With 16 warps of 8 lanes doing
 // the whole scalar step, 65,536 envs x 32 steps took 4,112 us (3,664 now).
-static_assert(kQtRecOff + kQtEnvs * sizeof(MotionRec) <= (uint32_t)(kQtEnvs * kHid * 2), "records fit the activation buffer");
-
 struct QtSmem {
   uint32_t hx, b0, b1, w3, bytes;
 };
 __host__ __device__ inline QtSmem qt_smem() {
   QtSmem t;
   t.hx = 0;
-  t.b0 = (uint32_t)(kQtEnvs * kHid * 2);
+  t.b0 = kQtRecOff + kQtEnvs * (uint32_t)sizeof(MotionRec);
   t.b1 = t.b0 + kQtBuf;
   t.w3 = t.b1 + kQtBuf;
   t.bytes = t.w3 + 16u * kHid * 2u;
@@ -973,22 +972,23 @@ __host__ __device__ inline QtSmem qt_smem() {
 }
 
 // Epilogue of a hidden layer by 32 warps: warp w takes the rows of lane
-// quarter w % 4 and columns [32 (w / 4), + 32).
-__device__ __forceinline__ void qt_epilogue(uint32_t tacc, const float* bias, uint8_t* hs, int warp, int lane) {
-  const int quarter = warp & 3, r = quarter * 32 + lane, c = (warp >> 2) * 32;
+// quarter w % 4 and columns [32 (w / 4), + 32) of the accumulators at tacc and
+// packs them into the first 16 of these columns.
+__device__ __forceinline__ void qt_epilogue(uint32_t tacc, const float* bias, int warp) {
+  const int c = (warp >> 2) * 32;
+  const uint32_t t = tacc + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c;
   float v[32];
-  tmem_ld32(tacc + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+  tmem_ld32(t, v);
+  uint32_t w[16];
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int k = c + 8 * g + 2 * j;
-      w[j] = pack_bf16x2(fmaxf(v[8 * g + 2 * j] + bias[k], 0.f), fmaxf(v[8 * g + 2 * j + 1] + bias[k + 1], 0.f));
-    }
-    *reinterpret_cast<uint4*>(hs + kmajor_offset(r, c + 8 * g, kQtEnvs)) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
+  for (int j = 0; j < 16; ++j)
+    w[j] = pack_bf16x2(fmaxf(v[2 * j] + bias[c + 2 * j], 0.f), fmaxf(v[2 * j + 1] + bias[c + 2 * j + 1], 0.f));
+  tmem_st16(t, w);
+  tmem_st_wait();
 }
+// Column (relative to the layer's accumulators) of K step ks of the packed
+// activations.
+__device__ __forceinline__ uint32_t qt_a_col(int ks) { return (uint32_t)((ks >> 1) * 32 + (ks & 1) * 8); }
 
 // This lane's share of an observation row into row r of the BF16 input tile.
 __device__ __forceinline__ void qt_obs_to_tile(uint8_t* xs, int r, float b0, float b1, float ex, int B, int lane) {
@@ -1021,11 +1021,11 @@ struct QtStream {
     bulk_g2s(buf[b], src, bytes, &ld[b]);
     ld_out[b] = true;
   }
-  // MMAs D[tacc] (+)= A x buffer b^T (Rb rows, K; A from its K step ks0,
-  // onto D when acc), then commits: the buffer's barrier, and the layer
-  // barrier when `last`
-  __device__ __forceinline__ void mma(int b, uint32_t tacc, const uint8_t* a, int Rb, int K, uint64_t* layer,
-                                      bool last, int ks0 = 0, bool acc = false) {
+  // MMAs D[tacc] (+)= A x buffer b^T (Rb rows, K; A in shared memory, or packed
+  // in tensor memory at ta from its K step ks0; onto D when acc), then commits:
+  // the buffer's barrier, and the layer barrier when `last`
+  __device__ __forceinline__ void mma(int b, uint32_t tacc, const uint8_t* a, uint32_t ta, int Rb, int K,
+                                      uint64_t* layer, bool last, int ks0 = 0, bool acc = false) {
     if (!ok) return;
     if (ld_out[b]) {
       ok = mbar_wait(&ld[b], pl[b], kTcTries);
@@ -1035,11 +1035,15 @@ struct QtStream {
     }
     tc_fence_after();
     const uint32_t idesc = idesc_bf16_f32(kQtEnvs, Rb);
-    const uint32_t sa = smem_u32(a), sb = smem_u32(buf[b]);
+    const uint32_t sb = smem_u32(buf[b]);
     const uint32_t la = kQtEnvs * 16, lb = (uint32_t)Rb * 16;
-    for (int ks = 0; ks < K / 16; ++ks)
-      tc_mma_bf16(tacc, smem_desc(sa + (uint32_t)(ks0 + ks) * 2 * la, la, 128),
-                  smem_desc(sb + (uint32_t)ks * 2 * lb, lb, 128), idesc, (acc || ks > 0) ? 1u : 0u);
+    for (int ks = 0; ks < K / 16; ++ks) {
+      const uint64_t db = smem_desc(sb + (uint32_t)ks * 2 * lb, lb, 128);
+      if (a)
+        tc_mma_bf16(tacc, smem_desc(smem_u32(a) + (uint32_t)ks * 2 * la, la, 128), db, idesc, ks > 0 ? 1u : 0u);
+      else
+        tc_mma_bf16_ta(tacc, ta + qt_a_col(ks0 + ks), db, idesc, (acc || ks > 0) ? 1u : 0u);
+    }
     tc_commit(&mm[b]);
     mm_out[b] = true;
     if (last) tc_commit(layer);
@@ -1112,9 +1116,9 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   __shared__ float sb1[kHid], sb2[kHid], sb3[kOutPad];
   const QtSmem T = qt_smem();
   const TcImg G = tc_img(L.k1);
-  uint8_t* hx = tsm + T.hx;  // the input tile, then H1, then H2
+  uint8_t* hx = tsm + T.hx;  // the input tile
   uint8_t* w3s = tsm + T.w3;
-  MotionRec* rec = reinterpret_cast<MotionRec*>(tsm + T.hx + kQtRecOff);  // during the env steps only
+  MotionRec* rec = reinterpret_cast<MotionRec*>(tsm + T.hx + kQtRecOff);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long n = c.n_envs;
   const int nblk = (int)((n + kQtEnvs - 1) / kQtEnvs);
@@ -1129,7 +1133,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   if (tid < kOutPad) sb3[tid] = __ldg(reinterpret_cast<const float*>(img + L.b3) + tid);
   for (int i = tid; i < (int)(16u * kHid * 2u / 16u); i += kQtThreads)
     reinterpret_cast<uint4*>(w3s)[i] = __ldg(reinterpret_cast<const uint4*>(timg + G.w3) + i);
-  if (warp == 0) tmem_alloc(&tslot, 256);
+  if (warp == 0) tmem_alloc(&tslot, 512);
   if (tid == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_ld[b], 1);
@@ -1142,7 +1146,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tacc = tslot;
+  const uint32_t tacc = tslot, tacc2 = tacc + 256u;
   QtStream S;  // meaningful in thread 0
   S.ld = bar_ld;
   S.mm = bar_mm;
@@ -1238,8 +1242,8 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       if (tid == 0) {
         if (!S.ld_out[0]) S.load(0, timg + G.w1h, w1h_bytes);
         if (!S.ld_out[1]) S.load(1, timg + G.w1h + w1h_bytes, w1h_bytes);
-        S.mma(0, tacc, hx, 128, L.k1, &bar_layer, false);
-        S.mma(1, tacc + 128u, hx, 128, L.k1, &bar_layer, true);
+        S.mma(0, tacc, hx, 0u, 128, L.k1, &bar_layer, false);
+        S.mma(1, tacc + 128u, hx, 0u, 128, L.k1, &bar_layer, true);
         S.load(0, timg + G.w2a, w2q_bytes);
         S.load(1, timg + G.w2a + w2q_bytes, w2q_bytes);
         if (!S.ok) ok_sh = 0;
@@ -1251,8 +1255,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       player ^= 1u;
       layer_out = false;
       tc_fence_after();
-      qt_epilogue(tacc, sb1, hx, warp, lane);  // H1 over the input tile
-      fence_async_smem();
+      qt_epilogue(tacc, sb1, warp);
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
@@ -1261,12 +1264,12 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       // of its rows through the buffers (piece c: K steps 8 c .. 8 c + 7);
       // the second half's pieces are both in flight before either is needed
       if (tid == 0) {
-        S.mma(0, tacc, hx, 128, kHid / 2, &bar_layer, false, 0, false);
-        S.mma(1, tacc, hx, 128, kHid / 2, &bar_layer, false, 8, true);
+        S.mma(0, tacc2, nullptr, tacc, 128, kHid / 2, &bar_layer, false, 0, false);
+        S.mma(1, tacc2, nullptr, tacc, 128, kHid / 2, &bar_layer, false, 8, true);
         S.load(0, timg + G.w2b, w2q_bytes);
         S.load(1, timg + G.w2b + w2q_bytes, w2q_bytes);
-        S.mma(0, tacc + 128u, hx, 128, kHid / 2, &bar_layer, false, 0, false);
-        S.mma(1, tacc + 128u, hx, 128, kHid / 2, &bar_layer, true, 8, true);
+        S.mma(0, tacc2 + 128u, nullptr, tacc, 128, kHid / 2, &bar_layer, false, 0, false);
+        S.mma(1, tacc2 + 128u, nullptr, tacc, 128, kHid / 2, &bar_layer, true, 8, true);
         if (!S.ok) ok_sh = 0;
       }
       layer_out = true;
@@ -1276,8 +1279,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       player ^= 1u;
       layer_out = false;
       tc_fence_after();
-      qt_epilogue(tacc, sb2, hx, warp, lane);  // H2 over H1 (layer 2 is complete)
-      fence_async_smem();
+      qt_epilogue(tacc2, sb2, warp);
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
@@ -1285,10 +1287,10 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       if (tid == 0) {
         tc_fence_after();
         const uint32_t idesc = idesc_bf16_f32(kQtEnvs, 16);
-        const uint32_t sa = smem_u32(hx), sw = smem_u32(w3s);
+        const uint32_t sw = smem_u32(w3s);
         for (int ks = 0; ks < kHid / 16; ++ks)
-          tc_mma_bf16(tacc, smem_desc(sa + (uint32_t)ks * 2 * (kQtEnvs * 16), kQtEnvs * 16, 128),
-                      smem_desc(sw + (uint32_t)ks * 2 * 256, 256, 128), idesc, ks > 0 ? 1u : 0u);
+          tc_mma_bf16_ta(tacc + 16u, tacc2 + qt_a_col(ks), smem_desc(sw + (uint32_t)ks * 2 * 256, 256, 128), idesc,
+                         ks > 0 ? 1u : 0u);
         tc_commit(&bar_layer);
         if (t + 1 < s1) {
           S.load(0, timg + G.w1h, w1h_bytes);
@@ -1305,13 +1307,13 @@ __global__ void __launch_bounds__(kQtThreads, 1)
       if (warp < 4) {
         float v[32];
         tc_fence_after();
-        tmem_ld32(tacc + ((uint32_t)(warp * 32) << 16), v);
+        tmem_ld32(tacc + 16u + ((uint32_t)(warp * 32) << 16), v);
         float o[kOut];
 #pragma unroll
         for (int j = 0; j < kOut; ++j) o[j] = v[j] + sb3[j];
         greedy[warp * 32 + lane] = (int)greedy_action(o, nullptr, L.plain);
       }
-      // the next input tile starts from zero (H2 is dead after the head)
+      // the next input tile starts from zero
       for (int i = tid; i < kQtEnvs * L.k1 / 8; i += kQtThreads)
         reinterpret_cast<uint4*>(hx)[i] = make_uint4(0u, 0u, 0u, 0u);
       if (tid == 0) scan_next = row_heavy = row_light = 0;
@@ -1436,7 +1438,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 0) tmem_free(tacc, 256);
+  if (warp == 0) tmem_free(tacc, 512);
   if (tid == 0) replay_advance(rp, use_replay, K);
 }
 
@@ -1444,7 +1446,7 @@ __global__ void __launch_bounds__(kQtThreads, 1)
 // Why a TD step produced no update (bits of a device word cleared at the
 // start of every step): a weight-image copy did not complete within its
 // bounded wait, or a sample's action index is outside the action table.
-// k_adam then writes NaN loss and gradient and leaves the parameters, the
+// The update then writes NaN loss and gradient and leaves the parameters, the
 // Adam moments and the image untouched; the step count does not advance.
 constexpr unsigned kTdFailCopy = 1u;
 constexpr unsigned kTdFailAction = 2u;
@@ -1516,7 +1518,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) mbar_init(&bar_img, 1);
   __syncthreads();
   if (!stage_image_bulk(sw, img, L.bytes, &bar_img, 0u, kTcTries)) {
-    // the image copy did not complete: no update this step (k_adam reads the
+    // the image copy did not complete: no gradient (k_grad_sum reads the
     // flag); one more bounded wait for the copy before the CTA exits
     if (threadIdx.x == 0) {
       atomicOr(fail, kTdFailCopy);
