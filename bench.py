@@ -432,7 +432,7 @@ def run_extras(flush, which, l2_read=None):
         "plain_rollout_same_workload": sim.n * Kq / (ms_r / 1e3),
         "fused_over_plain": ms_r / ms_q,
         "replay": f"{rp.capacity} transitions, 302 B each, appended every step",
-        "gpu_launches_per_call": 2,
+        "gpu_launches_per_call": 1,
     }
     # Q-value accuracy of the tensor-core forward against a float64 torch CPU forward
     th = q.get_params()
