@@ -785,15 +785,25 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_qnet_forward_tc(const uint8_t
 
 // One thread of every CTA of a rollout, after the CTA's last use of the ring's
 // step counter: the last CTA advances it by the K steps recorded and leaves
-// the CTA count (behind it) zero for the next launch.
+// the CTA count (behind it) zero for the next launch.  A learner on another
+// stream may read the counter at any moment (ring_steps): every CTA's entries
+// are ordered before the count, and the counts before the new value.
 __device__ __forceinline__ void replay_advance(const ReplayDev& rp, int use_replay, int K) {
   if (!use_replay) return;
   unsigned* done = reinterpret_cast<unsigned*>(rp.steps + 1);
   __threadfence();
   if (atomicAdd(done, 1u) == gridDim.x - 1u) {
+    __threadfence();
     *done = 0u;
     *rp.steps += (unsigned long long)K;
   }
+}
+// The counter as a learner reads it: the entries that it counts are visible
+// after this load.
+__device__ __forceinline__ unsigned long long ring_steps(const ReplayDev& rp) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(rp.steps) : "memory");
+  return v;
 }
 
 // VEM eps-greedy rollout with the network fused in: per step, the 16 envs of
@@ -1459,17 +1469,20 @@ __device__ __forceinline__ unsigned long long mod_inv(unsigned long long x, unsi
   if (r >= d) r -= d;
   return r;
 }
-// Ring entry of sample i of optimiser step `tstep` with st = *rp.steps: uniform over the
+// The draw of sample i of optimiser step `tstep`.
+__device__ __forceinline__ uint64_t sample_hash(unsigned long long seed, unsigned long long tstep, int i) {
+  return sm_at(sm_at(sm_at(sm_at(seed, kStreamSample), tstep), (uint64_t)i), 0ull);
+}
+// Ring entry of a sample with draw h and st steps recorded: uniform over the
 // V = min(steps, slots - reserve) most recently completed slots, so that a
 // rollout running concurrently (which writes the next slots) is never read.
 // With j = h mod (V n_envs): slot = (steps - 1 - j / n_envs) mod slots,
-// env = j mod n_envs.
-__device__ __forceinline__ long long sample_entry(unsigned long long seed, unsigned long long tstep,
-                                                  unsigned long long st, int i, const ReplayDev& rp) {
+// env = j mod n_envs.  Whoever reads parts of one sample uses one value of st
+// (share_steps): the counter may change between two loads.
+__device__ __forceinline__ long long sample_entry(uint64_t h, unsigned long long st, const ReplayDev& rp) {
   const unsigned long long usable = (unsigned long long)(rp.slots - rp.reserve);
   const unsigned long long V = st < usable ? st : usable;
   if (V == 0) return -1;
-  const uint64_t h = sm_at(sm_at(sm_at(sm_at(seed, kStreamSample), tstep), (uint64_t)i), 0ull);
   // the ring holds at most 2^31 entries, so j and its quotient fit 32 bits;
   // back < V <= slots, so one correction replaces the modulo of the difference
   const uint32_t n = (uint32_t)rp.n_envs;
@@ -1893,6 +1906,28 @@ __device__ __forceinline__ void st_cluster(float* p, uint32_t rank, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
 }
 
+// One reading of the ring's step counter for a learner's cluster, into every
+// CTA's slot: the CTAs gather s and s' of the same samples, and a rollout on
+// another stream may advance the counter between two loads.  Every thread of
+// the cluster, after its cluster_arrive() at the start.  The draws and the
+// weight copies go ahead of it; against a load in every CTA, batch 256 took
+// 14.6 -> 15.3 us.
+__device__ __forceinline__ unsigned long long share_steps(unsigned long long* slot, const ReplayDev& rp, uint32_t rank,
+                                                          int ranks) {
+  const bool reader = rank == 0 && threadIdx.x == 0;
+  const unsigned long long st = reader ? ring_steps(rp) : 0ull;
+  cluster_wait();  // every CTA of the cluster has started: remote stores from here on
+  if (reader)
+    for (int r = 0; r < ranks; ++r) {
+      uint32_t a;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(slot)), "r"(r));
+      asm volatile("st.shared::cluster.u64 [%0], %1;\n" ::"r"(a), "l"(st) : "memory");
+    }
+  cluster_arrive();
+  cluster_wait();
+  return *slot;
+}
+
 // dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
 __device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
   const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
@@ -1915,6 +1950,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ float next_q[2][2][kTile * kOutPad];  // rank 0: head outputs of s' by tile parity and network
   __shared__ int rows[kTile];
   __shared__ float hub[kTile];
+  __shared__ unsigned long long steps_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = lane & 3, g = lane >> 2;
   const uint32_t rank = cluster_rank();
@@ -1926,7 +1962,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   }
   pdl_wait();
   pdl_launch_dependents();
-  const unsigned long long tstep = __ldcg(step), st = __ldcg(rp.steps);
+  const unsigned long long tstep = __ldcg(step);
   if (tid == kThreads - 1) {
     // layer 1 starts when W1 and the vectors behind W2 are here
     const uint8_t* src = rank == 2 ? img_t : img;
@@ -1940,10 +1976,14 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   __syncthreads();
   const QW w = qw_at(sw, L);
   bool ok = true, first = true;
-  for (int tile = (int)blockIdx.x / kTpRanks, it = 0; tile < ntiles; tile += stride, ++it) {
+  int tile = (int)blockIdx.x / kTpRanks;
+  uint64_t h = sample_hash(seed, tstep, tile * kTile + warp);
+  const unsigned long long st = share_steps(&steps_sh, rp, rank, kTpRanks);
+  for (int it = 0; tile < ntiles; tile += stride, ++it) {
     {
       const int i = tile * kTile + warp;
-      const int e = i < batch ? (int)sample_entry(seed, tstep, st, i, rp) : -1;
+      if (it > 0) h = sample_hash(seed, tstep, i);
+      const int e = i < batch ? (int)sample_entry(h, st, rp) : -1;
       const float* src = (rank == 0 ? rp.s : rp.s2) + (long long)e * rp.obs_dim;
       for (int k = lane; k < L.ld1; k += 32)
         X[warp * L.ld1 + k] = __float2bfloat16_rn(e >= 0 && k < rp.obs_dim ? src[k] : 0.0f);
@@ -1968,7 +2008,6 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     __syncthreads();
     if (ok && warp == 0) head_layer(H2, w, O, lane);
     __syncthreads();
-    if (it == 0) cluster_wait();  // the start's arrival
     if (rank != 0 && tid < kTile * kOutPad)
       st_cluster(&next_q[it & 1][rank - 1][tid], 0u, ok ? O[tid] : __int_as_float(0x7fc00000));
     cluster_arrive();
@@ -2637,6 +2676,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ uint32_t tslot;
   __shared__ int rows_sh[kLtRows];
   __shared__ float dsum_sh[4][kOutPad];
+  __shared__ unsigned long long steps_sh;
   const LtSmem T = lt_smem(L.k1);
   const TcImg G = tc_img(L.k1);
   uint8_t* xs = tsm + T.x;
@@ -2660,7 +2700,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   }
   pdl_wait();
   pdl_launch_dependents();
-  const unsigned long long tstep = __ldcg(step), st = __ldcg(rp.steps);
+  const unsigned long long tstep = __ldcg(step);
   if (tid == kThreads - 1) {
     const uint8_t* src = rank == 2 ? timg_t : timg;
     mbar_expect_tx(&bar_w1, G.w2a);
@@ -2686,10 +2726,14 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     if (ok) mma_out = false;
     tc_fence_after();
   };
-  for (int tile = (int)blockIdx.x / kTpRanks, it = 0; tile < ntiles; tile += stride, ++it) {
+  int tile = (int)blockIdx.x / kTpRanks;
+  uint64_t h = sample_hash(seed, tstep, tile * kLtRows + tid);
+  const unsigned long long st = share_steps(&steps_sh, rp, rank, kTpRanks);
+  for (int it = 0; tile < ntiles; tile += stride, ++it) {
     if (tid < kLtRows) {
       const int i = tile * kLtRows + tid;
-      rows_sh[tid] = i < batch ? (int)sample_entry(seed, tstep, st, i, rp) : -1;
+      if (it > 0) h = sample_hash(seed, tstep, i);
+      rows_sh[tid] = i < batch ? (int)sample_entry(h, st, rp) : -1;
     }
     __syncthreads();
     {
@@ -2799,7 +2843,6 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kOut; ++j) o[j] = (ok ? __uint_as_float(v[j]) : __int_as_float(0x7fc00000)) + b3[j];
       greedy_action(o, qv, L.plain);
     }
-    if (it == 0) cluster_wait();  // the start's arrival
     if (rank != 0 && warp < 4) {
 #pragma unroll
       for (int a = 0; a < 5; ++a)
