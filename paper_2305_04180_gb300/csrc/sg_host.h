@@ -55,7 +55,10 @@ struct SgRange {
 #define SG_RANGE(name) SgRange sg_range_(name)
 
 // A launch whose kernel may start while the kernel before it on the stream
-// still runs (programmatic dependent launch: it waits at pdl_wait).
+// still runs (programmatic dependent launch: it waits at pdl_wait).  What that
+// kernel writes is written during the lifetime of this one, so the read-only
+// path (__ldg, const __restrict__ pointers) is not for it: __ldcg, or the
+// asynchronous copies.
 template <typename... P, typename... A>
 cudaError_t sg_launch_pdl(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};

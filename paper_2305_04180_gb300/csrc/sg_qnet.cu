@@ -1935,9 +1935,8 @@ __device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
 }
 
 __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
-    k_td_tile(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, ImgLayout L, ReplayDev rp,
-              unsigned long long seed, const unsigned long long* __restrict__ step, int batch, float gamma, TdFrag f,
-              unsigned* __restrict__ fail) {
+    k_td_tile(const uint8_t* img, const uint8_t* img_t, ImgLayout L, ReplayDev rp, unsigned long long seed,
+              const unsigned long long* step, int batch, float gamma, TdFrag f, unsigned* fail) {
   extern __shared__ __align__(16) uint8_t smem[];
   uint8_t* sw = smem;
   bf16* X = reinterpret_cast<bf16*>(smem + L.bytes);
@@ -2353,7 +2352,7 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
     if (o == kOut) {
 #pragma unroll
       for (int i = 0; i < kOut; ++i)
-        w3[i] = __bfloat162float(reinterpret_cast<const bf16*>(u.img + u.L.w3)[i * kLdh + n]);
+        w3[i] = __bfloat162float(__ldcg(reinterpret_cast<const bf16*>(u.img + u.L.w3) + i * kLdh + n));
     }
   } else {
     at = ve < kBigB3 ? u.P.b1 + ve : u.P.b3 + (ve - kBigB3);
@@ -2487,7 +2486,7 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
     for (int e = t; e <= kBigHub; e += 256) {
       float a = 0.0f;
 #pragma unroll 4
-      for (int i = t0; i < t1; ++i) a += f.vec[(long long)i * kVecLd + e];
+      for (int i = t0; i < t1; ++i) a += __ldcg(f.vec + (long long)i * kVecLd + e);
       blk[e] = a;
     }
   }
@@ -2667,10 +2666,9 @@ __device__ __forceinline__ void lt_epilogue(uint32_t t, const float* bias, uint4
 }
 
 __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
-    k_td_tc(const uint8_t* __restrict__ img, const uint8_t* __restrict__ img_t, const uint8_t* __restrict__ timg,
-            const uint8_t* __restrict__ timg_t, ImgLayout L, ReplayDev rp, unsigned long long seed,
-            const unsigned long long* __restrict__ step, int batch, float gamma, TdFrag f,
-            unsigned* __restrict__ fail) {
+    k_td_tc(const uint8_t* img, const uint8_t* img_t, const uint8_t* timg, const uint8_t* timg_t, ImgLayout L,
+            ReplayDev rp, unsigned long long seed, const unsigned long long* step, int batch, float gamma, TdFrag f,
+            unsigned* fail) {
   extern __shared__ __align__(1024) uint8_t tsm[];
   __shared__ uint64_t bar_w1, bar_w2, bar_mma;
   __shared__ uint32_t tslot;
@@ -2746,7 +2744,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const int k = lane + 32 * c;
-          v[u][c] = e >= 0 && k < L.n_in ? __ldg(src + (long long)e * L.n_in + k) : 0.0f;
+          v[u][c] = e >= 0 && k < L.n_in ? __ldcg(src + (long long)e * L.n_in + k) : 0.0f;
         }
       }
 #pragma unroll
@@ -2781,16 +2779,16 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     if (first) {
       // the vectors of this CTA's network, behind layer 1
       for (int i = tid; i < 2 * kHid; i += kThreads)
-        b1[i] = __ldg(reinterpret_cast<const float*>(im + (i < kHid ? L.b1 : L.b2)) + (i & (kHid - 1)));
+        b1[i] = __ldcg(reinterpret_cast<const float*>(im + (i < kHid ? L.b1 : L.b2)) + (i & (kHid - 1)));
       if (rank == 0) {
 #pragma unroll
         for (int i = 0; i < kOut * kHid / kThreads; ++i) {
           const int j = tid + i * kThreads;
-          w3f[j] = __bfloat162float(reinterpret_cast<const bf16*>(im + L.w3)[(j >> 8) * kLdh + (j & (kHid - 1))]);
+          w3f[j] = __bfloat162float(__ldcg(reinterpret_cast<const bf16*>(im + L.w3) + (j >> 8) * kLdh + (j & (kHid - 1))));
         }
       }
 #pragma unroll
-      for (int j = 0; j < kOut; ++j) b3[j] = __ldg(reinterpret_cast<const float*>(im + L.b3) + j);
+      for (int j = 0; j < kOut; ++j) b3[j] = __ldcg(reinterpret_cast<const float*>(im + L.b3) + j);
     }
     if (rank == 0) {
       // X's B fragments: a core matrix is an 8 x 8 block of 16-byte rows

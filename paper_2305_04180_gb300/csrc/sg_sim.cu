@@ -221,14 +221,22 @@ __global__ void __launch_bounds__(64) k_step_motion(const __grid_constant__ DevC
 constexpr int kFinishWarps = 4;
 template <bool kDyn>
 __global__ void __launch_bounds__(32 * kFinishWarps, kDyn ? 8 : 12)
-    k_step_finish(const __grid_constant__ DevCfg c, SimPtrs p, const MotionRec* __restrict__ rec,
-                  const Discs* __restrict__ drec, float* __restrict__ obs, float* __restrict__ rew,
-                  uint8_t* __restrict__ done, float* __restrict__ term) {
+    k_step_finish(const __grid_constant__ DevCfg c, SimPtrs p, const MotionRec* rec, const Discs* drec,
+                  float* __restrict__ obs, float* __restrict__ rew, uint8_t* __restrict__ done,
+                  float* __restrict__ term) {
+  __shared__ Discs dsh[kDyn ? kFinishWarps : 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e = blockIdx.x * kFinishWarps + warp;
   pdl_wait();
-  if (e < c.n_envs)
-    finish_step<kDyn, true, true>(c, p, rec + e, kDyn ? drec + e : nullptr, lane, obs, rew, done, term);
+  if (e >= c.n_envs) return;  // warp-uniform
+  if (kDyn) {
+    constexpr int kWords = (int)(sizeof(Discs) / sizeof(float));
+    static_assert(kWords <= 32, "one word a lane");
+    if (lane < kWords)
+      reinterpret_cast<float*>(&dsh[warp])[lane] = __ldcg(reinterpret_cast<const float*>(drec + e) + lane);
+    __syncwarp();
+  }
+  finish_step<kDyn, true, true>(c, p, rec + e, kDyn ? &dsh[warp] : nullptr, lane, obs, rew, done, term);
 }
 
 // K steps of one env with uniformly random actions drawn on the device; the
