@@ -2282,8 +2282,10 @@ inline int td_update_items(int k1) { return 256 + 16 * (k1 / 16) + (kVecHub + 1 
 // sums added in CTA order through distributed shared memory (each CTA updates
 // an eighth of the item).  Items: 64 x 64 blocks of W2 and W1 (a warp 16 x 32, so
 // that a fragment serves two or four warps; the tiles' operands, contiguous, by
-// bulk copies in two stages of eight tiles), W3 and b2 of 64 units, the
-// remaining vectors.  Bound by L2 reads (each operand four times) and the
+// cp.async in two stages of eight tiles), W3 and b2 of 64 units, the
+// remaining vectors.  Nothing here can fail: other items are updated meanwhile,
+// so whether the step counts is settled before this kernel (a bulk copy's
+// bounded wait would come too late).  Bound by L2 reads (each operand four times) and the
 // latency of the chain; 16 x 16 items of one CTA read each operand 16 times,
 // 88 MB at batch 4,096 (45.6 us a step, 34.5 now with the rolled epilogues).
 constexpr int kSplit = 8, kSplitBlk = 64;
@@ -2298,14 +2300,7 @@ __device__ __forceinline__ void split_bf16(float x, float (&t)[3]) {
     x -= t[i];
   }
 }
-// A word, and two floats, of another CTA's copy of a shared array.
-__device__ __forceinline__ int ld_cluster1(const int* p, uint32_t rank) {
-  uint32_t a;
-  int v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(v) : "r"(a) : "memory");
-  return v;
-}
+// Two floats of another CTA's copy of a shared array.
 __device__ __forceinline__ float2 ld_cluster2(const float* p, uint32_t rank) {
   uint32_t a;
   float2 v;
@@ -2313,6 +2308,14 @@ __device__ __forceinline__ float2 ld_cluster2(const float* p, uint32_t rank) {
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
   return v;
 }
+
+// 16 bytes from global memory (through L2) to shared memory, asynchronously;
+// commit groups the copies issued so far, wait1 waits for all groups but the last.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
 // Operands of kGroup fragment tiles in one stage: 2 KB of A, up to 2 KB of B a tile.
 constexpr int kGroup = 8, kStageTile = 4096;
@@ -2323,8 +2326,6 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
   extern __shared__ __align__(128) uint8_t usm[];
   float* blk = reinterpret_cast<float*>(usm);
   uint8_t* stage = usm + kSplitBlk * kSplitBlk * 4;
-  __shared__ uint64_t bar[2];
-  __shared__ int bad_sh;
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
   const int g = lane >> 2, q = lane & 3;
@@ -2365,14 +2366,9 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
     for (int h = 0; h < 2; ++h)
       if (live[h]) th[h] = u.th[at + h], m[h] = u.m[at + h], v[h] = u.v[at + h];
   }
-  if (t == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    bad_sh = 0;
-  }
-  __syncthreads();
   pdl_wait();
-  const unsigned fail = __ldcg(u.fail);
+  const bool failed = __ldcg(u.fail) != 0u;
+  upd_fail(failed, run);
   // fragment tiles of this CTA, or the vectors of 128-sample tiles
   const int nt = mat || head ? ntiles : (ntiles + kLtSub - 1) / kLtSub;
   const int per = (nt + kSplit - 1) / kSplit, t0 = (int)rank * per, t1 = min(nt, t0 + per);
@@ -2384,31 +2380,27 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
     const uint8_t* gb = head ? reinterpret_cast<const uint8_t*>(f.dout)
                              : reinterpret_cast<const uint8_t*>((w2 ? f.h1 : f.x) + 4 * nb * 32);
     const long long lb = head ? kTile * kOutPad * 4 : nbk * 512;
-    const uint32_t bb = head ? (uint32_t)(kTile * kOutPad * 4) : (uint32_t)bblk * 512u;
+    const int bb = head ? kTile * kOutPad * 4 : bblk * 512;
     const int ngroups = (t1 - t0 + kGroup - 1) / kGroup;
-    // warp 0: the copies of group i into its stage, a lane per copy
+    // group i into its stage: a 16-byte word per thread and tile, of A by the
+    // first four warps, of B by the others
+    const bool mine = t < 128 || (t - 128) * 16 < bb;
     auto issue = [&](int i) {
       const int g0 = t0 + i * kGroup, gn = min(kGroup, t1 - g0);
-      if (lane == 0) mbar_expect_tx(&bar[i & 1], (uint32_t)gn * (2048u + bb));
-      __syncwarp();
-      const int tile = lane >> 1;
-      if (tile < gn) {
-        uint8_t* dst = stage + ((i & 1) * kGroup + tile) * kStageTile;
-        if (lane & 1)
-          bulk_g2s(dst + 2048, gb + (long long)(g0 + tile) * lb, bb, &bar[i & 1]);
-        else
-          bulk_g2s(dst, ga + (long long)(g0 + tile) * (kFragTile * 16), 2048u, &bar[i & 1]);
-      }
+      const uint8_t* src = t < 128 ? ga + (long long)g0 * (kFragTile * 16) + t * 16 : gb + g0 * lb + (t - 128) * 16;
+      const long long ld = t < 128 ? kFragTile * 16 : lb;
+      uint8_t* dst = stage + (i & 1) * kGroup * kStageTile + t * 16;
+      if (mine)
+        for (int e = 0; e < gn; ++e) cp_async16(dst + e * kStageTile, src + e * ld);
+      cp_async_commit();
     };
-    if (warp == 0) {
-      if (ngroups > 0) issue(0);
-      if (ngroups > 1) issue(1);
-    }
+    issue(0);
+    issue(1);
     const bool have0 = mat && 2 * (warp & 1) < bblk, have1 = mat && 2 * (warp & 1) + 1 < bblk;
     float acc[2][2][4] = {};
-    bool ok = true;
     for (int i = 0; i < ngroups; ++i) {
-      ok = ok && mbar_wait(&bar[i & 1], (uint32_t)(i >> 1) & 1u, kTcTries);
+      cp_async_wait1();  // group i (i + 1 stays in flight)
+      __syncthreads();
       const int gn = min(kGroup, t1 - t0 - i * kGroup);
       const uint8_t* st = stage + (i & 1) * kGroup * kStageTile;
       if (mat) {
@@ -2457,15 +2449,8 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
           for (int j = 0; j < 4; ++j) acc[0][0][j] += sm[j];
         }
       }
-      fence_async_smem();  // these reads before the stage takes another copy
-      __syncthreads();
-      if (warp == 0 && i + 2 < ngroups) issue(i + 2);
-    }
-    if (!ok) {
-      // a copy did not complete: no update of this item; one more bounded wait
-      bad_sh = 1;
-      if (t == 0)
-        for (int i = max(0, ngroups - 2); i < ngroups; ++i) mbar_wait(&bar[i & 1], (uint32_t)(i >> 1) & 1u, kTcTries);
+      __syncthreads();  // these reads before the stage takes another copy
+      issue(i + 2);
     }
     if (mat) {
 #pragma unroll
@@ -2492,10 +2477,6 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
   }
   cluster_arrive();
   cluster_wait();
-  bool bad = false;
-  if (t < kSplit) bad = ld_cluster1(&bad_sh, (uint32_t)t) != 0;
-  const bool failed = __syncthreads_or(bad) || fail != 0u;
-  upd_fail(failed, run);
   // element i (even) and i + 1 of the item
   auto total = [&](int i) {
     float2 x[kSplit];

@@ -1,7 +1,9 @@
 """Kernels launched with sg_launch_pdl overlap the kernel before them on the
 stream: what that kernel writes is not constant during their lifetime, so they
 must not read it on the read-only path, which is what __ldg asks for and const
-__restrict__ pointer arguments permit.  Read from the sources (no GPU)."""
+__restrict__ pointer arguments permit.  And an update kernel changes parameters
+from its first finished CTA on, so whether the step counts must be settled before
+it: a wait that may run out has no place there.  Read from the sources (no GPU)."""
 
 import os
 import re
@@ -51,3 +53,11 @@ def test_no_read_only_loads_of_what_the_kernel_before_writes(name):
     assert "pdl_wait();" in body
     assert not re.search(r"const\s+[\w:]+\s*\*\s*__restrict__", args), "read-only pointer argument"
     assert "__ldg(" not in body
+
+
+@pytest.mark.parametrize("name", [n for n in sorted(KERNELS) if "update" in n])
+def test_updates_hold_no_wait_that_may_run_out(name):
+    body = KERNELS[name][1]
+    assert "mbar_wait" not in body and "kTcTries" not in body
+    # the one failure word is read once, before any parameter is written
+    assert body.count("u.fail") == 1 and body.index("u.fail") < body.index("upd_adam(")
