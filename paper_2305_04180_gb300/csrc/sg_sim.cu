@@ -169,7 +169,9 @@ __global__ void __launch_bounds__(128) k_reset(const __grid_constant__ DevCfg c,
 // beam j).  No warp waits on another.  Bound by the latency of one env's
 // chain (state, map, skip values), so kE = 1 while the warps fit the GPU: 16
 // envs took 24.3 us a step when a warp always took 6 to 8, 6.4 us now; 4,096
-// envs 26 and 14 us.
+// envs 26 and 14 us.  With march steps other than 1 (kFast false) the envs of a
+// warp wait for one another's bounds-tested marches, so the line is the same: march
+// step 2, 1,024 envs: 25.5 us with one env per warp, 33.8 with two, 91 with eight.
 constexpr int kStepWarps = 8;
 
 template <bool kDyn, bool kFast, int kE>
@@ -204,7 +206,9 @@ __global__ void __launch_bounds__(32 * kStepWarps, kFast ? 3 : 4) k_step(const _
 // env-step.  65,536 envs: 68.1 -> 43.5 us a step, 16,384 envs: 30.4 -> 19.3 us.
 // The second kernel waits on the latency of the march's loads (L2): 4 warps a
 // CTA and one record a warp keep the warp slots full (8 warps or 2 records:
-// 47-49 us); 36 registers spill (57 us).
+// 47-49 us); 36 registers spill (57 us).  The general march is no exception, and its
+// 48 warps pay although it spills a word: march step 2, 65,536 envs: 166.7 us as one
+// kernel (seven envs per warp), 142.8 with 40 warps, 133.9 with 48; 8,192 envs 38.7.
 template <bool kDyn>
 __global__ void __launch_bounds__(64) k_step_motion(const __grid_constant__ DevCfg c, SimPtrs p,
                                                     const int* __restrict__ rank, const uint8_t* __restrict__ act,
@@ -219,7 +223,7 @@ __global__ void __launch_bounds__(64) k_step_motion(const __grid_constant__ DevC
 }
 
 constexpr int kFinishWarps = 4;
-template <bool kDyn>
+template <bool kDyn, bool kFast>
 __global__ void __launch_bounds__(32 * kFinishWarps, kDyn ? 8 : 12)
     k_step_finish(const __grid_constant__ DevCfg c, SimPtrs p, const MotionRec* rec, const Discs* drec,
                   float* __restrict__ obs, float* __restrict__ rew, uint8_t* __restrict__ done,
@@ -236,7 +240,7 @@ __global__ void __launch_bounds__(32 * kFinishWarps, kDyn ? 8 : 12)
       reinterpret_cast<float*>(&dsh[warp])[lane] = __ldcg(reinterpret_cast<const float*>(drec + e) + lane);
     __syncwarp();
   }
-  finish_step<kDyn, true, true>(c, p, rec + e, kDyn ? &dsh[warp] : nullptr, lane, obs, rew, done, term);
+  finish_step<kDyn, kFast, true>(c, p, rec + e, kDyn ? &dsh[warp] : nullptr, lane, obs, rew, done, term);
 }
 
 // K steps of one env with uniformly random actions drawn on the device; the
@@ -1329,7 +1333,7 @@ extern "C" int sg_sim_create(const sg_sim_config* cfg, int32_t n_maps, const uin
   alloc((void**)&s->status_dev, sizeof(uint32_t));
   alloc((void**)&s->map_order_dev, sizeof(int) * n);
   if (cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess) s->sms = 1;
-  if (dc.scan_fast && n >= kStepSplitEnvs && n <= kStepSplitMax) {
+  if (n >= kStepSplitEnvs && n <= kStepSplitMax) {
     alloc((void**)&s->rank_dev, sizeof(int) * n);
     alloc((void**)&s->step_rec, sizeof(MotionRec) * (size_t)n);
     if (cfg->n_dyn > 0) alloc((void**)&s->step_discs, sizeof(Discs) * (size_t)n);
@@ -1471,6 +1475,13 @@ extern "C" int sg_sim_reset(sg_sim_t sim, uint64_t seed, float* obs_dev, sg_stre
   return SG_OK;
 }
 
+// One env per warp (and per CTA) while that leaves SMs idle, then two, and eight
+// for the batches beyond the two-kernel step.
+template <bool kDyn, bool kFast>
+static decltype(&k_step<kDyn, kFast, 1>) step_kernel(int e) {
+  return e == 1 ? k_step<kDyn, kFast, 1> : e == 2 ? k_step<kDyn, kFast, 2> : k_step<kDyn, kFast, 8>;
+}
+
 extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev, float* rew_dev,
                            uint8_t* done_dev, float* term_obs_dev, sg_stream_t stream) {
   SG_RANGE("sg_sim_step");
@@ -1484,20 +1495,17 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
     (dyn ? k_step_motion<true> : k_step_motion<false>)<<<(n + 63) / 64, 64, 0, stream>>>(
         dc, sp, sim->rank_dev, act_dev, sim->step_rec, sim->step_discs);
     SG_CUDA(cudaGetLastError());
-    SG_CUDA(sg_launch_pdl(dyn ? k_step_finish<true> : k_step_finish<false>, (n + kFinishWarps - 1) / kFinishWarps,
-                          32 * kFinishWarps, 0, stream, dc, sp, (const MotionRec*)sim->step_rec, (const Discs*)sim->step_discs, obs_dev, rew_dev,
-                       done_dev, term_obs_dev));
+    auto finish = fast ? (dyn ? k_step_finish<true, true> : k_step_finish<false, true>)
+                       : (dyn ? k_step_finish<true, false> : k_step_finish<false, false>);
+    SG_CUDA(sg_launch_pdl(finish, (n + kFinishWarps - 1) / kFinishWarps,
+                          32 * kFinishWarps, 0, stream, dc, sp, (const MotionRec*)sim->step_rec,
+                          (const Discs*)sim->step_discs, obs_dev, rew_dev, done_dev, term_obs_dev));
     return SG_OK;
   }
-  // one env per warp (and per CTA) while that leaves SMs idle, more as the
-  // warps fill the resident slots
-  const int e = !fast ? 8 : n <= 32 * sim->sms ? 1 : n <= 64 * sim->sms ? 2 : n <= 128 * sim->sms ? 4 : 8;
+  const int e = n <= 32 * sim->sms ? 1 : n < kStepSplitEnvs ? 2 : 8;
   const int wpb = std::min(kStepWarps, std::max(1, (n / e + sim->sms - 1) / sim->sms));
-  auto kern = !fast ? (dyn ? k_step<true, false, 8> : k_step<false, false, 8>)
-              : e == 1 ? (dyn ? k_step<true, true, 1> : k_step<false, true, 1>)
-              : e == 2 ? (dyn ? k_step<true, true, 2> : k_step<false, true, 2>)
-              : e == 4 ? (dyn ? k_step<true, true, 4> : k_step<false, true, 4>)
-                       : (dyn ? k_step<true, true, 8> : k_step<false, true, 8>);
+  auto kern = fast ? (dyn ? step_kernel<true, true>(e) : step_kernel<false, true>(e))
+                   : (dyn ? step_kernel<true, false>(e) : step_kernel<false, false>(e));
   const int per = wpb * e;
   kern<<<(n + per - 1) / per, 32 * wpb, 0, stream>>>(dc, sp, sim->map_order_dev, act_dev, obs_dev, rew_dev, done_dev,
                                                       term_obs_dev);
