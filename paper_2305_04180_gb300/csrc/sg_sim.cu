@@ -1495,11 +1495,11 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
     (dyn ? k_step_motion<true> : k_step_motion<false>)<<<(n + 63) / 64, 64, 0, stream>>>(
         dc, sp, sim->rank_dev, act_dev, sim->step_rec, sim->step_discs);
     SG_CUDA(cudaGetLastError());
-    auto finish = fast ? (dyn ? k_step_finish<true, true> : k_step_finish<false, true>)
-                       : (dyn ? k_step_finish<true, false> : k_step_finish<false, false>);
-    SG_CUDA(sg_launch_pdl(finish, (n + kFinishWarps - 1) / kFinishWarps,
-                          32 * kFinishWarps, 0, stream, dc, sp, (const MotionRec*)sim->step_rec,
-                          (const Discs*)sim->step_discs, obs_dev, rew_dev, done_dev, term_obs_dev));
+    SG_CUDA(sg_launch_pdl(fast ? (dyn ? k_step_finish<true, true> : k_step_finish<false, true>)
+                               : (dyn ? k_step_finish<true, false> : k_step_finish<false, false>),
+                          (n + kFinishWarps - 1) / kFinishWarps, 32 * kFinishWarps, 0, stream, dc, sp,
+                          (const MotionRec*)sim->step_rec, (const Discs*)sim->step_discs, obs_dev, rew_dev, done_dev,
+                          term_obs_dev));
     return SG_OK;
   }
   const int e = n <= 32 * sim->sms ? 1 : n < kStepSplitEnvs ? 2 : 8;
