@@ -224,8 +224,9 @@ int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t qnet, cons
 /*
  * Launch configuration of the network-free rollout (uneven batching and the
  * autotuner).  Results never depend on it: every kernel computes the same
- * float32 step.  Until one is set, each rollout chooses by its env count and
- * K between SG_ROLLOUT_GRID and an unsliced SG_ROLLOUT_PIPE
+ * float32 step.  Until one is set, each rollout chooses by its env count, K and
+ * whether there are moving obstacles between SG_ROLLOUT_GRID and an unsliced
+ * SG_ROLLOUT_PIPE
  * (sg_sim_get_launch then gives the SG_ROLLOUT_GRID default).  kernel:
  *   SG_ROLLOUT_GRID   one warp per env, warps_per_block envs per CTA
  *                     (1, 2, 4 (default), 8, 16).

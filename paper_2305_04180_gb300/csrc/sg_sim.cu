@@ -1517,17 +1517,33 @@ extern "C" int sg_sim_step(sg_sim_t sim, const uint8_t* act_dev, float* obs_dev,
 // on it, so it follows the size of the call.  With random actions the scans of
 // a step wait for the pose chain only, so several warps per env shorten a
 // rollout while the envs alone leave warp slots empty, and the pose chain's
-// run-ahead pays at every size once K fills a chunk.  us (one warp per env /
-// pipelined): 16 envs x 1,000 steps 2,515 / 204 (15 scan warps), 304 x 512 1,656 /
-// 158 (15; 180 with 7), 456 x 512 269 with 15 and 201 with 7, 1,024 x 512 1,951 /
-// 395 (7), 4,096 x 224 1,184 / 622 (7; 627 with 3), 16,384 x 32 599 /
-// 497 (3, two envs per CTA).  Few steps of many envs stay with one warp per
-// env (4,096 x 8: 59 / 75; 65,536 x 16: 1,078 / 1,179).
-static sg_launch auto_launch(int n, int K, int sms) {
+// run-ahead pays at every size once K is long enough: the line lies where the
+// two meet, higher with more envs (whose scans fill the GPU either way).  us,
+// one warp per env / 15 scan warps, 7, 3 (two envs per CTA), 32 maps, randomised:
+//   256 envs x 32      124 / 26.4, 29.6, 36.7   512 x 32      126 / 39.2, 32.5, 39.1
+//   1,024 x 2          16.6 / 31, 18.8, 13.0    1,024 x 32    130 / 63, 48.2, 43.9
+//   2,048 x 2          17.6 / 52, 30.9, 20.0    2,048 x 4     26.1 / 56, 33.2, 22.6
+//   4,096 x 8          50 / 114, 66, 51.7       4,096 x 16    89 / 147, 92.8, 76.7
+//   6,000 x 12         102 / -, 115, 89         8,192 x 12    118 / -, 153, 117
+//   8,192 x 8          83 / 216, 123, 94        8,192 x 16    153 / 280, 174, 140
+//   16,384 x 16        273 / 544, 337, 270      16,384 x 24   403 / 636, 426, 351
+//   65,536 x 16        994 / -, 1,325, 1,057    65,536 x 24   1,466 / -, 1,657, 1,356
+// Moving obstacles lengthen the pose chain, which three scan warps then follow
+// only in short rollouts, and many envs hide it better with one warp each:
+//   1,024 x 32         183 / 123, 91.3, 88.1    1,024 x 128   593 / 320, 231, 247
+//   3,000 x 16         118 / -, 132, 126        3,000 x 32    220 / -, 218, 219
+//   4,096 x 32         253 / 412, 285, 290      4,096 x 64    489 / 645, 453, 477
+//   16,384 x 48        1,327 / -, 1,452, 1,525  16,384 x 128  3,472 / -, 3,021, 3,383
+static sg_launch auto_launch(int n, int K, int sms, bool dyn) {
   sg_launch L = {SG_ROLLOUT_GRID, 4, 1, 0, 0, 0, 0, 0};
-  if (K < std::min(kPipeChunk, n / 256)) return L;
+  const int line = n <= 4 * sms                ? 1
+                   : n <= (dyn ? 16 : 20) * sms ? (n + 511) / 512
+                   : dyn                        ? (n <= 20 * sms ? 24 : n <= 64 * sms ? 56 : 72)
+                   : n <= 64 * sms              ? 10 + n / 2048
+                                                : 18;
+  if (K < line) return L;
   L.kernel = SG_ROLLOUT_PIPE;
-  L.obs_warps = n <= 2 * sms ? 15 : n <= 32 * sms ? 7 : 3;
+  L.obs_warps = n <= 2 * sms ? 15 : n <= 4 * sms || (dyn && K >= 48) ? 7 : 3;
   L.warps_per_block = n <= 2 * sms ? 16 : 8;
   L.order = 1;
   return L;
@@ -1546,7 +1562,7 @@ extern "C" int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t
   if (policy == SG_POLICY_RANDOM) {
     if (replay) return SG_E_INVAL;  // transitions are recorded by the Q-policy rollout
     const int n = sim->dc.n_envs;
-    const sg_launch L = sim->launch_set ? sim->launch : auto_launch(n, K, sim->sms);
+    const sg_launch L = sim->launch_set ? sim->launch : auto_launch(n, K, sim->sms, sim->dc.n_dyn > 0);
     const SimPtrs sp = sg_sim_ptrs(sim);
     switch (L.kernel) {
       case SG_ROLLOUT_PIPE: {
