@@ -226,8 +226,9 @@ int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t qnet, cons
  * autotuner).  Results never depend on it: every kernel computes the same
  * float32 step.  Until one is set, each rollout chooses by its env count, K and
  * whether there are moving obstacles between SG_ROLLOUT_GRID and an unsliced
- * SG_ROLLOUT_PIPE
- * (sg_sim_get_launch then gives the SG_ROLLOUT_GRID default).  kernel:
+ * SG_ROLLOUT_PIPE; sg_sim_get_launch then gives the SG_ROLLOUT_GRID default with
+ * blocks_per_sm SG_LAUNCH_BY_SIZE, which sg_sim_set_launch takes as "none set".
+ * kernel:
  *   SG_ROLLOUT_GRID   one warp per env, warps_per_block envs per CTA
  *                     (1, 2, 4 (default), 8, 16).
  *   SG_ROLLOUT_QUEUE  a persistent grid of warps_per_block-warp CTAs
@@ -271,6 +272,7 @@ int sg_sim_rollout(sg_sim_t sim, int32_t K, int32_t policy, sg_qnet_t qnet, cons
 #define SG_ROLLOUT_QUEUE 1
 #define SG_ROLLOUT_SPLIT 2
 #define SG_ROLLOUT_PIPE 3
+#define SG_LAUNCH_BY_SIZE (-1)
 typedef struct sg_launch {
   int32_t kernel;
   int32_t warps_per_block;

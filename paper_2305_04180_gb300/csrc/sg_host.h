@@ -30,7 +30,7 @@ struct sg_sim {
   float* dyn = nullptr;        // [4 n_dyn][n] dynamic obstacles (null when n_dyn = 0)
   uint32_t* status_dev = nullptr;
   // launch configuration of the random rollout (sg_sim_set_launch)
-  sg_launch launch = {SG_ROLLOUT_GRID, 4, 1, 0, 0, 0, 0, 0};  // no slicing, default wait bound
+  sg_launch launch = {SG_ROLLOUT_GRID, 4, 1, 0, SG_LAUNCH_BY_SIZE, 0, 0, 0};
   bool launch_set = false;  // else the library chooses by the size of the call
   int persistent_blocks = 0;
   int* order_dev = nullptr;      // work list (cost-sorted env indices) or null

@@ -1702,7 +1702,8 @@ extern "C" int sg_sim_set_launch(sg_sim_t sim, const sg_launch* cfg) {
   }
   if (L.kernel == SG_ROLLOUT_QUEUE && !sim->queue_dev) SG_CUDA(cudaMalloc(&sim->queue_dev, sizeof(unsigned)));
   sim->launch = L;
-  sim->launch_set = true;
+  // the launch that sg_sim_get_launch gives while none is set
+  sim->launch_set = !(L.kernel == SG_ROLLOUT_GRID && L.blocks_per_sm == SG_LAUNCH_BY_SIZE);
   sim->persistent_blocks =
       (L.kernel == SG_ROLLOUT_QUEUE || (L.kernel == SG_ROLLOUT_PIPE && L.segment > 0)) ? bps * sms : 0;
   return SG_OK;

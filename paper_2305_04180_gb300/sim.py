@@ -144,7 +144,9 @@ class Sim:
     def set_launch(self, kernel="grid", warps_per_block=4, warps_per_env=1, obs_warps=0, blocks_per_sm=0,
                    order="index", segment=0, wait_iters=0):
         """Launch configuration of the network-free rollout (sg_sim_set_launch);
-        accepts the keys of ``launch_config()``.  segment: time slicing of the
+        accepts the keys of ``launch_config()`` (before a launch is set that is
+        "grid" with blocks_per_sm -1, which leaves the choice to the library
+        again).  segment: time slicing of the
         pipelined kernel (steps, a multiple of 32; 0 = none); wait_iters: the
         bound of its waits (0 = about a second)."""
         # order 1 is "cost" (longest first) for the work-list kernel and "map"
