@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -1785,8 +1786,10 @@ extern "C" int sg_sim_get_atlas(sg_sim_t sim, uint32_t* atlas_host, size_t* word
 // The h x w interior of a skip plane (its cell (0, 0) at dev) in row order.
 static int download_plane(const MapDesc& d, const uint8_t* dev, uint8_t* host) {
   const long long corner = skip_corner(d.clr_ld);
-  std::vector<uint8_t> plane((size_t)skip_plane_bytes(d.clr_ld, d.h));
-  SG_CUDA(cudaMemcpy(plane.data(), dev - corner, plane.size(), cudaMemcpyDeviceToHost));
+  const size_t bytes = (size_t)skip_plane_bytes(d.clr_ld, d.h);
+  const std::unique_ptr<uint8_t[]> plane(new (std::nothrow) uint8_t[bytes]);  // up to 269 MB: no exception past the C ABI
+  if (!plane) return SG_E_OOM;
+  SG_CUDA(cudaMemcpy(plane.get(), dev - corner, bytes, cudaMemcpyDeviceToHost));
   for (int y = 0; y < d.h; ++y)
     for (int x = 0; x < d.w; ++x) host[(size_t)y * d.w + x] = plane[(size_t)(corner + skip_off(x, y, d.clr_ld))];
   return SG_OK;
