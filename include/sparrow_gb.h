@@ -422,15 +422,18 @@ int sg_qnet_set_rollout_rows(sg_qnet_t q, int32_t rows);
 
 /*
  * At most rollout_ctas CTAs (one per SM) for the tcgen05 fused rollout run
- * with this network, and at most learner_ctas (rounded to whole clusters of
- * three, one at least) for the tile kernel of its TD step (0 = every SM, the
- * default; negative: SG_E_INVAL).  The ASL framework runs the
- * actor and the learner in parallel (Sec. 3.1, Alg. 1 and 2): a rollout and
- * a learning step launched on concurrent streams (or graph branches) with
- * caps that add up to the SM count each keep SMs of their own instead of
- * taking turns.  Results do not depend on the caps (the rollout's items are
- * taken from a device counter by whichever CTAs run, the learner's clusters
- * loop over its tiles).
+ * with this network, and at most learner_ctas (one per SM) for the tile kernel
+ * of its TD step (0 = every SM, the default; negative: SG_E_INVAL).  The ASL
+ * framework runs the actor and the learner in parallel (Sec. 3.1, Alg. 1 and 2):
+ * a rollout and a learning step launched on concurrent streams (or graph
+ * branches) with caps that add up to the SM count each keep SMs of their own
+ * instead of taking turns.  Below the SM count the learner therefore runs as
+ * single CTAs, wherever SMs are free, instead of thread-block clusters, which
+ * need free SMs side by side: each takes the three forwards of a tile in turn.
+ * The update that follows is small CTAs that fit beside each other on an SM.
+ * Results do not depend on the caps (the rollout's items are taken from a device
+ * counter by whichever CTAs run, the learner loops over its tiles and sums them
+ * in the same order).
  */
 int sg_qnet_set_grid_limit(sg_qnet_t q, int32_t rollout_ctas, int32_t learner_ctas);
 

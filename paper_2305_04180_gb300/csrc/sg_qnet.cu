@@ -1912,9 +1912,8 @@ __device__ __forceinline__ void st_cluster(float* p, uint32_t rank, float v) {
 // the cluster, after its cluster_arrive() at the start.  The draws and the
 // weight copies go ahead of it; against a load in every CTA, batch 256 took
 // 14.6 -> 15.3 us.
-__device__ __forceinline__ unsigned long long share_steps(unsigned long long* slot, const ReplayDev& rp, uint32_t rank,
-                                                          int ranks) {
-  const bool reader = rank == 0 && threadIdx.x == 0;
+__device__ __forceinline__ unsigned long long share_steps(unsigned long long* slot, const ReplayDev& rp, int ranks) {
+  const bool reader = cluster_rank() == 0 && threadIdx.x == 0;
   const unsigned long long st = reader ? ring_steps(rp) : 0ull;
   cluster_wait();  // every CTA of the cluster has started: remote stores from here on
   if (reader)
@@ -1934,7 +1933,11 @@ __device__ __forceinline__ void load_do(const float* p, float (&d)[kOutPad]) {
   d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w, d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
 }
 
-__global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
+// kRanks = 1 (a learner with SMs of its own): one CTA takes the three roles of a
+// tile in turn, Q(s') first; the target network's image goes over the online one
+// and back (two copies a tile).  The same values.
+template <int kRanks>
+__global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     k_td_tile(const uint8_t* img, const uint8_t* img_t, ImgLayout L, ReplayDev rp, unsigned long long seed,
               const unsigned long long* step, int batch, float gamma, TdFrag f, unsigned* fail) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -1952,8 +1955,8 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ unsigned long long steps_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = lane & 3, g = lane >> 2;
-  const uint32_t rank = cluster_rank();
-  const int ntiles = (batch + kTile - 1) / kTile, stride = (int)gridDim.x / kTpRanks;
+  uint32_t rank = kRanks == 1 ? 1u : cluster_rank();
+  const int ntiles = (batch + kTile - 1) / kTile, stride = (int)gridDim.x / kRanks;
   cluster_arrive();  // every CTA of the cluster has started before the first remote store
   if (tid == kThreads - 1) {
     mbar_init(&bar_w1, 1);
@@ -1962,7 +1965,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   pdl_wait();
   pdl_launch_dependents();
   const unsigned long long tstep = __ldcg(step);
-  if (tid == kThreads - 1) {
+  auto load_image = [&]() {
     // layer 1 starts when W1 and the vectors behind W2 are here
     const uint8_t* src = rank == 2 ? img_t : img;
     mbar_expect_tx(&bar_w1, (uint32_t)(L.w2 + L.bytes - L.w3));
@@ -1971,24 +1974,37 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     mbar_expect_tx(&bar_w2, (uint32_t)(L.w3 - L.w2));
     for (int off = L.w2; off < L.w3; off += kStageChunk)
       bulk_g2s(sw + off, src + off, (uint32_t)min(kStageChunk, L.w3 - off), &bar_w2);
-  }
+  };
+  if (tid == kThreads - 1) load_image();
   __syncthreads();
   const QW w = qw_at(sw, L);
-  bool ok = true, first = true;
-  int tile = (int)blockIdx.x / kTpRanks;
+  bool ok = true, first = true;  // first: the image's copy is still to be waited for, its phase
+  uint32_t phase = 0u;
+  int tile = (int)blockIdx.x / kRanks;
   uint64_t h = sample_hash(seed, tstep, tile * kTile + warp);
-  const unsigned long long st = share_steps(&steps_sh, rp, rank, kTpRanks);
-  for (int it = 0; tile < ntiles; tile += stride, ++it) {
+  const unsigned long long st = share_steps(&steps_sh, rp, kRanks);
+  for (int turn = 0; tile < ntiles; ++turn, tile += kRanks == 1 && turn % 3 ? 0 : stride) {
+    const int it = kRanks == 1 ? turn / 3 : turn;
+    if (kRanks == 1) {
+      rank = (uint32_t)((turn + 1) % 3);
+      if (rank != 1u && ok) {
+        fence_async_smem();  // this thread's reads of the image before the copy overwrites it
+        __syncthreads();
+        if (tid == kThreads - 1) load_image();
+        phase ^= 1u;
+        first = true;
+      }
+    }
     {
       const int i = tile * kTile + warp;
-      if (it > 0) h = sample_hash(seed, tstep, i);
+      if (turn > 0) h = sample_hash(seed, tstep, i);
       const int e = i < batch ? (int)sample_entry(h, st, rp) : -1;
       const float* src = (rank == 0 ? rp.s : rp.s2) + (long long)e * rp.obs_dim;
       for (int k = lane; k < L.ld1; k += 32)
         X[warp * L.ld1 + k] = __float2bfloat16_rn(e >= 0 && k < rp.obs_dim ? src[k] : 0.0f);
       if (lane == 0) rows[warp] = e;
     }
-    ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w1, 0u, kTcTries)));
+    ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w1, phase, kTcTries)));
     // this sample's reward, flag and action on their way during the forward
     int e = -1, act = 0;
     float rwd = 0.0f, nt = 1.0f;
@@ -2001,7 +2017,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
       }
     }
     if (ok) hidden_layer(X, L.ld1, L.k1 / 16, w.W1, L.ld1, w.b1, H1, warp, lane);
-    ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w2, 0u, kTcTries)));
+    ok = __syncthreads_and(ok && (!first || mbar_wait(&bar_w2, phase, kTcTries)));
     first = false;
     if (ok) hidden_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, warp, lane);
     __syncthreads();
@@ -2150,8 +2166,8 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     // no update this step; a copy that timed out may still be writing: one
     // more bounded wait for each before the CTA exits
     atomicOr(fail, kTdFailCopy);
-    mbar_wait(&bar_w1, 0u, kTcTries);
-    mbar_wait(&bar_w2, 0u, kTcTries);
+    mbar_wait(&bar_w1, phase, kTcTries);
+    mbar_wait(&bar_w2, phase, kTcTries);
   }
 }
 
@@ -2317,162 +2333,186 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// Operands of kGroup fragment tiles in one stage: 2 KB of A, up to 2 KB of B a tile.
-constexpr int kGroup = 8, kStageTile = 4096;
-constexpr int kSplitSmem = kSplitBlk * kSplitBlk * 4 + 2 * kGroup * kStageTile;
+// Operands of a group of fragment tiles in one stage: 2 KB of A, up to 2 KB of B a
+// tile; two stages.
+constexpr int kStageTile = 4096;
+constexpr int kBlkFloats = kSplitBlk * kSplitBlk;
+inline constexpr int split_group(int ctas) { return ctas == 1 ? 4 : 8; }
+inline constexpr int split_threads(int ctas) { return ctas == 1 ? 512 : 256; }
+inline constexpr size_t split_smem(int ctas) {
+  return (size_t)kSplit / ctas * kBlkFloats * 4 + (size_t)split_threads(ctas) / 256 * 2 * split_group(ctas) * kStageTile;
+}
 
-__global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
+// kCtas = 1 (a learner with SMs of its own): one CTA takes the kSplit parts of an
+// item with the same sums, its two halves of 256 threads (each with stages and a
+// barrier of its own) every other part.
+template <int kCtas>
+__global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(split_threads(kCtas), kCtas == 1 ? 1 : 2)
     k_td_update_split(TdUpdate u, TdFrag f, int ntiles) {
   extern __shared__ __align__(128) uint8_t usm[];
+  constexpr int kParts = kSplit / kCtas, kHalves = split_threads(kCtas) / 256, kGroup = split_group(kCtas);
+  const int half = kHalves > 1 ? (int)threadIdx.x >> 8 : 0;
   float* blk = reinterpret_cast<float*>(usm);
-  uint8_t* stage = usm + kSplitBlk * kSplitBlk * 4;
+  uint8_t* stage = usm + kParts * kBlkFloats * 4 + half * 2 * kGroup * kStageTile;
+  auto sync = [&]() {
+    if (kHalves > 1)
+      group_barrier(1 + half, 256);
+    else
+      __syncthreads();
+  };
   pdl_launch_dependents();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
+  const int t = (int)threadIdx.x & 255, warp = t >> 5, lane = t & 31;
   const int g = lane >> 2, q = lane & 3;
-  const uint32_t rank = cluster_rank();
+  const int first = kCtas == 1 ? 0 : (int)cluster_rank();
   const int nx = u.L.k1 / 16, nb1 = (nx + 3) / 4, n2 = 16, n1 = 4 * nb1;
-  const int item = (int)blockIdx.x / kSplit;
+  const int item = (int)blockIdx.x / kCtas;
   const bool w2 = item < n2, mat = item < n2 + n1, head = !mat && item < n2 + n1 + 4;
   const int mb = w2 ? item >> 2 : (item - n2) / nb1, nb = w2 ? item & 3 : (item - n2) % nb1, hb = item - n2 - n1;
-  // this thread's parameters: columns k, k + 1 of row r; output o of unit n
-  // (o = 6: its bias); vector entry ve
-  const int r = mb * kSplitBlk + 8 * (int)rank + warp, k = nb * kSplitBlk + 2 * lane;
-  const int o = t >> 3, n = hb * kSplitBlk + 8 * (int)rank + (t & 7);
+  // this thread's parameters of a part: columns k, k + 1 of row r; output o of
+  // unit n (o = 6: its bias); vector entry ve
+  const int k = nb * kSplitBlk + 2 * lane, o = t >> 3;
   constexpr int kVe = (kBigHub + 1 + kSplit - 1) / kSplit;
-  const int ve = (int)rank * kVe + t;
-  int at = 0;
+  int r = 0, n = 0, ve = 0, at = 0;
   bool live[2] = {false, false};
   float w3[kOut] = {};  // the unit's column of W3, before this launch changes it
-  if (mat) {
-    at = w2 ? u.P.w2 + r * kHid + k : u.P.w1 + r * u.L.n_in + k;
-    live[0] = w2 || k < u.L.n_in;
-    live[1] = w2 || k + 1 < u.L.n_in;
-  } else if (head) {
-    at = o < kOut ? u.P.w3 + o * kHid + n : u.P.b2 + n;
-    live[0] = o <= kOut;
-    if (o == kOut) {
-#pragma unroll
-      for (int i = 0; i < kOut; ++i)
-        w3[i] = __bfloat162float(__ldcg(reinterpret_cast<const bf16*>(u.img + u.L.w3) + i * kLdh + n));
-    }
-  } else {
-    at = ve < kBigB3 ? u.P.b1 + ve : u.P.b3 + (ve - kBigB3);
-    live[0] = t < kVe && ve < kBigHub;
-  }
-  UpdRun run = upd_begin(u);
   float th[2] = {}, m[2] = {}, v[2] = {};
-  if (u.lr != 0.0f) {
+  auto old_values = [&](int part) {
+    r = mb * kSplitBlk + 8 * part + warp, n = hb * kSplitBlk + 8 * part + (t & 7), ve = part * kVe + t;
+    if (mat) {
+      at = w2 ? u.P.w2 + r * kHid + k : u.P.w1 + r * u.L.n_in + k;
+      live[0] = w2 || k < u.L.n_in;
+      live[1] = w2 || k + 1 < u.L.n_in;
+    } else if (head) {
+      at = o < kOut ? u.P.w3 + o * kHid + n : u.P.b2 + n;
+      live[0] = o <= kOut;
+      if (o == kOut) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (live[h]) th[h] = u.th[at + h], m[h] = u.m[at + h], v[h] = u.v[at + h];
-  }
+        for (int i = 0; i < kOut; ++i)
+          w3[i] = __bfloat162float(__ldcg(reinterpret_cast<const bf16*>(u.img + u.L.w3) + i * kLdh + n));
+      }
+    } else {
+      at = ve < kBigB3 ? u.P.b1 + ve : u.P.b3 + (ve - kBigB3);
+      live[0] = t < kVe && ve < kBigHub;
+    }
+    if (u.lr != 0.0f) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (live[h]) th[h] = u.th[at + h], m[h] = u.m[at + h], v[h] = u.v[at + h];
+    }
+  };
+  UpdRun run = upd_begin(u);
+  if (kCtas > 1) old_values(first);
   pdl_wait();
   const bool failed = __ldcg(u.fail) != 0u;
   upd_fail(failed, run);
-  // fragment tiles of this CTA, or the vectors of 128-sample tiles
+  // fragment tiles of a part, or the vectors of 128-sample tiles
   const int nt = mat || head ? ntiles : (ntiles + kLtSub - 1) / kLtSub;
-  const int per = (nt + kSplit - 1) / kSplit, t0 = (int)rank * per, t1 = min(nt, t0 + per);
-  if (mat || head) {
-    // a tile's operands are contiguous: four 16-unit blocks of A; four (or the
-    // rest of) 16-column blocks of B, or the 16 rows of dO
-    const int nbk = w2 ? 16 : nx, bblk = min(4, nbk - 4 * nb);
-    const uint8_t* ga = reinterpret_cast<const uint8_t*>(head ? f.h2 + 4 * hb * 32 : (w2 ? f.z2 : f.z1) + 4 * mb * 32);
-    const uint8_t* gb = head ? reinterpret_cast<const uint8_t*>(f.dout)
-                             : reinterpret_cast<const uint8_t*>((w2 ? f.h1 : f.x) + 4 * nb * 32);
-    const long long lb = head ? kTile * kOutPad * 4 : nbk * 512;
-    const int bb = head ? kTile * kOutPad * 4 : bblk * 512;
-    const int ngroups = (t1 - t0 + kGroup - 1) / kGroup;
-    // group i into its stage: a 16-byte word per thread and tile, of A by the
-    // first four warps, of B by the others
-    const bool mine = t < 128 || (t - 128) * 16 < bb;
-    auto issue = [&](int i) {
-      const int g0 = t0 + i * kGroup, gn = min(kGroup, t1 - g0);
-      const uint8_t* src = t < 128 ? ga + (long long)g0 * (kFragTile * 16) + t * 16 : gb + g0 * lb + (t - 128) * 16;
-      const long long ld = t < 128 ? kFragTile * 16 : lb;
-      uint8_t* dst = stage + (i & 1) * kGroup * kStageTile + t * 16;
-      if (mine)
-        for (int e = 0; e < gn; ++e) cp_async16(dst + e * kStageTile, src + e * ld);
-      cp_async_commit();
-    };
-    issue(0);
-    issue(1);
-    const bool have0 = mat && 2 * (warp & 1) < bblk, have1 = mat && 2 * (warp & 1) + 1 < bblk;
-    float acc[2][2][4] = {};
-    for (int i = 0; i < ngroups; ++i) {
-      cp_async_wait1();  // group i (i + 1 stays in flight)
-      __syncthreads();
-      const int gn = min(kGroup, t1 - t0 - i * kGroup);
-      const uint8_t* st = stage + (i & 1) * kGroup * kStageTile;
-      if (mat) {
+  const int per = (nt + kSplit - 1) / kSplit;
+  for (int p = half; p < kParts; p += kHalves) {
+    float* sums = blk + p * kBlkFloats;
+    const int t0 = (first + p) * per, t1 = min(nt, t0 + per);
+    if (mat || head) {
+      // a tile's operands are contiguous: four 16-unit blocks of A; four (or the
+      // rest of) 16-column blocks of B, or the 16 rows of dO
+      const int nbk = w2 ? 16 : nx, bblk = min(4, nbk - 4 * nb);
+      const uint8_t* ga = reinterpret_cast<const uint8_t*>(head ? f.h2 + 4 * hb * 32 : (w2 ? f.z2 : f.z1) + 4 * mb * 32);
+      const uint8_t* gb = head ? reinterpret_cast<const uint8_t*>(f.dout)
+                               : reinterpret_cast<const uint8_t*>((w2 ? f.h1 : f.x) + 4 * nb * 32);
+      const long long lb = head ? kTile * kOutPad * 4 : nbk * 512;
+      const int bb = head ? kTile * kOutPad * 4 : bblk * 512;
+      const int ngroups = (t1 - t0 + kGroup - 1) / kGroup;
+      // group i into its stage: a 16-byte word per thread and tile, of A by the
+      // first four warps, of B by the others
+      const bool mine = t < 128 || (t - 128) * 16 < bb;
+      auto issue = [&](int i) {
+        const int g0 = t0 + i * kGroup, gn = min(kGroup, t1 - g0);
+        const uint8_t* src = t < 128 ? ga + (long long)g0 * (kFragTile * 16) + t * 16 : gb + g0 * lb + (t - 128) * 16;
+        const long long ld = t < 128 ? kFragTile * 16 : lb;
+        uint8_t* dst = stage + (i & 1) * kGroup * kStageTile + t * 16;
+        if (mine)
+          for (int e = 0; e < gn; ++e) cp_async16(dst + e * kStageTile, src + e * ld);
+        cp_async_commit();
+      };
+      issue(0);
+      issue(1);
+      const bool have0 = mat && 2 * (warp & 1) < bblk, have1 = mat && 2 * (warp & 1) + 1 < bblk;
+      float acc[2][2][4] = {};
+      for (int i = 0; i < ngroups; ++i) {
+        cp_async_wait1();  // group i (i + 1 stays in flight)
+        sync();
+        const int gn = min(kGroup, t1 - t0 - i * kGroup);
+        const uint8_t* st = stage + (i & 1) * kGroup * kStageTile;
+        if (mat) {
 #pragma unroll 2
-        for (int e = 0; e < gn; ++e, st += kStageTile) {
-          const uint4 a = reinterpret_cast<const uint4*>(st + (warp >> 1) * 512)[lane];
-          const uint4* pb = reinterpret_cast<const uint4*>(st + 2048 + 2 * (warp & 1) * 512) + lane;
-          const uint4 z = make_uint4(0u, 0u, 0u, 0u), b0 = have0 ? pb[0] : z, b1 = have1 ? pb[32] : z;
-          const uint32_t ar[4] = {a.x, a.y, a.z, a.w};
-          float d[2][2][4] = {};
-          mma_bf16(d[0][0], ar, b0.x, b0.y);
-          mma_bf16(d[0][1], ar, b0.z, b0.w);
-          mma_bf16(d[1][0], ar, b1.x, b1.y);
-          mma_bf16(d[1][1], ar, b1.z, b1.w);
+          for (int e = 0; e < gn; ++e, st += kStageTile) {
+            const uint4 a = reinterpret_cast<const uint4*>(st + (warp >> 1) * 512)[lane];
+            const uint4* pb = reinterpret_cast<const uint4*>(st + 2048 + 2 * (warp & 1) * 512) + lane;
+            const uint4 z = make_uint4(0u, 0u, 0u, 0u), b0 = have0 ? pb[0] : z, b1 = have1 ? pb[32] : z;
+            const uint32_t ar[4] = {a.x, a.y, a.z, a.w};
+            float d[2][2][4] = {};
+            mma_bf16(d[0][0], ar, b0.x, b0.y);
+            mma_bf16(d[0][1], ar, b0.z, b0.w);
+            mma_bf16(d[1][0], ar, b1.x, b1.y);
+            mma_bf16(d[1][1], ar, b1.z, b1.w);
 #pragma unroll
-          for (int b = 0; b < 2; ++b)
+            for (int b = 0; b < 2; ++b)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+              for (int h = 0; h < 2; ++h)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) acc[b][h][j] += d[b][h][j];
-        }
-      } else {
-        // dW3[o][n] = sum_s dO[s][o] H2[s][n] (warps 0..3) and M[n][o], the same
-        // sum over the samples with H2[s][n] > 0, from which db2[n] = sum_o W3[o][n]
-        // M[n][o] (warps 4..7).  dO in three BF16 terms against the exact BF16 H2
-        // and 0 / 1: FP32 sums of exact products, as on the CUDA cores.
-#pragma unroll 2
-        for (int e = 0; e < gn; ++e, st += kStageTile) {
-          const uint4 a = reinterpret_cast<const uint4*>(st + (warp & 3) * 512)[lane];
-          const float* d = reinterpret_cast<const float*>(st + 2048) + 2 * q * kOutPad + g;
-          float x[4][3];
-          split_bf16(d[0], x[0]);
-          split_bf16(d[kOutPad], x[1]);
-          split_bf16(d[8 * kOutPad], x[2]);
-          split_bf16(d[9 * kOutPad], x[3]);
-          uint32_t ar[4] = {a.x, a.y, a.z, a.w};
-          if (warp >= 4) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              ar[j] = ((ar[j] & 0x7FFFu) ? 0x3F80u : 0u) | ((ar[j] & 0x7FFF0000u) ? 0x3F800000u : 0u);
+                for (int j = 0; j < 4; ++j) acc[b][h][j] += d[b][h][j];
           }
-          float sm[4] = {};
+        } else {
+          // dW3[o][n] = sum_s dO[s][o] H2[s][n] (warps 0..3) and M[n][o], the same
+          // sum over the samples with H2[s][n] > 0, from which db2[n] = sum_o W3[o][n]
+          // M[n][o] (warps 4..7).  dO in three BF16 terms against the exact BF16 H2
+          // and 0 / 1: FP32 sums of exact products, as on the CUDA cores.
+#pragma unroll 2
+          for (int e = 0; e < gn; ++e, st += kStageTile) {
+            const uint4 a = reinterpret_cast<const uint4*>(st + (warp & 3) * 512)[lane];
+            const float* d = reinterpret_cast<const float*>(st + 2048) + 2 * q * kOutPad + g;
+            float x[4][3];
+            split_bf16(d[0], x[0]);
+            split_bf16(d[kOutPad], x[1]);
+            split_bf16(d[8 * kOutPad], x[2]);
+            split_bf16(d[9 * kOutPad], x[3]);
+            uint32_t ar[4] = {a.x, a.y, a.z, a.w};
+            if (warp >= 4) {
 #pragma unroll
-          for (int c = 2; c >= 0; --c) mma_bf16(sm, ar, pack_bf16x2(x[0][c], x[1][c]), pack_bf16x2(x[2][c], x[3][c]));
+              for (int j = 0; j < 4; ++j)
+                ar[j] = ((ar[j] & 0x7FFFu) ? 0x3F80u : 0u) | ((ar[j] & 0x7FFF0000u) ? 0x3F800000u : 0u);
+            }
+            float sm[4] = {};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[0][0][j] += sm[j];
+            for (int c = 2; c >= 0; --c) mma_bf16(sm, ar, pack_bf16x2(x[0][c], x[1][c]), pack_bf16x2(x[2][c], x[3][c]));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[0][0][j] += sm[j];
+          }
         }
+        sync();  // these reads before the stage takes another copy
+        issue(i + 2);
       }
-      __syncthreads();  // these reads before the stage takes another copy
-      issue(i + 2);
-    }
-    if (mat) {
+      if (mat) {
 #pragma unroll
-      for (int b = 0; b < 2; ++b)
+        for (int b = 0; b < 2; ++b)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+          for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int j = 0; j < 2; ++j)
-            *reinterpret_cast<float2*>(blk + (16 * (warp >> 1) + g + 8 * j) * kSplitBlk + 32 * (warp & 1) + 16 * b + 8 * h + 2 * q) =
-                make_float2(acc[b][h][2 * j], acc[b][h][2 * j + 1]);
+            for (int j = 0; j < 2; ++j)
+              *reinterpret_cast<float2*>(sums + (16 * (warp >> 1) + g + 8 * j) * kSplitBlk + 32 * (warp & 1) + 16 * b + 8 * h + 2 * q) =
+                  make_float2(acc[b][h][2 * j], acc[b][h][2 * j + 1]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          *reinterpret_cast<float2*>(sums + (16 * (warp & 3) + g + 8 * j) * 16 + 8 * (warp >> 2) + 2 * q) =
+              make_float2(acc[0][0][2 * j], acc[0][0][2 * j + 1]);
+      }
     } else {
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-        *reinterpret_cast<float2*>(blk + (16 * (warp & 3) + g + 8 * j) * 16 + 8 * (warp >> 2) + 2 * q) =
-            make_float2(acc[0][0][2 * j], acc[0][0][2 * j + 1]);
-    }
-  } else {
-    for (int e = t; e <= kBigHub; e += 256) {
-      float a = 0.0f;
+      for (int e = t; e <= kBigHub; e += 256) {
+        float a = 0.0f;
 #pragma unroll 4
-      for (int i = t0; i < t1; ++i) a += __ldcg(f.vec + (long long)i * kVecLd + e);
-      blk[e] = a;
+        for (int i = t0; i < t1; ++i) a += __ldcg(f.vec + (long long)i * kVecLd + e);
+        sums[e] = a;
+      }
     }
   }
   cluster_arrive();
@@ -2481,54 +2521,62 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(256, 2)
   auto total = [&](int i) {
     float2 x[kSplit];
 #pragma unroll
-    for (int c = 0; c < kSplit; ++c) x[c] = ld_cluster2(blk + i, (uint32_t)c);
+    for (int c = 0; c < kSplit; ++c)
+      x[c] = kCtas == 1 ? *reinterpret_cast<const float2*>(blk + c * kBlkFloats + i) : ld_cluster2(blk + i, (uint32_t)c);
     float2 sum = x[0];
 #pragma unroll
     for (int c = 1; c < kSplit; ++c) sum.x += x[c].x, sum.y += x[c].y;
     if (failed) sum.x = sum.y = __int_as_float(0x7fc00000);
     return sum;
   };
-  if (mat) {
-    if (live[0]) {
-      const float2 gr = total((8 * (int)rank + warp) * kSplitBlk + 2 * lane);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (!live[h]) continue;
-        const float gh = h ? gr.y : gr.x;
-        upd_grad(u, at + h, gh);
-        if (run.adam) th[h] = upd_adam(u, run, at + h, gh, th[h], m[h], v[h]);
-        if (run.sync) u.tgt[at + h] = th[h];
-      }
-      // the padding column beside an odd last input stays zero
-      if (w2)
-        upd_images<2, 2>(u, run, r, k, th[0], th[1]);
-      else
-        upd_images<1, 2>(u, run, r, k, th[0], th[1]);
+  for (int p = half; p < kParts; p += kHalves) {
+    const int part = first + p;
+    if (kCtas == 1) {
+      old_values(part);
+      sync();  // the part's columns of W3 are read before other threads change them
     }
-  } else if (head) {
-    if (live[0]) {
-      const int e = (8 * (int)rank + (t & 7)) * 16;
-      float gr = 0.0f;
-      if (o < kOut) {
-        const float2 x = total(e + (o & ~1));
-        gr = (o & 1) ? x.y : x.x;
-      } else {
+    if (mat) {
+      if (live[0]) {
+        const float2 gr = total((8 * part + warp) * kSplitBlk + 2 * lane);
 #pragma unroll
-        for (int i = 0; i < kOut; i += 2) {
-          const float2 x = total(e + 8 + i);
-          gr += w3[i] * x.x;
-          gr += w3[i + 1] * x.y;
+        for (int h = 0; h < 2; ++h) {
+          if (!live[h]) continue;
+          const float gh = h ? gr.y : gr.x;
+          upd_grad(u, at + h, gh);
+          if (run.adam) th[h] = upd_adam(u, run, at + h, gh, th[h], m[h], v[h]);
+          if (run.sync) u.tgt[at + h] = th[h];
         }
+        // the padding column beside an odd last input stays zero
+        if (w2)
+          upd_images<2, 2>(u, run, r, k, th[0], th[1]);
+        else
+          upd_images<1, 2>(u, run, r, k, th[0], th[1]);
       }
-      upd_one(u, run, at, gr, th[0], m[0], v[0]);
+    } else if (head) {
+      if (live[0]) {
+        const int e = (8 * part + (t & 7)) * 16;
+        float gr = 0.0f;
+        if (o < kOut) {
+          const float2 x = total(e + (o & ~1));
+          gr = (o & 1) ? x.y : x.x;
+        } else {
+#pragma unroll
+          for (int i = 0; i < kOut; i += 2) {
+            const float2 x = total(e + 8 + i);
+            gr += w3[i] * x.x;
+            gr += w3[i + 1] * x.y;
+          }
+        }
+        upd_one(u, run, at, gr, th[0], m[0], v[0]);
+      }
+    } else if (t < kVe && ve <= kBigHub) {
+      const float2 x = total(ve & ~1);
+      const float gr = (ve & 1) ? x.y : x.x;
+      if (ve < kBigHub)
+        upd_one(u, run, at, gr, th[0], m[0], v[0]);
+      else if (u.loss)
+        *u.loss = gr / (float)u.batch;
     }
-  } else if (t < kVe && ve <= kBigHub) {
-    const float2 x = total(ve & ~1);
-    const float gr = (ve & 1) ? x.y : x.x;
-    if (ve < kBigHub)
-      upd_one(u, run, at, gr, th[0], m[0], v[0]);
-    else if (u.loss)
-      *u.loss = gr / (float)u.batch;
   }
   upd_end(u, failed);
   cluster_arrive();  // the others' reads of this CTA's sums are done
@@ -2646,7 +2694,9 @@ __device__ __forceinline__ void lt_epilogue(uint32_t t, const float* bias, uint4
   tmem_st_wait();
 }
 
-__global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
+// kRanks = 1: the three roles of a tile in turn, as in k_td_tile.
+template <int kRanks>
+__global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     k_td_tc(const uint8_t* img, const uint8_t* img_t, const uint8_t* timg, const uint8_t* timg_t, ImgLayout L,
             ReplayDev rp, unsigned long long seed, const unsigned long long* step, int batch, float gamma, TdFrag f,
             unsigned* fail) {
@@ -2667,11 +2717,10 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   float* next_q = reinterpret_cast<float*>(tsm + T.next);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, q = lane & 3, quarter = warp & 3, grp = warp >> 2;
-  const uint32_t rank = cluster_rank();
-  const int ntiles = (batch + kLtRows - 1) / kLtRows, stride = (int)gridDim.x / kTpRanks;
+  uint32_t rank = kRanks == 1 ? 1u : cluster_rank();
+  const int ntiles = (batch + kLtRows - 1) / kLtRows, stride = (int)gridDim.x / kRanks;
   cluster_arrive();  // every CTA of the cluster has started before the first remote store
   if (warp == 0) tmem_alloc(&tslot, 512);
-  const uint8_t* im = rank == 2 ? img_t : img;
   if (tid == kThreads - 1) {
     mbar_init(&bar_w1, 1);
     mbar_init(&bar_w2, 1);
@@ -2680,14 +2729,15 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   pdl_wait();
   pdl_launch_dependents();
   const unsigned long long tstep = __ldcg(step);
-  if (tid == kThreads - 1) {
+  auto load_image = [&]() {
     const uint8_t* src = rank == 2 ? timg_t : timg;
     mbar_expect_tx(&bar_w1, G.w2a);
     bulk_g2s(tsm + T.w1, src + G.w1, G.w2a, &bar_w1);
     mbar_expect_tx(&bar_w2, kHid * kHid * 2u + 16u * kHid * 2u);
     bulk_g2s(tsm + T.w2, src + G.w2f, kHid * kHid * 2u, &bar_w2);
     bulk_g2s(tsm + T.w3, src + G.w3, 16u * kHid * 2u, &bar_w2);
-  }
+  };
+  if (tid == kThreads - 1) load_image();
   lt_sync();
   const uint32_t tacc = tslot, tacc2 = tacc + 256u;
   const uint32_t tw = ((uint32_t)(quarter * 32) << 16) + (uint32_t)(64 * grp);  // this warp's lanes and columns
@@ -2696,7 +2746,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   const int nx = L.k1 / 16;
   float b3[kOut];
   bool ok = true, first = true, mma_out = false;
-  uint32_t phase = 0u;
+  uint32_t phase = 0u, wphase = 0u;
   // wait for the MMAs committed last, by every thread
   auto mma_wait = [&]() {
     mma_out = true;
@@ -2705,13 +2755,24 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
     if (ok) mma_out = false;
     tc_fence_after();
   };
-  int tile = (int)blockIdx.x / kTpRanks;
+  int tile = (int)blockIdx.x / kRanks;
   uint64_t h = sample_hash(seed, tstep, tile * kLtRows + tid);
-  const unsigned long long st = share_steps(&steps_sh, rp, rank, kTpRanks);
-  for (int it = 0; tile < ntiles; tile += stride, ++it) {
+  const unsigned long long st = share_steps(&steps_sh, rp, kRanks);
+  for (int turn = 0; tile < ntiles; ++turn, tile += kRanks == 1 && turn % 3 ? 0 : stride) {
+    const int it = kRanks == 1 ? turn / 3 : turn;
+    if (kRanks == 1) {
+      rank = (uint32_t)((turn + 1) % 3);
+      if (rank != 1u && ok) {
+        // only MMAs read the weights' operands, and every one is complete
+        if (tid == kThreads - 1) load_image();
+        wphase ^= 1u;
+        first = true;
+      }
+    }
+    const uint8_t* im = rank == 2 ? img_t : img;
     if (tid < kLtRows) {
       const int i = tile * kLtRows + tid;
-      if (it > 0) h = sample_hash(seed, tstep, i);
+      if (turn > 0) h = sample_hash(seed, tstep, i);
       rows_sh[tid] = i < batch ? (int)sample_entry(h, st, rp) : -1;
     }
     __syncthreads();
@@ -2749,7 +2810,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
         nt = rp.term[e] ? 0.0f : 1.0f;
       }
     }
-    if (tid == 0 && ok && (!first || mbar_wait(&bar_w1, 0u, kTcTries))) {
+    if (tid == 0 && ok && (!first || mbar_wait(&bar_w1, wphase, kTcTries))) {
       tc_fence_after();
       for (int ks = 0; ks < nx; ++ks)
         tc_mma_bf16(tacc, smem_desc(sx + (uint32_t)ks * 2u * kLtRows * 16u, kLtRows * 16u, 128),
@@ -2791,7 +2852,7 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
         lt_epilogue<0>(tacc + tw, b1 + 64 * grp, nullptr, mask1, lane);
     }
     lt_sync();
-    if (tid == 0 && ok && (!first || mbar_wait(&bar_w2, 0u, kTcTries))) {
+    if (tid == 0 && ok && (!first || mbar_wait(&bar_w2, wphase, kTcTries))) {
       tc_fence_after();
       tc_layer_ta(tacc2, tacc, sw2, kHid);
       tc_commit(&bar_mma);
@@ -2980,8 +3041,8 @@ __global__ void __cluster_dims__(kTpRanks, 1, 1) __launch_bounds__(kThreads, 1)
   if (!ok && tid == 0) {
     // no update this step; what is in flight gets one more bounded wait
     atomicOr(fail, kTdFailCopy);
-    mbar_wait(&bar_w1, 0u, kTcTries);
-    mbar_wait(&bar_w2, 0u, kTcTries);
+    mbar_wait(&bar_w1, wphase, kTcTries);
+    mbar_wait(&bar_w2, wphase, kTcTries);
     if (mma_out) mbar_wait(&bar_mma, phase ^ 1u, kTcTries);
   }
   lt_sync();
@@ -3121,9 +3182,12 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
       (rc = set_smem_attr((const void*)k_rollout_q<1, true, true>, roll_smem(widest, 16))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<2, true, false>, roll_smem(widest, 32))) ||
       (rc = set_smem_attr((const void*)k_rollout_q<2, true, true>, roll_smem(widest, 32))) ||
-      (rc = set_smem_attr((const void*)k_td_tile, grad_smem(widest))) ||
-      (rc = set_smem_attr((const void*)k_td_tc, lt_smem(80).bytes)) ||
-      (rc = set_smem_attr((const void*)k_td_update_split, kSplitSmem))) {
+      (rc = set_smem_attr((const void*)k_td_tile<1>, grad_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_td_tile<kTpRanks>, grad_smem(widest))) ||
+      (rc = set_smem_attr((const void*)k_td_tc<1>, lt_smem(80).bytes)) ||
+      (rc = set_smem_attr((const void*)k_td_tc<kTpRanks>, lt_smem(80).bytes)) ||
+      (rc = set_smem_attr((const void*)k_td_update_split<1>, split_smem(1))) ||
+      (rc = set_smem_attr((const void*)k_td_update_split<kSplit>, split_smem(kSplit)))) {
     free_qnet(q);
     return rc;
   }
@@ -3138,7 +3202,7 @@ extern "C" int sg_qnet_create(int32_t n_in, int32_t arch, int32_t max_batch, uin
   la[0].val.clusterDim.x = kTpRanks, la[0].val.clusterDim.y = 1, la[0].val.clusterDim.z = 1;
   lc.attrs = la;
   lc.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&q->td_clusters, k_td_tile, &lc) != cudaSuccess || q->td_clusters < 1) {
+  if (cudaOccupancyMaxActiveClusters(&q->td_clusters, k_td_tile<kTpRanks>, &lc) != cudaSuccess || q->td_clusters < 1) {
     cudaGetLastError();
     q->td_clusters = std::max(1, q->sms / (kTpRanks + 1));
   }
@@ -3500,24 +3564,35 @@ extern "C" int sg_td_train_step(sg_qnet_t q, sg_replay_t rp, int32_t batch, floa
   u.step = q->step, u.fail = q->td_fail, u.tick = q->td_fail + 1;
   u.lr = lr, u.every = target_every, u.loss = loss_dev, u.grad = grad_dev, u.batch = batch;
   u.P = q->PL, u.L = q->IL;
-  // a cluster per tile, evenly over the rounds
-  const int cap = q->lim_learner > 0 ? std::min(q->lim_learner, q->sms) : q->sms;
-  const int fit = std::max(1, std::min(q->td_clusters, cap / kTpRanks));
   const bool big = batch >= kLtMinBatch;
   const int rows = big ? kLtRows : kTile, ntiles = (batch + rows - 1) / rows;
-  const int rounds = (ntiles + fit - 1) / fit, grid = (ntiles + rounds - 1) / rounds * kTpRanks;
+  // a cluster per tile, or with a limit single CTAs: a cluster starts only where one
+  // GPC has that many SMs free, and what a rollout leaves free is spread over all of
+  // them.  The same for the update's clusters of eight up to three SMs a GPC.
+  // 65,536 envs x 32 steps beside 16 steps of batch 4,096, learner on 4 / 8 / 12 /
+  // 16 / 24 / 48 SMs, ms: clusters 10.9 / 7.2 / 5.4 / 5.2 / 4.4 / 4.4, CTAs for the
+  // tiles only 6.9 / 5.2 / 4.8 / 4.4 / 3.62 / 4.36, for both 6.0 / 3.9 / 3.27 / 3.36 /
+  // 3.56 / 4.41; one after the other 3.40.  Where the rollout ends early the
+  // update's clusters are faster: 19,456 envs x 8 beside 32 steps, 8 / 24 / 48 SMs: 8.7 /
+  // 2.79 / 1.77, 4.6 / 2.66 / 1.68, 5.7 / 3.78 / 2.81.
+  const bool own = q->lim_learner > 0 && q->lim_learner < q->sms, own_update = own && q->lim_learner < 24;
+  const int fit = own ? q->lim_learner : std::max(1, std::min(q->td_clusters, q->sms / kTpRanks));
+  // evenly over the rounds
+  const int rounds = (ntiles + fit - 1) / fit, grid = (ntiles + rounds - 1) / rounds * (own ? 1 : kTpRanks);
   const int frags = big ? ntiles * kLtSub : ntiles, items = td_update_items(q->IL.k1);
   const TdFrag f = td_frag(q->frag, frags, q->IL.k1);
   const uint8_t *im = q->img, *im_t = q->img_t, *tc = q->img_tc, *tc_t = q->img_tc_t;
   const unsigned long long* step = q->step;
   if (big) {
-    SG_CUDA(sg_launch_pdl(k_td_tc, grid, kThreads, lt_smem(q->IL.k1).bytes, stream, im, im_t, tc, tc_t, q->IL, rp->d,
-                          seed, step, batch, gamma, f, q->td_fail));
-    SG_CUDA(sg_launch_pdl(k_td_update_split, td_split_items(q->IL.k1) * kSplit, 256, kSplitSmem, stream, u, f, frags));
+    const int parts = own_update ? 1 : kSplit;
+    SG_CUDA(sg_launch_pdl(own ? k_td_tc<1> : k_td_tc<kTpRanks>, grid, kThreads, lt_smem(q->IL.k1).bytes, stream, im,
+                          im_t, tc, tc_t, q->IL, rp->d, seed, step, batch, gamma, f, q->td_fail));
+    SG_CUDA(sg_launch_pdl(own_update ? k_td_update_split<1> : k_td_update_split<kSplit>, td_split_items(q->IL.k1) * parts,
+                          split_threads(parts), split_smem(parts), stream, u, f, frags));
     return SG_OK;
   }
-  SG_CUDA(sg_launch_pdl(k_td_tile, grid, kThreads, grad_smem(q->IL), stream, im, im_t, q->IL, rp->d, seed, step, batch,
-                        gamma, f, q->td_fail));
+  SG_CUDA(sg_launch_pdl(own ? k_td_tile<1> : k_td_tile<kTpRanks>, grid, kThreads, grad_smem(q->IL), stream, im, im_t,
+                        q->IL, rp->d, seed, step, batch, gamma, f, q->td_fail));
   if (ntiles <= kTuSlots)
     SG_CUDA(sg_launch_pdl(k_td_update<4, true>, items, 128, 0, stream, u, f, ntiles));
   else

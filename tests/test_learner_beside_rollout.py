@@ -6,7 +6,8 @@ With lr = 0 nothing but the seed and the step counter decides a step's samples,
 so each step that ran beside the rollouts has the loss and the gradient, bit
 for bit, of a step that runs alone with the counter at one of the values it
 passed through (the ring never wraps: completed slots keep their contents).  One
-cluster takes all tiles, so that one reading of the counter covers the step."""
+cluster (a batch of one tile) or one CTA takes all tiles, so that one reading of
+the counter covers the step."""
 
 import numpy as np
 import pytest
@@ -18,8 +19,8 @@ from workloads.maps import make_map
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("batch,steps,n_roll", [(16, 400, 400), (2048, 40, 160)])
-def test_samples_come_from_one_entry_beside_rollouts(batch, steps, n_roll):
+@pytest.mark.parametrize("batch,steps,n_roll,ctas", [(16, 400, 400, 0), (40, 400, 400, 1), (2048, 40, 160, 1)])
+def test_samples_come_from_one_entry_beside_rollouts(batch, steps, n_roll, ctas):
     from paper_2305_04180_gb300 import QNet, Replay, Sim
 
     n, K, first = 16, 1, 3
@@ -28,7 +29,7 @@ def test_samples_come_from_one_entry_beside_rollouts(batch, steps, n_roll):
     actor = QNet(sim.obs_dim, 16, seed=1)
     q = QNet(sim.obs_dim, batch, seed=2)
     q.set_params(3.0 * q.get_params("online"), "target")
-    q.set_grid_limit(learner=3)
+    q.set_grid_limit(learner=ctas)
     rp = Replay(first + n_roll * K + 1, n, sim.obs_dim, reserve=1)
     eps = torch.full((n,), 0.5, device="cuda")
     for _ in range(first):
