@@ -1478,7 +1478,7 @@ __device__ __forceinline__ uint64_t sample_hash(unsigned long long seed, unsigne
 // rollout running concurrently (which writes the next slots) is never read.
 // With j = h mod (V n_envs): slot = (steps - 1 - j / n_envs) mod slots,
 // env = j mod n_envs.  Whoever reads parts of one sample uses one value of st
-// (share_steps): the counter may change between two loads.
+// (offer_steps): the counter may change between two loads.
 __device__ __forceinline__ long long sample_entry(uint64_t h, unsigned long long st, const ReplayDev& rp) {
   const unsigned long long usable = (unsigned long long)(rp.slots - rp.reserve);
   const unsigned long long V = st < usable ? st : usable;
@@ -1906,25 +1906,27 @@ __device__ __forceinline__ void st_cluster(float* p, uint32_t rank, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
 }
 
-// One reading of the ring's step counter for a learner's cluster, into every
-// CTA's slot: the CTAs gather s and s' of the same samples, and a rollout on
-// another stream may advance the counter between two loads.  Every thread of
-// the cluster, after its cluster_arrive() at the start.  The draws and the
-// weight copies go ahead of it; against a load in every CTA, batch 256 took
-// 14.6 -> 15.3 us.
-__device__ __forceinline__ unsigned long long share_steps(unsigned long long* slot, const ReplayDev& rp, int ranks) {
-  const bool reader = cluster_rank() == 0 && threadIdx.x == 0;
-  const unsigned long long st = reader ? ring_steps(rp) : 0ull;
-  cluster_wait();  // every CTA of the cluster has started: remote stores from here on
-  if (reader)
-    for (int r = 0; r < ranks; ++r) {
-      uint32_t a;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(slot)), "r"(r));
-      asm volatile("st.shared::cluster.u64 [%0], %1;\n" ::"r"(a), "l"(st) : "memory");
-    }
-  cluster_arrive();
-  cluster_wait();
-  return *slot;
+// The ring's step counter for a learner's cluster.  Its CTAs gather s and s' of
+// the same samples, and a rollout on another stream may advance the counter
+// between two loads, so they agree on the first CTA's reading.  A cluster barrier
+// before the gather costs 0.6 us of a step (batch 256: 15.8 -> 16.4, its fences);
+// instead each CTA goes on with its own reading (own[0], by one thread), one warp of
+// the first CTA sends the others its value while they are at the first tile's
+// head (to own[1], counted on their barrier bar), and a CTA that has read another
+// one repeats that tile: 15.7 us, 19.1 when it has to.
+constexpr int kOfferWarp = 8;
+__device__ __forceinline__ void offer_steps(unsigned long long* own, uint64_t* bar, int ranks) {
+  cluster_wait();  // every CTA of the cluster has started, its barrier is initialised
+  const int r = threadIdx.x & 31;
+  if (r > 0 && r < ranks) {
+    uint32_t a, b;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(own + 1)), "r"(r));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(b) : "r"(smem_u32(bar)), "r"(r));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];\n" ::"r"(a),
+                 "l"(own[0]), "r"(b)
+                 : "memory");
+  }
+  __syncwarp();
 }
 
 // dL/d(head outputs) of a sample, every thread the same (two 16-byte reads).
@@ -1952,19 +1954,24 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ float next_q[2][2][kTile * kOutPad];  // rank 0: head outputs of s' by tile parity and network
   __shared__ int rows[kTile];
   __shared__ float hub[kTile];
-  __shared__ unsigned long long steps_sh;
+  __shared__ uint64_t bar_steps;
+  __shared__ unsigned long long steps_sh[2];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = lane & 3, g = lane >> 2;
   uint32_t rank = kRanks == 1 ? 1u : cluster_rank();
   const int ntiles = (batch + kTile - 1) / kTile, stride = (int)gridDim.x / kRanks;
-  cluster_arrive();  // every CTA of the cluster has started before the first remote store
   if (tid == kThreads - 1) {
     mbar_init(&bar_w1, 1);
     mbar_init(&bar_w2, 1);
+    mbar_init(&bar_steps, 1);
+    if (kRanks > 1 && rank != 0) mbar_expect_tx(&bar_steps, 8u);
   }
+  __syncwarp();
+  cluster_arrive();  // every CTA of the cluster has started before the first remote store
   pdl_wait();
   pdl_launch_dependents();
   const unsigned long long tstep = __ldcg(step);
+  if (tid == 0) steps_sh[0] = ring_steps(rp);
   auto load_image = [&]() {
     // layer 1 starts when W1 and the vectors behind W2 are here
     const uint8_t* src = rank == 2 ? img_t : img;
@@ -1982,7 +1989,8 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
   uint32_t phase = 0u;
   int tile = (int)blockIdx.x / kRanks;
   uint64_t h = sample_hash(seed, tstep, tile * kTile + warp);
-  const unsigned long long st = share_steps(&steps_sh, rp, kRanks);
+  unsigned long long st = steps_sh[0];
+  bool agreed = rank == 0 || kRanks == 1;  // st is the cluster's
   for (int turn = 0; tile < ntiles; ++turn, tile += kRanks == 1 && turn % 3 ? 0 : stride) {
     const int it = kRanks == 1 ? turn / 3 : turn;
     if (kRanks == 1) {
@@ -2022,7 +2030,19 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     if (ok) hidden_layer(H1, kLdh, kHid / 16, w.W2, kLdh, w.b2, H2, warp, lane);
     __syncthreads();
     if (ok && warp == 0) head_layer(H2, w, O, lane);
+    if (kRanks > 1 && turn == 0 && rank == 0 && warp == kOfferWarp) offer_steps(steps_sh, &bar_steps, kRanks);
     __syncthreads();
+    if (!agreed) {
+      ok = __syncthreads_and(ok && mbar_wait(&bar_steps, 0u, kTcTries));
+      agreed = true;
+      if (ok && st != steps_sh[1]) {
+        // the first CTA read another value: the tile again
+        st = steps_sh[1];
+        turn = -1, tile -= stride;
+        continue;
+      }
+    }
+    if (kRanks > 1 && turn == 0 && !(rank == 0 && warp == kOfferWarp)) cluster_wait();  // the start's arrival
     if (rank != 0 && tid < kTile * kOutPad)
       st_cluster(&next_q[it & 1][rank - 1][tid], 0u, ok ? O[tid] : __int_as_float(0x7fc00000));
     cluster_arrive();
@@ -2168,6 +2188,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     atomicOr(fail, kTdFailCopy);
     mbar_wait(&bar_w1, phase, kTcTries);
     mbar_wait(&bar_w2, phase, kTcTries);
+    if (kRanks > 1 && rank != 0) mbar_wait(&bar_steps, 0u, kTcTries);
   }
 }
 
@@ -2705,7 +2726,8 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ uint32_t tslot;
   __shared__ int rows_sh[kLtRows];
   __shared__ float dsum_sh[4][kOutPad];
-  __shared__ unsigned long long steps_sh;
+  __shared__ uint64_t bar_steps;
+  __shared__ unsigned long long steps_sh[2];
   const LtSmem T = lt_smem(L.k1);
   const TcImg G = tc_img(L.k1);
   uint8_t* xs = tsm + T.x;
@@ -2719,16 +2741,20 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
   const int g = lane >> 2, q = lane & 3, quarter = warp & 3, grp = warp >> 2;
   uint32_t rank = kRanks == 1 ? 1u : cluster_rank();
   const int ntiles = (batch + kLtRows - 1) / kLtRows, stride = (int)gridDim.x / kRanks;
-  cluster_arrive();  // every CTA of the cluster has started before the first remote store
-  if (warp == 0) tmem_alloc(&tslot, 512);
   if (tid == kThreads - 1) {
     mbar_init(&bar_w1, 1);
     mbar_init(&bar_w2, 1);
     mbar_init(&bar_mma, 1);
+    mbar_init(&bar_steps, 1);
+    if (kRanks > 1 && rank != 0) mbar_expect_tx(&bar_steps, 8u);
   }
+  __syncwarp();
+  cluster_arrive();  // every CTA of the cluster has started before the first remote store
+  if (warp == 0) tmem_alloc(&tslot, 512);
   pdl_wait();
   pdl_launch_dependents();
   const unsigned long long tstep = __ldcg(step);
+  if (tid == 0) steps_sh[0] = ring_steps(rp);
   auto load_image = [&]() {
     const uint8_t* src = rank == 2 ? timg_t : timg;
     mbar_expect_tx(&bar_w1, G.w2a);
@@ -2757,7 +2783,8 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
   };
   int tile = (int)blockIdx.x / kRanks;
   uint64_t h = sample_hash(seed, tstep, tile * kLtRows + tid);
-  const unsigned long long st = share_steps(&steps_sh, rp, kRanks);
+  unsigned long long st = steps_sh[0];
+  bool agreed = rank == 0 || kRanks == 1;  // st is the cluster's
   for (int turn = 0; tile < ntiles; ++turn, tile += kRanks == 1 && turn % 3 ? 0 : stride) {
     const int it = kRanks == 1 ? turn / 3 : turn;
     if (kRanks == 1) {
@@ -2870,6 +2897,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
       tc_layer_ta(tacc + 32u, tacc2, sw3, 16);
       tc_commit(&bar_mma);
     }
+    if (kRanks > 1 && turn == 0 && rank == 0 && warp == kOfferWarp) offer_steps(steps_sh, &bar_steps, kRanks);
     mma_wait();
     float qv[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
     if (warp < 4) {
@@ -2883,6 +2911,18 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kOut; ++j) o[j] = (ok ? __uint_as_float(v[j]) : __int_as_float(0x7fc00000)) + b3[j];
       greedy_action(o, qv, L.plain);
     }
+    if (!agreed) {
+      ok = __syncthreads_and(ok && mbar_wait(&bar_steps, 0u, kTcTries));
+      agreed = true;
+      if (ok && st != steps_sh[1]) {
+        // the first CTA read another value: the tile again (its head is read)
+        st = steps_sh[1];
+        lt_sync();
+        turn = -1, tile -= stride;
+        continue;
+      }
+    }
+    if (kRanks > 1 && turn == 0 && !(rank == 0 && warp == kOfferWarp)) cluster_wait();  // the start's arrival
     if (rank != 0 && warp < 4) {
 #pragma unroll
       for (int a = 0; a < 5; ++a)
@@ -3044,6 +3084,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     mbar_wait(&bar_w1, wphase, kTcTries);
     mbar_wait(&bar_w2, wphase, kTcTries);
     if (mma_out) mbar_wait(&bar_mma, phase ^ 1u, kTcTries);
+    if (kRanks > 1 && rank != 0) mbar_wait(&bar_steps, 0u, kTcTries);
   }
   lt_sync();
   if (warp == 0) tmem_free(tacc, 512);
