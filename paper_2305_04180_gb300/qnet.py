@@ -78,7 +78,7 @@ class QNet:
         check(self.L.sg_qnet_set_rollout_rows(self.handle, int(rows)), "sg_qnet_set_rollout_rows")
 
     def set_grid_limit(self, rollout: int = 0, learner: int = 0):
-        """CTA caps of the tcgen05 fused rollout and TD step run with this
+        """CTA caps of the tcgen05 fused rollout and of the TD step run with this
         network (0 = every SM): concurrent actor and learner keep SMs of
         their own."""
         check(self.L.sg_qnet_set_grid_limit(self.handle, int(rollout), int(learner)), "sg_qnet_set_grid_limit")
