@@ -2038,6 +2038,8 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
       if (ok && st != steps_sh[1]) {
         // the first CTA read another value: the tile again
         st = steps_sh[1];
+        if (tid == 0) ring_steps(rp);  // acquire: what the gather above left in L1 may be older than st
+        __syncthreads();
         turn = -1, tile -= stride;
         continue;
       }
@@ -2916,6 +2918,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
       if (ok && st != steps_sh[1]) {
         // the first CTA read another value: the tile again (its head is read)
         st = steps_sh[1];
+        if (tid == 0) ring_steps(rp);  // acquire, as in k_td_tile
         lt_sync();
         turn = -1, tile -= stride;
         continue;

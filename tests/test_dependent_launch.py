@@ -61,3 +61,12 @@ def test_updates_hold_no_wait_that_may_run_out(name):
     assert "mbar_wait" not in body and "kTcTries" not in body
     # the one failure word is read once, before any parameter is written
     assert body.count("u.fail") == 1 and body.index("u.fail") < body.index("upd_adam(")
+
+
+@pytest.mark.parametrize("name", ["k_td_tile", "k_td_tc"])
+def test_a_repeated_tile_is_gathered_behind_an_acquire(name):
+    """A CTA that repeats its first tile with a later step counter has read rows
+    that lie beside the new ones: its L1 must not answer for those."""
+    body = KERNELS[name][1]
+    assert len(re.findall(r"st = steps_sh\[1\];", body)) == 1
+    assert re.search(r"st = steps_sh\[1\];\s*if \(tid == 0\) ring_steps\(rp\);\s*(__syncthreads|lt_sync)\(\);", body)
