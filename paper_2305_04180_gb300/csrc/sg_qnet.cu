@@ -2625,7 +2625,7 @@ __global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(split_threads(kC
 // Bound by the latency of its chain (gather, three layers, dO, dH1, about 18 K
 // cycles).  In place of the learner whose jobs streamed W2 through two 32 KB
 // buffers, ran a forward for each of two roles a tile and wrote a 330 KB
-// gradient row per tile: batch 4,096 76 -> 33.7 us.
+// gradient row per tile: batch 4,096 76 -> 32.3 us.
 // Below this batch the 16-sample learner, whose CTAs spread over more SMs: 24.3
 // against 27.2 us at batch 1,024 (35.8 against 31.3 at 2,000, where the line
 // stays so that the batches keep their summation order).
@@ -2758,8 +2758,9 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
   if (tid == 0) steps_sh[0] = ring_steps(rp);
   auto load_image = [&]() {
     const uint8_t* src = rank == 2 ? timg_t : timg;
-    mbar_expect_tx(&bar_w1, G.w2a);
+    mbar_expect_tx(&bar_w1, G.w2a + 2u * kHid * 4u);
     bulk_g2s(tsm + T.w1, src + G.w1, G.w2a, &bar_w1);
+    bulk_g2s(b1, (rank == 2 ? img_t : img) + L.b1, 2u * kHid * 4u, &bar_w1);  // b1 and b2
     mbar_expect_tx(&bar_w2, kHid * kHid * 2u + 16u * kHid * 2u);
     bulk_g2s(tsm + T.w2, src + G.w2f, kHid * kHid * 2u, &bar_w2);
     bulk_g2s(tsm + T.w3, src + G.w3, 16u * kHid * 2u, &bar_w2);
@@ -2791,7 +2792,9 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     if (kRanks == 1) {
       rank = (uint32_t)((turn + 1) % 3);
       if (rank != 1u && ok) {
-        // only MMAs read the weights' operands, and every one is complete
+        // every MMA that read the weights is complete
+        fence_async_smem();  // this thread's reads of the biases before the copy overwrites them
+        __syncthreads();
         if (tid == kThreads - 1) load_image();
         wphase ^= 1u;
         first = true;
@@ -2846,20 +2849,6 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
                     ks > 0 ? 1u : 0u);
       tc_commit(&bar_mma);
     }
-    if (first) {
-      // the vectors of this CTA's network, behind layer 1
-      for (int i = tid; i < 2 * kHid; i += kThreads)
-        b1[i] = __ldcg(reinterpret_cast<const float*>(im + (i < kHid ? L.b1 : L.b2)) + (i & (kHid - 1)));
-      if (rank == 0) {
-#pragma unroll
-        for (int i = 0; i < kOut * kHid / kThreads; ++i) {
-          const int j = tid + i * kThreads;
-          w3f[j] = __bfloat162float(__ldcg(reinterpret_cast<const bf16*>(im + L.w3) + (j >> 8) * kLdh + (j & (kHid - 1))));
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kOut; ++j) b3[j] = __ldcg(reinterpret_cast<const float*>(im + L.b3) + j);
-    }
     if (rank == 0) {
       // X's B fragments: a core matrix is an 8 x 8 block of 16-byte rows
       for (int w = warp; w < kLtSub * nx; w += kThreads / 32) {
@@ -2873,6 +2862,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
     // this warp's fragment tiles: samples 32 quarter .., units 64 grp ..
     const long long fo = (long long)(tile * kLtSub + 2 * quarter) * kFragTile + 4 * grp * 32;
     uint32_t mask1[2] = {0u, 0u}, mask2[2] = {0u, 0u};
+    if (ok && first) mbar_wait(&bar_w1, wphase, kTcTries);  // complete: the biases are visible to this thread
     if (ok) {
       if (rank == 0)
         lt_epilogue<1>(tacc + tw, b1 + 64 * grp, f.h1 + fo, mask1, lane);
@@ -2884,6 +2874,19 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1)
       tc_fence_after();
       tc_layer_ta(tacc2, tacc, sw2, kHid);
       tc_commit(&bar_mma);
+    }
+    if (first) {
+      // behind layer 2 (with the biases, behind layer 1 they took 1.3 us of batch 4,096)
+      if (rank == 0) {
+        // W3 in FP32 for dZ2
+#pragma unroll
+        for (int i = 0; i < kOut * kHid / kThreads; ++i) {
+          const int j = tid + i * kThreads;
+          w3f[j] = __bfloat162float(__ldcg(reinterpret_cast<const bf16*>(im + L.w3) + (j >> 8) * kLdh + (j & (kHid - 1))));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kOut; ++j) b3[j] = __ldcg(reinterpret_cast<const float*>(im + L.b3) + j);
     }
     first = false;
     mma_wait();
